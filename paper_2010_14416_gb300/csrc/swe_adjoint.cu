@@ -39,7 +39,7 @@ struct AdjArgs {
     const V4<double>* __restrict__ U;     // state U^n, internal order
     const V4<double>* __restrict__ geoA;
     const V4<double>* __restrict__ geoB;
-    const V4<double>* __restrict__ geoR;  // 1/|L n| of the three edges (the forward's)
+    const V4<double>* __restrict__ geoR;  // lengths of the three edges
     const int4* __restrict__ topo;
     const double* __restrict__ gm2;
     V4<double>* __restrict__ lam;         // lambda (h, hu, hv, -)
@@ -57,7 +57,7 @@ struct AdjArgs {
     const int4* __restrict__ eidx;
     long long n_edges;
     // phase 2 on transposes: the interior edges (canonical orientation), their
-    // L n and 1/|L n|, and per edge the adjoints of its two cells' states
+    // unit normals and lengths, and per edge the adjoints of its two cells' states
     const int2* __restrict__ ecells;
     const double* __restrict__ eln;
     const double* __restrict__ erl;
@@ -78,78 +78,78 @@ __device__ __forceinline__ int adj_code(const AdjArgs& a, int c) {
     return c;
 }
 
-// the forward's unit normal and length of an edge, from its 1/|L n|
-__device__ __forceinline__ void unit_normal(double lx, double ly, double rl, double& n1, double& n2, double& len) {
-    const double l2 = edge_l2(lx, ly);
-    len = l2 * rl;
-    n1 = lx * rl;
-    n2 = ly * rl;
+// the outward unit normal and length of local edge j
+__device__ __forceinline__ void edge_geo(const V4<double>& gA, const V4<double>& gB, const V4<double>& gR, int j,
+                                         double& n1, double& n2, double& len) {
+    n1 = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);
+    n2 = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
+    len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
 }
 
-__device__ __forceinline__ void edge_ln(const V4<double>& gA, const V4<double>& gB, int j, double& lx, double& ly) {
-    lx = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);
-    ly = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
-}
-
-// Reverse of the semi-implicit friction update (friction_update, Eq 33-37,
-// the literal formulas) at (h, qx, qy, g m^2, Rh, Rx, Ry): for the adjoints
-// (bdh, bdqx, bdqy) of (dh, dqx, dqy), the adjoints w[0..6] of the seven
-// inputs, in the order of the dual-number seeds.
+// Reverse of the semi-implicit friction update (f64::update, Eq 33-37) at
+// (h, qx, qy, g m^2, Rh, Rx, Ry): for the adjoints (bdh, bdqx, bdqy) of
+// (dh, dqx, dqy), the adjoints w[0..6] of the seven inputs, in the order of
+// the dual-number seeds.  Reciprocals and roots as in the forward
+// (swe_f64.cuh): the FP64 pipe bounds this kernel too.
 __device__ void friction_rev(double hi, double qx, double qy, double gm2, double Rh, double Rx, double Ry, double dt,
                              double h_dry, double bdh, double bdqx, double bdqy, double w[7]) {
-    const double dh = dt * Rh, dqx0 = dt * Rx, dqy0 = dt * Ry;
-    const double qq = qx * qx + qy * qy;
-    const bool act = gt_pos(hi, h_dry) && gt_zero(gm2) && gt_zero(qq);
+    const double qq = f64::fma(qx, qx, f64::mul(qy, qy));
+    const bool act = gt_pos(hi, h_dry) && gt_zero(gm2) && gt_pos(qq, 1e-300);
 #pragma unroll
     for (int k = 0; k < 7; ++k) w[k] = 0.0;
     if (!act) {
         w[4] = bdh * dt; w[5] = bdqx * dt; w[6] = bdqy * dt;
         return;
     }
+    const double dh = dt * Rh, dqx0 = dt * Rx, dqy0 = dt * Ry;
     // forward
-    const double qn = sqrt(qq);
-    const double p = 1.0 / (hi * hi * cbrt(hi));                // h^(-7/3)
-    const double cf = gm2 * p, rh = 1.0 / hi;
-    const double al = 0.5 * dt * cf;
-    const double P = 7.0 / 6.0 * dh * rh - 1.0;
-    const double k = dt * cf * qn * P;
+    double rq;
+    const double qn = f64::sqrt_rsqrt(qq, rq);                  // |q|, 1/|q|
+    const double r = f64::rcbrt(hi);
+    const double rh = r * r * r;                                // 1/h
+    const double p = rh * rh * r;                               // h^(-7/3)
+    const double cf = gm2 * p;
+    const double dtc = dt * cf, al = f64::half(dtc);
+    const double P = (7.0 / 6.0) * dh * rh - 1.0;
+    const double c1 = dtc * qn, k = c1 * P;
     const double bx = dqx0 + k * qx, by = dqy0 + k * qy;
-    const double d1 = 1.0 + al * qn, d2 = d1 + al * qn;
-    const double rqd2 = 1.0 / (qn * d2), rd1 = 1.0 / d1;
+    const double rd1 = f64::rcp(f64::fma(0.5, c1, 1.0)), rd2 = f64::rcp(1.0 + c1);
+    const double rqd2 = rq * rd2;
     const double S = bx * qx + by * qy;
     const double proj = S * al * rqd2;
     // reverse: dq = (b - proj q) / d1
-    const double b_rd1 = bdqx * (bx - proj * qx) + bdqy * (by - proj * qy);
+    const double ox = (bx - proj * qx) * rd1, oy = (by - proj * qy) * rd1;
+    const double bd1 = -(bdqx * ox + bdqy * oy) * rd1;          // of d1, through 1/d1
     double b_bx = bdqx * rd1, b_by = bdqy * rd1;
-    const double b_proj = -(bdqx * qx + bdqy * qy) * rd1;
-    double b_qx = -bdqx * proj * rd1, b_qy = -bdqy * proj * rd1;
+    const double b_proj = -(b_bx * qx + b_by * qy);
+    double b_qx = -b_bx * proj, b_qy = -b_by * proj;
     // proj = S al / (|q| d2)
     const double b_S = b_proj * al * rqd2;
+    const double b_pp = b_proj * proj;
     double b_al = b_proj * S * rqd2;
-    const double b_rqd2 = b_proj * S * al;
     b_bx += b_S * qx; b_qx += b_S * bx;
     b_by += b_S * qy; b_qy += b_S * by;
-    double b_qn = -b_rqd2 * rqd2 * rqd2 * d2;
-    const double b_d2 = -b_rqd2 * rqd2 * rqd2 * qn;
-    double b_d1 = -b_rd1 * rd1 * rd1 + b_d2;
-    b_al += b_d2 * qn + b_d1 * qn;
-    b_qn += b_d2 * al + b_d1 * al;
+    double b_qn = -b_pp * rq;
+    const double b_d2 = -b_pp * rd2;
+    // d1 = 1 + al |q|, d2 = d1 + al |q|
+    const double b_aq = bd1 + b_d2 + b_d2;
+    b_al += b_aq * qn;
+    b_qn += b_aq * al;
     // b = dt R_q + k q
     const double b_k = b_bx * qx + b_by * qy;
     b_qx += b_bx * k; b_qy += b_by * k;
     // k = dt c |q| P, P = (7/6) dh / h - 1
-    double b_cf = b_k * dt * qn * P + b_al * 0.5 * dt;
-    b_qn += b_k * dt * cf * P;
-    const double b_P = b_k * dt * cf * qn;
-    const double b_dh = bdh + b_P * 7.0 / 6.0 * rh;
-    const double b_rh = b_P * 7.0 / 6.0 * dh;
-    // c = g m^2 h^(-7/3), 1/h, |q| = sqrt(qx^2 + qy^2)
-    const double b_h = -b_rh * rh * rh - b_cf * gm2 * (7.0 / 3.0) * p * rh;
-    const double b_gm2 = b_cf * p;
-    const double b_qq = b_qn / (2.0 * qn);
-    b_qx += 2.0 * b_qq * qx;
-    b_qy += 2.0 * b_qq * qy;
-    w[0] = b_h; w[1] = b_qx; w[2] = b_qy; w[3] = b_gm2;
+    const double b_kP = b_k * P;
+    const double b_cf = dt * (b_kP * qn + f64::half(b_al));
+    b_qn += b_kP * dtc;
+    const double b_P = b_k * c1 * (7.0 / 6.0);
+    const double b_dh = bdh + b_P * rh;
+    // c = g m^2 h^(-7/3), 1/h, |q|
+    const double b_h = -rh * (b_P * dh * rh + (7.0 / 3.0) * b_cf * cf);
+    const double b_qq = b_qn * rq;
+    b_qx += b_qq * qx;
+    b_qy += b_qq * qy;
+    w[0] = b_h; w[1] = b_qx; w[2] = b_qy; w[3] = b_cf * p;
     w[4] = b_dh * dt; w[5] = b_bx * dt; w[6] = b_by * dt;
 }
 
@@ -170,24 +170,22 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
     double ui, vi;
     cell_velocity<double>(hi, own.y, own.z, h_dry, ui, vi);
     // the forward's explicit right-hand side R_i
-    double f0 = 0.0, f1 = 0.0, f2 = 0.0, sx = 0.0, sy = 0.0;
+    const double g2 = f64::mul(0.5, g);
+    const f64::Side own_side{hi, ui, vi, zi};
+    double m = 0.0, x = 0.0, y = 0.0;
     int4 ei = make_int4(-1, -1, -1, 0);
     if constexpr (EDGES) ei = a.eidx[i];
     for (int j = 0; j < 3; ++j) {
-        double lx, ly, n1, n2, len;
-        edge_ln(gA, gB, j, lx, ly);
-        unit_normal(lx, ly, j == 0 ? gR.x : (j == 1 ? gR.y : gR.z), n1, n2, len);
-        double F0, F1, F2;
+        double n1, n2, len;
+        edge_geo(gA, gB, gR, j, n1, n2, len);
+        double tm = 0.0, tx, ty;
         const int c = code[j];
         if (c >= 0) {
             const V4<double> o = a.U[c & kNbrMask];
-            double src;
+            const bool flip = (c & kFlipBit) != 0;
             if constexpr (EDGES) {
-                if (!(hi > h_dry) && !(o.x > h_dry)) {
-                    const double zs = tmax(zi, o.w);
-                    const double hsi = tmax(0.0, hi + zi - zs);
-                    F0 = 0.0; F1 = 0.0; F2 = 0.0;
-                    src = 0.5 * g * (hsi * hsi - hi * hi);
+                if (!gt_pos(hi, h_dry) && !gt_pos(o.x, h_dry)) {
+                    f64::dry_edge(hi, zi, o.w, n1, n2, len, g2, tx, ty);
                 } else {
                     int e = j == 0 ? ei.x : (j == 1 ? ei.y : ei.z);
                     if (a.debug && !(e >= 0 && e < a.n_edges)) {
@@ -195,38 +193,37 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
                         e = 0;
                     }
                     const V4<double> fl = a.eflux[e];
-                    if (c & kFlipBit) {
-                        F0 = -fl.x; F1 = -fl.y; F2 = -fl.z;
-                        src = a.esrc[e];
-                    } else {
-                        F0 = fl.x; F1 = fl.y; F2 = fl.z;
-                        src = fl.w;
-                    }
+                    tm = flip ? -fl.x : fl.x;
+                    tx = flip ? -fl.w : fl.y;
+                    ty = flip ? -a.esrc[e] : fl.z;
                 }
             } else {
-                edge_interior<double>(hi, ui, vi, zi, o.x, o.y, o.z, o.w, n1, n2, (c & kFlipBit) != 0, g, h_dry, F0,
-                                      F1, F2, src, a.hll != 0);
+                f64::Side other{o.x, 0.0, 0.0, o.w};
+                f64::velocity(o.x, o.y, o.z, h_dry, other.u, other.v);
+                f64::EdgeTerms t;
+                f64::edge(flip ? other : own_side, flip ? own_side : other, flip ? -n1 : n1, flip ? -n2 : n2, len, g2,
+                          h_dry, a.hll != 0, t);
+                tm = flip ? -t.m : t.m;
+                tx = flip ? -t.xR : t.xL;
+                ty = flip ? -t.yR : t.yL;
             }
-            sx += src * lx;
-            sy += src * ly;
         } else {
             const int grp = -1 - c;
-            edge_boundary<double>(a.bc.kind[grp], a.bc.value[grp], hi, ui, vi, zi, n1, n2, g, h_dry, F0, F1, F2,
-                                  a.hll != 0);
+            f64::boundary(a.bc.kind[grp], a.bc.value[grp], own_side, n1, n2, len, g2, h_dry, a.hll != 0, tm, tx, ty);
         }
-        f0 += len * F0;
-        f1 += len * F1;
-        f2 += len * F2;
+        m = f64::add(m, tm);
+        x = f64::add(x, tx);
+        y = f64::add(y, ty);
     }
     const double ia = gB.z;
-    const double Rh = -f0 * ia, Rx = (sx - f1) * ia, Ry = (sy - f2) * ia;
+    const double Rh = -m * ia, Rx = -x * ia, Ry = -y * ia;
     const V4<double> L = a.lam[i];
     double lh = L.x, lx_ = L.y, ly_ = L.z;
     double w[7];
     if constexpr (TRANSPOSE) {
         // the forward's clamps (h < 0 zeroes the cell, h <= h_dry zeroes momentum) on
         // the new depth, then the friction update's transpose
-        const double hn = hi + a.dt * Rh;
+        const double hn = f64::add(hi, -f64::mul(m, f64::mul(a.dt, ia)));   // f64::update
         if (hn < 0.0) { lh = 0.0; lx_ = 0.0; ly_ = 0.0; }
         else if (hn <= h_dry) { lx_ = 0.0; ly_ = 0.0; }
         friction_rev(hi, own.y, own.z, a.gm2[i], Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
@@ -272,9 +269,9 @@ __global__ void __launch_bounds__(128) adj_phase2_kernel(const AdjArgs a) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
     for (int j = 0; j < 3; ++j) {
-        double lx, ly, n1, n2, len;
-        edge_ln(gA, gB, j, lx, ly);
-        unit_normal(lx, ly, j == 0 ? gR.x : (j == 1 ? gR.y : gR.z), n1, n2, len);
+        double n1, n2, len;
+        edge_geo(gA, gB, gR, j, n1, n2, len);
+        const double lx = len * n1, ly = len * n2;
         const int c = code[j];
         D4 F0, F1, F2;
         if (c >= 0) {
@@ -327,193 +324,236 @@ __global__ void __launch_bounds__(128) adj_phase2_kernel(const AdjArgs a) {
 // d(nu_L . E_L + nu_R . E_R) / d(h, hu, hv, z) of both cells.  One forward
 // evaluation of the edge and one reverse sweep through it give both, where
 // the dual-number kernels evaluate the edge from each side on four-component
-// duals.  The forward is recomputed here with the literal formulas of
-// Eq 12-30 (the ones the dual-number kernels differentiate) and every branch
-// is taken as the forward takes it; the derivative of a max at a tie is that
-// of the operand the forward returns.
+// duals.  The forward is recomputed here with the arithmetic of swe_f64.cuh,
+// whose reciprocals and inverse roots the reverse uses again (no division),
+// and every branch is taken as the forward takes it; the derivative of a max
+// at a tie is that of the operand the forward returns.
 
-// Reverse of riemann_hllc (Eq 17-26) at (hL, unL, utL, hR, unR, utR): adds
+// Reverse of f64::riemann (Eq 17-26) at (hL, unL, utL, hR, unR, utR): adds
 // the adjoints of the six inputs for the flux adjoints (bG1, bG2, bG3).
-__device__ void riemann_rev(double hL, double unL, double utL, double hR, double unR, double utR, double g,
-                            double h_dry, bool hll_only, double bG1, double bG2, double bG3, double& bhL,
-                            double& bunL, double& butL, double& bhR, double& bunR, double& butR) {
+__device__ __forceinline__ void riemann_rev(double hL, double unL, double utL, double hR, double unR, double utR,
+                                            double g2, double h_dry, bool hll_only, double bG1, double bG2, double bG3,
+                                            double& bhL, double& bunL, double& butL, double& bhR, double& bunR,
+                                            double& butR) {
     const bool wetL = gt_pos(hL, h_dry), wetR = gt_pos(hR, h_dry);
     if (!wetL && !wetR) return;   // no flux on either side
+    const bool wet = wetL && wetR;
     // ---- forward values
-    const double aL = sqrt(g * hL), aR = sqrt(g * hR);
-    double SL, SR, Ss, h0 = 0.0, hs = 0.0, pL = 1.0, pR = 1.0, gL = 0.0, gR = 0.0, b = 0.0;
-    const double hsum = hL + hR, asum = aL + aR, du = unR - unL;
-    bool rare = false, shL = false, shR = false, base_pos = false;
-    if (!wetL) {
-        SL = unR - 2.0 * aR; SR = unR + aR; Ss = SL;
-    } else if (!wetR) {
-        SL = unL - aL; SR = unL + 2.0 * aL; Ss = SR;
-    } else {
-        h0 = 0.5 * hsum - 0.25 * du * hsum / asum;                              // Eq 21
-        rare = le_pos(h0, min_nonneg(hL, hR));
-        if (rare) {                                                            // Eq 22
-            const double base = 0.5 * asum + 0.25 * (unL - unR);
-            base_pos = !lt_zero(base);
-            b = base_pos ? base : 0.0;
-            hs = b * b / g;
-        } else {                                                               // Eq 23
-            gL = sqrt(g * (h0 + hL) / (2.0 * h0 * hL));
-            gR = sqrt(g * (h0 + hR) / (2.0 * h0 * hR));
-            hs = (hL * gL + hR * gR + unL - unR) / (gL + gR);
+    const double ghL = f64::mul(g2, hL), ghR = f64::mul(g2, hR);
+    const double PL0 = f64::mul(ghL, hL), PR0 = f64::mul(ghR, hR);
+    double yL, yR;                                                              // 1/a_K (0 where a_K = 0)
+    const double aL = f64::sqrt_rsqrt(f64::twice(ghL), yL), aR = f64::sqrt_rsqrt(f64::twice(ghR), yR);
+    double SL, SR;
+    double hw = 0.0, w = 0.0, asum = 0.0, hsum = 0.0, rhw = 0.0, rh0 = 0.0, rL = 0.0, rR = 0.0, gL = 0.0, gR = 0.0,
+           ygL = 0.0, ygR = 0.0, rDg = 0.0, hs = 0.0, ycL = 0.0, ycR = 0.0;
+    bool shock = false, shL = false, shR = false;
+    if (wet) {
+        SL = f64::sub(unL, aL);
+        SR = f64::add(unR, aR);
+        asum = f64::add(aL, aR);
+        hsum = f64::add(hL, hR);
+        const double du = f64::sub(unR, unL);
+        w = f64::fma(2.0, asum, -du);
+        hw = f64::mul(hsum, w);
+        const double asum4 = f64::four_times(asum);
+        shock = gt_pos(hw, f64::mul(min_nonneg(hL, hR), asum4));                // Eq 21
+        if (shock) {                                                            // Eq 23
+            rhw = f64::rcp(hw);
+            rh0 = f64::mul(asum4, rhw);
+            rL = f64::rcp(hL);
+            rR = f64::rcp(hR);
+            gL = f64::sqrt_rsqrt(f64::mul(g2, f64::add(rh0, rL)), ygL);
+            gR = f64::sqrt_rsqrt(f64::mul(g2, f64::add(rh0, rR)), ygR);
+            rDg = f64::rcp(f64::add(gL, gR));
+            hs = f64::mul(f64::fma(hL, gL, f64::fma(hR, gR, -du)), rDg);
+            const double ghs = f64::mul(g2, hs);
+            shL = gt_pos(hs, hL);
+            shR = gt_pos(hs, hR);
+            if (shL) SL = f64::sub(unL, f64::sqrt_rsqrt(f64::mul(ghs, f64::fma(hs, rL, 1.0)), ycL));   // Eq 20
+            if (shR) SR = f64::add(unR, f64::sqrt_rsqrt(f64::mul(ghs, f64::fma(hs, rR, 1.0)), ycR));
         }
-        shL = gt_pos(hs, hL);                                                  // Eq 20
-        shR = gt_pos(hs, hR);
-        if (shL) pL = sqrt(0.5 * hs * (hs + hL)) / hL;
-        if (shR) pR = sqrt(0.5 * hs * (hs + hR)) / hR;
-        SL = unL - aL * pL;                                                    // Eq 19
-        SR = unR + aR * pR;
-        const double mL = hL * (unL - SL), mR = hR * (unR - SR);
-        Ss = (SL * mR - SR * mL) / (mR - mL);                                  // Eq 25
+    } else if (wetL) {                                                          // Eq 26
+        SL = f64::sub(unL, aL);
+        SR = f64::fma(2.0, aL, unL);
+    } else {
+        SL = f64::fma(-2.0, aR, unR);
+        SR = f64::add(unR, aR);
     }
-    const double qL = hL * unL, qR = hR * unR;
-    const double PL = qL * unL + 0.5 * g * hL * hL, PR = qR * unR + 0.5 * g * hR * hR;
-    const bool supL = ge_zero(SL), supR = !supL && le_zero(SR);              // Eq 17
-    const double D = SR - SL;
-    double G1;
-    if (supL) G1 = qL;
-    else if (supR) G1 = qR;
-    else G1 = (SR * qL - SL * qR + SR * SL * (hR - hL)) / D;
+    const double qL = f64::mul(hL, unL), qR = f64::mul(hR, unR);
+    const bool supL = ge_zero(SL), supR = !supL && le_zero(SR);               // Eq 17
     // ---- reverse
     double bSL = 0.0, bSR = 0.0, bqL = 0.0, bqR = 0.0, bPL = 0.0, bPR = 0.0;
-    if (!hll_only) {                                                           // Eq 24
-        const bool up = ge_zero(Ss);
-        bG1 += bG3 * (up ? utL : utR);
-        if (up) butL += bG3 * G1;
-        else butR += bG3 * G1;
-    } else if (supL) {
-        bqL += bG3 * utL; butL += bG3 * qL;
-    } else if (supR) {
-        bqR += bG3 * utR; butR += bG3 * qR;
-    } else {
-        const double N3 = SR * qL * utL - SL * qR * utR + SR * SL * (hR * utR - hL * utL);
-        const double bN3 = bG3 / D;
-        const double dh = hR * utR - hL * utL;
-        bSR += bN3 * (qL * utL + SL * dh) - bG3 * N3 / (D * D);
-        bSL += bN3 * (-qR * utR + SR * dh) + bG3 * N3 / (D * D);
-        bqL += bN3 * SR * utL;
-        bqR -= bN3 * SL * utR;
-        butL += bN3 * (SR * qL - SR * SL * hL);
-        butR += bN3 * (-SL * qR + SR * SL * hR);
-        bhR += bN3 * SR * SL * utR;
-        bhL -= bN3 * SR * SL * utL;
-    }
-    if (supL) {                                                                // Eq 17-18
-        bqL += bG1; bPL += bG2;
-    } else if (supR) {
-        bqR += bG1; bPR += bG2;
-    } else {
-        const double G2 = (SR * PL - SL * PR + SR * SL * (qR - qL)) / D;
-        const double bN1 = bG1 / D, bN2 = bG2 / D, bD = -(bG1 * G1 + bG2 * G2) / D;
-        bSR += bN1 * (qL + SL * (hR - hL)) + bN2 * (PL + SL * (qR - qL)) + bD;
-        bSL += bN1 * (-qR + SR * (hR - hL)) + bN2 * (-PR + SR * (qR - qL)) - bD;
-        bqL += bN1 * SR - bN2 * SR * SL;
-        bqR += -bN1 * SL + bN2 * SR * SL;
-        bPL += bN2 * SR;
-        bPR -= bN2 * SL;
-        bhR += bN1 * SR * SL;
-        bhL -= bN1 * SR * SL;
-    }
-    // P_K = q_K un_K + g h_K^2 / 2, q_K = h_K un_K
-    bqL += bPL * unL; bunL += bPL * qL; bhL += bPL * g * hL;
-    bqR += bPR * unR; bunR += bPR * qR; bhR += bPR * g * hR;
-    bhL += bqL * unL; bunL += bqL * hL;
-    bhR += bqR * unR; bunR += bqR * hR;
-    double baL = 0.0, baR = 0.0;
-    if (!wetL) {                                                               // Eq 26
-        bunR += bSL + bSR; baR += -2.0 * bSL + bSR;
-    } else if (!wetR) {
-        bunL += bSL + bSR; baL += -bSL + 2.0 * bSR;
-    } else {
-        bunL += bSL; baL -= bSL * pL;
-        bunR += bSR; baR += bSR * pR;
-        const double bpL = -bSL * aL, bpR = bSR * aR;
-        double bhs = 0.0;
-        if (shL) {   // p_L = r / h_L, r = sqrt(h* (h* + h_L) / 2)
-            const double r = pL * hL;
-            bhs += bpL * (hs + 0.5 * hL) / (2.0 * r * hL);
-            bhL += bpL * (hs / (4.0 * r * hL) - pL / hL);
+    if (supL || supR) {
+        const double q = supL ? qL : qR, ut = supL ? utL : utR;
+        double bq = bG1 + bG3 * ut;   // G3 = q ut for either flux
+        double but = bG3 * q;
+        if (supR && !hll_only && wetL && !wetR && ge_zero(SR)) {   // S* = S_R = 0: the left side's ut (Eq 24)
+            bq = bG1 + bG3 * utL;
+            but = 0.0;
+            butL += bG3 * q;
         }
-        if (shR) {
-            const double r = pR * hR;
-            bhs += bpR * (hs + 0.5 * hR) / (2.0 * r * hR);
-            bhR += bpR * (hs / (4.0 * r * hR) - pR / hR);
-        }
-        if (rare) {
-            if (base_pos) {
-                const double bb = bhs * 2.0 * b / g;
-                baL += 0.5 * bb; baR += 0.5 * bb;
-                bunL += 0.25 * bb; bunR -= 0.25 * bb;
-            }
+        if (supL) { bqL = bq; bPL = bG2; butL += but; }
+        else { bqR = bq; bPR = bG2; butR += but; }
+    } else {
+        const double r = f64::rcp(f64::sub(SR, SL));
+        const double ss = f64::mul(SR, SL);
+        const double fL = f64::fma(qL, unL, PL0), fR = f64::fma(qR, unR, PR0);
+        const double dh = f64::sub(hR, hL), dq = f64::sub(qR, qL);
+        const double G1 = f64::mul(f64::fma(ss, dh, f64::fma(-SL, qR, f64::mul(SR, qL))), r);
+        const double G2 = f64::mul(f64::fma(ss, dq, f64::fma(-SL, fR, f64::mul(SR, fL))), r);
+        if (!hll_only) {                                                        // Eq 24
+            const bool upL = wetL && (!wetR || ge_zero(G1));
+            bG1 += bG3 * (upL ? utL : utR);
+            if (upL) butL += bG3 * G1;
+            else butR += bG3 * G1;
         } else {
-            // h* = N / (g_L + g_R), N = h_L g_L + h_R g_R + un_L - un_R
-            const double Dg = gL + gR;
-            const double bN = bhs / Dg, bDg = -bhs * hs / Dg;
-            bhL += bN * gL; bhR += bN * gR;
-            bunL += bN; bunR -= bN;
-            const double bgL = bN * hL + bDg, bgR = bN * hR + bDg;
-            // g_K = sqrt(X_K), X_K = g (h0 + h_K) / (2 h0 h_K) = (g/2)(1/h_K + 1/h0)
-            const double bXL = bgL / (2.0 * gL), bXR = bgR / (2.0 * gR);
-            const double bh0 = -(bXL + bXR) * 0.5 * g / (h0 * h0);
-            bhL -= bXL * 0.5 * g / (hL * hL);
-            bhR -= bXR * 0.5 * g / (hR * hR);
-            // h0 = hsum/2 - du hsum / (4 asum)
-            const double bhsum = bh0 * (0.5 - 0.25 * du / asum);
-            const double bdu = -bh0 * 0.25 * hsum / asum;
-            const double basum = bh0 * 0.25 * du * hsum / (asum * asum);
-            bhL += bhsum; bhR += bhsum;
-            bunR += bdu; bunL -= bdu;
-            baL += basum; baR += basum;
+            const double tL = qL * utL, tR = qR * utR, dt3 = hR * utR - hL * utL;
+            const double G3 = (SR * tL - SL * tR + ss * dt3) * r;
+            const double bN3 = bG3 * r;
+            bSR += bN3 * (tL + SL * dt3 - G3);
+            bSL += bN3 * (SR * dt3 - tR + G3);
+            bqL += bN3 * SR * utL;
+            bqR -= bN3 * SL * utR;
+            butL += bN3 * (SR * qL - ss * hL);
+            butR += bN3 * (ss * hR - SL * qR);
+            bhR += bN3 * ss * utR;
+            bhL -= bN3 * ss * utL;
         }
+        // G = N / (S_R - S_L)
+        const double bN1 = bG1 * r, bN2 = bG2 * r;
+        bSR += bN1 * (qL + SL * dh - G1) + bN2 * (fL + SL * dq - G2);
+        bSL += bN1 * (SR * dh - qR + G1) + bN2 * (SR * dq - fR + G2);
+        const double b2s = bN2 * ss, b1s = bN1 * ss;
+        bqL += bN1 * SR - b2s;
+        bqR += b2s - bN1 * SL;
+        bPL = bN2 * SR;
+        bPR = -bN2 * SL;
+        bhR += b1s;
+        bhL -= b1s;
     }
-    if (aL > 0.0) bhL += baL * g / (2.0 * aL);                                 // a_K = sqrt(g h_K)
-    if (aR > 0.0) bhR += baR * g / (2.0 * aR);
+    // f_K = q_K un_K + g h_K^2 / 2, q_K = h_K un_K
+    bqL += bPL * unL; bunL += bPL * qL + bqL * hL; bhL += f64::twice(ghL) * bPL + bqL * unL;
+    bqR += bPR * unR; bunR += bPR * qR + bqR * hR; bhR += f64::twice(ghR) * bPR + bqR * unR;
+    double baL = 0.0, baR = 0.0;
+    if (wet) {
+        bunL += bSL;
+        bunR += bSR;
+        if (!shL) baL = -bSL;
+        if (!shR) baR = bSR;
+        if (shock) {
+            double bhs = 0.0;
+            if (shL) {   // c_L = sqrt(g/2 (h*^2 / h_L + h*))
+                const double t = -bSL * g2 * f64::half(ycL), x = hs * rL;
+                bhs += t * f64::fma(2.0, x, 1.0);
+                bhL -= t * x * x;
+            }
+            if (shR) {
+                const double t = bSR * g2 * f64::half(ycR), x = hs * rR;
+                bhs += t * f64::fma(2.0, x, 1.0);
+                bhR -= t * x * x;
+            }
+            // h* = N / (g_L + g_R), N = h_L g_L + h_R g_R - du
+            const double bN = bhs * rDg;
+            bhL += bN * gL; bhR += bN * gR;
+            double bdu = -bN;
+            // g_K = sqrt(g/2 (1/h0 + 1/h_K))
+            const double xL = bN * (hL - hs) * f64::half(ygL) * g2, xR = bN * (hR - hs) * f64::half(ygR) * g2;
+            bhL -= xL * rL * rL;
+            bhR -= xR * rR * rR;
+            // 1/h0 = 4 asum / (hsum w), w = 2 asum - du
+            const double b0 = xL + xR, b0r = b0 * rh0 * rhw;
+            const double bw = -b0r * hsum, bhsum = -b0r * w;
+            const double ba = f64::four_times(b0 * rhw) + f64::twice(bw);
+            bdu -= bw;
+            bhL += bhsum; bhR += bhsum;
+            baL += ba; baR += ba;
+            bunR += bdu; bunL -= bdu;
+        }
+    } else if (wetL) {                                                          // Eq 26
+        bunL += bSL + bSR;
+        baL = 2.0 * bSR - bSL;
+    } else {
+        bunR += bSL + bSR;
+        baR = bSR - 2.0 * bSL;
+    }
+    bhL += baL * g2 * yL;                                                       // a_K = sqrt(g h_K)
+    bhR += baR * g2 * yR;
 }
 
 // Reverse of one interior edge in canonical orientation (left cell L, its
 // outward unit normal (n1, n2)): for the adjoints (wF0, wF1, wF2) of the flux
-// leaving L and (sL, sR) of the two cells' bed source factors, adds the
-// adjoints of (h, hu, hv, z) of L to dL and of R to dR.
-__device__ void edge_interior_rev(const V4<double>& L, const V4<double>& R, double n1, double n2, double g,
-                                  double h_dry, bool hll_only, double wF0, double wF1, double wF2, double sL,
-                                  double sR, V4<double>& dL, V4<double>& dR) {
+// leaving L and (sL, sR) of the two cells' bed source factors, the adjoints
+// of (h, hu, hv, z) of L in dL and of R in dR.
+__device__ __forceinline__ void edge_interior_rev(const V4<double>& L, const V4<double>& R, double n1, double n2,
+                                                  double g2, double h_dry, bool hll_only, double wF0, double wF1,
+                                                  double wF2, double sL, double sR, V4<double>& dL, V4<double>& dR) {
     // forward: velocities (R9), hydrostatic reconstruction (Eq 28), rotation (Eq 12)
     const bool wL = gt_pos(L.x, h_dry), wR = gt_pos(R.x, h_dry);
-    const double rL = wL ? 1.0 / L.x : 0.0, rR = wR ? 1.0 / R.x : 0.0;
-    const double uL = L.y * rL, vL = L.z * rL, uR = R.y * rR, vR = R.z * rR;
-    const bool zleft = L.w > R.w;   // z* = max(z_L, z_R); a tie takes z_R, as the forward
-    const double zs = zleft ? L.w : R.w;
-    const double xL = L.x + L.w - zs, xR = R.x + R.w - zs;
+    const double rL = wL ? f64::rcp(L.x) : 0.0, rR = wR ? f64::rcp(R.x) : 0.0;
+    const double uL = f64::mul(L.y, rL), vL = f64::mul(L.z, rL), uR = f64::mul(R.y, rR), vR = f64::mul(R.z, rR);
+    const double zs = max_finite(L.w, R.w);   // a tie takes z_R, as the forward
+    const bool zleft = __double_as_longlong(zs) != __double_as_longlong(R.w);
+    const double xL = f64::sub(f64::add(L.x, L.w), zs), xR = f64::sub(f64::add(R.x, R.w), zs);
     const bool pL = !lt_zero(xL), pR = !lt_zero(xR);
     const double hL = pL ? xL : 0.0, hR = pR ? xR : 0.0;
-    const double unL = uL * n1 + vL * n2, utL = vL * n1 - uL * n2;
-    const double unR = uR * n1 + vR * n2, utR = vR * n1 - uR * n2;
+    const double unL = f64::fma(uL, n1, f64::mul(vL, n2)), utL = f64::fma(vL, n1, -f64::mul(uL, n2));
+    const double unR = f64::fma(uR, n1, f64::mul(vR, n2)), utR = f64::fma(vR, n1, -f64::mul(uR, n2));
     // reverse: back from (x, y) (Eq 12 inverse)
-    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2, bG3 = -wF1 * n2 + wF2 * n1;
-    double bhL = 0.0, bunL = 0.0, butL = 0.0, bhR = 0.0, bunR = 0.0, butR = 0.0;
-    riemann_rev(hL, unL, utL, hR, unR, utR, g, h_dry, hll_only, bG1, bG2, bG3, bhL, bunL, butL, bhR, bunR, butR);
+    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2, bG3 = wF2 * n1 - wF1 * n2;
     // bed source factors (Eq 30 with 1/2): src_K = (g/2)(h**_K^2 - h_K^2)
-    bhL += sL * g * hL;
-    bhR += sR * g * hR;
-    double bh0L = -sL * g * L.x, bh0R = -sR * g * R.x;
-    // rotation
-    const double buL = bunL * n1 - butL * n2, bvL = bunL * n2 + butL * n1;
-    const double buR = bunR * n1 - butR * n2, bvR = bunR * n2 + butR * n1;
-    double bqxL = 0.0, bqyL = 0.0, bqxR = 0.0, bqyR = 0.0;
-    if (wL) { bqxL = buL * rL; bqyL = bvL * rL; bh0L -= (buL * uL + bvL * vL) * rL; }
-    if (wR) { bqxR = buR * rR; bqyR = bvR * rR; bh0R -= (buR * uR + bvR * vR) * rR; }
-    // reconstruction
-    double bzL = 0.0, bzR = 0.0, bzs = 0.0;
-    if (pL) { bh0L += bhL; bzL += bhL; bzs -= bhL; }
-    if (pR) { bh0R += bhR; bzR += bhR; bzs -= bhR; }
-    if (zleft) bzL += bzs;
-    else bzR += bzs;
-    dL.x += bh0L; dL.y += bqxL; dL.z += bqyL; dL.w += bzL;
-    dR.x += bh0R; dR.y += bqxR; dR.z += bqyR; dR.w += bzR;
+    const double gsL = f64::twice(g2) * sL, gsR = f64::twice(g2) * sR;
+    double bhL = gsL * hL, bunL = 0.0, butL = 0.0, bhR = gsR * hR, bunR = 0.0, butR = 0.0;
+    riemann_rev(hL, unL, utL, hR, unR, utR, g2, h_dry, hll_only, bG1, bG2, bG3, bhL, bunL, butL, bhR, bunR, butR);
+    double bh0L = -gsL * L.x, bh0R = -gsR * R.x;
+    // rotation and velocities (r_K = 0 on a dry side)
+    dL.y = (bunL * n1 - butL * n2) * rL;
+    dL.z = (bunL * n2 + butL * n1) * rL;
+    bh0L -= dL.y * uL + dL.z * vL;
+    dR.y = (bunR * n1 - butR * n2) * rR;
+    dR.z = (bunR * n2 + butR * n1) * rR;
+    bh0R -= dR.y * uR + dR.z * vR;
+    // reconstruction: h*_K = h_K + z_K - z*, z* the higher bed
+    if (!pL) bhL = 0.0;
+    if (!pR) bhR = 0.0;
+    dL.x = bh0L + bhL;
+    dR.x = bh0R + bhR;
+    dL.w = zleft ? -bhR : bhL;
+    dR.w = zleft ? bhR : -bhL;
+}
+
+// Reverse of a boundary edge's flux (f64::boundary_flux): adds to d the
+// adjoints of cell c's (h, hu, hv, z) for the adjoints of the flux leaving it.
+__device__ __forceinline__ void boundary_rev(int kind, double value, const V4<double>& c, double n1, double n2,
+                                             double g2, double h_dry, bool hll_only, double wF0, double wF1, double wF2,
+                                             double d[4]) {
+    const bool wet = gt_pos(c.x, h_dry);
+    const double r = wet ? f64::rcp(c.x) : 0.0;
+    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2, bG3 = wF2 * n1 - wF1 * n2;
+    const double gh = f64::twice(g2) * c.x;
+    if (kind == kBcWall) {
+        d[0] += bG2 * gh;
+        return;
+    }
+    if (kind == kBcInflow) {   // G2 = g h^2 / 2 + q^2 / h
+        const double qr = value * r;
+        d[0] += bG2 * (gh - qr * qr);
+        return;
+    }
+    const double u = f64::mul(c.y, r), v = f64::mul(c.z, r);
+    const double un = f64::fma(u, n1, f64::mul(v, n2)), ut = f64::fma(v, n1, -f64::mul(u, n2));
+    const double x = f64::sub(value, c.w);
+    const double hg = kind == kBcStage ? max_zero(x) : c.x;
+    double bh = 0.0, bun = 0.0, but = 0.0, bhg = 0.0;
+    riemann_rev(c.x, un, ut, hg, un, ut, g2, h_dry, hll_only, bG1, bG2, bG3, bh, bun, but, bhg, bun, but);
+    if (kind == kBcStage) {
+        if (!lt_zero(x)) d[3] -= bhg;
+    } else {
+        bh += bhg;
+    }
+    const double bx = (bun * n1 - but * n2) * r, by = (bun * n2 + but * n1) * r;
+    d[0] += bh - (bx * u + by * v);
+    d[1] += bx;
+    d[2] += by;
 }
 
 // Phase 2, edges: each interior edge once, the adjoints of both cells' states
@@ -532,12 +572,10 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
             continue;
         }
         const V4<double> L = a.U[lr.x], R = a.U[lr.y];
-        const double lx = a.eln[2 * e], ly = a.eln[2 * e + 1];
-        double n1, n2, len;
-        unit_normal(lx, ly, a.erl[e], n1, n2, len);
+        const double n1 = a.eln[2 * e], n2 = a.eln[2 * e + 1], len = a.erl[e];
         const V4<double> nl = a.nu[lr.x], nr = a.nu[lr.y];
-        const double sL = nl.y * lx + nl.z * ly, sR = -(nr.y * lx + nr.z * ly);
-        edge_interior_rev(L, R, n1, n2, a.g, a.h_dry, a.hll != 0, len * (nr.x - nl.x), len * (nr.y - nl.y),
+        const double sL = len * (nl.y * n1 + nl.z * n2), sR = -len * (nr.y * n1 + nr.z * n2);
+        edge_interior_rev(L, R, n1, n2, 0.5 * a.g, a.h_dry, a.hll != 0, len * (nr.x - nl.x), len * (nr.y - nl.y),
                           len * (nr.z - nl.z), sL, sR, dl, dr);
         a.ed[2 * e] = dl;
         a.ed[2 * e + 1] = dr;
@@ -545,8 +583,8 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
 }
 
 // Phase 2, cells: lambda^n_j = own term + the contributions of j's interior
-// edges (in local edge order) + its boundary edges' (on duals, own state
-// only); dL/dz_j likewise.
+// edges (in local edge order) + its boundary edges' (own state only);
+// dL/dz_j likewise.
 __global__ void __launch_bounds__(128) adj_cell_kernel(const AdjArgs a) {
     const long long jc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (jc >= a.n) return;
@@ -571,26 +609,17 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const AdjArgs a) {
         }
     }
     if (any_boundary) {
-        const double g = a.g, h_dry = a.h_dry;
         const V4<double> own = a.U[jc];
         const V4<double> gA = a.geoA[jc], gB = a.geoB[jc], gR = a.geoR[jc];
         const V4<double> nuj = a.nu[jc];
-        const D4 H = D4::seed(own.x, 0), QX = D4::seed(own.y, 1), QY = D4::seed(own.z, 2), Z = D4::seed(own.w, 3);
-        D4 U, V;
-        cell_velocity<D4>(H, QX, QY, D4(h_dry), U, V);
         for (int j = 0; j < 3; ++j) {
             const int c = code[j];
             if (c >= 0) continue;
-            double lx, ly, n1, n2, len;
-            edge_ln(gA, gB, j, lx, ly);
-            unit_normal(lx, ly, j == 0 ? gR.x : (j == 1 ? gR.y : gR.z), n1, n2, len);
+            double n1, n2, len;
+            edge_geo(gA, gB, gR, j, n1, n2, len);
             const int grp = -1 - c;
-            D4 F0, F1, F2;
-            edge_boundary<D4>(a.bc.kind[grp], a.bc.value[grp], H, U, V, Z, D4(n1), D4(n2), D4(g), D4(h_dry), F0, F1,
-                              F2, a.hll != 0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                acc[k] += -len * (nuj.x * F0.d[k] + nuj.y * F1.d[k] + nuj.z * F2.d[k]);
+            boundary_rev(a.bc.kind[grp], a.bc.value[grp], own, n1, n2, 0.5 * a.g, a.h_dry, a.hll != 0, -len * nuj.x,
+                         -len * nuj.y, -len * nuj.z, acc);
         }
     }
     const V4<double> aw = a.aw[jc];

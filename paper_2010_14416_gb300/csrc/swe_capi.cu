@@ -2,8 +2,9 @@
 //
 // Device layout of one mesh (n cells, precision T, internal locality order):
 //   state[2]  V4<T>[n]   (h, hu, hv, z) ping-pong pair
-//   geoA      V4<T>[n]   L n of edges 0 and 1
-//   geoB      V4<T>[n]   L n of edge 2, 1/|Omega|, inscribed radius
+//   geoA      V4<T>[n]   L n of edges 0 and 1 (FP64: n)
+//   geoB      V4<T>[n]   L n of edge 2 (FP64: n), 1/|Omega|, inscribed radius
+//   geoR      V4<T>[n]   FP64: L of the three edges
 //   topo      int4[n]    neighbour codes
 //   gm2       T[n]       g m^2
 //   perm      int64[n]   internal -> caller index
@@ -116,24 +117,20 @@ template <typename T>
 int upload_static(swe_mesh* m) {
     const HostMesh& H = m->hm;
     const int64_t n = H.n_cells;
-    if (sizeof(T) == 8) {
-        std::vector<V4<double>> R(n);
-        for (int64_t c = 0; c < n; ++c) {
-            R[c].x = host_edge_rl(H.ln[6 * c + 0], H.ln[6 * c + 1]);
-            R[c].y = host_edge_rl(H.ln[6 * c + 2], H.ln[6 * c + 3]);
-            R[c].z = host_edge_rl(H.ln[6 * c + 4], H.ln[6 * c + 5]);
-            R[c].w = 0.0;
-        }
-        cudaError_t e = cudaMemcpy(m->geoR, R.data(), n * sizeof(V4<double>), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(e, "swe_mesh_create: upload");
-    }
-    std::vector<V4<T>> A(n), B(n);
+    std::vector<V4<T>> A(n), B(n), R(n);
     std::vector<T> gm2(n), zt(n);
     const std::vector<int4> topo = make_topo(m);
     for (int64_t c = 0; c < n; ++c) {
-        A[c].x = (T)H.ln[6 * c + 0]; A[c].y = (T)H.ln[6 * c + 1];
-        A[c].z = (T)H.ln[6 * c + 2]; A[c].w = (T)H.ln[6 * c + 3];
-        B[c].x = (T)H.ln[6 * c + 4]; B[c].y = (T)H.ln[6 * c + 5];
+        double ln[6], len[3] = {0.0, 0.0, 0.0};
+        for (int j = 0; j < 3; ++j) {
+            ln[2 * j] = H.ln[6 * c + 2 * j];
+            ln[2 * j + 1] = H.ln[6 * c + 2 * j + 1];
+            if (sizeof(T) == 8) len[j] = host_unit_normal(ln[2 * j], ln[2 * j + 1]);
+        }
+        A[c].x = (T)ln[0]; A[c].y = (T)ln[1];
+        A[c].z = (T)ln[2]; A[c].w = (T)ln[3];
+        B[c].x = (T)ln[4]; B[c].y = (T)ln[5];
+        R[c].x = (T)len[0]; R[c].y = (T)len[1]; R[c].z = (T)len[2]; R[c].w = (T)0;
         B[c].z = (T)H.inv_area[c]; B[c].w = (T)H.rin[c];
         gm2[c] = (T)(m->cfg.g * H.m[c] * H.m[c]);
         zt[c] = (T)H.z[c];
@@ -141,6 +138,8 @@ int upload_static(swe_mesh* m) {
     cudaError_t e;
     if ((e = cudaMemcpy(m->geoA, A.data(), n * sizeof(V4<T>), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(m->geoB, B.data(), n * sizeof(V4<T>), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (sizeof(T) == 8 &&
+         (e = cudaMemcpy(m->geoR, R.data(), n * sizeof(V4<T>), cudaMemcpyHostToDevice)) != cudaSuccess) ||
         (e = cudaMemcpy(m->gm2, gm2.data(), n * sizeof(T), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(m->zdev, zt.data(), n * sizeof(T), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(m->topo, topo.data(), n * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -428,10 +427,16 @@ cudaError_t launch_step_raw(swe_mesh* m, const void* in, void* out, unsigned lon
                                       eflux_out, esrc_out);
 }
 
-double host_edge_rl(double lx, double ly) { return 1.0 / std::sqrt(std::fma(lx, lx, ly * ly)); }
+double host_unit_normal(double& lx, double& ly) {
+    const double l2 = std::fma(lx, lx, ly * ly);
+    const double rl = 1.0 / std::sqrt(l2);
+    lx *= rl;
+    ly *= rl;
+    return l2 * rl;
+}
 
 void append_edges(const HostMesh& H, int64_t base, std::vector<int2>& cells, std::vector<double>& ln, int4* eidx,
-                  std::vector<double>* rl) {
+                  std::vector<double>* len) {
     const int64_t n = H.n_cells;
     for (int64_t c = 0; c < n; ++c) eidx[c] = make_int4(-1, -1, -1, 0);
     for (int64_t c = 0; c < n; ++c)
@@ -441,9 +446,10 @@ void append_edges(const HostMesh& H, int64_t base, std::vector<int2>& cells, std
                 const int e = (int)cells.size();
                 const int k = code & kNbrMask;
                 cells.push_back(make_int2((int)(base + c), (int)(base + k)));
-                ln.push_back(H.ln[6 * c + 2 * j]);
-                ln.push_back(H.ln[6 * c + 2 * j + 1]);
-                if (rl) rl->push_back(host_edge_rl(H.ln[6 * c + 2 * j], H.ln[6 * c + 2 * j + 1]));
+                double lx = H.ln[6 * c + 2 * j], ly = H.ln[6 * c + 2 * j + 1];
+                if (len) len->push_back(host_unit_normal(lx, ly));
+                ln.push_back(lx);
+                ln.push_back(ly);
                 (j == 0 ? eidx[c].x : (j == 1 ? eidx[c].y : eidx[c].z)) = e;
                 for (int jk = 0; jk < 3; ++jk)
                     if ((H.code[3 * k + jk] & kNbrMask) == (int32_t)c && H.code[3 * k + jk] >= 0)

@@ -96,19 +96,24 @@ __global__ void diag_boundary_kernel(const V4<T>* __restrict__ cur, const V4<T>*
     const V4<T> gA = geoA[i], gB = geoB[i];
     const T lx = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);
     const T ly = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
-    const T l2 = edge_l2(lx, ly);
-    T pre = T(0);
+    T len, n1, n2;   // the step's own
     if constexpr (sizeof(T) == 8) {
         const V4<T> gR = geoR[i];
-        pre = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
+        len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
+        n1 = lx;
+        n2 = ly;
+    } else {
+        const T l2 = edge_l2(lx, ly);
+        const T rl = rsqrtf(l2);
+        len = l2 * rl;
+        n1 = lx * rl;
+        n2 = ly * rl;
     }
-    const T rl = edge_rl<T>(pre, l2);   // the step's own edge scale
-    const T len = l2 * rl;
     T ui, vi;
     cell_velocity<T>(c.x, c.y, c.z, h_dry, ui, vi);
     const int grp = groups[k];
     T F0, F1, F2;
-    edge_boundary<T>(bc.kind[grp], bc.value[grp], c.x, ui, vi, c.w, lx * rl, ly * rl, g, h_dry, F0, F1, F2, hll != 0);
+    edge_boundary<T>(bc.kind[grp], bc.value[grp], c.x, ui, vi, c.w, n1, n2, g, h_dry, F0, F1, F2, hll != 0);
     q[k] = (double)len * (double)F0;
 }
 

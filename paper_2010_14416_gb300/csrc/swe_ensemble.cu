@@ -40,7 +40,7 @@ struct swe_ensemble {
     void* state[2] = {nullptr, nullptr};
     void* geoA = nullptr;
     void* geoB = nullptr;
-    void* geoR = nullptr;             // FP64: 1/|L n| of the three edges
+    void* geoR = nullptr;             // FP64: lengths of the three edges
     int4* topo = nullptr;
     void* gm2 = nullptr;
     long long* perm = nullptr;        // per member, relative to the member's base

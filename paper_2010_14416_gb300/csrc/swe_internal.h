@@ -96,12 +96,13 @@ int build_edges(swe_mesh* m);
 // Appends the interior edges of H, its cells numbered from `base`, in canonical
 // orientation (each once, from its left cell, in the order of that cell):
 // (left, right), the left cell's L n, and into eidx[0 .. H.n_cells) each
-// cell's edge per local edge (-1 on the boundary).
+// cell's edge per local edge (-1 on the boundary).  With `len` (FP64), ln
+// receives the unit normals and len the lengths.
 void append_edges(const HostMesh& H, int64_t base, std::vector<int2>& cells, std::vector<double>& ln, int4* eidx,
-                  std::vector<double>* rl = nullptr);
-// 1/|L n| of an edge as every FP64 kernel takes it: 1/sqrt(fma(lx, lx, ly ly)),
-// formed on the host with one rounding per operation (the same on every host).
-double host_edge_rl(double lx, double ly);
+                  std::vector<double>* len = nullptr);
+// Makes (lx, ly) = L n a unit normal and returns L, with one rounding per
+// operation (the same on every host; L n and -L n give opposite normals).
+double host_unit_normal(double& lx, double& ly);
 // The activity kernel indexes cells with 32 bits: meshes below this size.
 constexpr int64_t kActivityMaxCells = int64_t(1) << 29;
 // Applies pending boundary-group changes of m to the device.
@@ -120,7 +121,7 @@ struct swe_mesh {
     void* state[2] = {nullptr, nullptr};
     void* geoA = nullptr;
     void* geoB = nullptr;
-    void* geoR = nullptr;              // FP64: V4<double> 1/|L n| of the three edges
+    void* geoR = nullptr;              // FP64: V4<double> lengths of the three edges
     int4* topo = nullptr;
     void* gm2 = nullptr;
     void* zdev = nullptr;
@@ -151,8 +152,8 @@ struct swe_mesh {
     // edge pass (cfg.edge_pass): interior edges in canonical orientation
     int64_t n_edges = 0;
     int2* ecells = nullptr;            // (left, right)
-    void* eln = nullptr;               // [E][2] T, L n outward from the left cell
-    void* erl = nullptr;               // FP64: [E] 1/|L n|
+    void* eln = nullptr;               // [E][2] T, L n (FP64: n) outward from the left cell
+    void* erl = nullptr;               // FP64: [E] length
     void* eflux = nullptr;             // V4<T>[E]
     void* esrc = nullptr;              // T[E]
     int4* eidx = nullptr;              // per cell, the edge of each local edge (-1: boundary)

@@ -20,7 +20,9 @@
 
 #include <type_traits>
 
+#include "swe_compare.cuh"
 #include "swe_f32.cuh"
+#include "swe_f64.cuh"
 
 namespace swe {
 
@@ -63,9 +65,9 @@ template <typename T>
 struct StepArgs {
     const V4<T>* __restrict__ s_in;    // (h, hu, hv, z) per cell
     V4<T>* __restrict__ s_out;
-    const V4<T>* __restrict__ geoA;    // (L n)_0 x, y, (L n)_1 x, y : outward normals times length
-    const V4<T>* __restrict__ geoB;    // (L n)_2 x, y, 1/|Omega|, inscribed radius
-    const V4<T>* __restrict__ geoR;    // FP64: 1/|L n| of the three edges (x, y, z)
+    const V4<T>* __restrict__ geoA;    // (L n)_0 x, y, (L n)_1 x, y : outward normals times length (FP64: n alone)
+    const V4<T>* __restrict__ geoB;    // (L n)_2 x, y (FP64: n), 1/|Omega|, inscribed radius
+    const V4<T>* __restrict__ geoR;    // FP64: the three edges' lengths L (x, y, z)
     const int4* __restrict__ topo;     // neighbour codes of the 3 edges; .w = g m^2 bits (FP32)
     const T* __restrict__ gm2;         // g m^2 per cell (Manning factor of Eq 32), FP64 only
     const double* dt_read;             // min_i R_i/(c_i+|u_i|) of the current state
@@ -89,10 +91,10 @@ struct StepArgs {
     // edge pass (step_kernel with EDGES): interior edges in canonical orientation,
     // evaluated once per step by edge_flux_kernel before the cell pass
     const int2* ecells;                // (left, right) cell of each interior edge
-    const T* eln;                      // [E][2] L n of the edge, outward from the left cell
-    const T* erl;                      // FP64: 1/|L n| of the edge
-    V4<T>* eflux;                      // (F0, F1, F2, bed source factor of the left cell) per edge
-    T* esrc;                           // bed source factor of the right cell per edge
+    const T* eln;                      // [E][2] L n of the edge (FP64: n alone), outward from the left cell
+    const T* erl;                      // FP64: the edge's length
+    V4<T>* eflux;                      // (F0, F1, F2, bed source factor of the left cell) per edge; FP64: m, xL, yL, xR
+    T* esrc;                           // bed source factor of the right cell per edge; FP64: yR
     const int4* eidx;                  // per cell: the interior edge of each local edge (x, y, z)
     long long n_edges;
     T g, h_dry;
@@ -114,7 +116,7 @@ struct EnsArgs {
     V4<T>* __restrict__ s_out;
     const V4<T>* __restrict__ geoA;
     const V4<T>* __restrict__ geoB;
-    const V4<T>* __restrict__ geoR;    // FP64: 1/|L n| of the three edges
+    const V4<T>* __restrict__ geoR;    // FP64: the three edges' lengths
     const int4* __restrict__ topo;     // neighbour codes offset to the concatenated numbering
     const T* __restrict__ gm2;         // FP64 only
     const int* __restrict__ tile_member;               // member of each kEnsPad-cell span
@@ -179,155 +181,9 @@ template <> struct Ar<double> {
     static __device__ __forceinline__ double pow_m73(double h) { return 1.0 / (h * h * cbrt(h)); }
 };
 
-template <typename T>
-__device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
-template <typename T>
-__device__ __forceinline__ T tmin(T a, T b) { return a < b ? a : b; }
-
-// FP64 (the double instantiation only): where the paper's formulas divide by
-// several quantities in turn, one division by their product and
-// multiplications replace them.  A double division or square root is an
-// iteration of several operations on the FP64 unit, which bounds that path;
-// the products stay far inside the double range for depths of 1e-6 to 1e4 m.
-// Results move by a few ulps.  FP32 divisions are single hardware
-// approximations, and the adjoint's duals keep the formulas as written.
-template <typename T>
-constexpr bool kOneDivision = std::is_same<T, double>::value;
-
-// h^(-1/3) in double without a division or a double cube root, for the
-// friction factor h^(-7/3) = r^7 and 1/h = r^3 (Eq 33-35): Newton's iteration
-// for r^-3 = h, r <- r (4 - h r^3) / 3, started from the FP32 reciprocal cube
-// root (relative error about 2^-22) and taken twice (the error squares each
-// time, to the rounding of the last step).  For positive normal h in the FP32
-// range; friction calls it for wet cells only (h > h_dry).
-__device__ __forceinline__ double inv_cbrt_newton(double h) {
-    double r = (double)rcbrtf((float)h);
-    r = r * fma(-h, r * r * r, 4.0) * (1.0 / 3.0);
-    r = r * fma(-h, r * r * r, 4.0) * (1.0 / 3.0);
-    return r;
-}
-
-// ---- comparisons of the flux path ------------------------------------------------
-// On GB300 the FP64 unit (2 operations per clock per SM) executes compares and
-// min/max of doubles as well as their arithmetic, and it bounds the FP64 step.
-// For doubles each helper below forms exactly the IEEE result of its
-// comparison (NaN, infinities and signed zeros included) from the bit
-// patterns, with 64-bit integer operations, which the FP64 kernels leave
-// idle; the selects return the same operand the plain expression returns, so
-// results are bit for bit those of the plain operators.  Other scalars (float,
-// the adjoint's dual numbers) use the plain operators.
-namespace cmp {
-constexpr unsigned long long kPosInf = 0x7FF0000000000000ULL;   // bits of +inf
-constexpr unsigned long long kNegZero = 0x8000000000000000ULL;  // bits of -0
-__device__ __forceinline__ unsigned long long bits(double x) { return (unsigned long long)__double_as_longlong(x); }
-template <typename T>
-constexpr bool kInt = std::is_same<T, double>::value;
-}  // namespace cmp
-
-// x > c for c finite and > 0
-template <typename T>
-__device__ __forceinline__ bool gt_pos(T x, T c) {
-    if constexpr (cmp::kInt<T>) {
-        const unsigned long long xb = cmp::bits(x), cb = cmp::bits(c);
-        return xb - cb - 1ULL < cmp::kPosInf - cb;          // c < x <= +inf
-    } else {
-        return x > c;
-    }
-}
-// x <= c for c finite and > 0
-template <typename T>
-__device__ __forceinline__ bool le_pos(T x, T c) {
-    if constexpr (cmp::kInt<T>) {
-        const unsigned long long xb = cmp::bits(x), cb = cmp::bits(c);
-        return xb <= cb || xb - cmp::kNegZero <= cmp::kPosInf;   // +0 <= x <= c, or -inf <= x <= -0
-    } else {
-        return x <= c;
-    }
-}
-// x < c for c finite and > 0
-template <typename T>
-__device__ __forceinline__ bool lt_pos(T x, T c) {
-    if constexpr (cmp::kInt<T>) {
-        const unsigned long long xb = cmp::bits(x), cb = cmp::bits(c);
-        return xb < cb || xb - cmp::kNegZero <= cmp::kPosInf;
-    } else {
-        return x < c;
-    }
-}
-// |x| < c for c finite and > 0
-template <typename T>
-__device__ __forceinline__ bool abs_lt_pos(T x, T c) {
-    if constexpr (cmp::kInt<T>) {
-        return (cmp::bits(x) & ~cmp::kNegZero) < cmp::bits(c);
-    } else {
-        return fabs(x) < c;
-    }
-}
-template <typename T>
-__device__ __forceinline__ bool gt_zero(T x) {
-    if constexpr (cmp::kInt<T>) return cmp::bits(x) - 1ULL < cmp::kPosInf;            // smallest denormal .. +inf
-    else return x > T(0);
-}
-template <typename T>
-__device__ __forceinline__ bool ge_zero(T x) {
-    if constexpr (cmp::kInt<T>) {
-        const unsigned long long xb = cmp::bits(x);
-        return xb <= cmp::kPosInf || xb == cmp::kNegZero;
-    } else {
-        return x >= T(0);
-    }
-}
-template <typename T>
-__device__ __forceinline__ bool le_zero(T x) {
-    if constexpr (cmp::kInt<T>) {
-        const unsigned long long xb = cmp::bits(x);
-        return xb == 0ULL || xb - cmp::kNegZero <= cmp::kPosInf;
-    } else {
-        return x <= T(0);
-    }
-}
-template <typename T>
-__device__ __forceinline__ bool lt_zero(T x) {
-    if constexpr (cmp::kInt<T>) return cmp::bits(x) - (cmp::kNegZero + 1ULL) < cmp::kPosInf;  // -inf .. -denormal
-    else return x < T(0);
-}
-// tmax(0, x)
-template <typename T>
-__device__ __forceinline__ T max_zero(T x) {
-    if constexpr (cmp::kInt<T>) return lt_zero(x) ? T(0) : x;
-    else return tmax(T(0), x);
-}
-// tmin(a, b) for a, b >= +0 (or +inf), e.g. CFL candidates and depths
-template <typename T>
-__device__ __forceinline__ T min_nonneg(T a, T b) {
-    if constexpr (cmp::kInt<T>) return cmp::bits(a) < cmp::bits(b) ? a : b;
-    else return tmin(a, b);
-}
-// tmax(a, b) for finite a, b (bed elevations)
-template <typename T>
-__device__ __forceinline__ T max_finite(T a, T b) {
-    if constexpr (cmp::kInt<T>) {
-        // the sign-magnitude bits, turned into a two's-complement key, order
-        // finite doubles except that -0 sorts below +0, where IEEE has a tie
-        const long long ab = __double_as_longlong(a), bb = __double_as_longlong(b);
-        const long long ka = ab ^ ((ab >> 63) & 0x7FFFFFFFFFFFFFFFLL), kb = bb ^ ((bb >> 63) & 0x7FFFFFFFFFFFFFFFLL);
-        const bool both_zero = (((unsigned long long)ab | (unsigned long long)bb) << 1) == 0ULL;
-        return (ka > kb && !both_zero) ? a : b;
-    } else {
-        return tmax(a, b);
-    }
-}
-
-// 1/|L n| of an edge.  FP64 takes it precomputed (the host forms
-// 1/sqrt(fma(lx, lx, ly ly)) once per cell edge, the same on every host): the
-// square root and division are a quarter of the flux pass's FP64 work, and the
-// FP64 pipe bounds that path.  FP32 forms it with the hardware reciprocal
-// square root, since memory bounds that path.
-template <typename T>
-__device__ __forceinline__ T edge_rl(T pre, T l2) {
-    if constexpr (sizeof(T) == 8) return pre;
-    else return Ar<T>::rsqrt_(l2);
-}
+// h^(-1/3) in double, for the friction factor h^(-7/3) = r^7 and 1/h = r^3
+// (Eq 33-35): positive normal h in the FP32 range.
+__device__ __forceinline__ double inv_cbrt_newton(double h) { return f64::rcbrt(h); }
 
 // |L n|^2 of an edge, written as one fused multiply-add so that every kernel
 // (and both cells of an edge, whose L n differ only in sign) forms the same
@@ -349,7 +205,11 @@ __device__ __forceinline__ void riemann_hllc(T hL, T unL, T utL, T hR, T unR, T 
     if constexpr (std::is_same<T, float>::value) {   // FP32: swe_f32.cuh, branch-free and explicitly rounded
         f32::riemann<float>(hL, unL, utL, hR, unR, utR, g, f32::mul(0.5f, g), h_dry, G1, G2, G3, speeds, hll_only);
         return;
-    }
+    } else if constexpr (std::is_same<T, double>::value) {   // FP64: swe_f64.cuh
+        double PL, PR;
+        f64::riemann<false>(hL, unL, utL, hR, unR, utR, 0.5 * g, h_dry, 1.0, G1, G2, G3, PL, PR, speeds, hll_only);
+        return;
+    } else {
     using A = Ar<T>;
     const bool wetL = gt_pos(hL, h_dry), wetR = gt_pos(hR, h_dry);
     if (!wetL && !wetR) {
@@ -366,39 +226,16 @@ __device__ __forceinline__ void riemann_hllc(T hL, T unL, T utL, T hR, T unR, T 
     } else {
         const T hsum = hL + hR;
         const T h0 = T(0.5) * hsum - T(0.25) * A::div_((unR - unL) * hsum, aL + aR);  // Eq 21
-        T hs;
-        if (le_pos(h0, min_nonneg(hL, hR))) {                                      // Eq 22
-            const T b = max_zero(T(0.5) * (aL + aR) + T(0.25) * (unL - unR));
-            hs = A::div_(b * b, g);
-        } else if constexpr (!kOneDivision<T>) {                                    // Eq 23
+        T pL = T(1), pR = T(1);                                                     // Eq 20
+        // Eq 22's two-rarefaction estimate is at most min(h_L, h_R) where Eq 21
+        // chooses it: p_L = p_R = 1 there
+        if (!le_pos(h0, min_nonneg(hL, hR))) {                                       // Eq 23
             const T r2h0 = A::rcp_(T(2) * h0);
             const T gL = A::sqrt_(g * (h0 + hL) * r2h0 * A::rcp_(hL));
             const T gR = A::sqrt_(g * (h0 + hR) * r2h0 * A::rcp_(hR));
-            hs = A::div_(hL * gL + hR * gR + unL - unR, gL + gR);
-        } else {
-            // one division gives 1/(2 h0 h_L) and 1/(2 h0 h_R) (h0 > min(h_L, h_R) > 0 here)
-            const T h02 = T(2) * h0;
-            const T inv = A::rcp_(h02 * hL * hR);
-            const T gL = A::sqrt_(g * (h0 + hL) * (hR * inv));
-            const T gR = A::sqrt_(g * (h0 + hR) * (hL * inv));
-            hs = A::div_(hL * gL + hR * gR + unL - unR, gL + gR);
-        }
-        T pL = T(1), pR = T(1);                                                     // Eq 20
-        if constexpr (!kOneDivision<T>) {
+            const T hs = A::div_(hL * gL + hR * gR + unL - unR, gL + gR);
             if (gt_pos(hs, hL)) pL = A::div_(A::sqrt_(T(0.5) * hs * (hs + hL)), hL);
             if (gt_pos(hs, hR)) pR = A::div_(A::sqrt_(T(0.5) * hs * (hs + hR)), hR);
-        } else {
-            // sqrt(h*(h*+h_K)/2)/h_K = sqrt(h*(h*+h_K)/(2 h_K^2)); both shocks share a division
-            const bool shL = gt_pos(hs, hL), shR = gt_pos(hs, hR);
-            if (shL && shR) {
-                const T inv = A::rcp_(hL * hR);
-                pL = A::sqrt_(T(0.5) * hs * (hs + hL)) * (hR * inv);
-                pR = A::sqrt_(T(0.5) * hs * (hs + hR)) * (hL * inv);
-            } else if (shL) {
-                pL = A::div_(A::sqrt_(T(0.5) * hs * (hs + hL)), hL);
-            } else if (shR) {
-                pR = A::div_(A::sqrt_(T(0.5) * hs * (hs + hR)), hR);
-            }
         }
         SL = unL - aL * pL;                                                          // Eq 19
         SR = unR + aR * pR;
@@ -423,6 +260,7 @@ __device__ __forceinline__ void riemann_hllc(T hL, T unL, T utL, T hR, T unR, T 
     }
     if (!hll_only) G3 = G1 * (ge_zero(Ss) ? utL : utR);                              // Eq 24
     if (speeds) { speeds[0] = SL; speeds[1] = SR; speeds[2] = Ss; }
+    }
 }
 
 template <typename T>
@@ -522,9 +360,13 @@ __device__ __forceinline__ void cp_async_wait() {
 
 template <typename T>
 __device__ __forceinline__ void cell_velocity(T h, T hu, T hv, T h_dry, T& u, T& v) {
-    u = T(0);
-    v = T(0);
-    if (gt_pos(h, h_dry)) { const T r = Ar<T>::rcp_(h); u = hu * r; v = hv * r; }
+    if constexpr (std::is_same<T, double>::value) {
+        f64::velocity(h, hu, hv, h_dry, u, v);
+    } else {
+        u = T(0);
+        v = T(0);
+        if (gt_pos(h, h_dry)) { const T r = Ar<T>::rcp_(h); u = hu * r; v = hv * r; }
+    }
 }
 
 // Flux leaving cell i through an interior edge (per unit length, x-y frame)
@@ -540,6 +382,7 @@ __device__ __forceinline__ void edge_interior(T hi, T ui, T vi, T zi, T hk, T hu
                                   F2, src, hll_only, src_k);
         return;
     }
+    static_assert(!std::is_same<T, double>::value, "FP64 edges: f64::edge");
     T uk, vk;
     cell_velocity<T>(hk, huk, hvk, h_dry, uk, vk);
     // hydrostatic reconstruction (Eq 28): z* = max(z_i, z_k)
@@ -572,7 +415,16 @@ __device__ __forceinline__ void edge_boundary(int kind, double value, T hi, T ui
     if constexpr (std::is_same<T, float>::value) {   // FP32: swe_f32.cuh
         f32::edge_boundary(kind, value, hi, ui, vi, zi, n1, n2, g, f32::mul(0.5f, g), h_dry, F0, F1, F2, hll_only);
         return;
-    }
+    } else if constexpr (std::is_same<T, double>::value) {   // FP64: swe_f64.cuh
+        const f64::Side c{hi, ui, vi, zi};
+        const double un = f64::fma(ui, n1, f64::mul(vi, n2)), ut = f64::fma(vi, n1, -f64::mul(ui, n2));
+        double G1, G2, G3;
+        f64::boundary_flux(kind, value, c, un, ut, 0.5 * g, h_dry, hll_only, G1, G2, G3);
+        F0 = G1;
+        F1 = f64::fma(G2, n1, -f64::mul(G3, n2));
+        F2 = f64::fma(G2, n2, f64::mul(G3, n1));
+        return;
+    } else {
     const T un = ui * n1 + vi * n2, ut = vi * n1 - ui * n2;
     T G1, G2, G3;
     if (kind == kBcWall) {
@@ -590,9 +442,10 @@ __device__ __forceinline__ void edge_boundary(int kind, double value, T hi, T ui
     F0 = G1;
     F1 = G2 * n1 - G3 * n2;
     F2 = G2 * n2 + G3 * n1;
+    }
 }
 
-// Semi-implicit friction (Eq 33-37): dU solving [I - dt/2 J_f] dU = dt (R + S_f)
+// Semi-implicit friction (Eq 33-37), for the adjoint's duals: dU solving [I - dt/2 J_f] dU = dt (R + S_f)
 // with R = (Rh, Rx, Ry) the explicit right-hand side per unit area.
 template <typename T>
 __device__ __forceinline__ void friction_update(T hi, T qx, T qy, T gm2, T Rh, T Rx, T Ry, T dt, T h_dry, T& dh,
@@ -605,15 +458,7 @@ __device__ __forceinline__ void friction_update(T hi, T qx, T qy, T gm2, T Rh, T
         const T qq = qx * qx + qy * qy;
         if (gt_zero(qq)) {
             const T qn = A::sqrt_(qq);
-            T cf, rh;                                       // c = g m^2 h^(-7/3), 1/h
-            if constexpr (kOneDivision<T>) {
-                const T r = inv_cbrt_newton(hi), r3 = r * r * r;   // h^(-1/3), 1/h
-                cf = gm2 * (r3 * r3 * r);                            // h^(-7/3) = r^7
-                rh = r3;
-            } else {
-                cf = gm2 * A::pow_m73(hi);
-                rh = A::rcp_(hi);
-            }
+            const T cf = gm2 * A::pow_m73(hi), rh = A::rcp_(hi);   // c = g m^2 h^(-7/3), 1/h
             const T al = T(0.5) * dt * cf;                  // alpha = dt c / 2
             // rhs: dt (R_q + S_f) + dt/2 J_qh dh, with S_f = -c|q|q and
             // J_qh = (7/3) c |q| q / h
@@ -622,15 +467,7 @@ __device__ __forceinline__ void friction_update(T hi, T qx, T qy, T gm2, T Rh, T
             // (1 + a|q|) I + a q q^T/|q| has eigenvalue 1 + 2a|q| along q
             // and 1 + a|q| across it
             const T d1 = T(1) + al * qn, d2 = d1 + al * qn;
-            T rqd2, rd1;                                    // 1/(|q| d2), 1/d1
-            if constexpr (kOneDivision<T>) {
-                const T qd2 = qn * d2, inv = A::rcp_(qd2 * d1);
-                rqd2 = d1 * inv;
-                rd1 = qd2 * inv;
-            } else {
-                rqd2 = A::rcp_(qn * d2);
-                rd1 = A::rcp_(d1);
-            }
+            const T rqd2 = A::rcp_(qn * d2), rd1 = A::rcp_(d1);
             const T proj = (bx * qx + by * qy) * al * rqd2;
             dqx = (bx - proj * qx) * rd1;
             dqy = (by - proj * qy) * rd1;
@@ -638,54 +475,29 @@ __device__ __forceinline__ void friction_update(T hi, T qx, T qy, T gm2, T Rh, T
     }
 }
 
-// ---- the end of one cell update -----------------------------------------------------
-// From the summed edge terms (f = sum of L_ij F_ij, s = sum of the bed source
-// factors times L_ij n_ij) to the new state (Eq 37 with friction, Eq 33-36),
-// its checks, and the cell's next CFL candidate R_i/(sqrt(g h)+|u|) (Eq 15;
-// +inf when the new state is dry).  Every cell kernel ends here, so their
-// arithmetic is the same.
-template <typename T, typename Args>
-__device__ __forceinline__ T finish_cell(const Args& a, long long i, const V4<T>& own, T f0, T f1, T f2, T sx, T sy,
-                                         T ia, T rin, T gm2, T dt, unsigned long long* n_clamped, unsigned* status) {
-    using A = Ar<T>;
-    const T g = a.g, h_dry = a.h_dry;
-    const T hi = own.x;
-    V4<T> out;
+// ---- the end of one FP64 cell update --------------------------------------------------
+// From the sums of the edges' terms (f64::EdgeTerms) to the new state, its
+// checks, and the cell's next CFL candidate R_i/(sqrt(g h)+|u|) (Eq 15; +inf
+// when the new state is dry).  Every FP64 cell kernel ends here.
+template <typename Args>
+__device__ __forceinline__ double finish_cell(const Args& a, long long i, const V4<double>& own, double m, double x,
+                                              double y, double ia, double rin, double gm2, double dt,
+                                              unsigned long long* n_clamped, unsigned* status) {
+    const double g = a.g, h_dry = a.h_dry;
+    V4<double> out;
     out.w = own.w;
-    const T Rh = -f0 * ia;
-    const T Rx = (sx - f1) * ia;
-    const T Ry = (sy - f2) * ia;
-    const T qx = own.y, qy = own.z;
-    T dh, dqx, dqy;
-    friction_update<T>(hi, qx, qy, gm2, Rh, Rx, Ry, dt, h_dry, dh, dqx, dqy);
-    out.x = hi + dh;
-    out.y = qx + dqx;
-    out.z = qy + dqy;
+    f64::update(own.x, own.y, own.z, m, x, y, ia, gm2, dt, h_dry, out.x, out.y, out.z);
     if (lt_zero(out.x)) {
-        out.x = T(0); out.y = T(0); out.z = T(0);
+        out.x = 0.0; out.y = 0.0; out.z = 0.0;
         atomicAdd(n_clamped, 1ULL);
     } else if (le_pos(out.x, h_dry)) {
-        out.y = T(0); out.z = T(0);
+        out.y = 0.0; out.z = 0.0;
     }
-    const T big = T(3.0e38);
+    const double big = 3.0e38;
     if (!lt_pos(out.x, big) || !abs_lt_pos(out.y, big) || !abs_lt_pos(out.z, big))
         atomicOr(status, kStatusNonFinite);
     a.s_out[i] = out;
-    // next CFL candidate (Eq 15), R_i / (sqrt(g h) + |u|) on the new state
-    T cand = inf_of<T>();
-    if (gt_pos(out.x, h_dry)) {
-        if constexpr (kOneDivision<T>) {
-            // R h / (h sqrt(g h) + |q|): the velocity's division folded into the candidate's
-            const T qm = A::sqrt_(out.y * out.y + out.z * out.z);
-            cand = A::div_(rin * out.x, out.x * A::sqrt_(g * out.x) + qm);
-        } else {
-            const T r = A::rcp_(out.x);
-            const T u = out.y * r, v = out.z * r;
-            const T den = A::sqrt_(g * out.x) + A::sqrt_(u * u + v * v);
-            cand = A::div_(rin, den);
-        }
-    }
-    return cand;
+    return gt_pos(out.x, h_dry) ? f64::cfl_candidate(out.x, out.y, out.z, rin, g) : inf_of<double>();
 }
 
 // ---- one FP32 cell of the fused step -------------------------------------------------
@@ -838,19 +650,18 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
 // at the price of geometry traffic for quiet cells too); otherwise they are
 // issued after the quiet test.  Both give the same results.
 //
-// EDGES takes the interior fluxes from the edge pass (edge_flux_kernel, the
-// same edge_interior arithmetic evaluated once per edge from the left cell)
-// instead of evaluating them here; an edge with both cells dry has no flux and
-// its bed source factor is formed inline, as edge_interior would form it.
+// EDGES takes the interior edges' terms from the edge pass (edge_flux_kernel,
+// the same arithmetic evaluated once per edge) instead of evaluating them
+// here; an edge with both cells dry has no flux and its bed source term is
+// formed inline, with the same bits.
 template <typename T, bool GEO_EARLY, bool EDGES = false, typename Args>
 __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>& own, const int4& tp, T dt,
                                          unsigned& active, unsigned long long* n_clamped, unsigned* status) {
     if constexpr (std::is_same<T, float>::value) {
         return update_cell_f32<GEO_EARLY, EDGES>(a, i, own, tp, dt, active, n_clamped, status);
     } else {
-    using A = Ar<T>;
-    const T g = a.g, h_dry = a.h_dry;
-    const T hi = own.x, zi = own.w;
+    const double h_dry = a.h_dry, g2 = f64::mul(0.5, a.g);
+    const double hi = own.x, zi = own.w;
     int code[3] = {tp.x, tp.y, tp.z};
     if (a.debug) {   // an unusable code is flagged and taken as a wall (group 0)
 #pragma unroll
@@ -861,16 +672,16 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
             }
     }
     // issue the three neighbour gathers before any arithmetic
-    V4<T> nb[3];
+    V4<double> nb[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) nb[j] = code[j] >= 0 ? a.s_in[code[j] & kNbrMask] : own;
-    V4<T> gA, gB, gR;
-    T gm2;
+    V4<double> gA, gB, gR;   // unit normals, 1/|Omega| and R, lengths
+    double gm2;
     if constexpr (GEO_EARLY) {
         gA = a.geoA[i];
         gB = a.geoB[i];
-        if constexpr (sizeof(T) == 8) gR = a.geoR[i];
-        gm2 = load_gm2(a, i, tp, T(0));
+        gR = a.geoR[i];
+        gm2 = a.gm2[i];
     }
     bool quiet = !gt_pos(hi, h_dry);
 #pragma unroll
@@ -882,76 +693,73 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
             quiet = quiet && (kind == kBcWall || kind == kBcTransmissive);
         }
     }
-    V4<T> out;
-    out.w = zi;
     if (quiet) {
-        out.x = hi; out.y = T(0); out.z = T(0);
+        V4<double> out;
+        out.x = hi; out.y = 0.0; out.z = 0.0; out.w = zi;
         a.s_out[i] = out;
-        return inf_of<T>();
+        return inf_of<double>();
     }
     active += 1u;
     if constexpr (!GEO_EARLY) {
         gA = a.geoA[i];
         gB = a.geoB[i];
-        if constexpr (sizeof(T) == 8) gR = a.geoR[i];
-        gm2 = load_gm2(a, i, tp, T(0));
+        gR = a.geoR[i];
+        gm2 = a.gm2[i];
     }
-    if constexpr (sizeof(T) != 8) gR = gA;   // unused: FP32 forms 1/|L n| itself
-    T ui, vi;
-    cell_velocity<T>(hi, own.y, own.z, h_dry, ui, vi);
-    T f0 = T(0), f1 = T(0), f2 = T(0), sx = T(0), sy = T(0);
+    f64::Side own_side{hi, 0.0, 0.0, zi};
+    // with EDGES only boundary edges need the cell's own velocity
+    if (!EDGES || code[0] < 0 || code[1] < 0 || code[2] < 0)
+        f64::velocity(hi, own.y, own.z, h_dry, own_side.u, own_side.v);
+    double m = 0.0, x = 0.0, y = 0.0;
     int4 ei = make_int4(-1, -1, -1, 0);
     if constexpr (EDGES) ei = a.eidx[i];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const int c = j == 0 ? code[0] : (j == 1 ? code[1] : code[2]);
-        const V4<T> o = j == 0 ? nb[0] : (j == 1 ? nb[1] : nb[2]);
-        const T lx = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);
-        const T ly = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
-        const T l2 = edge_l2(lx, ly);
-        const T rl = edge_rl<T>(j == 0 ? gR.x : (j == 1 ? gR.y : gR.z), l2);
-        const T len = l2 * rl;
-        const T n1 = lx * rl, n2 = ly * rl;     // this cell's outward unit normal
-        T F0, F1, F2;
+        const int c = code[j];
+        const V4<double> o = nb[j];
+        const double n1 = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);   // this cell's outward unit normal
+        const double n2 = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
+        const double len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
+        double tm = 0.0, tx, ty;
         if (c >= 0) {
-            T src;
+            const bool flip = (c & kFlipBit) != 0;
             if constexpr (EDGES) {
                 if (!gt_pos(hi, h_dry) && !gt_pos(o.x, h_dry)) {
-                    const T zs = max_finite(zi, o.w);
-                    const T hsi = max_zero(hi + zi - zs);
-                    F0 = T(0); F1 = T(0); F2 = T(0);
-                    src = T(0.5) * g * (hsi * hsi - hi * hi);
+                    f64::dry_edge(hi, zi, o.w, n1, n2, len, g2, tx, ty);
                 } else {
                     int e = j == 0 ? ei.x : (j == 1 ? ei.y : ei.z);
                     if (a.debug && !(e >= 0 && e < a.n_edges)) {
                         atomicOr(status, kStatusBadIndex);
                         e = 0;
                     }
-                    const V4<T> fl = a.eflux[e];
-                    if (c & kFlipBit) {
-                        F0 = -fl.x; F1 = -fl.y; F2 = -fl.z;
-                        src = a.esrc[e];
-                    } else {
-                        F0 = fl.x; F1 = fl.y; F2 = fl.z;
-                        src = fl.w;
-                    }
+                    const V4<double> fl = a.eflux[e];
+                    tm = flip ? -fl.x : fl.x;
+                    tx = flip ? -fl.w : fl.y;
+                    ty = flip ? -a.esrc[e] : fl.z;
                 }
             } else {
-                edge_interior<T>(hi, ui, vi, zi, o.x, o.y, o.z, o.w, n1, n2, (c & kFlipBit) != 0, g, h_dry, F0, F1,
-                                 F2, src, a.hll != 0);
+                f64::Side nb_side{o.x, 0.0, 0.0, o.w};
+                f64::velocity(o.x, o.y, o.z, h_dry, nb_side.u, nb_side.v);
+                f64::Side L, R;   // the canonical orientation: left = lower caller index
+                L.h = flip ? nb_side.h : own_side.h; R.h = flip ? own_side.h : nb_side.h;
+                L.u = flip ? nb_side.u : own_side.u; R.u = flip ? own_side.u : nb_side.u;
+                L.v = flip ? nb_side.v : own_side.v; R.v = flip ? own_side.v : nb_side.v;
+                L.z = flip ? nb_side.z : own_side.z; R.z = flip ? own_side.z : nb_side.z;
+                f64::EdgeTerms t;
+                f64::edge(L, R, flip ? -n1 : n1, flip ? -n2 : n2, len, g2, h_dry, a.hll != 0, t);
+                tm = flip ? -t.m : t.m;
+                tx = flip ? -t.xR : t.xL;
+                ty = flip ? -t.yR : t.yL;
             }
-            sx += src * lx;
-            sy += src * ly;
         } else {
             const int grp = -1 - c;
-            edge_boundary<T>(a.bc_kind(grp), a.bc_value(grp), hi, ui, vi, zi, n1, n2, g, h_dry, F0, F1, F2,
-                             a.hll != 0);
+            f64::boundary(a.bc_kind(grp), a.bc_value(grp), own_side, n1, n2, len, g2, h_dry, a.hll != 0, tm, tx, ty);
         }
-        f0 += len * F0;
-        f1 += len * F1;
-        f2 += len * F2;
+        m = f64::add(m, tm);
+        x = f64::add(x, tx);
+        y = f64::add(y, ty);
     }
-    return finish_cell<T>(a, i, own, f0, f1, f2, sx, sy, gB.z, gB.w, gm2, dt, n_clamped, status);
+    return finish_cell(a, i, own, m, x, y, gB.z, gB.w, gm2, dt, n_clamped, status);
     }
 }
 
@@ -1079,9 +887,9 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_pair(const StepArgs<f
 // ---- edge pass: each interior edge's flux once per step ----------------------------
 // The canonical evaluation of an interior edge (from its left cell, Eq 12-30)
 // is the one both of its cells make in step_kernel; here one thread makes it
-// and stores the flux leaving the left cell and both cells' bed source
-// factors, which the cell pass (step_kernel with EDGES) applies with the
-// left/right sign.  Edges with both cells dry are skipped: the cells form
+// and stores, FP32, the flux leaving the left cell and both cells' bed source
+// factors, or, FP64, both cells' terms (f64::EdgeTerms), which the cell pass
+// (step_kernel with EDGES) applies with the left/right sign.  Edges with both cells dry are skipped: the cells form
 // them inline.  Worth it where the flux arithmetic, not memory, bounds the
 // step (the FP64 pipe).
 template <typename T, int BLOCK>
@@ -1096,19 +904,24 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
         }
         const V4<T> L = a.s_in[lr.x], R = a.s_in[lr.y];
         if (!gt_pos(L.x, h_dry) && !gt_pos(R.x, h_dry)) continue;
-        const T lx = a.eln[2 * e], ly = a.eln[2 * e + 1];
-        const T l2 = edge_l2(lx, ly);
-        T pre = T(0);
-        if constexpr (sizeof(T) == 8) pre = a.erl[e];
-        const T rl = edge_rl<T>(pre, l2);
-        const T n1 = lx * rl, n2 = ly * rl;
-        T ui, vi;
-        cell_velocity<T>(L.x, L.y, L.z, h_dry, ui, vi);
-        T F0, F1, F2, sl, sr;
-        edge_interior<T>(L.x, ui, vi, L.w, R.x, R.y, R.z, R.w, n1, n2, false, g, h_dry, F0, F1, F2, sl, a.hll != 0,
-                         &sr);
         V4<T> f;
-        f.x = F0; f.y = F1; f.z = F2; f.w = sl;
+        T sr;
+        if constexpr (sizeof(T) == 8) {
+            f64::Side l{L.x, 0.0, 0.0, L.w}, r{R.x, 0.0, 0.0, R.w};
+            f64::velocity(L.x, L.y, L.z, h_dry, l.u, l.v);
+            f64::velocity(R.x, R.y, R.z, h_dry, r.u, r.v);
+            f64::EdgeTerms t;
+            f64::edge(l, r, a.eln[2 * e], a.eln[2 * e + 1], a.erl[e], f64::mul(0.5, g), h_dry, a.hll != 0, t);
+            f.x = t.m; f.y = t.xL; f.z = t.yL; f.w = t.xR;
+            sr = t.yR;
+        } else {
+            const T lx = a.eln[2 * e], ly = a.eln[2 * e + 1];
+            const T rl = rsqrtf(edge_l2(lx, ly));
+            T ui, vi;
+            cell_velocity<T>(L.x, L.y, L.z, h_dry, ui, vi);
+            edge_interior<T>(L.x, ui, vi, L.w, R.x, R.y, R.z, R.w, lx * rl, ly * rl, false, g, h_dry, f.x, f.y, f.z,
+                             f.w, a.hll != 0, &sr);
+        }
         a.eflux[e] = f;
         a.esrc[e] = sr;
     }

@@ -1,0 +1,31 @@
+"""The FP64 kernels' reciprocal and roots (swe_f64.cuh): one third-order
+correction of a hardware seed.  Bounds, in units of 2^-52 relative: the last
+operation rounds by at most 1/2 and the correction leaves under 0.02, so the
+reciprocal is within 0.52 and the root and its inverse (whose first product
+rounds too) within 0.77; the reference itself is within 1/2 (quotient, root),
+1 (inverse root) or 2 (inverse cube root, from cbrt's own bound of 1)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2010_14416_gb300 import build as libbuild
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(HERE, "..", "paper_2010_14416_gb300", "csrc")
+
+
+def test_fp64_reciprocal_and_roots_within_their_bounds(tmp_path):
+    exe = str(tmp_path / "f64_arith_check")
+    cmd = [libbuild.nvcc()] + libbuild.ARCH + ["-O3", "-std=c++17", "-I", CSRC,
+                                                os.path.join(HERE, "cuda", "f64_arith_check.cu"), "-o", exe]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
+    got = {k: float(v) for k, v in (line.split() for line in r.stdout.splitlines())}
+    bounds = dict(rcp=1.02, rcp_negative=1.02, sqrt=1.27, rsqrt=1.77, rcbrt=3.0, scale=0.0, special=0.0)
+    assert got.keys() == bounds.keys()
+    assert all(got[k] <= bounds[k] for k in bounds), got

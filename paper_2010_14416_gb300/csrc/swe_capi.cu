@@ -66,6 +66,15 @@ __global__ void init_small_kernel(unsigned long long* small, double t) {
 
 using namespace swe;
 
+int swe::status_code(unsigned long long st) {
+    if (st & kStatusBadIndex) {
+        set_error("swe_step: a neighbour index, edge index or boundary group out of range (debug checks)");
+        return SWE_EMESH;
+    }
+    if (st & kStatusNonFinite) { set_error("swe_step: non-finite state"); return SWE_ENONFINITE; }
+    if (st & kStatusDry) { set_error("swe_step: every cell is dry, no CFL time step"); return SWE_EDRY; }
+    return SWE_OK;
+}
 
 namespace {
 
@@ -163,6 +172,7 @@ int flush_topo(swe_mesh* m) {
     }
     m->topo_dirty = false;
     m->act_valid = false;   // static activity may have changed
+    drop_diag_workspace(m);   // the boundary edges' groups
     drop_graph(m);
     return SWE_OK;
 }
@@ -296,16 +306,6 @@ int read_small(swe_mesh* m, unsigned long long out[kSmallWords]) {
                                     cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "swe: reading the status block");
-    return SWE_OK;
-}
-
-int status_code(unsigned long long st) {
-    if (st & kStatusBadIndex) {
-        set_error("swe_step: a neighbour index, edge index or boundary group out of range (debug checks)");
-        return SWE_EMESH;
-    }
-    if (st & kStatusNonFinite) { set_error("swe_step: non-finite state"); return SWE_ENONFINITE; }
-    if (st & kStatusDry) { set_error("swe_step: every cell is dry, no CFL time step"); return SWE_EDRY; }
     return SWE_OK;
 }
 
@@ -577,6 +577,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     DeviceGuard dg(m->cfg.device);
     if (m->stream) cudaStreamSynchronize(m->stream);
     drop_graph(m);
+    drop_diag_workspace(m);
     void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
                     m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl};

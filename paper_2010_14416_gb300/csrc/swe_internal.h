@@ -107,6 +107,10 @@ double host_unit_normal(double& lx, double& ly);
 constexpr int64_t kActivityMaxCells = int64_t(1) << 29;
 // Applies pending boundary-group changes of m to the device.
 int flush_mesh_bc(swe_mesh* m);
+// The error code (and message) of a status word.
+int status_code(unsigned long long status);
+// Frees m's diagnostics workspace.
+void drop_diag_workspace(swe_mesh* m);
 // Drops m's captured CUDA graph (after a change of launch shape).
 void drop_mesh_graph(swe_mesh* m);
 }  // namespace swe
@@ -157,6 +161,11 @@ struct swe_mesh {
     void* eflux = nullptr;             // V4<T>[E]
     void* esrc = nullptr;              // T[E]
     int4* eidx = nullptr;              // per cell, the edge of each local edge (-1: boundary)
+    // diagnostics workspace (swe_diag.cu)
+    double *diag_dev = nullptr, *diag_partial = nullptr, *diag_host = nullptr;
+    long long* diag_slots = nullptr;
+    int* diag_groups = nullptr;
+    std::vector<int> diag_edge_group;
     // reverse step of swe_adjoint: SWE_ADJOINT_TRANSPOSE or SWE_ADJOINT_DUAL
     int adjoint_method = SWE_ADJOINT_TRANSPOSE;
 };

@@ -712,6 +712,7 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
         const long long need = (units + c.block_size - 1) / c.block_size;
         const long long wave = (long long)std::max(per_sm, 1) * std::max(sms, 1);
         m->grid = (unsigned)std::min(need, c.grid > 0 ? (long long)c.grid : wave);
+        if (c.grid == 0 && c.precision == SWE_FP64 && !c.activity && n <= kSpreadCells) m->grid = spread_grid(n);
         // launches without activity bytes: the same shape, or the default one
         // when the configured shape exists only as an activity kernel
         m->plain = LaunchShape{c.block_size, c.min_blocks, c.stages, c.geometry_early, c.edge_pass, m->grid,
@@ -729,6 +730,7 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
                     : Launch<double>::resident_blocks(d.block, d.min_blocks, d.stages, 0, 0, 0, &pb);
             if (e != cudaSuccess) { swe_mesh_destroy(m); return cuda_fail(e, "swe_mesh_create: occupancy"); }
             d.grid = (unsigned)std::min((long long)((n + d.block - 1) / d.block), (long long)std::max(pb, 1) * std::max(sms, 1));
+            if (c.precision == SWE_FP64 && n <= kSpreadCells) d.grid = spread_grid(n);
             m->plain = d;
         }
     }

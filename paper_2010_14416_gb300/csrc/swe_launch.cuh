@@ -69,7 +69,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
         if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_EDGE(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0, true><<<grid, B, 0, st>>>(a);            \
+        step_kernel<T, B, M, S, G != 0, true><<<grid, step_threads(a.n, grid, B), 0, st>>>(a);            \
         return cudaGetLastError();                                                \
     }
         if constexpr (sizeof(T) == 4) {
@@ -82,7 +82,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
     }
 #define SWE_LAUNCH(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0><<<grid, B, 0, st>>>(a);                  \
+        step_kernel<T, B, M, S, G != 0><<<grid, step_threads(a.n, grid, B), 0, st>>>(a);                  \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {
@@ -203,9 +203,11 @@ int Launch<T>::pair_variants(int (*out)[4], int max) {
 template <typename T>
 cudaError_t Launch<T>::edge_flux(const StepArgs<T>& a, cudaStream_t st) {
     if (a.n_edges <= 0) return cudaSuccess;
-    const long long eb = (a.n_edges + kEdgeBlock - 1) / kEdgeBlock;
+    // (step_threads says why)
+    const int block = sizeof(T) == 8 && a.n_edges <= kSpreadCells ? 32 : kEdgeBlock;
+    const long long eb = (a.n_edges + block - 1) / block;
     const unsigned egrid = (unsigned)(eb < 65536 ? eb : 65536);
-    edge_flux_kernel<T, kEdgeBlock><<<egrid, kEdgeBlock, 0, st>>>(a);
+    edge_flux_kernel<T, kEdgeBlock><<<egrid, block, 0, st>>>(a);
     return cudaGetLastError();
 }
 

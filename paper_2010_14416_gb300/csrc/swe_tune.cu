@@ -5,7 +5,8 @@
 // compiled (block, min_blocks, stages, geometry early) shape of the step
 // kernel, every (block, min_blocks, geometry early) shape of the cell-pair
 // step (FP32) and of the activity kernel, each with several grid sizes (one or two resident waves looping
-// over the cells, or 1, 2 or 4 cells per thread), is timed with CUDA events
+// over the cells, or 1, 2 or 4 cells
+// per thread, or, on a small FP64 mesh, blocks of one to three warps), is timed with CUDA events
 // on the mesh's current state.  The trial steps read the current state and
 // write a scratch state buffer and a scratch copy of the status block; trials
 // of the activity kernel also write the mesh's next activity buffers, with
@@ -79,10 +80,13 @@ int candidate_shapes(const swe_mesh* m, std::vector<Shape>& cand) {
         const long long units = pairs ? (n + 1) / 2 : n;
         const long long need = (units + block - 1) / block;
         const long long wave = (long long)std::max(per_sm, 1) * std::max(sms, 1);
-        const long long grids[] = {wave, 2 * wave, need, (need + 1) / 2, (need + 3) / 4};
+        std::vector<long long> grids = {wave, 2 * wave, need, (need + 1) / 2, (need + 3) / 4};
+        for (long long& gsz : grids) gsz = std::max(1LL, std::min(gsz, need));
+        // a small FP64 mesh: the smallest compiled block run with fewer threads too
+        if (sizeof(T) == 8 && block == 128 && !act && n <= kSpreadCells)
+            for (int t : {32, 64, 96}) grids.push_back((n + t - 1) / t);
         for (long long gsz : grids) {
-            const Shape sh{block, minb, stages, geo, act, edges,
-                           (unsigned)std::max(1LL, std::min(gsz, need)), pairs};
+            const Shape sh{block, minb, stages, geo, act, edges, (unsigned)gsz, pairs};
             bool seen = false;
             for (const Shape& c : cand) seen = seen || same_shape(c, sh);
             if (!seen) cand.push_back(sh);

@@ -219,6 +219,8 @@ StepArgs<T> make_args(swe_mesh* m, int64_t step_index, double cfl) {
     a.act_in = nullptr;
     a.act_next = nullptr;
     a.act_clear = nullptr;
+    a.act_list = m->act_list;
+    a.act_count = m->act_count;
     if (m->cfg.activity && m->act[0]) {
         a.act_in = m->act[p3];
         a.act_next = m->act[(p3 + 1) % 3];
@@ -510,16 +512,19 @@ int init_activity(swe_mesh* m) {
             e = cudaMalloc((void**)&m->act[k], len);
             if (e == cudaSuccess) e = cudaMemsetAsync(m->act[k], 0, len, m->stream);
         }
+        if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_list, n * sizeof(unsigned));
+        if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_count, 2 * sizeof(unsigned));
+        if (e == cudaSuccess) e = cudaMemsetAsync(m->act_count, 0, 2 * sizeof(unsigned), m->stream);
         if (e != cudaSuccess) {
-            for (auto& p : m->act) {
+            for (void* p : {(void*)m->act[0], (void*)m->act[1], (void*)m->act[2], (void*)m->act_list, (void*)m->act_count})
                 if (p) cudaFree(p);
-                p = nullptr;
-            }
+            for (auto& p : m->act) p = nullptr;
+            m->act_list = m->act_count = nullptr;
             set_error("activity bytes: device allocation failed");
             return SWE_ENOMEM;
         }
         m->act_len = len;
-        m->device_bytes += 3 * len;
+        m->device_bytes += 3 * len + (int64_t)((n + 2) * sizeof(unsigned));
     }
     const int p3 = (int)(m->nstep % 3);
     e = cudaMemsetAsync(m->act[p3], 2, m->act_len, m->stream);   // bit 1: rebuilt (act_init_kernel)
@@ -580,7 +585,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     drop_diag_workspace(m);
     void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
-                    m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl};
+                    m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);

@@ -149,6 +149,8 @@ struct swe_mesh {
     unsigned char* act[3] = {nullptr, nullptr, nullptr};
     int64_t act_len = 0;
     bool act_valid = false;
+    unsigned* act_list = nullptr;      // n cells: those that run the flux path in a step
+    unsigned* act_count = nullptr;     // 2 words, 0 between steps
     // shape of the steps that run without activity bytes (launch_step_raw for
     // other buffers: adjoint, frozen time steps); equals the cfg shape when
     // activity is off

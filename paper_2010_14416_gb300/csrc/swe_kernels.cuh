@@ -47,6 +47,7 @@ __host__ __device__ __forceinline__ bool code_ok(int code, long long n, int n_gr
 
 constexpr int kBcWall = 0, kBcInflow = 1, kBcTransmissive = 2, kBcStage = 3;
 
+constexpr int kScanBlock = 256;   // threads of act_scan_kernel, 16 cells each
 constexpr int kEnsPad = 256;  // ensemble members are padded to whole multiples of this many cells
 
 template <typename T>
@@ -88,6 +89,8 @@ struct StepArgs {
     const unsigned char* act_in;
     unsigned char* act_next;
     unsigned char* act_clear;
+    unsigned* act_list;                // cells that run the flux path (act_scan_kernel), in [0, *act_count)
+    unsigned* act_count;               // and a count of the blocks that have used it; both 0 between steps
     // edge pass (step_kernel with EDGES): interior edges in canonical orientation,
     // evaluated once per step by edge_flux_kernel before the cell pass
     const int2* ecells;                // (left, right) cell of each interior edge
@@ -940,136 +943,160 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
 // record or its neighbours' states -- the same result the neighbour test of
 // update_cell gives, bit for bit.
 //
-// Per-thread cp.async pipeline over the thread's cells c_k = i0 + k stride:
-// iteration k issues the topology of c_{k+1} (only if its byte is set), then
-// the activity bytes of c_{k+PF+1} (8 lanes copy the warp's 32 bytes) and the
-// state record of c_{k+PF}; it then processes c_k.  PF (the prefetch
-// distance of the streamed state, >= 2) is a compiled shape parameter.
+// Two launches.  act_scan_kernel reads the bytes (2 per cell, 16 cells a
+// thread) and gathers the cells that run the flux path into a list, a block's
+// 4,096 cells in their order; a quiet cell costs it nothing more unless its
+// state has to be written: where the cell was quiet in the previous step too,
+// the output buffer (the state of two steps ago, itself dry at rest with the
+// same h) holds it already.  step_kernel_act then updates the listed cells,
+// dealt evenly to the threads.  On a mostly dry mesh the channel's cells lie
+// together in the mesh order, so dealing out the cells by their place instead
+// leaves some SMs with several times the average work and makes every quiet
+// cell cost a state record read: that kernel, a cp.async pipeline over all
+// cells, took 96 us a step on the 13M-cell river, 6 % of it wet.
+template <typename T>
+__global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> a) {
+    const long long c0 = ((long long)blockIdx.x * kScanBlock + threadIdx.x) * 16;
+    const bool in = c0 < a.n;
+    uint4 now = make_uint4(0u, 0u, 0u, 0u), prev = now;
+    if (in) {
+        now = *(const uint4*)(a.act_in + c0);      // the buffers reach past n in whole 32 bytes
+        prev = *(const uint4*)(a.act_clear + c0);
+    }
+    // whether there is a step (warp_step_dt), by the bits alone: in 25,000 warps
+    // of a 13M-cell mesh an FP64 product each takes microseconds
+    const double dt = a.dt_fixed ? *a.dt_fixed : *a.dt_read;
+    if (!((unsigned long long)__double_as_longlong(dt) < kInfBits)) {
+        // no step: the state and its activity carry over unchanged
+        if (in) {
+            *(uint4*)(a.act_next + c0) = now;
+            *(uint4*)(a.act_clear + c0) = make_uint4(0u, 0u, 0u, 0u);
+            for (long long c = c0; c < c0 + 16 && c < a.n; ++c) a.s_out[c] = a.s_in[c];
+        }
+        return;
+    }
+    // bit 0 of a byte: the cell runs the flux path in this step; a previous
+    // byte that is not 0: it ran it in the previous step, or the bytes were
+    // rebuilt less than two steps ago
+    const unsigned w[4] = {now.x, now.y, now.z, now.w}, v[4] = {prev.x, prev.y, prev.z, prev.w};
+    // the low bits of a word's four bytes, as a 4-bit number
+    auto low_bits = [](unsigned x) { return ((x & 0x01010101u) * 0x01020408u) >> 24; };
+    unsigned runs = 0u, rewrite = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        runs |= low_bits(w[q]) << (4 * q);
+        rewrite |= low_bits(v[q] | (v[q] >> 1)) << (4 * q);   // bytes are 0 to 3
+    }
+    if (rewrite) *(uint4*)(a.act_clear + c0) = make_uint4(0u, 0u, 0u, 0u);
+    rewrite &= ~runs;
+    // a warp whose 512 cells are all to be rewritten (the two steps after the
+    // bytes are rebuilt) copies them side by side
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (__all_sync(0xffffffffu, rewrite == 0xFFFFu && c0 + 16 <= a.n)) {
+        const long long w0 = c0 - 16 * lane;
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            V4<T> s = a.s_in[w0 + 32 * k + lane];
+            s.y = T(0); s.z = T(0);
+            a.s_out[w0 + 32 * k + lane] = s;
+        }
+    } else {
+        for (unsigned m = rewrite; m; m &= m - 1u) {
+            const long long c = c0 + __ffs(m) - 1;
+            if (c < a.n) {
+                V4<T> s = a.s_in[c];
+                s.y = T(0); s.z = T(0);
+                a.s_out[c] = s;
+            }
+        }
+    }
+    const unsigned cnt = __popc(runs);
+    if (!__syncthreads_or(cnt)) return;
+    unsigned pos = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned up = __shfl_up_sync(0xffffffffu, pos, o);
+        if (lane >= o) pos += up;
+    }
+    __shared__ unsigned total[kScanBlock / 32], base;
+    if (lane == 31) total[warp] = pos;
+    __syncthreads();
+    unsigned before = 0u, all = 0u;
+#pragma unroll
+    for (int q = 0; q < kScanBlock / 32; ++q) {
+        if (q == warp) before = all;
+        all += total[q];
+    }
+    if (threadIdx.x == 0) base = atomicAdd(a.act_count, all);
+    __syncthreads();
+    unsigned at = base + before + pos - cnt;
+    for (unsigned m = runs; m; m &= m - 1u) a.act_list[at++] = (unsigned)c0 + __ffs(m) - 1;
+}
+
+// The listed cells' update and marks.  Each thread keeps the state and
+// topology records of its next PF - 1 entries in flight through cp.async into
+// its own shared-memory slots.
 template <typename T, int BLOCK, int MINB, bool GEO_EARLY, int PF>
 __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_act(const StepArgs<T> a) {
     static_assert(BLOCK % 32 == 0, "warps of whole cells");
-    static_assert(PF >= 2, "the wait counts below assume a prefetch distance of at least two cells");
-    constexpr int NS = PF + 1;  // state and activity slots
+    static_assert(PF >= 2, "at least one entry ahead");
     const WarpDt<T> wdt = warp_step_dt<T>(a.cfl, a.dt_read, a.dt_fixed);
-    const double dt_d = wdt.d;
     const bool have_dt = wdt.have;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *a.dt_reset = kInfBits;
-        if (have_dt) *a.t += dt_d;
+        if (have_dt) *a.t += wdt.d;
         else atomicOr(a.status, kStatusDry);
-        if (a.dt_log) *a.dt_log = dt_d;
+        if (a.dt_log) *a.dt_log = wdt.d;
     }
     T cand = inf_of<T>();
     unsigned active = 0u;
-    // 32-bit cell indices: the host allows this kernel only for n < 2^29, so
-    // c + (PF + 1) stride < 2^32 with stride <= n + BLOCK and PF <= 5
+    const int tid = threadIdx.x;
     const unsigned stride = gridDim.x * BLOCK;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned i0 = blockIdx.x * BLOCK + tid;
-    const unsigned n = (unsigned)a.n;
-    if (!have_dt) {
-        // no step: the state and its activity carry over unchanged
-        for (unsigned c = i0; c < n; c += stride) {
-            a.s_out[c] = a.s_in[c];
-            a.act_next[c] = a.act_in[c];
-            a.act_clear[c] = 0;
+    const unsigned n_list = have_dt ? *(volatile const unsigned*)a.act_count : 0u;
+    __shared__ V4<T> st_own[PF][BLOCK];
+    __shared__ int4 st_topo[PF][BLOCK];
+    __shared__ unsigned st_cell[PF][BLOCK];
+    auto fetch = [&](int slot, unsigned k) {
+        if (k < n_list) {
+            const unsigned c = a.act_list[k];
+            st_cell[slot][tid] = c;
+            cp_async_record<sizeof(V4<T>)>(&st_own[slot][tid], &a.s_in[c]);
+            cp_async_record<16>(&st_topo[slot][tid], &a.topo[c]);
         }
-    } else {
-        static_assert(PF <= 5, "32-bit indices");
-        __shared__ V4<T> st_own[NS][BLOCK];
-        __shared__ int4 st_topo[2][BLOCK];
-        __shared__ unsigned st_act[NS][BLOCK / 4];  // 32 activity bytes per warp per stage
-        __shared__ unsigned st_prev[NS][BLOCK / 4]; // and the previous step's (act_clear) bytes
-        const T dt = wdt.t;
-        // warp w of the block owns st_act[.][8 w .. 8 w + 7]; lanes 0..7 copy 4 bytes each
-        auto act_copy = [&](int slot, unsigned c) {
-            const unsigned base = c - lane;
-            if (lane < 8 && base < n) {
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
-                                 (unsigned)__cvta_generic_to_shared(&st_act[slot][warp * 8 + lane])),
-                             "l"(a.act_in + base + 4 * lane)
-                             : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
-                                 (unsigned)__cvta_generic_to_shared(&st_prev[slot][warp * 8 + lane])),
-                             "l"(a.act_clear + base + 4 * lane)
-                             : "memory");
-            }
-        };
-        // bit 0: the cell runs the flux path in this step (bit 0 of its byte);
-        // bit 1: the previous step's byte is not 0 (the cell ran the flux path
-        // then, or the bytes were rebuilt less than two steps ago)
-        auto act_byte = [&](int slot) -> unsigned {
-            return (((const unsigned char*)&st_act[slot][warp * 8])[lane] & 1u) |
-                   (((const unsigned char*)&st_prev[slot][warp * 8])[lane] ? 2u : 0u);
-        };
-        // prologue: activity of c_0 .. c_PF and states of c_0 .. c_{PF-1}; then topology of c_0
-#pragma unroll
-        for (int q = 0; q <= PF; ++q) act_copy(q, i0 + q * stride);
-#pragma unroll
-        for (int q = 0; q < PF; ++q)
-            if (i0 + q * stride < n) cp_async_record<sizeof(V4<T>)>(&st_own[q][tid], &a.s_in[i0 + q * stride]);
         cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
-        unsigned f_cur = act_byte(0);
-        if ((f_cur & 1u) && i0 < n) cp_async_record<16>(&st_topo[0][tid], &a.topo[i0]);
-        cp_async_commit();                                       // T_{-1}
-        cp_async_commit();                                       // H_{-1} (empty: its copies were in the first group)
-        int ks = 0, k2 = 0;  // k mod NS, k mod 2
-        for (unsigned c = i0; c - lane < n; c += stride) {
-            const int ks1 = ks + 1 == NS ? 0 : ks + 1;          // slot of c_{k+1}
-            const int ksp = ks == 0 ? NS - 1 : ks - 1;          // slot of c_{k+PF} (c_{k-1}'s, consumed)
-            // groups so far: ..., T_{k-1}, H_{k-1}; H_{k-PF} and older (activity of
-            // c_{k+1}, state of c_k) must be complete, which H_{k-2} implies
-            cp_async_wait<2>();
-            __syncwarp();
-            const unsigned f_next = act_byte(ks1);
-            const unsigned c1 = c + stride, cp = c + PF * stride, cp1 = c + (PF + 1) * stride;
-            if ((f_next & 1u) && c1 < n) cp_async_record<16>(&st_topo[k2 ^ 1][tid], &a.topo[c1]);
-            cp_async_commit();                                   // T_k
-            __syncwarp();                                        // every lane has read slot ks before it refills
-            act_copy(ks, cp1);
-            if (cp < n) cp_async_record<sizeof(V4<T>)>(&st_own[ksp][tid], &a.s_in[cp]);
-            cp_async_commit();                                   // H_k
-            cp_async_wait<3>();                                  // T_{k-1}: the topology of c_k
-            if (c < n) {
-                const V4<T> own = st_own[ks][tid];
-                if (!(f_cur & 1u)) {
-                    // quiet: the new state is (h, 0, 0); if the cell was quiet in the
-                    // previous step too, the output buffer (the state of two steps
-                    // ago, itself dry at rest with the same h) holds it already
-                    if (f_cur & 2u) {
-                        V4<T> out;
-                        out.x = own.x; out.y = T(0); out.z = T(0); out.w = own.w;
-                        a.s_out[c] = out;
-                    }
-                } else {
-                    const T r = update_cell<T, GEO_EARLY>(a, c, own, st_topo[k2][tid], dt, active, a.n_clamped,
-                                                          a.status);
-                    cand = min_nonneg(cand, r);
-                    const bool wet = r < inf_of<T>();
-                    // the topology record is read again from shared memory rather than kept
-                    // live in registers across the update
-                    const volatile int* tv = (const volatile int*)&st_topo[k2][tid];
-                    if (wet || (tv[3] & kStaticBit)) a.act_next[c] = 1;
-                    if (wet) {
+    };
+    unsigned k = blockIdx.x * BLOCK + tid;   // host: n < 2^29, so k + PF stride < 2^32
 #pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-                            const int code = tv[j];
-                            if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups)))
-                                a.act_next[code & kNbrMask] = 1;
-                        }
-                    }
-                }
-                a.act_clear[c] = 0;
+    for (int s = 0; s < PF - 1; ++s) fetch(s, k + s * stride);
+    const T dt = wdt.t;
+    int slot = 0;
+    for (; k < n_list; k += stride) {
+        fetch(slot == 0 ? PF - 1 : slot - 1, k + (PF - 1) * stride);
+        cp_async_wait<PF - 1>();
+        const unsigned c = st_cell[slot][tid];
+        const V4<T> own = st_own[slot][tid];
+        const T r = update_cell<T, GEO_EARLY>(a, c, own, st_topo[slot][tid], dt, active, a.n_clamped, a.status);
+        cand = min_nonneg(cand, r);
+        const bool wet = r < inf_of<T>();
+        // the topology record and the cell are read again from shared memory
+        // rather than kept live in registers across the update
+        const volatile int* tv = (const volatile int*)&st_topo[slot][tid];
+        if (wet || (tv[3] & kStaticBit)) a.act_next[((const volatile unsigned*)st_cell[slot])[tid]] = 1;
+        if (wet) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int code = tv[j];
+                if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups))) a.act_next[code & kNbrMask] = 1;
             }
-            f_cur = f_next;
-            ks = ks1;
-            k2 ^= 1;
         }
-        cp_async_wait<0>();
+        slot = slot == PF - 1 ? 0 : slot + 1;
     }
-    block_min_publish<BLOCK>(cand, a.dt_write, active, a.n_active);
+    cp_async_wait<0>();
+    block_min_publish<BLOCK>(cand, a.dt_write, active, a.n_active);   // (a barrier: every thread has read the count)
+    // the last block to get here empties the list for the next scan
+    if (tid == 0 && atomicAdd(a.act_count + 1, 1u) == gridDim.x - 1) {
+        a.act_count[0] = 0u;
+        a.act_count[1] = 0u;
+    }
 }
 
 // Activity bytes of a state (into a buffer filled with 2): a wet cell marks

@@ -32,8 +32,8 @@ static inline unsigned grid_for(long long n, int block) {
 constexpr int kEdgeBlock = 256;
 
 // (block, min blocks per SM, geometry early, stages) shapes of the activity
-// kernel; stages = the state's prefetch distance + 1.  Shared memory per
-// thread: `stages` state records and activity bytes, 2 topology records.
+// kernel; stages - 1 = list entries whose records a thread holds or has in
+// flight (state, topology and index in shared memory).
 #define SWE_ACT_VARIANTS_F32(X)                                                                     \
     X(128, 8, 0, 3) X(256, 4, 0, 3) X(512, 2, 0, 3) X(128, 8, 1, 3) X(256, 4, 1, 3) X(128, 8, 1, 4) \
     X(128, 8, 1, 5) X(256, 4, 1, 4) X(128, 8, 0, 4)
@@ -51,6 +51,9 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
     const unsigned grid = a.grid;
     if (grid == 0) return cudaErrorInvalidValue;
     if (a.act_in) {
+        act_scan_kernel<T><<<grid_for<T>(a.n, 16 * kScanBlock), kScanBlock, 0, st>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_ACT(B, M, G, S) \
     if (block == B && min_blocks == M && geo_early == G && stages == S) {         \
         step_kernel_act<T, B, M, G != 0, S - 1><<<grid, B, 0, st>>>(a);          \

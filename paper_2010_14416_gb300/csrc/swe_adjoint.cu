@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "swe_dual.cuh"
@@ -688,6 +689,41 @@ struct DevBuf {
     ~DevBuf() { if (p) cudaFree(p); }
 };
 
+// The buffers of one adjoint call, laid out in one allocation that the mesh
+// keeps (up to kAdjKeep) for its next call: allocating and freeing them took
+// 0.4 ms a call and more with the checkpoints' size.
+constexpr size_t kAdjKeep = (size_t)3 << 29;   // 1.5 GiB of the device's 280
+struct AdjArena {
+    swe_mesh* m;
+    std::vector<std::pair<void**, size_t>> parts;   // (pointer, offset)
+    size_t bytes = 0;
+    explicit AdjArena(swe_mesh* mesh) : m(mesh) {}
+    void add(void** p, size_t b) {
+        parts.push_back({p, bytes});
+        bytes += (std::max<size_t>(b, 16) + 255) / 256 * 256;
+    }
+    cudaError_t place() {
+        cudaError_t e = cudaSuccess;
+        if (m->adj_bytes < bytes) {
+            drop_adjoint_workspace(m);
+            e = cudaMalloc(&m->adj_arena, bytes);
+            if (e != cudaSuccess) {
+                m->adj_arena = nullptr;
+                return e;
+            }
+            m->adj_bytes = bytes;
+        }
+        for (auto& q : parts) *q.first = (char*)m->adj_arena + q.second;
+        return e;
+    }
+    // nothing uses the buffers after the call (it may leave early, and the
+    // mesh may change its stream before the next)
+    ~AdjArena() {
+        cudaStreamSynchronize(m->stream);
+        if (m->adj_bytes > kAdjKeep) drop_adjoint_workspace(m);
+    }
+};
+
 struct AdjDeviceGuard {
     int prev = -1;
     explicit AdjDeviceGuard(int dev) {
@@ -724,91 +760,108 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         if (gauge_cells[k] < 0 || gauge_cells[k] >= n) { set_error("swe_adjoint: gauge cell out of range"); return SWE_EINVAL; }
         gint[k] = m->hm.inv[gauge_cells[k]];
     }
-    const int K = checkpoint_every > 0 ? checkpoint_every : 50;
-    const int64_t nseg = (nsteps + K - 1) / K;
     AdjDeviceGuard dg(m->cfg.device);
     int rc = flush_mesh_bc(m);
     if (rc) return rc;
     cudaStream_t st = m->stream;
     const size_t sb = (size_t)n * sizeof(V4<double>);
-    DevBuf ckpt, seg, dtlog, small, lam, aw, nu, gmv, gzv, dg_idx, dtarget, dloss, ed;
     const bool transposes = m->adjoint_method == SWE_ADJOINT_TRANSPOSE;
     if (transposes) {   // the interior edge list of the edge-by-edge reverse step
         rc = build_edges(m);
         if (rc) return rc;
     }
+    // With the edge pass, a segment's steps keep their edge terms (40 B per
+    // interior edge and step), so phase 1 reads those of U^n that the step
+    // n -> n+1 formed instead of running the edge pass again; without room for
+    // them, phase 1 runs it.
+    const bool edges = m->plain.edges && m->eflux;
+    const size_t Eb = (size_t)std::max<int64_t>(m->n_edges, 1);
+    bool keep = edges && transposes;
+    void *p_ckpt, *p_seg, *p_dtlog, *p_small, *p_lam, *p_aw, *p_nu, *p_gm, *p_gz, *p_idx, *p_target, *p_loss, *p_ed,
+        *p_flux = nullptr, *p_src = nullptr;
     cudaError_t e = cudaSuccess;
-    auto alloc = [&](DevBuf& b, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(&b.p, bytes ? bytes : 16);
+    AdjArena arena(m);
+    // K steps a segment, segments recomputed from their checkpoints in reverse:
+    // one segment of all steps (nothing recomputed, the same bits) where its
+    // states and edge terms fit the kept workspace, else what was asked for.
+    const int K_asked = checkpoint_every > 0 ? checkpoint_every : 50;
+    int64_t K = K_asked;
+    auto layout = [&](int64_t k, bool with_flux) {
+        K = k;
+        arena.parts.clear();
+        arena.bytes = 0;
+        arena.add(&p_ckpt, (size_t)((nsteps + K - 1) / K) * sb);
+        arena.add(&p_seg, (size_t)K * sb);
+        arena.add(&p_dtlog, nsteps * sizeof(double));
+        arena.add(&p_small, kSmallWords * sizeof(unsigned long long));
+        for (void** p : {&p_lam, &p_aw, &p_nu}) arena.add(p, sb);
+        for (void** p : {&p_gm, &p_gz}) arena.add(p, n * sizeof(double));
+        arena.add(&p_idx, n_gauges * sizeof(long long));
+        arena.add(&p_target, (size_t)n_obs * n_gauges * sizeof(double));
+        arena.add(&p_loss, sizeof(double));
+        arena.add(&p_ed, transposes ? Eb * 2 * sizeof(V4<double>) : 0);
+        if (with_flux) {
+            arena.add(&p_flux, (size_t)K * Eb * sizeof(V4<double>));
+            arena.add(&p_src, (size_t)K * Eb * sizeof(double));
+        }
     };
-    alloc(ckpt, nseg * sb);
-    alloc(seg, (size_t)K * sb);
-    alloc(dtlog, nsteps * sizeof(double));
-    alloc(small, kSmallWords * sizeof(unsigned long long));
-    alloc(lam, sb);
-    alloc(aw, sb);
-    alloc(nu, sb);
-    alloc(gmv, n * sizeof(double));
-    alloc(gzv, n * sizeof(double));
-    alloc(dg_idx, n_gauges * sizeof(long long));
-    alloc(dtarget, (size_t)n_obs * n_gauges * sizeof(double));
-    alloc(dloss, sizeof(double));
-    if (transposes) alloc(ed, (size_t)std::max<int64_t>(m->n_edges, 1) * 2 * sizeof(V4<double>));
+    auto place = [&]() {
+        e = arena.place();
+        if (e != cudaSuccess) (void)cudaGetLastError();   // clear the failed allocation's error
+        return e == cudaSuccess;
+    };
+    layout(nsteps, keep);
+    if (nsteps <= K_asked || arena.bytes > kAdjKeep || !place()) {
+        layout(std::min<int64_t>(K_asked, nsteps), keep);
+        if (!place() && keep) {
+            keep = false;
+            layout(std::min<int64_t>(K_asked, nsteps), false);
+            place();
+        }
+    }
     if (e != cudaSuccess) {
         set_error(std::string("swe_adjoint: device allocation failed: ") + cudaGetErrorString(e));
         return SWE_ENOMEM;
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(dloss.p, 0, sizeof(double), st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dg_idx.p, gint.data(), n_gauges * sizeof(long long), cudaMemcpyHostToDevice, st);
+    const int64_t nseg = (nsteps + K - 1) / K;
+    if (e == cudaSuccess) e = cudaMemsetAsync(p_loss, 0, sizeof(double), st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p_idx, gint.data(), n_gauges * sizeof(long long), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(dtarget.p, targets, (size_t)n_obs * n_gauges * sizeof(double), cudaMemcpyHostToDevice, st);
-    const long long* gi = (const long long*)dg_idx.p;
-    const double* tg = (const double*)dtarget.p;
-    // With the edge pass, the recomputation of a segment keeps each step's edge
-    // fluxes (64 B per interior edge and step), so phase 1 reads the fluxes of
-    // U^n that the recomputed step n -> n+1 formed instead of running the edge
-    // pass again; without room for them, phase 1 runs it.
-    const bool edges = m->plain.edges && m->eflux;
-    DevBuf segflux, segsrc;
-    const size_t Eb = (size_t)std::max<int64_t>(m->n_edges, 1);
-    bool keep = edges && transposes;
-    if (keep) {
-        keep = cudaMalloc(&segflux.p, (size_t)K * Eb * sizeof(V4<double>)) == cudaSuccess &&
-               cudaMalloc(&segsrc.p, (size_t)K * Eb * sizeof(double)) == cudaSuccess;
-        if (!keep) (void)cudaGetLastError();   // clear the failed allocation's error
-    }
-    V4<double>* const sflux = (V4<double>*)segflux.p;
-    double* const ssrc = (double*)segsrc.p;
+        e = cudaMemcpyAsync(p_target, targets, (size_t)n_obs * n_gauges * sizeof(double), cudaMemcpyHostToDevice, st);
+    const long long* gi = (const long long*)p_idx;
+    const double* tg = (const double*)p_target;
+    V4<double>* const sflux = (V4<double>*)p_flux;
+    double* const ssrc = (double*)p_src;
     // forward run: checkpoints every K steps, step sizes logged, loss summed
     // over the observations.  The last segment's states (and, with the edge
     // pass, the fluxes its steps form) are kept as the reverse sweep's segment
     // buffer: recomputing them would give the same bits (the same kernels and
     // step sizes), so the reverse sweep starts without a recomputation.
     const int64_t last0 = (nseg - 1) * K;   // first step of the last segment
-    char* const segp = (char*)seg.p;
+    char* const segp = (char*)p_seg;
     for (int64_t s = 0; s < nsteps && e == cudaSuccess; ++s) {
         void* cur = m->state[m->nstep % 2];
         void* nxt = m->state[(m->nstep + 1) % 2];
-        if (s % K == 0) e = cudaMemcpyAsync((char*)ckpt.p + (s / K) * sb, cur, sb, cudaMemcpyDeviceToDevice, st);
+        if (s % K == 0) e = cudaMemcpyAsync((char*)p_ckpt + (s / K) * sb, cur, sb, cudaMemcpyDeviceToDevice, st);
         const bool in_last = s >= last0;
         if (e == cudaSuccess && in_last)
             e = cudaMemcpyAsync(segp + (s - last0) * sb, cur, sb, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess)
-            e = launch_step_raw(m, cur, nxt, m->small, m->nstep, cfl, nullptr, (double*)dtlog.p + s, st, false,
+            e = launch_step_raw(m, cur, nxt, m->small, m->nstep, cfl, nullptr, (double*)p_dtlog + s, st, false,
                                 keep && in_last ? (void*)(sflux + (s - last0) * Eb) : nullptr,
                                 keep && in_last ? (void*)(ssrc + (s - last0) * Eb) : nullptr);
         ++m->nstep;
         m->act_valid = false;   // stepped without the activity bytes
         if (e == cudaSuccess && (s + 1) % obs_every == 0) {
             adj_loss_kernel<<<1, 32, 0, st>>>((const V4<double>*)nxt, gi, tg + ((s + 1) / obs_every - 1) * n_gauges,
-                                             n_gauges, (double*)dloss.p);
+                                             n_gauges, (double*)p_loss);
             e = cudaGetLastError();
         }
     }
     if (e != cudaSuccess) return afail(e, "swe_adjoint: forward");
     std::vector<double> dts(nsteps);
     std::vector<unsigned long long> fstat(kSmallWords);
-    e = cudaMemcpyAsync(dts.data(), dtlog.p, nsteps * sizeof(double), cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(dts.data(), p_dtlog, nsteps * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(fstat.data(), m->small, kSmallWords * 8, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return afail(e, "swe_adjoint: forward");
@@ -821,15 +874,15 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         if (!std::isfinite(d)) { set_error("swe_adjoint: forward run went dry"); return SWE_EDRY; }
     if (dts_out) std::memcpy(dts_out, dts.data(), nsteps * sizeof(double));
     // lambda^N = d(last observation)/dU^N
-    e = cudaMemsetAsync(lam.p, 0, sb, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(gmv.p, 0, n * sizeof(double), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(gzv.p, 0, n * sizeof(double), st);
+    e = cudaMemsetAsync(p_lam, 0, sb, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p_gm, 0, n * sizeof(double), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p_gz, 0, n * sizeof(double), st);
     if (e == cudaSuccess) {
         adj_inject_kernel<<<1, 32, 0, st>>>((const V4<double>*)m->state[m->nstep % 2], gi,
-                                           tg + (n_obs - 1) * n_gauges, n_gauges, (V4<double>*)lam.p);
+                                           tg + (n_obs - 1) * n_gauges, n_gauges, (V4<double>*)p_lam);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) { small_init_kernel<<<1, 32, 0, st>>>((unsigned long long*)small.p); e = cudaGetLastError(); }
+    if (e == cudaSuccess) { small_init_kernel<<<1, 32, 0, st>>>((unsigned long long*)p_small); e = cudaGetLastError(); }
     if (e != cudaSuccess) return afail(e, "swe_adjoint: loss");
     AdjArgs a;
     a.geoA = (const V4<double>*)m->geoA;
@@ -837,11 +890,11 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     a.geoR = (const V4<double>*)m->geoR;
     a.topo = m->topo;
     a.gm2 = (const double*)m->gm2;
-    a.lam = (V4<double>*)lam.p;
-    a.aw = (V4<double>*)aw.p;
-    a.nu = (V4<double>*)nu.p;
-    a.gm = (double*)gmv.p;
-    a.gz = (double*)gzv.p;
+    a.lam = (V4<double>*)p_lam;
+    a.aw = (V4<double>*)p_aw;
+    a.nu = (V4<double>*)p_nu;
+    a.gm = (double*)p_gm;
+    a.gz = (double*)p_gz;
     a.n = n;
     a.g = m->cfg.g;
     a.h_dry = m->cfg.h_dry;
@@ -850,7 +903,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     a.n_edges = m->n_edges;
     a.debug = m->cfg.debug_checks;
     a.n_groups = m->n_groups;
-    a.status = (unsigned*)((unsigned long long*)small.p + kSlotStatus);
+    a.status = (unsigned*)((unsigned long long*)p_small + kSlotStatus);
     // with the edge pass, phase 1 takes R's interior fluxes from one evaluation per edge
     a.eflux = edges ? (const V4<double>*)m->eflux : nullptr;
     a.esrc = edges ? (const double*)m->esrc : nullptr;
@@ -858,7 +911,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     a.ecells = m->ecells;
     a.eln = (const double*)m->eln;
     a.erl = (const double*)m->erl;
-    a.ed = (V4<double>*)ed.p;
+    a.ed = (V4<double>*)p_ed;
     StepArgs<double> ea{};
     if (edges) {
         ea.ecells = m->ecells;
@@ -875,17 +928,21 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         ea.n_groups = a.n_groups;
         ea.status = a.status;
     }
-    const unsigned egrid = (unsigned)std::min<int64_t>((std::max<int64_t>(m->n_edges, 1) + 127) / 128, 65535);
-    const unsigned grid = (unsigned)((n + 127) / 128);
+    // one-warp blocks on a small mesh: 128 threads leave some SMs with twice the
+    // others' share (step_threads has the measurements)
+    const unsigned eblock = m->n_edges <= kSpreadCells ? 32 : 128, block = n <= kSpreadCells ? 32 : 128;
+    const unsigned egrid =
+        (unsigned)std::min<int64_t>((std::max<int64_t>(m->n_edges, 1) + eblock - 1) / eblock, 65535);
+    const unsigned grid = (unsigned)((n + block - 1) / block);
     // reverse sweep, segment by segment
     for (int64_t sgi = nseg - 1; sgi >= 0 && e == cudaSuccess; --sgi) {
         const int64_t n0 = sgi * K, n1 = std::min<int64_t>(n0 + K, nsteps);
         const bool from_forward = sgi == nseg - 1;   // the forward run kept this segment
         if (!from_forward)
-            e = cudaMemcpyAsync(segp, (char*)ckpt.p + sgi * sb, sb, cudaMemcpyDeviceToDevice, st);
+            e = cudaMemcpyAsync(segp, (char*)p_ckpt + sgi * sb, sb, cudaMemcpyDeviceToDevice, st);
         for (int64_t k = 0; !from_forward && k + 1 < n1 - n0 && e == cudaSuccess; ++k)
-            e = launch_step_raw(m, segp + k * sb, segp + (k + 1) * sb, (unsigned long long*)small.p, k, cfl,
-                                (const double*)dtlog.p + n0 + k, nullptr, st, false,
+            e = launch_step_raw(m, segp + k * sb, segp + (k + 1) * sb, (unsigned long long*)p_small, k, cfl,
+                                (const double*)p_dtlog + n0 + k, nullptr, st, false,
                                 keep ? (void*)(sflux + k * Eb) : nullptr, keep ? (void*)(ssrc + k * Eb) : nullptr);
         if (keep && !from_forward && e == cudaSuccess) {   // the segment's last state has no recomputed step
             const int64_t k = n1 - n0 - 1;
@@ -900,22 +957,22 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
             if (keep) {
                 a.eflux = sflux + k * Eb;
                 a.esrc = ssrc + k * Eb;
-                adj_phase1_kernel<true, true><<<grid, 128, 0, st>>>(a);
+                adj_phase1_kernel<true, true><<<grid, block, 0, st>>>(a);
             } else if (edges) {
                 ea.s_in = a.U;
                 e = Launch<double>::edge_flux(ea, st);
                 if (e != cudaSuccess) break;
-                if (transposes) adj_phase1_kernel<true, true><<<grid, 128, 0, st>>>(a);
-                else adj_phase1_kernel<true, false><<<grid, 128, 0, st>>>(a);
+                if (transposes) adj_phase1_kernel<true, true><<<grid, block, 0, st>>>(a);
+                else adj_phase1_kernel<true, false><<<grid, block, 0, st>>>(a);
             } else {
-                if (transposes) adj_phase1_kernel<false, true><<<grid, 128, 0, st>>>(a);
-                else adj_phase1_kernel<false, false><<<grid, 128, 0, st>>>(a);
+                if (transposes) adj_phase1_kernel<false, true><<<grid, block, 0, st>>>(a);
+                else adj_phase1_kernel<false, false><<<grid, block, 0, st>>>(a);
             }
             if (transposes) {
-                adj_edge_kernel<<<egrid, 128, 0, st>>>(a);
-                adj_cell_kernel<<<grid, 128, 0, st>>>(a);
+                adj_edge_kernel<<<egrid, eblock, 0, st>>>(a);
+                adj_cell_kernel<<<grid, block, 0, st>>>(a);
             } else {
-                adj_phase2_kernel<<<grid, 128, 0, st>>>(a);
+                adj_phase2_kernel<<<grid, block, 0, st>>>(a);
             }
             const int64_t nn = n0 + k;  // lambda now holds lambda^nn
             if (nn > 0 && nn % obs_every == 0)
@@ -926,7 +983,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     if (e != cudaSuccess) return afail(e, "swe_adjoint: reverse sweep");
     if (m->cfg.debug_checks) {
         unsigned long long rs[kSmallWords];
-        e = cudaMemcpyAsync(rs, small.p, sizeof rs, cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(rs, p_small, sizeof rs, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return afail(e, "swe_adjoint: reverse sweep status");
         if (rs[kSlotStatus] & kStatusBadIndex) {
@@ -936,16 +993,16 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     }
     // outputs
     if (where == SWE_DEVICE) {
-        adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)gmv.p, (const double*)gzv.p,
+        adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)p_gm, (const double*)p_gz,
                                                                        (const double*)m->gm2, m->perm, m->cfg.g,
                                                                        grad_manning, grad_bathy, n);
         e = cudaGetLastError();
     } else {
         DevBuf om, oz;
-        alloc(om, n * sizeof(double));
-        alloc(oz, n * sizeof(double));
+        e = cudaMalloc(&om.p, n * sizeof(double));
+        if (e == cudaSuccess) e = cudaMalloc(&oz.p, n * sizeof(double));
         if (e == cudaSuccess) {
-            adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)gmv.p, (const double*)gzv.p,
+            adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)p_gm, (const double*)p_gz,
                                                                            (const double*)m->gm2, m->perm, m->cfg.g,
                                                                            (double*)om.p, (double*)oz.p, n);
             e = cudaGetLastError();
@@ -956,13 +1013,19 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
             e = cudaMemcpyAsync(grad_bathy, oz.p, n * sizeof(double), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(loss, dloss.p, sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(loss, p_loss, sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return afail(e, "swe_adjoint: output");
     return SWE_OK;
 }
 
 }  // namespace
+
+void swe::drop_adjoint_workspace(swe_mesh* m) {
+    if (m->adj_arena) cudaFree(m->adj_arena);
+    m->adj_arena = nullptr;
+    m->adj_bytes = 0;
+}
 
 extern "C" {
 

@@ -583,6 +583,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     if (m->stream) cudaStreamSynchronize(m->stream);
     drop_graph(m);
     drop_diag_workspace(m);
+    drop_adjoint_workspace(m);
     void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
                     m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count};

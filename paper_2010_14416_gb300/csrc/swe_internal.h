@@ -109,6 +109,8 @@ constexpr int64_t kActivityMaxCells = int64_t(1) << 29;
 int flush_mesh_bc(swe_mesh* m);
 // The error code (and message) of a status word.
 int status_code(unsigned long long status);
+// Frees m's adjoint workspace.
+void drop_adjoint_workspace(swe_mesh* m);
 // Frees m's diagnostics workspace.
 void drop_diag_workspace(swe_mesh* m);
 // Drops m's captured CUDA graph (after a change of launch shape).
@@ -163,6 +165,9 @@ struct swe_mesh {
     void* eflux = nullptr;             // V4<T>[E]
     void* esrc = nullptr;              // T[E]
     int4* eidx = nullptr;              // per cell, the edge of each local edge (-1: boundary)
+    // adjoint workspace (swe_adjoint.cu), kept between calls
+    void* adj_arena = nullptr;
+    size_t adj_bytes = 0;
     // diagnostics workspace (swe_diag.cu)
     double *diag_dev = nullptr, *diag_partial = nullptr, *diag_host = nullptr;
     long long* diag_slots = nullptr;

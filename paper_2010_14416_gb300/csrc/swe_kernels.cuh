@@ -209,8 +209,7 @@ __device__ __forceinline__ void riemann_hllc(T hL, T unL, T utL, T hR, T unR, T 
         f32::riemann<float>(hL, unL, utL, hR, unR, utR, g, f32::mul(0.5f, g), h_dry, G1, G2, G3, speeds, hll_only);
         return;
     } else if constexpr (std::is_same<T, double>::value) {   // FP64: swe_f64.cuh
-        double PL, PR;
-        f64::riemann<false>(hL, unL, utL, hR, unR, utR, 0.5 * g, h_dry, 1.0, G1, G2, G3, PL, PR, speeds, hll_only);
+        f64::riemann_any(hL, unL, utL, hR, unR, utR, 0.5 * g, h_dry, G1, G2, G3, speeds, hll_only);
         return;
     } else {
     using A = Ar<T>;
@@ -717,10 +716,10 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
     double m = 0.0, x = 0.0, y = 0.0;
     int4 ei = make_int4(-1, -1, -1, 0);
     if constexpr (EDGES) ei = a.eidx[i];
-#pragma unroll
+#pragma unroll(EDGES ? 3 : 1)   // an edge's evaluation is some 2,500 instructions
     for (int j = 0; j < 3; ++j) {
-        const int c = code[j];
-        const V4<double> o = nb[j];
+        const int c = j == 0 ? code[0] : (j == 1 ? code[1] : code[2]);
+        const V4<double> o = j == 0 ? nb[0] : (j == 1 ? nb[1] : nb[2]);
         const double n1 = j == 0 ? gA.x : (j == 1 ? gA.z : gB.x);   // this cell's outward unit normal
         const double n2 = j == 0 ? gA.y : (j == 1 ? gA.w : gB.y);
         const double len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);

@@ -92,67 +92,74 @@ __device__ __forceinline__ void edge_geo(const V4<double>& gA, const V4<double>&
 // (dh, dqx, dqy), the adjoints w[0..6] of the seven inputs, in the order of
 // the dual-number seeds.  Reciprocals and roots as in the forward
 // (swe_f64.cuh): the FP64 pipe bounds this kernel too.
-__device__ void friction_rev(double hi, double qx, double qy, double gm2, double Rh, double Rx, double Ry, double dt,
-                             double h_dry, double bdh, double bdqx, double bdqy, double w[7]) {
-    const double qq = f64::fma(qx, qx, f64::mul(qy, qy));
+template <class A>
+__device__ __forceinline__ void friction_rev(double hi, double qx, double qy, double gm2, double Rh, double Rx,
+                                             double Ry, double dt, double h_dry, double bdh, double bdqx, double bdqy,
+                                             double w[7]) {
+    using f64::add, f64::fma;
+    const double qq = fma(qx, qx, A::mul(qy, qy));
     const bool act = gt_pos(hi, h_dry) && gt_zero(gm2) && gt_pos(qq, 1e-300);
 #pragma unroll
     for (int k = 0; k < 7; ++k) w[k] = 0.0;
     if (!act) {
-        w[4] = bdh * dt; w[5] = bdqx * dt; w[6] = bdqy * dt;
+        w[4] = A::mul(bdh, dt); w[5] = A::mul(bdqx, dt); w[6] = A::mul(bdqy, dt);
         return;
     }
-    const double dh = dt * Rh, dqx0 = dt * Rx, dqy0 = dt * Ry;
+    const double dh = A::mul(dt, Rh);
     // forward
     double rq;
-    const double qn = f64::sqrt_rsqrt(qq, rq);                  // |q|, 1/|q|
-    const double r = f64::rcbrt(hi);
-    const double rh = r * r * r;                                // 1/h
-    const double p = rh * rh * r;                               // h^(-7/3)
-    const double cf = gm2 * p;
-    const double dtc = dt * cf, al = f64::half(dtc);
-    const double P = (7.0 / 6.0) * dh * rh - 1.0;
-    const double c1 = dtc * qn, k = c1 * P;
-    const double bx = dqx0 + k * qx, by = dqy0 + k * qy;
-    const double rd1 = f64::rcp(f64::fma(0.5, c1, 1.0)), rd2 = f64::rcp(1.0 + c1);
-    const double rqd2 = rq * rd2;
-    const double S = bx * qx + by * qy;
-    const double proj = S * al * rqd2;
+    const double qn = A::sqrt_rsqrt(qq, rq);                    // |q|, 1/|q|
+    const double r = f64::rcbrt<A>(hi);
+    const double rh = A::mul(A::mul(r, r), r);                  // 1/h
+    const double p = A::mul(A::mul(rh, rh), r);                 // h^(-7/3)
+    const double cf = A::mul(gm2, p);
+    const double dtc = A::mul(dt, cf), al = f64::half(dtc);
+    const double dhr = A::mul(dh, rh);
+    const double P = fma(7.0 / 6.0, dhr, -1.0);
+    const double c1 = A::mul(dtc, qn), k = A::mul(c1, P);
+    const double bx = fma(k, qx, A::mul(dt, Rx)), by = fma(k, qy, A::mul(dt, Ry));
+    const double rd1 = A::rcp(fma(0.5, c1, 1.0)), rd2 = A::rcp(add(1.0, c1));
+    const double alq = A::mul(al, A::mul(rq, rd2));             // al / (|q| d2)
+    const double S = fma(bx, qx, A::mul(by, qy));
+    const double proj = A::mul(S, alq);
     // reverse: dq = (b - proj q) / d1
-    const double ox = (bx - proj * qx) * rd1, oy = (by - proj * qy) * rd1;
-    const double bd1 = -(bdqx * ox + bdqy * oy) * rd1;          // of d1, through 1/d1
-    double b_bx = bdqx * rd1, b_by = bdqy * rd1;
-    const double b_proj = -(b_bx * qx + b_by * qy);
-    double b_qx = -b_bx * proj, b_qy = -b_by * proj;
+    const double ox = A::mul(fma(-proj, qx, bx), rd1), oy = A::mul(fma(-proj, qy, by), rd1);
+    double b_bx = A::mul(bdqx, rd1), b_by = A::mul(bdqy, rd1);
+    const double bd1 = -fma(b_bx, ox, A::mul(b_by, oy));        // of d1, through 1/d1
+    const double b_proj = -fma(b_bx, qx, A::mul(b_by, qy));
+    double b_qx = -A::mul(b_bx, proj), b_qy = -A::mul(b_by, proj);
     // proj = S al / (|q| d2)
-    const double b_S = b_proj * al * rqd2;
-    const double b_pp = b_proj * proj;
-    double b_al = b_proj * S * rqd2;
-    b_bx += b_S * qx; b_qx += b_S * bx;
-    b_by += b_S * qy; b_qy += b_S * by;
-    double b_qn = -b_pp * rq;
-    const double b_d2 = -b_pp * rd2;
-    // d1 = 1 + al |q|, d2 = d1 + al |q|
-    const double b_aq = bd1 + b_d2 + b_d2;
-    b_al += b_aq * qn;
-    b_qn += b_aq * al;
+    const double b_S = A::mul(b_proj, alq);
+    const double b_pp = A::mul(b_proj, proj);
+    const double b_d2 = -A::mul(b_pp, rd2);
+    double b_qn = -A::mul(b_pp, rq);
+    // al in proj, and in d1 = 1 + al |q|, d2 = d1 + al |q|
+    const double b_aq = fma(2.0, b_d2, bd1);
+    const double b_al = fma(b_aq, qn, A::mul(A::mul(b_proj, S), A::mul(rq, rd2)));
+    b_qn = fma(b_aq, al, b_qn);
+    b_bx = fma(b_S, qx, b_bx); b_qx = fma(b_S, bx, b_qx);
+    b_by = fma(b_S, qy, b_by); b_qy = fma(b_S, by, b_qy);
     // b = dt R_q + k q
-    const double b_k = b_bx * qx + b_by * qy;
-    b_qx += b_bx * k; b_qy += b_by * k;
+    const double b_k = fma(b_bx, qx, A::mul(b_by, qy));
+    b_qx = fma(b_bx, k, b_qx); b_qy = fma(b_by, k, b_qy);
     // k = dt c |q| P, P = (7/6) dh / h - 1
-    const double b_kP = b_k * P;
-    const double b_cf = dt * (b_kP * qn + f64::half(b_al));
-    b_qn += b_kP * dtc;
-    const double b_P = b_k * c1 * (7.0 / 6.0);
-    const double b_dh = bdh + b_P * rh;
+    const double b_kP = A::mul(b_k, P);
+    const double b_cf = A::mul(dt, fma(b_kP, qn, f64::half(b_al)));
+    b_qn = fma(b_kP, dtc, b_qn);
+    const double b_P = A::mul(A::mul(b_k, c1), 7.0 / 6.0);
+    const double b_dh = fma(b_P, rh, bdh);
     // c = g m^2 h^(-7/3), 1/h, |q|
-    const double b_h = -rh * (b_P * dh * rh + (7.0 / 3.0) * b_cf * cf);
-    const double b_qq = b_qn * rq;
-    b_qx += b_qq * qx;
-    b_qy += b_qq * qy;
-    w[0] = b_h; w[1] = b_qx; w[2] = b_qy; w[3] = b_cf * p;
-    w[4] = b_dh * dt; w[5] = b_bx * dt; w[6] = b_by * dt;
+    const double b_qq = A::mul(b_qn, rq);
+    w[0] = -A::mul(rh, fma(b_P, dhr, A::mul(7.0 / 3.0, A::mul(b_cf, cf))));
+    w[1] = fma(b_qq, qx, b_qx);
+    w[2] = fma(b_qq, qy, b_qy);
+    w[3] = A::mul(b_cf, p);
+    w[4] = A::mul(b_dh, dt); w[5] = A::mul(b_bx, dt); w[6] = A::mul(b_by, dt);
 }
+
+// The range of adjoints (and of the forward's right-hand side) that Soft
+// takes: beyond it, and beyond the forward's ranges, the FP64 pipe.
+__device__ __forceinline__ bool soft_adjoint(double x) { return f64::in_range<-400, 200>(x); }
 
 // EDGES reads R_i's interior fluxes from the edge pass (the forward's own
 // edge-pass arithmetic) instead of evaluating them; R_i is the same bit for bit.
@@ -162,6 +169,16 @@ template <bool EDGES, bool TRANSPOSE>
 __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
+    const V4<double> L = a.lam[i];
+    if (TRANSPOSE && ((__double_as_longlong(L.x) | __double_as_longlong(L.y) | __double_as_longlong(L.z)) << 1) == 0LL &&
+        !a.debug) {
+        // a cell that no gauge's influence has reached yet passes nothing on
+        V4<double> zero;
+        zero.x = zero.y = zero.z = zero.w = 0.0;
+        a.aw[i] = zero;
+        a.nu[i] = zero;
+        return;
+    }
     const double g = a.g, h_dry = a.h_dry;
     const V4<double> own = a.U[i];
     const V4<double> gA = a.geoA[i], gB = a.geoB[i], gR = a.geoR[i];
@@ -218,7 +235,6 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
     }
     const double ia = gB.z;
     const double Rh = -m * ia, Rx = -x * ia, Ry = -y * ia;
-    const V4<double> L = a.lam[i];
     double lh = L.x, lx_ = L.y, ly_ = L.z;
     double w[7];
     if constexpr (TRANSPOSE) {
@@ -227,7 +243,14 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
         const double hn = f64::add(hi, -f64::mul(m, f64::mul(a.dt, ia)));   // f64::update
         if (hn < 0.0) { lh = 0.0; lx_ = 0.0; ly_ = 0.0; }
         else if (hn <= h_dry) { lx_ = 0.0; ly_ = 0.0; }
-        friction_rev(hi, own.y, own.z, a.gm2[i], Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
+        const double gm2 = a.gm2[i];
+        if (f64::in_range<-64, 24>(hi) && f64::in_range<-64, 24>(own.y) && f64::in_range<-64, 24>(own.z) &&
+            f64::in_range<-64, 16>(gm2) && f64::in_range<-64, 24>(a.dt) && f64::in_range<-192, 128>(Rh) &&
+            f64::in_range<-192, 128>(Rx) && f64::in_range<-192, 128>(Ry) && soft_adjoint(lh) && soft_adjoint(lx_) &&
+            soft_adjoint(ly_))
+            friction_rev<f64::SoftFlush>(hi, own.y, own.z, gm2, Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
+        else
+            friction_rev<f64::Hard>(hi, own.y, own.z, gm2, Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
     } else {
         // Phi on duals: seeds h, hu, hv, g m^2, Rh, Rx, Ry
         D7 dh, dqx, dqy;
@@ -328,196 +351,209 @@ __global__ void __launch_bounds__(128) adj_phase2_kernel(const AdjArgs a) {
 // duals.  The forward is recomputed here with the arithmetic of swe_f64.cuh,
 // whose reciprocals and inverse roots the reverse uses again (no division),
 // and every branch is taken as the forward takes it; the derivative of a max
-// at a tie is that of the operand the forward returns.
+// at a tie is that of the operand the forward returns.  The FP64 pipe bounds
+// these kernels too: products, reciprocals and roots run on the integer unit
+// (f64::SoftFlush), and an edge or cell whose adjoints are still zero is
+// passed over (48 steps back, 64 gauges have reached half of 250k cells):
+// 375k edges 188 us before, 1,181 us a step of that adjoint at first, 390
+// before these two, 192 with them.
 
 // Reverse of f64::riemann (Eq 17-26) at (hL, unL, utL, hR, unR, utR): adds
 // the adjoints of the six inputs for the flux adjoints (bG1, bG2, bG3).
+template <class A>
 __device__ __forceinline__ void riemann_rev(double hL, double unL, double utL, double hR, double unR, double utR,
                                             double g2, double h_dry, bool hll_only, double bG1, double bG2, double bG3,
                                             double& bhL, double& bunL, double& butL, double& bhR, double& bunR,
                                             double& butR) {
+    using f64::add, f64::sub, f64::fma;
     const bool wetL = gt_pos(hL, h_dry), wetR = gt_pos(hR, h_dry);
     if (!wetL && !wetR) return;   // no flux on either side
     const bool wet = wetL && wetR;
     // ---- forward values
-    const double ghL = f64::mul(g2, hL), ghR = f64::mul(g2, hR);
-    const double PL0 = f64::mul(ghL, hL), PR0 = f64::mul(ghR, hR);
+    const double ghL = A::mul(g2, hL), ghR = A::mul(g2, hR);
     double yL, yR;                                                              // 1/a_K (0 where a_K = 0)
-    const double aL = f64::sqrt_rsqrt(f64::twice(ghL), yL), aR = f64::sqrt_rsqrt(f64::twice(ghR), yR);
+    const double aL = A::sqrt_rsqrt(f64::twice(ghL), yL), aR = A::sqrt_rsqrt(f64::twice(ghR), yR);
     double SL, SR;
-    double hw = 0.0, w = 0.0, asum = 0.0, hsum = 0.0, rhw = 0.0, rh0 = 0.0, rL = 0.0, rR = 0.0, gL = 0.0, gR = 0.0,
-           ygL = 0.0, ygR = 0.0, rDg = 0.0, hs = 0.0, ycL = 0.0, ycR = 0.0;
+    double w = 0.0, hsum = 0.0, rhw = 0.0, rh0 = 0.0, rL = 0.0, rR = 0.0, gL = 0.0, gR = 0.0, ygL = 0.0, ygR = 0.0,
+           rDg = 0.0, hs = 0.0, ycL = 0.0, ycR = 0.0;
     bool shock = false, shL = false, shR = false;
     if (wet) {
-        SL = f64::sub(unL, aL);
-        SR = f64::add(unR, aR);
-        asum = f64::add(aL, aR);
-        hsum = f64::add(hL, hR);
-        const double du = f64::sub(unR, unL);
-        w = f64::fma(2.0, asum, -du);
-        hw = f64::mul(hsum, w);
+        SL = sub(unL, aL);
+        SR = add(unR, aR);
+        const double asum = add(aL, aR);
+        hsum = add(hL, hR);
+        const double du = sub(unR, unL);
+        w = fma(2.0, asum, -du);
+        const double hw = A::mul(hsum, w);
         const double asum4 = f64::four_times(asum);
-        shock = gt_pos(hw, f64::mul(min_nonneg(hL, hR), asum4));                // Eq 21
+        shock = gt_pos(hw, A::mul(min_nonneg(hL, hR), asum4));                  // Eq 21
         if (shock) {                                                            // Eq 23
-            rhw = f64::rcp(hw);
-            rh0 = f64::mul(asum4, rhw);
-            rL = f64::rcp(hL);
-            rR = f64::rcp(hR);
-            gL = f64::sqrt_rsqrt(f64::mul(g2, f64::add(rh0, rL)), ygL);
-            gR = f64::sqrt_rsqrt(f64::mul(g2, f64::add(rh0, rR)), ygR);
-            rDg = f64::rcp(f64::add(gL, gR));
-            hs = f64::mul(f64::fma(hL, gL, f64::fma(hR, gR, -du)), rDg);
-            const double ghs = f64::mul(g2, hs);
+            rhw = A::rcp(hw);
+            rh0 = A::mul(asum4, rhw);
+            rL = A::rcp(hL);
+            rR = A::rcp(hR);
+            gL = A::sqrt_rsqrt(A::mul(g2, add(rh0, rL)), ygL);
+            gR = A::sqrt_rsqrt(A::mul(g2, add(rh0, rR)), ygR);
+            rDg = A::rcp(add(gL, gR));
+            hs = A::mul(fma(hL, gL, fma(hR, gR, -du)), rDg);
+            const double ghs = A::mul(g2, hs);
             shL = gt_pos(hs, hL);
             shR = gt_pos(hs, hR);
-            if (shL) SL = f64::sub(unL, f64::sqrt_rsqrt(f64::mul(ghs, f64::fma(hs, rL, 1.0)), ycL));   // Eq 20
-            if (shR) SR = f64::add(unR, f64::sqrt_rsqrt(f64::mul(ghs, f64::fma(hs, rR, 1.0)), ycR));
+            if (shL) SL = sub(unL, A::sqrt_rsqrt(A::mul(ghs, fma(hs, rL, 1.0)), ycL));   // Eq 20
+            if (shR) SR = add(unR, A::sqrt_rsqrt(A::mul(ghs, fma(hs, rR, 1.0)), ycR));
         }
     } else if (wetL) {                                                          // Eq 26
-        SL = f64::sub(unL, aL);
-        SR = f64::fma(2.0, aL, unL);
+        SL = sub(unL, aL);
+        SR = fma(2.0, aL, unL);
     } else {
-        SL = f64::fma(-2.0, aR, unR);
-        SR = f64::add(unR, aR);
+        SL = fma(-2.0, aR, unR);
+        SR = add(unR, aR);
     }
-    const double qL = f64::mul(hL, unL), qR = f64::mul(hR, unR);
+    const double qL = A::mul(hL, unL), qR = A::mul(hR, unR);
     const bool supL = ge_zero(SL), supR = !supL && le_zero(SR);               // Eq 17
     // ---- reverse
     double bSL = 0.0, bSR = 0.0, bqL = 0.0, bqR = 0.0, bPL = 0.0, bPR = 0.0;
     if (supL || supR) {
-        const double q = supL ? qL : qR, ut = supL ? utL : utR;
-        double bq = bG1 + bG3 * ut;   // G3 = q ut for either flux
-        double but = bG3 * q;
-        if (supR && !hll_only && wetL && !wetR && ge_zero(SR)) {   // S* = S_R = 0: the left side's ut (Eq 24)
-            bq = bG1 + bG3 * utL;
-            but = 0.0;
-            butL += bG3 * q;
-        }
-        if (supL) { bqL = bq; bPL = bG2; butL += but; }
-        else { bqR = bq; bPR = bG2; butR += but; }
+        // G3 = q ut for either flux; where S* = S_R = 0 the left side's ut (Eq 24)
+        const bool left_ut = supL || (!hll_only && wetL && !wetR && ge_zero(SR));
+        const double q = supL ? qL : qR;
+        const double bq = fma(bG3, left_ut ? utL : utR, bG1);
+        if (left_ut) butL = fma(bG3, q, butL);
+        else butR = fma(bG3, q, butR);
+        if (supL) { bqL = bq; bPL = bG2; }
+        else { bqR = bq; bPR = bG2; }
     } else {
-        const double r = f64::rcp(f64::sub(SR, SL));
-        const double ss = f64::mul(SR, SL);
-        const double fL = f64::fma(qL, unL, PL0), fR = f64::fma(qR, unR, PR0);
-        const double dh = f64::sub(hR, hL), dq = f64::sub(qR, qL);
-        const double G1 = f64::mul(f64::fma(ss, dh, f64::fma(-SL, qR, f64::mul(SR, qL))), r);
-        const double G2 = f64::mul(f64::fma(ss, dq, f64::fma(-SL, fR, f64::mul(SR, fL))), r);
+        const double r = A::rcp(sub(SR, SL));
+        const double ss = A::mul(SR, SL);
+        const double fL = fma(qL, unL, A::mul(ghL, hL)), fR = fma(qR, unR, A::mul(ghR, hR));
+        const double dh = sub(hR, hL), dq = sub(qR, qL);
+        const double SRqL = A::mul(SR, qL);
+        const double G1 = A::mul(fma(ss, dh, fma(-SL, qR, SRqL)), r);
+        const double G2 = A::mul(fma(ss, dq, fma(-SL, fR, A::mul(SR, fL))), r);
         if (!hll_only) {                                                        // Eq 24
             const bool upL = wetL && (!wetR || ge_zero(G1));
-            bG1 += bG3 * (upL ? utL : utR);
-            if (upL) butL += bG3 * G1;
-            else butR += bG3 * G1;
+            bG1 = fma(bG3, upL ? utL : utR, bG1);
+            if (upL) butL = fma(bG3, G1, butL);
+            else butR = fma(bG3, G1, butR);
         } else {
-            const double tL = qL * utL, tR = qR * utR, dt3 = hR * utR - hL * utL;
-            const double G3 = (SR * tL - SL * tR + ss * dt3) * r;
-            const double bN3 = bG3 * r;
-            bSR += bN3 * (tL + SL * dt3 - G3);
-            bSL += bN3 * (SR * dt3 - tR + G3);
-            bqL += bN3 * SR * utL;
-            bqR -= bN3 * SL * utR;
-            butL += bN3 * (SR * qL - ss * hL);
-            butR += bN3 * (ss * hR - SL * qR);
-            bhR += bN3 * ss * utR;
-            bhL -= bN3 * ss * utL;
+            const double tL = A::mul(qL, utL), tR = A::mul(qR, utR), dt3 = fma(hR, utR, -A::mul(hL, utL));
+            const double G3 = A::mul(fma(ss, dt3, fma(-SL, tR, A::mul(SR, tL))), r);
+            const double bN3 = A::mul(bG3, r);
+            bSR = fma(bN3, sub(fma(SL, dt3, tL), G3), bSR);
+            bSL = fma(bN3, add(fma(SR, dt3, -tR), G3), bSL);
+            bqL = fma(A::mul(bN3, SR), utL, bqL);
+            bqR = fma(-A::mul(bN3, SL), utR, bqR);
+            butL = fma(bN3, fma(-ss, hL, SRqL), butL);
+            butR = fma(bN3, fma(ss, hR, -A::mul(SL, qR)), butR);
+            const double b3s = A::mul(bN3, ss);
+            bhR = fma(b3s, utR, bhR);
+            bhL = fma(-b3s, utL, bhL);
         }
         // G = N / (S_R - S_L)
-        const double bN1 = bG1 * r, bN2 = bG2 * r;
-        bSR += bN1 * (qL + SL * dh - G1) + bN2 * (fL + SL * dq - G2);
-        bSL += bN1 * (SR * dh - qR + G1) + bN2 * (SR * dq - fR + G2);
-        const double b2s = bN2 * ss, b1s = bN1 * ss;
-        bqL += bN1 * SR - b2s;
-        bqR += b2s - bN1 * SL;
-        bPL = bN2 * SR;
-        bPR = -bN2 * SL;
-        bhR += b1s;
-        bhL -= b1s;
+        const double bN1 = A::mul(bG1, r), bN2 = A::mul(bG2, r);
+        bSR = fma(bN1, sub(fma(SL, dh, qL), G1), fma(bN2, sub(fma(SL, dq, fL), G2), bSR));
+        bSL = fma(bN1, add(fma(SR, dh, -qR), G1), fma(bN2, add(fma(SR, dq, -fR), G2), bSL));
+        const double b2s = A::mul(bN2, ss), b1s = A::mul(bN1, ss);
+        bqL = add(bqL, fma(bN1, SR, -b2s));
+        bqR = add(bqR, fma(-bN1, SL, b2s));
+        bPL = A::mul(bN2, SR);
+        bPR = -A::mul(bN2, SL);
+        bhR = add(bhR, b1s);
+        bhL = sub(bhL, b1s);
     }
     // f_K = q_K un_K + g h_K^2 / 2, q_K = h_K un_K
-    bqL += bPL * unL; bunL += bPL * qL + bqL * hL; bhL += f64::twice(ghL) * bPL + bqL * unL;
-    bqR += bPR * unR; bunR += bPR * qR + bqR * hR; bhR += f64::twice(ghR) * bPR + bqR * unR;
+    bqL = fma(bPL, unL, bqL);
+    bunL = fma(bPL, qL, fma(bqL, hL, bunL));
+    bhL = fma(f64::twice(ghL), bPL, fma(bqL, unL, bhL));
+    bqR = fma(bPR, unR, bqR);
+    bunR = fma(bPR, qR, fma(bqR, hR, bunR));
+    bhR = fma(f64::twice(ghR), bPR, fma(bqR, unR, bhR));
     double baL = 0.0, baR = 0.0;
     if (wet) {
-        bunL += bSL;
-        bunR += bSR;
+        bunL = add(bunL, bSL);
+        bunR = add(bunR, bSR);
         if (!shL) baL = -bSL;
         if (!shR) baR = bSR;
         if (shock) {
             double bhs = 0.0;
             if (shL) {   // c_L = sqrt(g/2 (h*^2 / h_L + h*))
-                const double t = -bSL * g2 * f64::half(ycL), x = hs * rL;
-                bhs += t * f64::fma(2.0, x, 1.0);
-                bhL -= t * x * x;
+                const double t = A::mul(A::mul(-bSL, g2), f64::half(ycL)), x = A::mul(hs, rL);
+                bhs = A::mul(t, fma(2.0, x, 1.0));
+                bhL = fma(-A::mul(t, x), x, bhL);
             }
             if (shR) {
-                const double t = bSR * g2 * f64::half(ycR), x = hs * rR;
-                bhs += t * f64::fma(2.0, x, 1.0);
-                bhR -= t * x * x;
+                const double t = A::mul(A::mul(bSR, g2), f64::half(ycR)), x = A::mul(hs, rR);
+                bhs = fma(t, fma(2.0, x, 1.0), bhs);
+                bhR = fma(-A::mul(t, x), x, bhR);
             }
             // h* = N / (g_L + g_R), N = h_L g_L + h_R g_R - du
-            const double bN = bhs * rDg;
-            bhL += bN * gL; bhR += bN * gR;
-            double bdu = -bN;
+            const double bN = A::mul(bhs, rDg), bNg = A::mul(bN, g2);
             // g_K = sqrt(g/2 (1/h0 + 1/h_K))
-            const double xL = bN * (hL - hs) * f64::half(ygL) * g2, xR = bN * (hR - hs) * f64::half(ygR) * g2;
-            bhL -= xL * rL * rL;
-            bhR -= xR * rR * rR;
+            const double xL = A::mul(A::mul(bNg, sub(hL, hs)), f64::half(ygL));
+            const double xR = A::mul(A::mul(bNg, sub(hR, hs)), f64::half(ygR));
             // 1/h0 = 4 asum / (hsum w), w = 2 asum - du
-            const double b0 = xL + xR, b0r = b0 * rh0 * rhw;
-            const double bw = -b0r * hsum, bhsum = -b0r * w;
-            const double ba = f64::four_times(b0 * rhw) + f64::twice(bw);
-            bdu -= bw;
-            bhL += bhsum; bhR += bhsum;
-            baL += ba; baR += ba;
-            bunR += bdu; bunL -= bdu;
+            const double b0 = add(xL, xR), b0r = A::mul(A::mul(b0, rh0), rhw);
+            const double bw = -A::mul(b0r, hsum);
+            bhL = fma(bN, gL, fma(-A::mul(xL, rL), rL, fma(-b0r, w, bhL)));
+            bhR = fma(bN, gR, fma(-A::mul(xR, rR), rR, fma(-b0r, w, bhR)));
+            const double ba = fma(4.0, A::mul(b0, rhw), f64::twice(bw));
+            const double bdu = add(bN, bw);   // of -du
+            baL = add(baL, ba); baR = add(baR, ba);
+            bunR = sub(bunR, bdu); bunL = add(bunL, bdu);
         }
     } else if (wetL) {                                                          // Eq 26
-        bunL += bSL + bSR;
-        baL = 2.0 * bSR - bSL;
+        bunL = add(bunL, add(bSL, bSR));
+        baL = fma(2.0, bSR, -bSL);
     } else {
-        bunR += bSL + bSR;
-        baR = bSR - 2.0 * bSL;
+        bunR = add(bunR, add(bSL, bSR));
+        baR = fma(-2.0, bSL, bSR);
     }
-    bhL += baL * g2 * yL;                                                       // a_K = sqrt(g h_K)
-    bhR += baR * g2 * yR;
+    bhL = fma(A::mul(baL, g2), yL, bhL);                                        // a_K = sqrt(g h_K)
+    bhR = fma(A::mul(baR, g2), yR, bhR);
 }
 
 // Reverse of one interior edge in canonical orientation (left cell L, its
 // outward unit normal (n1, n2)): for the adjoints (wF0, wF1, wF2) of the flux
 // leaving L and (sL, sR) of the two cells' bed source factors, the adjoints
 // of (h, hu, hv, z) of L in dL and of R in dR.
+template <class A>
 __device__ __forceinline__ void edge_interior_rev(const V4<double>& L, const V4<double>& R, double n1, double n2,
-                                                  double g2, double h_dry, bool hll_only, double wF0, double wF1,
-                                                  double wF2, double sL, double sR, V4<double>& dL, V4<double>& dR) {
+                                                  double len, double g2, double h_dry, bool hll_only,
+                                                  const V4<double>& nl, const V4<double>& nr, V4<double>& dL,
+                                                  V4<double>& dR) {
+    using f64::add, f64::sub, f64::fma;
+    // adjoints of the flux leaving L (F in the left cell's term -len F, +len F
+    // in the right cell's) and of the bed source factors
+    const double bG1 = A::mul(len, sub(nr.x, nl.x));
+    const double d1 = A::mul(len, sub(nr.y, nl.y)), d2 = A::mul(len, sub(nr.z, nl.z));
+    const double gl = A::mul(f64::twice(g2), len);
+    const double gsL = A::mul(gl, fma(nl.y, n1, A::mul(nl.z, n2))), gsR = -A::mul(gl, fma(nr.y, n1, A::mul(nr.z, n2)));
     // forward: velocities (R9), hydrostatic reconstruction (Eq 28), rotation (Eq 12)
     const bool wL = gt_pos(L.x, h_dry), wR = gt_pos(R.x, h_dry);
-    const double rL = wL ? f64::rcp(L.x) : 0.0, rR = wR ? f64::rcp(R.x) : 0.0;
-    const double uL = f64::mul(L.y, rL), vL = f64::mul(L.z, rL), uR = f64::mul(R.y, rR), vR = f64::mul(R.z, rR);
+    const double rL = wL ? A::rcp(L.x) : 0.0, rR = wR ? A::rcp(R.x) : 0.0;
+    const double uL = A::mul(L.y, rL), vL = A::mul(L.z, rL), uR = A::mul(R.y, rR), vR = A::mul(R.z, rR);
     const double zs = max_finite(L.w, R.w);   // a tie takes z_R, as the forward
     const bool zleft = __double_as_longlong(zs) != __double_as_longlong(R.w);
-    const double xL = f64::sub(f64::add(L.x, L.w), zs), xR = f64::sub(f64::add(R.x, R.w), zs);
+    const double xL = sub(add(L.x, L.w), zs), xR = sub(add(R.x, R.w), zs);
     const bool pL = !lt_zero(xL), pR = !lt_zero(xR);
     const double hL = pL ? xL : 0.0, hR = pR ? xR : 0.0;
-    const double unL = f64::fma(uL, n1, f64::mul(vL, n2)), utL = f64::fma(vL, n1, -f64::mul(uL, n2));
-    const double unR = f64::fma(uR, n1, f64::mul(vR, n2)), utR = f64::fma(vR, n1, -f64::mul(uR, n2));
+    const double unL = fma(uL, n1, A::mul(vL, n2)), utL = fma(vL, n1, -A::mul(uL, n2));
+    const double unR = fma(uR, n1, A::mul(vR, n2)), utR = fma(vR, n1, -A::mul(uR, n2));
     // reverse: back from (x, y) (Eq 12 inverse)
-    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2, bG3 = wF2 * n1 - wF1 * n2;
+    const double bG2 = fma(d1, n1, A::mul(d2, n2)), bG3 = fma(d2, n1, -A::mul(d1, n2));
     // bed source factors (Eq 30 with 1/2): src_K = (g/2)(h**_K^2 - h_K^2)
-    const double gsL = f64::twice(g2) * sL, gsR = f64::twice(g2) * sR;
-    double bhL = gsL * hL, bunL = 0.0, butL = 0.0, bhR = gsR * hR, bunR = 0.0, butR = 0.0;
-    riemann_rev(hL, unL, utL, hR, unR, utR, g2, h_dry, hll_only, bG1, bG2, bG3, bhL, bunL, butL, bhR, bunR, butR);
-    double bh0L = -gsL * L.x, bh0R = -gsR * R.x;
+    double bhL = A::mul(gsL, hL), bunL = 0.0, butL = 0.0, bhR = A::mul(gsR, hR), bunR = 0.0, butR = 0.0;
+    riemann_rev<A>(hL, unL, utL, hR, unR, utR, g2, h_dry, hll_only, bG1, bG2, bG3, bhL, bunL, butL, bhR, bunR, butR);
     // rotation and velocities (r_K = 0 on a dry side)
-    dL.y = (bunL * n1 - butL * n2) * rL;
-    dL.z = (bunL * n2 + butL * n1) * rL;
-    bh0L -= dL.y * uL + dL.z * vL;
-    dR.y = (bunR * n1 - butR * n2) * rR;
-    dR.z = (bunR * n2 + butR * n1) * rR;
-    bh0R -= dR.y * uR + dR.z * vR;
+    dL.y = A::mul(fma(bunL, n1, -A::mul(butL, n2)), rL);
+    dL.z = A::mul(fma(bunL, n2, A::mul(butL, n1)), rL);
+    dR.y = A::mul(fma(bunR, n1, -A::mul(butR, n2)), rR);
+    dR.z = A::mul(fma(bunR, n2, A::mul(butR, n1)), rR);
     // reconstruction: h*_K = h_K + z_K - z*, z* the higher bed
     if (!pL) bhL = 0.0;
     if (!pR) bhR = 0.0;
-    dL.x = bh0L + bhL;
-    dR.x = bh0R + bhR;
+    dL.x = fma(-gsL, L.x, fma(-dL.y, uL, fma(-dL.z, vL, bhL)));
+    dR.x = fma(-gsR, R.x, fma(-dR.y, uR, fma(-dR.z, vR, bhR)));
     dL.w = zleft ? -bhR : bhL;
     dR.w = zleft ? bhR : -bhL;
 }
@@ -544,8 +580,10 @@ __device__ __forceinline__ void boundary_rev(int kind, double value, const V4<do
     const double un = f64::fma(u, n1, f64::mul(v, n2)), ut = f64::fma(v, n1, -f64::mul(u, n2));
     const double x = f64::sub(value, c.w);
     const double hg = kind == kBcStage ? max_zero(x) : c.x;
-    double bh = 0.0, bun = 0.0, but = 0.0, bhg = 0.0;
-    riemann_rev(c.x, un, ut, hg, un, ut, g2, h_dry, hll_only, bG1, bG2, bG3, bh, bun, but, bhg, bun, but);
+    double bh = 0.0, bun = 0.0, but = 0.0, bhg = 0.0, bung = 0.0, butg = 0.0;
+    riemann_rev<f64::Hard>(c.x, un, ut, hg, un, ut, g2, h_dry, hll_only, bG1, bG2, bG3, bh, bun, but, bhg, bung, butg);
+    bun += bung;
+    but += butg;
     if (kind == kBcStage) {
         if (!lt_zero(x)) d[3] -= bhg;
     } else {
@@ -555,6 +593,14 @@ __device__ __forceinline__ void boundary_rev(int kind, double value, const V4<do
     d[0] += bh - (bx * u + by * v);
     d[1] += bx;
     d[2] += by;
+}
+
+__device__ __forceinline__ bool zero3(const V4<double>& v) {
+    return ((__double_as_longlong(v.x) | __double_as_longlong(v.y) | __double_as_longlong(v.z)) << 1) == 0LL;
+}
+__device__ __forceinline__ bool soft_state(const V4<double>& s) {
+    return f64::in_range<-64, 24>(s.x) && f64::in_range<-64, 24>(s.y) && f64::in_range<-64, 24>(s.z) &&
+           f64::in_range<-64, 24>(s.w);
 }
 
 // Phase 2, edges: each interior edge once, the adjoints of both cells' states
@@ -572,12 +618,22 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
             a.ed[2 * e + 1] = dr;
             continue;
         }
+        // both cells' adjoints zero (no gauge's influence has come this far back):
+        // so is the edge's
+        const V4<double> nl = a.nu[lr.x], nr = a.nu[lr.y];
+        if (zero3(nl) && zero3(nr)) {
+            a.ed[2 * e] = dl;
+            a.ed[2 * e + 1] = dr;
+            continue;
+        }
         const V4<double> L = a.U[lr.x], R = a.U[lr.y];
         const double n1 = a.eln[2 * e], n2 = a.eln[2 * e + 1], len = a.erl[e];
-        const V4<double> nl = a.nu[lr.x], nr = a.nu[lr.y];
-        const double sL = len * (nl.y * n1 + nl.z * n2), sR = -len * (nr.y * n1 + nr.z * n2);
-        edge_interior_rev(L, R, n1, n2, 0.5 * a.g, a.h_dry, a.hll != 0, len * (nr.x - nl.x), len * (nr.y - nl.y),
-                          len * (nr.z - nl.z), sL, sR, dl, dr);
+        const double g2 = f64::mul(0.5, a.g);
+        if (soft_state(L) && soft_state(R) && f64::soft_edge(n1, n2, len, g2) && soft_adjoint(nl.x) &&
+            soft_adjoint(nl.y) && soft_adjoint(nl.z) && soft_adjoint(nr.x) && soft_adjoint(nr.y) && soft_adjoint(nr.z))
+            edge_interior_rev<f64::SoftFlush>(L, R, n1, n2, len, g2, a.h_dry, a.hll != 0, nl, nr, dl, dr);
+        else
+            edge_interior_rev<f64::Hard>(L, R, n1, n2, len, g2, a.h_dry, a.hll != 0, nl, nr, dl, dr);
         a.ed[2 * e] = dl;
         a.ed[2 * e + 1] = dr;
     }

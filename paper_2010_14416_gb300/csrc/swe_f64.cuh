@@ -123,8 +123,10 @@ struct Soft {
     }
     static __device__ __forceinline__ unsigned significand_hi(int hi) { return ((unsigned)hi & 0xFFFFFu) | 0x100000u; }
 
-    // a b, rounded to nearest even: zero operands, or normal ones with a normal product
-    static __device__ __forceinline__ double mul(double a, double b) {
+    // a b, rounded to nearest even: zero operands, or normal ones with a normal
+    // product; with FLUSH a smaller product gives zero
+    template <bool FLUSH>
+    static __device__ __forceinline__ double product(double a, double b) {
         const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
         const unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
         const unsigned bm = significand_hi(bh);
@@ -147,9 +149,10 @@ struct Soft {
         const unsigned q = (l0 != 0u) | (h0 & 1u);
         const unsigned long long r = (((unsigned long long)h1 << 32) | h0) + (l1 >= 0x80000001u - q ? 1ULL : 0ULL);
         unsigned rh = (unsigned)(r >> 32) + ea + eb + top - (1024u << 20), rl = (unsigned)r;
-        if (ea == 0u || eb == 0u) { rh = 0u; rl = 0u; }
+        if (ea == 0u || eb == 0u || (FLUSH && ea + eb <= (1024u << 20))) { rh = 0u; rl = 0u; }
         return __hiloint2double((int)(rh | ((ah ^ bh) & 0x80000000u)), (int)rl);
     }
+    static __device__ __forceinline__ double mul(double a, double b) { return product<false>(a, b); }
 
     // an FP32 seed in (1/2, 1] as a 32-bit fraction
     static __device__ __forceinline__ unsigned fraction(float r) {
@@ -224,6 +227,11 @@ struct Soft {
         return root<false>(x, y);
     }
     static __device__ __forceinline__ double sqrt_rsqrt(double x, double& y) { return root<true>(x, y); }
+};
+
+// For adjoints, whose products may become as small as they like.
+struct SoftFlush : Soft {
+    static __device__ __forceinline__ double mul(double a, double b) { return product<true>(a, b); }
 };
 
 // for operands of any kind

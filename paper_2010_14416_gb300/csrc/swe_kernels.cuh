@@ -657,11 +657,93 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
 // the same arithmetic evaluated once per edge) instead of evaluating them
 // here; an edge with both cells dry has no flux and its bed source term is
 // formed inline, with the same bits.
+
+// The FP64 cell of the edge-pass step.  It reads its neighbours' depths only,
+// and normals and lengths only for boundary edges and edges with both cells
+// dry: with whole neighbour and geometry records the kernel held 138 registers
+// (12 warps an SM) and waited on its chain of operations (48 us for 250k wet
+// cells; a step of the 1M-cell canal 182 us then, 163 now).
+template <typename Args>
+__device__ __forceinline__ double update_cell_edges(const Args& a, long long i, const V4<double>& own, const int4& tp,
+                                                    double dt, unsigned& active, unsigned long long* n_clamped,
+                                                    unsigned* status) {
+    const double h_dry = a.h_dry;
+    const double hi = own.x, zi = own.w;
+    int code[3] = {tp.x, tp.y, tp.z};
+    if (a.debug) {   // an unusable code is flagged and taken as a wall (group 0)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (!code_ok(code[j], a.cell_bound(), a.n_groups)) {
+                atomicOr(status, kStatusBadIndex);
+                code[j] = -1;
+            }
+    }
+    const int4 ei = a.eidx[i];
+    const bool wet = gt_pos(hi, h_dry);
+    bool flux[3];   // the edge pass evaluated the edge
+    bool quiet = !wet;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        flux[j] = false;
+        if (code[j] >= 0) {
+            flux[j] = wet || gt_pos(a.s_in[code[j] & kNbrMask].x, h_dry);
+            quiet = quiet && !flux[j];
+        } else {
+            const int kind = a.bc_kind(-1 - code[j]);
+            quiet = quiet && (kind == kBcWall || kind == kBcTransmissive);
+        }
+    }
+    if (quiet) {
+        V4<double> out;
+        out.x = hi; out.y = 0.0; out.z = 0.0; out.w = zi;
+        a.s_out[i] = out;
+        return inf_of<double>();
+    }
+    active += 1u;
+    const double2 tail = ((const double2*)&a.geoB[i])[1];   // 1/|Omega|, R
+    const double gm2 = a.gm2[i];
+    double m = 0.0, x = 0.0, y = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int c = code[j];
+        double tm = 0.0, tx, ty;
+        if (flux[j]) {
+            int e = j == 0 ? ei.x : (j == 1 ? ei.y : ei.z);
+            if (a.debug && !(e >= 0 && e < a.n_edges)) {
+                atomicOr(status, kStatusBadIndex);
+                e = 0;
+            }
+            const V4<double> fl = a.eflux[e];
+            const bool flip = (c & kFlipBit) != 0;
+            tm = flip ? -fl.x : fl.x;
+            tx = flip ? -fl.w : fl.y;
+            ty = flip ? -a.esrc[e] : fl.z;
+        } else {
+            const double2 n = j == 2 ? *(const double2*)&a.geoB[i] : ((const double2*)&a.geoA[i])[j];
+            const double len = ((const double*)&a.geoR[i])[j], g2 = f64::mul(0.5, a.g);
+            if (c >= 0) {
+                f64::dry_edge(hi, zi, a.s_in[c & kNbrMask].w, n.x, n.y, len, g2, tx, ty);
+            } else {
+                const int grp = -1 - c;
+                f64::Side side{hi, 0.0, 0.0, zi};
+                f64::velocity(hi, own.y, own.z, h_dry, side.u, side.v);
+                f64::boundary(a.bc_kind(grp), a.bc_value(grp), side, n.x, n.y, len, g2, h_dry, a.hll != 0, tm, tx, ty);
+            }
+        }
+        m = f64::add(m, tm);
+        x = f64::add(x, tx);
+        y = f64::add(y, ty);
+    }
+    return finish_cell(a, i, own, m, x, y, tail.x, tail.y, gm2, dt, n_clamped, status);
+}
+
 template <typename T, bool GEO_EARLY, bool EDGES = false, typename Args>
 __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>& own, const int4& tp, T dt,
                                          unsigned& active, unsigned long long* n_clamped, unsigned* status) {
     if constexpr (std::is_same<T, float>::value) {
         return update_cell_f32<GEO_EARLY, EDGES>(a, i, own, tp, dt, active, n_clamped, status);
+    } else if constexpr (EDGES) {
+        return update_cell_edges(a, i, own, tp, dt, active, n_clamped, status);
     } else {
     const double h_dry = a.h_dry, g2 = f64::mul(0.5, a.g);
     const double hi = own.x, zi = own.w;
@@ -710,13 +792,9 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
         gm2 = a.gm2[i];
     }
     f64::Side own_side{hi, 0.0, 0.0, zi};
-    // with EDGES only boundary edges need the cell's own velocity
-    if (!EDGES || code[0] < 0 || code[1] < 0 || code[2] < 0)
-        f64::velocity(hi, own.y, own.z, h_dry, own_side.u, own_side.v);
+    f64::velocity(hi, own.y, own.z, h_dry, own_side.u, own_side.v);
     double m = 0.0, x = 0.0, y = 0.0;
-    int4 ei = make_int4(-1, -1, -1, 0);
-    if constexpr (EDGES) ei = a.eidx[i];
-#pragma unroll(EDGES ? 3 : 1)   // an edge's evaluation is some 2,500 instructions
+#pragma unroll 1   // an edge's evaluation is some 2,500 instructions
     for (int j = 0; j < 3; ++j) {
         const int c = j == 0 ? code[0] : (j == 1 ? code[1] : code[2]);
         const V4<double> o = j == 0 ? nb[0] : (j == 1 ? nb[1] : nb[2]);
@@ -726,34 +804,18 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
         double tm = 0.0, tx, ty;
         if (c >= 0) {
             const bool flip = (c & kFlipBit) != 0;
-            if constexpr (EDGES) {
-                if (!gt_pos(hi, h_dry) && !gt_pos(o.x, h_dry)) {
-                    f64::dry_edge(hi, zi, o.w, n1, n2, len, g2, tx, ty);
-                } else {
-                    int e = j == 0 ? ei.x : (j == 1 ? ei.y : ei.z);
-                    if (a.debug && !(e >= 0 && e < a.n_edges)) {
-                        atomicOr(status, kStatusBadIndex);
-                        e = 0;
-                    }
-                    const V4<double> fl = a.eflux[e];
-                    tm = flip ? -fl.x : fl.x;
-                    tx = flip ? -fl.w : fl.y;
-                    ty = flip ? -a.esrc[e] : fl.z;
-                }
-            } else {
-                f64::Side nb_side{o.x, 0.0, 0.0, o.w};
-                f64::velocity(o.x, o.y, o.z, h_dry, nb_side.u, nb_side.v);
-                f64::Side L, R;   // the canonical orientation: left = lower caller index
-                L.h = flip ? nb_side.h : own_side.h; R.h = flip ? own_side.h : nb_side.h;
-                L.u = flip ? nb_side.u : own_side.u; R.u = flip ? own_side.u : nb_side.u;
-                L.v = flip ? nb_side.v : own_side.v; R.v = flip ? own_side.v : nb_side.v;
-                L.z = flip ? nb_side.z : own_side.z; R.z = flip ? own_side.z : nb_side.z;
-                f64::EdgeTerms t;
-                f64::edge(L, R, flip ? -n1 : n1, flip ? -n2 : n2, len, g2, h_dry, a.hll != 0, t);
-                tm = flip ? -t.m : t.m;
-                tx = flip ? -t.xR : t.xL;
-                ty = flip ? -t.yR : t.yL;
-            }
+            f64::Side nb_side{o.x, 0.0, 0.0, o.w};
+            f64::velocity(o.x, o.y, o.z, h_dry, nb_side.u, nb_side.v);
+            f64::Side L, R;   // the canonical orientation: left = lower caller index
+            L.h = flip ? nb_side.h : own_side.h; R.h = flip ? own_side.h : nb_side.h;
+            L.u = flip ? nb_side.u : own_side.u; R.u = flip ? own_side.u : nb_side.u;
+            L.v = flip ? nb_side.v : own_side.v; R.v = flip ? own_side.v : nb_side.v;
+            L.z = flip ? nb_side.z : own_side.z; R.z = flip ? own_side.z : nb_side.z;
+            f64::EdgeTerms t;
+            f64::edge(L, R, flip ? -n1 : n1, flip ? -n2 : n2, len, g2, h_dry, a.hll != 0, t);
+            tm = flip ? -t.m : t.m;
+            tx = flip ? -t.xR : t.xL;
+            ty = flip ? -t.yR : t.yL;
         } else {
             const int grp = -1 - c;
             f64::boundary(a.bc_kind(grp), a.bc_value(grp), own_side, n1, n2, len, g2, h_dry, a.hll != 0, tm, tx, ty);
@@ -766,13 +828,22 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
     }
 }
 
+// Blocks per SM that a step kernel's registers are held to.  The FP64 cell
+// pass after the edge pass is a chain of integer and FP64 operations: the more
+// warps the better until it spills (20 an SM, 96 registers; 16 for the
+// ensemble's).
+template <typename T, bool EDGES, bool ENSEMBLE>
+__host__ __device__ constexpr int min_blocks_of(int block, int min_blocks) {
+    return sizeof(T) == 8 && EDGES ? (ENSEMBLE ? 16 : 20) * 32 / block : min_blocks;
+}
+
 // ---- the fused step: fluxes + bed source + BCs + friction + update + next dt ------
 // Grid-stride over cells with about one resident wave of blocks, so the block
 // reduction (and its barrier) runs once per block.  With STAGES > 1 each
 // thread keeps its next STAGES-1 cells' state and topology records in flight
 // through cp.async into its own shared-memory slots.
 template <typename T, int BLOCK, int MINB, int STAGES, bool GEO_EARLY, bool EDGES = false>
-__global__ void __launch_bounds__(BLOCK, MINB) step_kernel(const StepArgs<T> a) {
+__global__ void __launch_bounds__(BLOCK, (min_blocks_of<T, EDGES, false>(BLOCK, MINB))) step_kernel(const StepArgs<T> a) {
     const WarpDt<T> wdt = warp_step_dt<T>(a.cfl, a.dt_read, a.dt_fixed);
     const double dt_d = wdt.d;
     const bool have_dt = wdt.have;
@@ -1143,7 +1214,7 @@ __device__ __forceinline__ long long ens_tile_of(long long k, long long nchunk_s
 }
 
 template <typename T, int BLOCK, int MINB, int STAGES, bool GEO_EARLY, bool EDGES = false>
-__global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel(const EnsArgs<T> a) {
+__global__ void __launch_bounds__(BLOCK, (min_blocks_of<T, EDGES, true>(BLOCK, MINB))) ensemble_step_kernel(const EnsArgs<T> a) {
     static_assert(kEnsPad % BLOCK == 0, "a tile must not straddle two members");
     const long long G = gridDim.x, b = blockIdx.x;
     const int cl2 = a.chunk_log2;

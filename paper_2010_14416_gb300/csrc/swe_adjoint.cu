@@ -563,14 +563,14 @@ __device__ __forceinline__ void edge_interior_rev(const V4<double>& L, const V4<
 __device__ __forceinline__ void boundary_rev(int kind, double value, const V4<double>& c, double n1, double n2,
                                              double g2, double h_dry, bool hll_only, double wF0, double wF1, double wF2,
                                              double d[4]) {
-    const bool wet = gt_pos(c.x, h_dry);
-    const double r = wet ? f64::rcp(c.x) : 0.0;
-    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2, bG3 = wF2 * n1 - wF1 * n2;
+    const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2;
     const double gh = f64::twice(g2) * c.x;
     if (kind == kBcWall) {
         d[0] += bG2 * gh;
         return;
     }
+    const double r = gt_pos(c.x, h_dry) ? f64::rcp(c.x) : 0.0;
+    const double bG3 = wF2 * n1 - wF1 * n2;
     if (kind == kBcInflow) {   // G2 = g h^2 / 2 + q^2 / h
         const double qr = value * r;
         d[0] += bG2 * (gh - qr * qr);
@@ -715,11 +715,11 @@ __global__ void adj_inject_kernel(const V4<double>* __restrict__ U, const long l
 
 // caller-order gradients: dL/dm = dL/d(g m^2) * 2 g m, dL/dz as is
 __global__ void adj_output_kernel(const double* __restrict__ gm, const double* __restrict__ gz,
-                                  const double* __restrict__ gm2, const long long* __restrict__ perm, double g,
+                                  const double* __restrict__ gm2, const unsigned* __restrict__ inv, double g,
                                   double* __restrict__ out_m, double* __restrict__ out_z, long long n) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n) {
-        const long long o = perm[c];
+    const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o < n) {
+        const long long c = inv[o];
         // g m = sqrt(g * g m^2) for m >= 0
         if (out_m) out_m[o] = gm[c] * 2.0 * sqrt(g * gm2[c]);
         if (out_z) out_z[o] = gz[c];
@@ -899,17 +899,23 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         void* cur = m->state[m->nstep % 2];
         void* nxt = m->state[(m->nstep + 1) % 2];
         if (s % K == 0) e = cudaMemcpyAsync((char*)p_ckpt + (s / K) * sb, cur, sb, cudaMemcpyDeviceToDevice, st);
+        // in the last segment the steps go from one of its states to the next
         const bool in_last = s >= last0;
-        if (e == cudaSuccess && in_last)
-            e = cudaMemcpyAsync(segp + (s - last0) * sb, cur, sb, cudaMemcpyDeviceToDevice, st);
+        const void* in = in_last ? segp + (s - last0) * sb : cur;
+        void* out = in_last && s + 1 < nsteps ? segp + (s + 1 - last0) * sb : nxt;
+        if (e == cudaSuccess && s == last0)
+            e = cudaMemcpyAsync(segp, cur, sb, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess)
-            e = launch_step_raw(m, cur, nxt, m->small, m->nstep, cfl, nullptr, (double*)p_dtlog + s, st, false,
+            e = launch_step_raw(m, in, out, m->small, m->nstep, cfl, nullptr, (double*)p_dtlog + s, st, false,
                                 keep && in_last ? (void*)(sflux + (s - last0) * Eb) : nullptr,
                                 keep && in_last ? (void*)(ssrc + (s - last0) * Eb) : nullptr);
+        // and the mesh is left with the last two
+        if (e == cudaSuccess && in_last && s + 1 == nsteps && s > last0)
+            e = cudaMemcpyAsync(cur, in, sb, cudaMemcpyDeviceToDevice, st);
         ++m->nstep;
         m->act_valid = false;   // stepped without the activity bytes
         if (e == cudaSuccess && (s + 1) % obs_every == 0) {
-            adj_loss_kernel<<<1, 32, 0, st>>>((const V4<double>*)nxt, gi, tg + ((s + 1) / obs_every - 1) * n_gauges,
+            adj_loss_kernel<<<1, 32, 0, st>>>((const V4<double>*)out, gi, tg + ((s + 1) / obs_every - 1) * n_gauges,
                                              n_gauges, (double*)p_loss);
             e = cudaGetLastError();
         }
@@ -1050,7 +1056,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
     // outputs
     if (where == SWE_DEVICE) {
         adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)p_gm, (const double*)p_gz,
-                                                                       (const double*)m->gm2, m->perm, m->cfg.g,
+                                                                       (const double*)m->gm2, m->inv, m->cfg.g,
                                                                        grad_manning, grad_bathy, n);
         e = cudaGetLastError();
     } else {
@@ -1059,7 +1065,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         if (e == cudaSuccess) e = cudaMalloc(&oz.p, n * sizeof(double));
         if (e == cudaSuccess) {
             adj_output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double*)p_gm, (const double*)p_gz,
-                                                                           (const double*)m->gm2, m->perm, m->cfg.g,
+                                                                           (const double*)m->gm2, m->inv, m->cfg.g,
                                                                            (double*)om.p, (double*)oz.p, n);
             e = cudaGetLastError();
         }

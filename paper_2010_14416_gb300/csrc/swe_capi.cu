@@ -7,7 +7,7 @@
 //   geoR      V4<T>[n]   FP64: L of the three edges
 //   topo      int4[n]    neighbour codes
 //   gm2       T[n]       g m^2
-//   perm      int64[n]   internal -> caller index
+//   perm, inv u32[n]     internal -> caller index and back
 //   small     u64[8]     dt slots 0..2 (double bits), t, status, clamp count
 // Step n reads state[n % 2] and dt slot n % 3, writes state[(n+1) % 2] and
 // slot (n+1) % 3, and clears slot (n+2) % 3, so a graph of a multiple of six
@@ -128,6 +128,7 @@ int upload_static(swe_mesh* m) {
     const int64_t n = H.n_cells;
     std::vector<V4<T>> A(n), B(n), R(n);
     std::vector<T> gm2(n), zt(n);
+    std::vector<unsigned> perm(n), inv(n);
     const std::vector<int4> topo = make_topo(m);
     for (int64_t c = 0; c < n; ++c) {
         double ln[6], len[3] = {0.0, 0.0, 0.0};
@@ -143,6 +144,8 @@ int upload_static(swe_mesh* m) {
         B[c].z = (T)H.inv_area[c]; B[c].w = (T)H.rin[c];
         gm2[c] = (T)(m->cfg.g * H.m[c] * H.m[c]);
         zt[c] = (T)H.z[c];
+        perm[c] = (unsigned)H.perm[c];
+        inv[H.perm[c]] = (unsigned)c;
     }
     cudaError_t e;
     if ((e = cudaMemcpy(m->geoA, A.data(), n * sizeof(V4<T>), cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -152,7 +155,8 @@ int upload_static(swe_mesh* m) {
         (e = cudaMemcpy(m->gm2, gm2.data(), n * sizeof(T), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(m->zdev, zt.data(), n * sizeof(T), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(m->topo, topo.data(), n * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(m->perm, H.perm.data(), n * sizeof(long long), cudaMemcpyHostToDevice)) != cudaSuccess)
+        (e = cudaMemcpy(m->perm, perm.data(), n * sizeof(unsigned), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(m->inv, inv.data(), n * sizeof(unsigned), cudaMemcpyHostToDevice)) != cudaSuccess)
         return cuda_fail(e, "swe_mesh_create: upload");
     return SWE_OK;
 }
@@ -219,12 +223,19 @@ StepArgs<T> make_args(swe_mesh* m, int64_t step_index, double cfl) {
     a.act_in = nullptr;
     a.act_next = nullptr;
     a.act_clear = nullptr;
+    a.span_in = nullptr;
+    a.span_next = nullptr;
+    a.span_clear = nullptr;
     a.act_list = m->act_list;
     a.act_count = m->act_count;
     if (m->cfg.activity && m->act[0]) {
         a.act_in = m->act[p3];
         a.act_next = m->act[(p3 + 1) % 3];
         a.act_clear = m->act[(p3 + 2) % 3];
+        // the flags lie behind the bytes
+        a.span_in = a.act_in + m->act_len;
+        a.span_next = a.act_next + m->act_len;
+        a.span_clear = a.act_clear + m->act_len;
     }
     a.g = (T)m->cfg.g;
     a.h_dry = (T)m->cfg.h_dry;
@@ -343,8 +354,8 @@ int set_state_t(swe_mesh* m, const void* h, const void* hu, const void* hv, int 
     }
     // z rides in the state record (copied from the static z array)
     e = Launch<T>::pack(src[0], src[1], src[2], m->perm, (const T*)m->zdev, (V4<T>*)m->state[0], n, m->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(m->state[1], m->state[0], n * sizeof(V4<T>),
-                                              cudaMemcpyDeviceToDevice, m->stream);
+    // (the other buffer holds nothing that is read: a step writes every record,
+    // with the activity bytes the first two after a set_state do)
     if (e == cudaSuccess) { init_small_kernel<<<1, 32, 0, m->stream>>>(m->small, t); e = cudaGetLastError(); }
     if (e == cudaSuccess)
         e = Launch<T>::dt((const V4<T>*)m->state[0], (const V4<T>*)m->geoB, n, (T)m->cfg.g, (T)m->cfg.h_dry,
@@ -363,13 +374,13 @@ int get_state_t(swe_mesh* m, void* h, void* hu, void* hv, int where) {
     const V4<T>* cur = (const V4<T>*)m->state[m->nstep % 2];
     cudaError_t e;
     if (where == SWE_DEVICE) {
-        e = Launch<T>::unpack(cur, m->perm, (T*)h, (T*)hu, (T*)hv, n, m->stream);
+        e = Launch<T>::unpack(cur, m->inv, (T*)h, (T*)hu, (T*)hv, n, m->stream);
         if (e != cudaSuccess) return cuda_fail(e, "swe_get_state");
         return SWE_OK;
     }
     int rc = ensure_stage(m);
     if (rc) return rc;
-    e = Launch<T>::unpack(cur, m->perm, (T*)m->stage[0], (T*)m->stage[1], (T*)m->stage[2], n, m->stream);
+    e = Launch<T>::unpack(cur, m->inv, (T*)m->stage[0], (T*)m->stage[1], (T*)m->stage[2], n, m->stream);
     void* dst[3] = {h, hu, hv};
     for (int k = 0; k < 3 && e == cudaSuccess; ++k)
         e = cudaMemcpyAsync(dst[k], m->stage[k], n * sizeof(T), cudaMemcpyDeviceToHost, m->stream);
@@ -507,11 +518,9 @@ int init_activity(swe_mesh* m) {
     const int64_t n = m->hm.n_cells;
     cudaError_t e = cudaSuccess;
     if (!m->act[0]) {
-        const int64_t len = (n + 31) / 32 * 32 + 32;
-        for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-            e = cudaMalloc((void**)&m->act[k], len);
-            if (e == cudaSuccess) e = cudaMemsetAsync(m->act[k], 0, len, m->stream);
-        }
+        const int64_t len = (n + 31) / 32 * 32 + 32;   // bytes, then a flag per span
+        const int64_t all = len + ((n + (1 << kScanLog) - 1) >> kScanLog);
+        for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMalloc((void**)&m->act[k], all);
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_list, n * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_count, 2 * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMemsetAsync(m->act_count, 0, 2 * sizeof(unsigned), m->stream);
@@ -524,14 +533,15 @@ int init_activity(swe_mesh* m) {
             return SWE_ENOMEM;
         }
         m->act_len = len;
-        m->device_bytes += 3 * len + (int64_t)((n + 2) * sizeof(unsigned));
+        m->device_bytes += 3 * all + (int64_t)((n + 2) * sizeof(unsigned));
     }
     const int p3 = (int)(m->nstep % 3);
-    e = cudaMemsetAsync(m->act[p3], 2, m->act_len, m->stream);   // bit 1: rebuilt (act_init_kernel)
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->act[(p3 + 1) % 3], 0, m->act_len, m->stream);
+    const int64_t all = m->act_len + ((n + (1 << kScanLog) - 1) >> kScanLog);
+    e = cudaMemsetAsync(m->act[p3], 2, all, m->stream);   // bit 1: rebuilt (act_init_kernel)
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->act[(p3 + 1) % 3], 0, all, m->stream);
     // the previous step's bytes: all 1, so the next step writes every cell's
     // state (its output buffer holds no step's result yet)
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->act[(p3 + 2) % 3], 1, m->act_len, m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->act[(p3 + 2) % 3], 1, all, m->stream);
     if (e == cudaSuccess)
         e = m->cfg.precision == SWE_FP32
                 ? Launch<float>::act_init((const V4<float>*)m->state[m->nstep % 2], m->topo, n, (float)m->cfg.h_dry,
@@ -584,7 +594,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     drop_graph(m);
     drop_diag_workspace(m);
     drop_adjoint_workspace(m);
-    void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm,
+    void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm, m->inv,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
                     m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count};
     for (void* b : bufs)
@@ -645,6 +655,12 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
         set_error("swe_mesh_create: edge_pass and activity exclude each other");
         return SWE_EINVAL;
     }
+    // FP64 with nothing chosen: the edge pass.  Its 1.5 evaluations a cell in
+    // place of 3 halve the step's work (and 4,000 cells are one chain of
+    // instructions a warp: 18.3 us a step without it); the results are the same.
+    const bool implied_edges = c.precision == SWE_FP64 && c.block_size == 0 && c.min_blocks == 0 && c.stages == 0 &&
+                               c.grid == 0 && !c.geometry_early && !c.activity;
+    if (implied_edges) c.edge_pass = 1;
     if (c.block_size == 0) c.block_size = c.precision == SWE_FP32 ? 256 : 128;
     if (c.block_size != 128 && c.block_size != 256 && c.block_size != 512) {
         set_error("swe_mesh_create: block_size must be 128, 256 or 512");
@@ -686,7 +702,8 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
         (rc = dev_alloc(m, (void**)&m->topo, n * sizeof(int4), "topology")) ||
         (rc = dev_alloc(m, &m->gm2, n * m->esz, "manning")) ||
         (rc = dev_alloc(m, &m->zdev, n * m->esz, "bed")) ||
-        (rc = dev_alloc(m, (void**)&m->perm, n * sizeof(long long), "permutation")) ||
+        (rc = dev_alloc(m, (void**)&m->perm, n * sizeof(unsigned), "permutation")) ||
+        (rc = dev_alloc(m, (void**)&m->inv, n * sizeof(unsigned), "permutation")) ||
         (rc = dev_alloc(m, (void**)&m->small, kSmallWords * sizeof(unsigned long long), "status"))) {
         swe_mesh_destroy(m);
         return rc;
@@ -695,6 +712,11 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
     if (rc) { swe_mesh_destroy(m); return rc; }
     if (c.edge_pass) {
         rc = build_edges(m);
+        if (rc == SWE_ENOMEM && implied_edges && !(cfg && cfg->edge_pass)) {   // without the edges' arrays, then
+            (void)cudaGetLastError();
+            c.edge_pass = m->cfg.edge_pass = 0;
+            rc = SWE_OK;
+        }
         if (rc) { swe_mesh_destroy(m); return rc; }
     }
     {

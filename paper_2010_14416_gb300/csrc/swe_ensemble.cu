@@ -43,7 +43,7 @@ struct swe_ensemble {
     void* geoR = nullptr;             // FP64: lengths of the three edges
     int4* topo = nullptr;
     void* gm2 = nullptr;
-    long long* perm = nullptr;        // per member, relative to the member's base
+    unsigned* inv = nullptr;          // per member, caller -> internal index, relative to the member's base
     int* tile_member = nullptr;
     long long* member_first_tile = nullptr;
     double* cfl = nullptr;
@@ -144,17 +144,6 @@ __global__ void count_wet_kernel(const V4<T>* __restrict__ s, long long n, T h_d
         c += s[i].x > h_dry ? 1u : 0u;
     c = __reduce_add_sync(0xffffffffu, c);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, (unsigned long long)c);
-}
-
-template <typename T>
-__global__ void ens_unpack_kernel(const V4<T>* __restrict__ s, const long long* __restrict__ perm, long long base,
-                                  T* __restrict__ h, T* __restrict__ hu, T* __restrict__ hv, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const long long o = perm[base + i];
-        const V4<T> v = s[base + i];
-        h[o] = v.x; hu[o] = v.y; hv[o] = v.z;
-    }
 }
 
 template <typename T>
@@ -300,7 +289,7 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
         (sizeof(T) == 8 && (rc = ens_alloc(E, &E->geoR, off * v4, "geometry"))) ||
         (rc = ens_alloc(E, (void**)&E->topo, off * sizeof(int4), "topology")) ||
         (rc = ens_alloc(E, &E->gm2, off * sizeof(T), "manning")) ||
-        (rc = ens_alloc(E, (void**)&E->perm, off * sizeof(long long), "permutation")) ||
+        (rc = ens_alloc(E, (void**)&E->inv, off * sizeof(unsigned), "permutation")) ||
         (rc = ens_alloc(E, (void**)&E->tile_member, E->n_tiles * sizeof(int), "tiles")) ||
         (rc = ens_alloc(E, (void**)&E->member_first_tile, nm * sizeof(long long), "tiles")) ||
         (rc = ens_alloc(E, (void**)&E->cfl, nm * sizeof(double), "cfl")) ||
@@ -337,7 +326,7 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
     for (int k = 0; k < nm; ++k) E->debug = E->debug || M[k]->cfg.debug_checks;
     // per-member device copies and host-built topology / tile tables
     std::vector<int4> topo(off);
-    std::vector<long long> perm(off, 0);
+    std::vector<unsigned> inv(off, 0u);
     std::vector<int> tile_member(E->n_tiles);
     const int wall_code = -1;  // global group 0
     for (int k = 0; k < nm; ++k) {
@@ -368,7 +357,7 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
                 if (code[j] < 0 && (kinds[-1 - code[j]] == kBcInflow || kinds[-1 - code[j]] == kBcStage))
                     w |= kStaticBit;
             topo[b + c] = make_int4(code[0], code[1], code[2], w);
-            perm[b + c] = m->hm.perm[c];
+            inv[b + m->hm.perm[c]] = (unsigned)c;
         }
         for (int64_t c = n; c < (E->n_cells[k] + kEnsPad - 1) / kEnsPad * kEnsPad; ++c)
             topo[b + c] = make_int4(wall_code, wall_code, wall_code, 0);
@@ -378,7 +367,7 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
     }
     std::vector<long long> mft(E->first_tile.begin(), E->first_tile.end());
     e = cudaMemcpyAsync(E->topo, topo.data(), off * sizeof(int4), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(E->perm, perm.data(), off * sizeof(long long), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(E->inv, inv.data(), off * sizeof(unsigned), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(E->tile_member, tile_member.data(), E->n_tiles * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
@@ -500,12 +489,11 @@ int ens_capture(swe_ensemble* E, int64_t start, int64_t len, const EnsPhysics& p
 template <typename T>
 int ens_get_state(swe_ensemble* E, int k, void* h, void* hu, void* hv, int where) {
     const int64_t n = E->n_cells[k];
-    const V4<T>* cur = (const V4<T>*)E->state[E->nstep % 2];
+    const V4<T>* cur = (const V4<T>*)E->state[E->nstep % 2] + E->base[k];
+    const unsigned* inv = E->inv + E->base[k];
     cudaError_t e;
-    const unsigned grid = (unsigned)((n + 255) / 256);
     if (where == SWE_DEVICE) {
-        ens_unpack_kernel<T><<<grid, 256, 0, E->stream>>>(cur, E->perm, E->base[k], (T*)h, (T*)hu, (T*)hv, n);
-        e = cudaGetLastError();
+        e = Launch<T>::unpack(cur, inv, (T*)h, (T*)hu, (T*)hv, n, E->stream);
         return e == cudaSuccess ? SWE_OK : efail(e, "swe_ensemble_get_state");
     }
     if (E->stage_cells < n) {
@@ -517,9 +505,7 @@ int ens_get_state(swe_ensemble* E, int k, void* h, void* hu, void* hv, int where
         }
         E->stage_cells = n;
     }
-    ens_unpack_kernel<T><<<grid, 256, 0, E->stream>>>(cur, E->perm, E->base[k], (T*)E->stage[0], (T*)E->stage[1],
-                                                      (T*)E->stage[2], n);
-    e = cudaGetLastError();
+    e = Launch<T>::unpack(cur, inv, (T*)E->stage[0], (T*)E->stage[1], (T*)E->stage[2], n, E->stream);
     void* dst[3] = {h, hu, hv};
     for (int j = 0; j < 3 && e == cudaSuccess; ++j)
         e = cudaMemcpyAsync(dst[j], E->stage[j], n * sizeof(T), cudaMemcpyDeviceToHost, E->stream);
@@ -875,7 +861,7 @@ void swe_ensemble_destroy(swe_ensemble* E) {
     EnsDeviceGuard dg(E->device);
     if (E->stream) cudaStreamSynchronize(E->stream);
     drop_graphs(E);
-    void* bufs[] = {E->state[0], E->state[1], E->geoA, E->geoB, E->topo, E->gm2, E->perm, E->tile_member,
+    void* bufs[] = {E->state[0], E->state[1], E->geoA, E->geoB, E->topo, E->gm2, E->inv, E->tile_member,
                     E->member_first_tile, E->cfl, E->small, E->n_active, E->kind, E->value,
                     E->stage[0], E->stage[1], E->stage[2], E->act[0], E->act[1], E->act[2],
                     E->ecells, E->eln, E->eflux, E->esrc, E->eidx, E->geoR, E->erl, E->sched};

@@ -131,7 +131,7 @@ struct swe_mesh {
     int4* topo = nullptr;
     void* gm2 = nullptr;
     void* zdev = nullptr;
-    long long* perm = nullptr;
+    unsigned *perm = nullptr, *inv = nullptr;   // internal -> caller index and back
     void* stage[3] = {nullptr, nullptr, nullptr};
     unsigned long long* small = nullptr;
     swe::BcTable bc{};

@@ -48,6 +48,7 @@ __host__ __device__ __forceinline__ bool code_ok(int code, long long n, int n_gr
 constexpr int kBcWall = 0, kBcInflow = 1, kBcTransmissive = 2, kBcStage = 3;
 
 constexpr int kScanBlock = 256;   // threads of act_scan_kernel, 16 cells each
+constexpr int kScanLog = 12;      // a block's span: 2^kScanLog = 16 kScanBlock cells
 constexpr int kEnsPad = 256;  // ensemble members are padded to whole multiples of this many cells
 
 template <typename T>
@@ -89,6 +90,10 @@ struct StepArgs {
     const unsigned char* act_in;
     unsigned char* act_next;
     unsigned char* act_clear;
+    // one flag per kScanSpan cells and buffer: the span has a byte that is not 0
+    const unsigned char* span_in;
+    unsigned char* span_next;
+    unsigned char* span_clear;
     unsigned* act_list;                // cells that run the flux path (act_scan_kernel), in [0, *act_count)
     unsigned* act_count;               // and a count of the blocks that have used it; both 0 between steps
     // edge pass (step_kernel with EDGES): interior edges in canonical orientation,
@@ -309,7 +314,7 @@ __device__ __forceinline__ void block_min_publish(T cand, unsigned long long* ds
                                                   unsigned long long* count_dst = nullptr) {
     __shared__ T warp_min[BLOCK / 32];
     __shared__ unsigned warp_cnt[BLOCK / 32];
-    for (int o = 16; o > 0; o >>= 1) cand = tmin(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+    for (int o = 16; o > 0; o >>= 1) cand = min_nonneg(cand, __shfl_xor_sync(0xffffffffu, cand, o));
     if (count_dst) cnt = __reduce_add_sync(0xffffffffu, cnt);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) { warp_min[wid] = cand; warp_cnt[wid] = cnt; }
@@ -318,7 +323,7 @@ __device__ __forceinline__ void block_min_publish(T cand, unsigned long long* ds
         const int warps = (int)blockDim.x >> 5;   // at most BLOCK / 32
         T v = lane < warps ? warp_min[lane] : inf_of<T>();
         unsigned c = lane < warps ? warp_cnt[lane] : 0u;
-        for (int o = 16; o > 0; o >>= 1) v = tmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+        for (int o = 16; o > 0; o >>= 1) v = min_nonneg(v, __shfl_xor_sync(0xffffffffu, v, o));
         if (count_dst) c = __reduce_add_sync(0xffffffffu, c);
         if (lane == 0 && v < inf_of<T>())
             atomicMin(dst, (unsigned long long)__double_as_longlong((double)v));
@@ -354,6 +359,21 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
+}
+
+// ---- a cell update's view of the mesh: states in, state out, geometry ----------------
+template <typename Args>
+__device__ __forceinline__ auto load_state(const Args& a, long long i) {
+    return a.s_in[i];
+}
+template <typename Args, typename V>
+__device__ __forceinline__ void store_state(const Args& a, long long i, const V& v) {
+    a.s_out[i] = v;
+}
+template <typename Args, typename V>
+__device__ __forceinline__ void load_geometry(const Args& a, long long i, V& gA, V& gB) {
+    gA = a.geoA[i];
+    gB = a.geoB[i];
 }
 
 // ---- pieces of one cell update, shared by the step kernels and the adjoint ----------
@@ -499,7 +519,7 @@ __device__ __forceinline__ double finish_cell(const Args& a, long long i, const 
     const double big = 3.0e38;
     if (!lt_pos(out.x, big) || !abs_lt_pos(out.y, big) || !abs_lt_pos(out.z, big))
         atomicOr(status, kStatusNonFinite);
-    a.s_out[i] = out;
+    store_state(a, i, out);
     return gt_pos(out.x, h_dry) ? f64::cfl_candidate(out.x, out.y, out.z, rin, g) : inf_of<double>();
 }
 
@@ -532,12 +552,11 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
     }
     V4<float> nb[3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) nb[j] = code[j] >= 0 ? a.s_in[code[j] & kNbrMask] : own;
+    for (int j = 0; j < 3; ++j) nb[j] = code[j] >= 0 ? load_state(a, code[j] & kNbrMask) : own;
     V4<float> gA, gB;
     float gm2;
     if constexpr (GEO_EARLY) {
-        gA = a.geoA[i];
-        gB = a.geoB[i];
+        load_geometry(a, i, gA, gB);
         gm2 = load_gm2(a, i, tp, 0.0f);
     }
     bool quiet = !(hi > h_dry);
@@ -554,13 +573,12 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
     out.w = zi;
     if (quiet) {
         out.x = hi; out.y = 0.0f; out.z = 0.0f;
-        a.s_out[i] = out;
+        store_state(a, i, out);
         return inf_of<float>();
     }
     active += 1u;
     if constexpr (!GEO_EARLY) {
-        gA = a.geoA[i];
-        gB = a.geoB[i];
+        load_geometry(a, i, gA, gB);
         gm2 = load_gm2(a, i, tp, 0.0f);
     }
     float ui, vi;
@@ -633,7 +651,7 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
                                           h_dry, out.x, out.y, out.z, clamped, nonfinite);
     if (clamped) atomicAdd(n_clamped, 1ULL);
     if (nonfinite) atomicOr(status, kStatusNonFinite);
-    a.s_out[i] = out;
+    store_state(a, i, out);
     return cand;
 }
 
@@ -1014,8 +1032,9 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
 // update_cell gives, bit for bit.
 //
 // Two launches.  act_scan_kernel reads the bytes (2 per cell, 16 cells a
-// thread) and gathers the cells that run the flux path into a list, a block's
-// 4,096 cells in their order; a quiet cell costs it nothing more unless its
+// thread, a block's 4,096 at a time, and none of a span whose flags say that
+// they are all 0) and gathers the cells that run the flux path into a list, a
+// span's cells in their order; a quiet cell costs it nothing more unless its
 // state has to be written: where the cell was quiet in the previous step too,
 // the output buffer (the state of two steps ago, itself dry at rest with the
 // same h) holds it already.  step_kernel_act then updates the listed cells,
@@ -1023,27 +1042,36 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
 // together in the mesh order, so dealing out the cells by their place instead
 // leaves some SMs with several times the average work and makes every quiet
 // cell cost a state record read: that kernel, a cp.async pipeline over all
-// cells, took 96 us a step on the 13M-cell river, 6 % of it wet.
+// cells, took 96 us a step on the 13M-cell river, 6 % of it wet; the two take
+// 11 (without the flags) and 24 us.
 template <typename T>
 __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> a) {
-    const long long c0 = ((long long)blockIdx.x * kScanBlock + threadIdx.x) * 16;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ unsigned total[kScanBlock / 32], base;
+    // whether there is a step (warp_step_dt), by the bits alone: in thousands of
+    // warps an FP64 product each takes microseconds
+    const double dt = a.dt_fixed ? *a.dt_fixed : *a.dt_read;
+    const bool have_dt = (unsigned long long)__double_as_longlong(dt) < kInfBits;
+    const unsigned sp = blockIdx.x;   // the block's span
+    const unsigned char fl = a.span_in[sp], fp = a.span_clear[sp];
+    const long long c0 = ((long long)sp << kScanLog) + threadIdx.x * 16;
+    if (!have_dt) {
+        // no step: the state and its activity carry over unchanged
+        for (long long c = c0; c < c0 + 16 && c < a.n; ++c) {
+            a.s_out[c] = a.s_in[c];
+            a.act_next[c] = a.act_in[c];
+            a.act_clear[c] = 0;
+        }
+        __syncthreads();   // every thread has read the flags
+        if (threadIdx.x == 0) { a.span_next[sp] = fl; a.span_clear[sp] = 0; }
+        return;
+    }
+    if (!(fl | fp)) return;
     const bool in = c0 < a.n;
     uint4 now = make_uint4(0u, 0u, 0u, 0u), prev = now;
     if (in) {
         now = *(const uint4*)(a.act_in + c0);      // the buffers reach past n in whole 32 bytes
         prev = *(const uint4*)(a.act_clear + c0);
-    }
-    // whether there is a step (warp_step_dt), by the bits alone: in 25,000 warps
-    // of a 13M-cell mesh an FP64 product each takes microseconds
-    const double dt = a.dt_fixed ? *a.dt_fixed : *a.dt_read;
-    if (!((unsigned long long)__double_as_longlong(dt) < kInfBits)) {
-        // no step: the state and its activity carry over unchanged
-        if (in) {
-            *(uint4*)(a.act_next + c0) = now;
-            *(uint4*)(a.act_clear + c0) = make_uint4(0u, 0u, 0u, 0u);
-            for (long long c = c0; c < c0 + 16 && c < a.n; ++c) a.s_out[c] = a.s_in[c];
-        }
-        return;
     }
     // bit 0 of a byte: the cell runs the flux path in this step; a previous
     // byte that is not 0: it ran it in the previous step, or the bytes were
@@ -1061,7 +1089,6 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
     rewrite &= ~runs;
     // a warp whose 512 cells are all to be rewritten (the two steps after the
     // bytes are rebuilt) copies them side by side
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (__all_sync(0xffffffffu, rewrite == 0xFFFFu && c0 + 16 <= a.n)) {
         const long long w0 = c0 - 16 * lane;
 #pragma unroll 4
@@ -1081,22 +1108,23 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
         }
     }
     const unsigned cnt = __popc(runs);
-    if (!__syncthreads_or(cnt)) return;
     unsigned pos = cnt;
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned up = __shfl_up_sync(0xffffffffu, pos, o);
         if (lane >= o) pos += up;
     }
-    __shared__ unsigned total[kScanBlock / 32], base;
     if (lane == 31) total[warp] = pos;
-    __syncthreads();
+    __syncthreads();   // (every thread has read the flags, too)
     unsigned before = 0u, all = 0u;
 #pragma unroll
     for (int q = 0; q < kScanBlock / 32; ++q) {
         if (q == warp) before = all;
         all += total[q];
     }
-    if (threadIdx.x == 0) base = atomicAdd(a.act_count, all);
+    if (threadIdx.x == 0) {
+        base = atomicAdd(a.act_count, all);
+        a.span_clear[sp] = 0;
+    }
     __syncthreads();
     unsigned at = base + before + pos - cnt;
     for (unsigned m = runs; m; m &= m - 1u) a.act_list[at++] = (unsigned)c0 + __ffs(m) - 1;
@@ -1150,12 +1178,20 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_act(const StepArgs<T>
         // the topology record and the cell are read again from shared memory
         // rather than kept live in registers across the update
         const volatile int* tv = (const volatile int*)&st_topo[slot][tid];
-        if (wet || (tv[3] & kStaticBit)) a.act_next[((const volatile unsigned*)st_cell[slot])[tid]] = 1;
-        if (wet) {
+        if (wet || (tv[3] & kStaticBit)) {
+            const unsigned me = ((const volatile unsigned*)st_cell[slot])[tid];
+            a.act_next[me] = 1;
+            a.span_next[me >> kScanLog] = 1;
+            if (wet) {
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const int code = tv[j];
-                if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups))) a.act_next[code & kNbrMask] = 1;
+                for (int j = 0; j < 3; ++j) {
+                    const int code = tv[j];
+                    if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups))) {
+                        const unsigned nb = (unsigned)code & kNbrMask;
+                        a.act_next[nb] = 1;
+                        if ((nb ^ me) >> kScanLog) a.span_next[nb >> kScanLog] = 1;
+                    }
+                }
             }
         }
         slot = slot == PF - 1 ? 0 : slot + 1;
@@ -1198,7 +1234,7 @@ __global__ void act_init_kernel(const V4<T>* __restrict__ s, const int4* __restr
 // widening is monotone), which keeps FP32 kernels off the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ void warp_min_publish(T cand, unsigned long long* dst) {
-    for (int o = 16; o > 0; o >>= 1) cand = tmin(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+    for (int o = 16; o > 0; o >>= 1) cand = min_nonneg(cand, __shfl_xor_sync(0xffffffffu, cand, o));
     if ((threadIdx.x & 31) == 0 && cand < inf_of<T>())
         atomicMin(dst, (unsigned long long)__double_as_longlong((double)cand));
 }
@@ -1663,14 +1699,19 @@ __global__ void __launch_bounds__(BLOCK) dt_kernel(const V4<T>* __restrict__ s, 
 }
 
 // ---- layout conversion between caller arrays and the packed internal state --------
-// pack: s[new] = (h[perm[new]], hu[..], hv[..], z[new])
+// Each direction makes its random accesses reads (13M cells numbered by an
+// unstructured mesher): packing gathers the caller's three values by internal
+// order, perm[internal] = caller (scattering whole records by the caller's
+// order took 420 us, 16-byte writes into 32-byte sectors); unpacking gathers a
+// record by the caller's order, inv[caller] = internal, and writes side by
+// side (204 us).
 template <typename T>
 __global__ void pack_state_kernel(const T* __restrict__ h, const T* __restrict__ hu, const T* __restrict__ hv,
-                                  const long long* __restrict__ perm, const T* __restrict__ z,
-                                  V4<T>* __restrict__ s, long long n) {
+                                  const unsigned* __restrict__ perm, const T* __restrict__ z, V4<T>* __restrict__ s,
+                                  long long n) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        const long long o = perm[i];
+        const unsigned o = perm[i];
         V4<T> v;
         v.x = h[o]; v.y = hu[o]; v.z = hv[o]; v.w = z[i];
         s[i] = v;
@@ -1678,12 +1719,11 @@ __global__ void pack_state_kernel(const T* __restrict__ h, const T* __restrict__
 }
 
 template <typename T>
-__global__ void unpack_state_kernel(const V4<T>* __restrict__ s, const long long* __restrict__ perm,
-                                    T* __restrict__ h, T* __restrict__ hu, T* __restrict__ hv, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const long long o = perm[i];
-        const V4<T> v = s[i];
+__global__ void unpack_state_kernel(const V4<T>* __restrict__ s, const unsigned* __restrict__ inv, T* __restrict__ h,
+                                    T* __restrict__ hu, T* __restrict__ hv, long long n) {
+    const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o < n) {
+        const V4<T> v = s[inv[o]];
         h[o] = v.x; hu[o] = v.y; hv[o] = v.z;
     }
 }
@@ -1781,9 +1821,9 @@ struct Launch {
     static int default_min_blocks(int block);
     static cudaError_t dt(const V4<T>* s, const V4<T>* geoB, long long n, T g, T h_dry,
                           unsigned long long* dt_write, cudaStream_t st);
-    static cudaError_t pack(const T* h, const T* hu, const T* hv, const long long* perm, const T* z,
+    static cudaError_t pack(const T* h, const T* hu, const T* hv, const unsigned* perm, const T* z,
                             V4<T>* s, long long n, cudaStream_t st);
-    static cudaError_t unpack(const V4<T>* s, const long long* perm, T* h, T* hu, T* hv, long long n,
+    static cudaError_t unpack(const V4<T>* s, const unsigned* inv, T* h, T* hu, T* hv, long long n,
                               cudaStream_t st);
     static cudaError_t riemann(long long n, const T* hL, const T* unL, const T* utL, const T* hR,
                                const T* unR, const T* utR, T g, T h_dry, T* G1, T* G2, T* G3, T* S,

@@ -51,12 +51,14 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
     const unsigned grid = a.grid;
     if (grid == 0) return cudaErrorInvalidValue;
     if (a.act_in) {
-        act_scan_kernel<T><<<grid_for<T>(a.n, 16 * kScanBlock), kScanBlock, 0, st>>>(a);
+        // a block per span: most spans of a dry mesh cost it one look at their flags
+        const unsigned spans = grid_for<T>(a.n, 1 << kScanLog);
+        act_scan_kernel<T><<<spans, kScanBlock, 0, st>>>(a);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_ACT(B, M, G, S) \
     if (block == B && min_blocks == M && geo_early == G && stages == S) {         \
-        step_kernel_act<T, B, M, G != 0, S - 1><<<grid, B, 0, st>>>(a);          \
+        step_kernel_act<T, B, M, G != 0, S - 1><<<grid, B, 0, st>>>(a);           \
         return cudaGetLastError();                                                \
     }
         if constexpr (sizeof(T) == 4) {
@@ -72,7 +74,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
         if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_EDGE(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0, true><<<grid, step_threads(a.n, grid, B), 0, st>>>(a);            \
+        step_kernel<T, B, M, S, G != 0, true><<<grid, step_threads(a.n, grid, B), 0, st>>>(a); \
         return cudaGetLastError();                                                \
     }
         if constexpr (sizeof(T) == 4) {
@@ -85,7 +87,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
     }
 #define SWE_LAUNCH(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0><<<grid, step_threads(a.n, grid, B), 0, st>>>(a);                  \
+        step_kernel<T, B, M, S, G != 0><<<grid, step_threads(a.n, grid, B), 0, st>>>(a); \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {
@@ -169,8 +171,8 @@ cudaError_t Launch<T>::step_pair(const StepArgs<T>& a, int block, int min_blocks
         if (a.grid == 0) return cudaErrorInvalidValue;
 #define SWE_LAUNCH_PAIR(B, M, G, S) \
     if (block == B && min_blocks == M && geo_early == G && stages == S) {      \
-        step_kernel_pair<B, M, G != 0><<<a.grid, B, 0, st>>>(a);            \
-        return cudaGetLastError();                                              \
+        step_kernel_pair<B, M, G != 0><<<a.grid, B, 0, st>>>(a);                  \
+        return cudaGetLastError();                                                \
     }
         SWE_PAIR_VARIANTS_F32(SWE_LAUNCH_PAIR)
 #undef SWE_LAUNCH_PAIR
@@ -345,7 +347,7 @@ cudaError_t Launch<T>::ensemble_step(const EnsArgs<T>& a, int block, int min_blo
         if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_EDGE(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        ensemble_step_kernel<T, B, M, S, G != 0, true><<<grid, B, 0, st>>>(a);   \
+        ensemble_step_kernel<T, B, M, S, G != 0, true><<<grid, B, 0, st>>>(a);    \
         return cudaGetLastError();                                                \
     }
         if constexpr (sizeof(T) == 4) {
@@ -358,7 +360,7 @@ cudaError_t Launch<T>::ensemble_step(const EnsArgs<T>& a, int block, int min_blo
     }
 #define SWE_LAUNCH(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        ensemble_step_kernel<T, B, M, S, G != 0><<<grid, B, 0, st>>>(a);         \
+        ensemble_step_kernel<T, B, M, S, G != 0><<<grid, B, 0, st>>>(a);          \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {
@@ -403,8 +405,8 @@ cudaError_t Launch<T>::ensemble_step_act(const EnsArgs<T>& a, int block, int min
 #define SWE_LAUNCH(B, M, G) \
     if (block == B && min_blocks == M && geo_early == G) {                                       \
         if (dynamic) ensemble_step_kernel_act<T, B, M, G != 0, true, true><<<grid, B, 0, st>>>(a); \
-        else ensemble_step_kernel_act<T, B, M, G != 0, false, true><<<grid, B, 0, st>>>(a);     \
-        return cudaGetLastError();                                                               \
+        else ensemble_step_kernel_act<T, B, M, G != 0, false, true><<<grid, B, 0, st>>>(a); \
+        return cudaGetLastError();                                                \
     }
             SWE_ENS_ACTQ_VARIANTS_F32(SWE_LAUNCH)
 #undef SWE_LAUNCH
@@ -414,7 +416,7 @@ cudaError_t Launch<T>::ensemble_step_act(const EnsArgs<T>& a, int block, int min
 #define SWE_LAUNCH(B, M, G) \
     if (block == B && min_blocks == M && geo_early == G) {                        \
         if (dynamic) ensemble_step_kernel_act<T, B, M, G != 0, true><<<grid, B, 0, st>>>(a); \
-        else ensemble_step_kernel_act<T, B, M, G != 0><<<grid, B, 0, st>>>(a);   \
+        else ensemble_step_kernel_act<T, B, M, G != 0><<<grid, B, 0, st>>>(a);    \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {
@@ -495,7 +497,7 @@ cudaError_t Launch<T>::ensemble_step_dyn(const EnsArgs<T>& a, int block, int min
     if (grid == 0 || !a.sched) return cudaErrorInvalidValue;
 #define SWE_LAUNCH(B, M, G) \
     if (block == B && min_blocks == M && geo_early == G) {                        \
-        ensemble_step_kernel_dyn<T, B, M, G != 0><<<grid, B, 0, st>>>(a);        \
+        ensemble_step_kernel_dyn<T, B, M, G != 0><<<grid, B, 0, st>>>(a);         \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {
@@ -548,8 +550,8 @@ cudaError_t Launch<T>::ensemble_step_pair(const EnsArgs<T>& a, int min_blocks, i
         if (a.pair_spans == 0) return cudaSuccess;
 #define SWE_LAUNCH(M, G) \
     if (min_blocks == M && geo_early == G) {                                             \
-        ensemble_step_kernel_pair<128, M, G != 0><<<grid, 128, 0, st>>>(a);             \
-        return cudaGetLastError();                                                       \
+        ensemble_step_kernel_pair<128, M, G != 0><<<grid, 128, 0, st>>>(a);       \
+        return cudaGetLastError();                                                \
     }
         SWE_ENS_PAIR_VARIANTS_F32(SWE_LAUNCH)
 #undef SWE_LAUNCH
@@ -590,16 +592,16 @@ cudaError_t Launch<T>::dt(const V4<T>* s, const V4<T>* geoB, long long n, T g, T
 }
 
 template <typename T>
-cudaError_t Launch<T>::pack(const T* h, const T* hu, const T* hv, const long long* perm, const T* z,
+cudaError_t Launch<T>::pack(const T* h, const T* hu, const T* hv, const unsigned* perm, const T* z,
                             V4<T>* s, long long n, cudaStream_t st) {
     pack_state_kernel<T><<<grid_for<T>(n, 256), 256, 0, st>>>(h, hu, hv, perm, z, s, n);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t Launch<T>::unpack(const V4<T>* s, const long long* perm, T* h, T* hu, T* hv, long long n,
+cudaError_t Launch<T>::unpack(const V4<T>* s, const unsigned* inv, T* h, T* hu, T* hv, long long n,
                               cudaStream_t st) {
-    unpack_state_kernel<T><<<grid_for<T>(n, 256), 256, 0, st>>>(s, perm, h, hu, hv, n);
+    unpack_state_kernel<T><<<grid_for<T>(n, 256), 256, 0, st>>>(s, inv, h, hu, hv, n);
     return cudaGetLastError();
 }
 

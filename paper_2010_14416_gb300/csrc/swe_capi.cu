@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "swe_internal.h"
+#include "swe_loop.cuh"
 
 namespace swe {
 
@@ -71,6 +72,7 @@ int swe::status_code(unsigned long long st) {
         set_error("swe_step: a neighbour index, edge index or boundary group out of range (debug checks)");
         return SWE_EMESH;
     }
+    if (st & kStatusStall) { set_error("swe_step: the step loop gave up waiting for its blocks"); return SWE_ECUDA; }
     if (st & kStatusNonFinite) { set_error("swe_step: non-finite state"); return SWE_ENONFINITE; }
     if (st & kStatusDry) { set_error("swe_step: every cell is dry, no CFL time step"); return SWE_EDRY; }
     return SWE_OK;
@@ -273,8 +275,112 @@ int capture_graph(swe_mesh* m, int len, double cfl) {
     return SWE_OK;
 }
 
+static_assert(kLoopSlotT == kSlotT && kLoopSlotStatus == kSlotStatus && kLoopSlotClamp == kSlotClamp &&
+                  kLoopSlotActive == kSlotActive && kLoopSlotDtLast == kSlotDtLast,
+              "words of the status block");
+
+// The edges that touch each block's cells, for the FP64 step loop.
+int build_loop_edges(swe_mesh* m) {
+    const HostMesh& H = m->hm;
+    const int64_t n = H.n_cells, nb = (n + kLoopCells - 1) / kLoopCells;
+    std::vector<int2> ecell(nb * kLoopEdges, make_int2(-1, -1));
+    std::vector<double> egeo(nb * 3 * kLoopEdges, 0.0);
+    std::vector<uchar4> eslot(n, make_uchar4(0, 0, 0, 0));
+    auto slot = [&](int64_t c, int j) -> unsigned char& { return j == 0 ? eslot[c].x : (j == 1 ? eslot[c].y : eslot[c].z); };
+    for (int64_t b = 0; b < nb; ++b) {
+        const int64_t c0 = b * kLoopCells, c1 = std::min(n, c0 + kLoopCells);
+        int ne = 0;
+        for (int64_t c = c0; c < c1; ++c)
+            for (int j = 0; j < 3; ++j) {
+                const int32_t code = H.code[3 * c + j];
+                if (code < 0) continue;
+                const int64_t k = code & kNbrMask;
+                if (k >= c0 && k < c) {   // listed from k already
+                    for (int jk = 0; jk < 3; ++jk)
+                        if (H.code[3 * k + jk] >= 0 && (H.code[3 * k + jk] & kNbrMask) == c) slot(c, j) = slot(k, jk);
+                    continue;
+                }
+                const bool flip = (code & kFlipBit) != 0;
+                double lx = H.ln[6 * c + 2 * j], ly = H.ln[6 * c + 2 * j + 1];
+                const double len = host_unit_normal(lx, ly);
+                ecell[b * kLoopEdges + ne] = flip ? make_int2((int)k, (int)c) : make_int2((int)c, (int)k);
+                double* g = &egeo[b * 3 * kLoopEdges + ne];
+                g[0] = flip ? -lx : lx;
+                g[kLoopEdges] = flip ? -ly : ly;
+                g[2 * kLoopEdges] = len;
+                slot(c, j) = (unsigned char)ne++;
+            }
+    }
+    cudaError_t e = cudaMalloc((void**)&m->loop_ecell, ecell.size() * sizeof(int2));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&m->loop_egeo, egeo.size() * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&m->loop_eslot, eslot.size() * sizeof(uchar4));
+    if (e == cudaSuccess) e = cudaMemcpy(m->loop_ecell, ecell.data(), ecell.size() * sizeof(int2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(m->loop_egeo, egeo.data(), egeo.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(m->loop_eslot, eslot.data(), eslot.size() * sizeof(uchar4), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? SWE_OK : cuda_fail(e, "swe_step: step loop");
+}
+
+// Whether the next steps run as one loop launch: a small mesh, nothing chosen
+// about its launches, no debug checks and no capture of the stream (a
+// cooperative launch is not for every graph).  From 4 steps on: the loop's
+// launch and first reads cost about what two step launches do.
+template <typename T>
+bool use_loop(swe_mesh* m, int64_t nsteps) {
+    if (!m->loop_allowed || nsteps < 4) return false;
+    if (m->loop_cells < 0) {
+        long long cells = 0;
+        if (Launch<T>::loop_capacity(m->cfg.device, &cells) != cudaSuccess) { (void)cudaGetLastError(); cells = 0; }
+        m->loop_cells = cells;
+        if (m->hm.n_cells <= cells) {
+            bool ok = cudaMalloc((void**)&m->loop_barrier, sizeof(unsigned)) == cudaSuccess;
+            if (ok && sizeof(T) == 8) ok = build_loop_edges(m) == SWE_OK;
+            if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
+        }
+    }
+    if (m->hm.n_cells > m->loop_cells) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
+template <typename T>
+int run_loop(swe_mesh* m, int64_t nsteps, double cfl) {
+    LoopArgs<T> a;
+    a.state[0] = (V4<T>*)m->state[0];
+    a.state[1] = (V4<T>*)m->state[1];
+    a.geoA = (const V4<T>*)m->geoA;
+    a.geoB = (const V4<T>*)m->geoB;
+    a.geoR = (const V4<T>*)m->geoR;
+    a.topo = m->topo;
+    a.gm2 = (const T*)m->gm2;
+    a.small = m->small;
+    a.barrier = m->loop_barrier;
+    a.n = m->hm.n_cells;
+    a.cfl = cfl;
+    a.g = (T)m->cfg.g;
+    a.h_dry = (T)m->cfg.h_dry;
+    a.hll = m->cfg.flux == SWE_FLUX_HLL ? 1 : 0;
+    a.debug = 0;
+    a.n_groups = m->n_groups;
+    a.bc = m->bc;
+    a.ecell = m->loop_ecell;
+    a.egeo = m->loop_egeo;
+    a.eslot = m->loop_eslot;
+    m->act_valid = false;   // steps without activity bytes do not maintain them
+    while (nsteps > 0) {
+        a.step0 = m->nstep;
+        a.steps = (int)std::min<int64_t>(nsteps, 2000);   // some milliseconds a launch
+        const cudaError_t e = Launch<T>::loop(a, m->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "swe_step: loop launch");
+        m->nstep += a.steps;
+        nsteps -= a.steps;
+    }
+    return SWE_OK;
+}
+
 template <typename T>
 int run_steps(swe_mesh* m, int64_t nsteps, double cfl) {
+    if (use_loop<T>(m, nsteps)) return run_loop<T>(m, nsteps, cfl);
     if (m->cfg.activity) {
         if (!m->act_valid) {
             int rc = init_activity(m);
@@ -594,7 +700,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     drop_graph(m);
     drop_diag_workspace(m);
     drop_adjoint_workspace(m);
-    void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm, m->inv,
+    void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm, m->inv, m->loop_barrier, m->loop_ecell, m->loop_egeo, m->loop_eslot,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
                     m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count};
     for (void* b : bufs)
@@ -660,6 +766,9 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
     // instructions a warp: 18.3 us a step without it); the results are the same.
     const bool implied_edges = c.precision == SWE_FP64 && c.block_size == 0 && c.min_blocks == 0 && c.stages == 0 &&
                                c.grid == 0 && !c.geometry_early && !c.activity;
+    const bool nothing_chosen = c.block_size == 0 && c.min_blocks == 0 && c.stages == 0 && c.grid == 0 &&
+                                !c.geometry_early && !c.activity && !c.edge_pass && !c.cell_pairs &&
+                                c.graph_steps == 0;
     if (implied_edges) c.edge_pass = 1;
     if (c.block_size == 0) c.block_size = c.precision == SWE_FP32 ? 256 : 128;
     if (c.block_size != 128 && c.block_size != 256 && c.block_size != 512) {
@@ -679,6 +788,7 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
     swe_mesh* m = new (std::nothrow) swe_mesh();
     if (!m) { set_error("swe_mesh_create: out of host memory"); return SWE_ENOMEM; }
     m->cfg = c;
+    m->loop_allowed = nothing_chosen && !c.debug_checks;
     m->esz = c.precision == SWE_FP32 ? 4 : 8;
     std::string err;
     int rc;
@@ -888,6 +998,7 @@ int swe_get_info(swe_mesh* m, swe_info* info) {
     info->n_clamped = (int64_t)s[kSlotClamp];
     info->n_active = (int64_t)s[kSlotActive];
     info->status = s[kSlotStatus] & kStatusBadIndex    ? SWE_EMESH
+                   : s[kSlotStatus] & kStatusStall     ? SWE_ECUDA
                    : s[kSlotStatus] & kStatusNonFinite ? SWE_ENONFINITE
                    : (s[kSlotStatus] & kStatusDry ? SWE_EDRY : SWE_OK);
     return SWE_OK;

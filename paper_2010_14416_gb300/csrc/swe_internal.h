@@ -165,6 +165,15 @@ struct swe_mesh {
     void* eflux = nullptr;             // V4<T>[E]
     void* esrc = nullptr;              // T[E]
     int4* eidx = nullptr;              // per cell, the edge of each local edge (-1: boundary)
+    // the step loop (swe_loop.cuh), for a small mesh with nothing chosen about its
+    // launches: the largest mesh it takes (-1: not asked yet), its arrival count
+    // and, FP64, its blocks' edges
+    bool loop_allowed = false;
+    long long loop_cells = -1;
+    unsigned* loop_barrier = nullptr;
+    int2* loop_ecell = nullptr;
+    double* loop_egeo = nullptr;
+    uchar4* loop_eslot = nullptr;
     // adjoint workspace (swe_adjoint.cu), kept between calls
     void* adj_arena = nullptr;
     size_t adj_bytes = 0;

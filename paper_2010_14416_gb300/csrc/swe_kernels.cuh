@@ -35,6 +35,7 @@ constexpr unsigned long long kInfBits = 0x7FF0000000000000ULL;  // +inf as doubl
 // status word bits
 constexpr unsigned kStatusNonFinite = 1u;
 constexpr unsigned kStatusDry = 2u;
+constexpr unsigned kStatusStall = 8u;      // a wait of the step loop gave up
 constexpr unsigned kStatusBadIndex = 4u;   // debug checks: an index or boundary group out of range
 
 // Debug checks: whether a neighbour code can be used on a mesh of n cells with
@@ -1761,6 +1762,9 @@ inline unsigned spread_grid(long long n) { return (unsigned)((n + 31) / 32); }
 
 // ---- host-side launchers, one set per precision ------------------------------------
 template <typename T>
+struct LoopArgs;
+
+template <typename T>
 struct Launch {
     // (block, min_blocks) pairs with a compiled kernel; see step_variants()
     // with a.act_in set, the activity kernel (stages ignored) runs
@@ -1819,6 +1823,10 @@ struct Launch {
     static int ensemble_pair_variants(int (*out)[2], int max);
     static void ensemble_default(int* block, int* min_blocks, int* stages, int* geo_early);
     static int default_min_blocks(int block);
+    // many steps in one cooperative launch (swe_loop.cuh): the largest mesh whose
+    // grid is resident, and the launch
+    static cudaError_t loop_capacity(int device, long long* cells);
+    static cudaError_t loop(const LoopArgs<T>& a, cudaStream_t st);
     static cudaError_t dt(const V4<T>* s, const V4<T>* geoB, long long n, T g, T h_dry,
                           unsigned long long* dt_write, cudaStream_t st);
     static cudaError_t pack(const T* h, const T* hu, const T* hv, const unsigned* perm, const T* z,

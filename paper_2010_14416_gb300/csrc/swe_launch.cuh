@@ -3,6 +3,7 @@
 #pragma once
 
 #include "swe_kernels.cuh"
+#include "swe_loop.cuh"
 
 namespace swe {
 
@@ -582,6 +583,42 @@ int Launch<T>::ensemble_pair_variants(int (*out)[2], int max) {
 #undef SWE_LIST
     }
     return k;
+}
+
+// Shape of the step loop: FP32 128 threads, 6 blocks an SM (80 registers); FP64
+// 96 threads, 5 blocks (128).
+constexpr int kLoopBlock32 = 128, kLoopMin32 = 6, kLoopMin64 = 5;
+
+template <typename T>
+cudaError_t Launch<T>::loop_capacity(int device, long long* cells) {
+    int per_sm = 0, sms = 0, coop = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
+    if constexpr (sizeof(T) == 4) {
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_loop_f32<kLoopBlock32, kLoopMin32>,
+                                                              kLoopBlock32, 0);
+        *cells = (long long)per_sm * sms * kLoopBlock32;
+    } else {
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_loop_f64<kLoopMin64>, kLoopEdges, 0);
+        *cells = (long long)per_sm * sms * kLoopCells;
+    }
+    if (e != cudaSuccess || !coop) *cells = 0;
+    return e;
+}
+
+template <typename T>
+cudaError_t Launch<T>::loop(const LoopArgs<T>& a, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(a.barrier, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    void* args[] = {(void*)&a};
+    if constexpr (sizeof(T) == 4)
+        return cudaLaunchCooperativeKernel((const void*)step_loop_f32<kLoopBlock32, kLoopMin32>,
+                                           dim3(grid_for<T>(a.n, kLoopBlock32)), dim3(kLoopBlock32), args, 0, st);
+    else
+        return cudaLaunchCooperativeKernel((const void*)step_loop_f64<kLoopMin64>, dim3(grid_for<T>(a.n, kLoopCells)),
+                                           dim3(kLoopEdges), args, 0, st);
 }
 
 template <typename T>

@@ -1,0 +1,78 @@
+"""The step loop of small meshes (swe_loop.cuh: all steps of a call in one
+cooperative launch) against the kernels launched step by step, bit for bit.
+A mesh with nothing chosen about its launches takes the loop from 4 steps on;
+graph_steps=-1 (no graphs) keeps it on single launches."""
+import numpy as np
+import pytest
+
+from paper_2010_14416_gb300 import build as libbuild
+from paper_2010_14416_gb300 import capi
+from paper_2010_14416_gb300 import meshgen as mg
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    libbuild.build()
+    return capi.load()
+
+
+def _mesh(mi, precision, **kw):
+    m = capi.Mesh(mi.nodes, mi.tris, mi.z, mi.manning, precision=precision, **kw)
+    for pairs, kind, value in mi.bcs:
+        m.set_bc(pairs, kind, value)
+    m.set_state(mi.h.astype(m.dtype), mi.hu.astype(m.dtype), mi.hv.astype(m.dtype))
+    return m
+
+
+def _equal(a, b):
+    assert all(np.array_equal(x, y) for x, y in zip(a.get_state(), b.get_state()))
+    ia, ib = a.info(), b.info()
+    for k in ("t", "dt_next", "n_steps", "n_clamped", "n_active", "status"):
+        assert ia[k] == ib[k], k
+
+
+# one block, a block and a ragged one, whole blocks; the last sizes fill most of
+# the resident grid (FP64 about 24,000 cells, FP32 about 116,000)
+CASES = [("canal", 3, 1), ("canal", 17, 1), ("canal", 16, 4), ("canal", 65, 3), ("dam4k", 0, 0),
+         ("river", 90, 13), ("river_wet", 60, 12), ("river", 300, 37)]
+
+
+def _make(kind, nx, ny):
+    if kind == "canal":
+        return mg.canal(nx, ny, float(nx), float(ny), 0.2, seed=3, hL=2.0, hR=0.0, x_dam=nx / 2.0, manning=0.03)
+    if kind == "dam4k":
+        return mg.dam_break_4k()
+    return mg.river(nx, ny, seed=4, n_bumps=20, fully_wet=kind == "river_wet")
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+@pytest.mark.parametrize("kind,nx,ny", CASES)
+def test_loop_matches_single_launches_bitwise(kind, nx, ny, precision):
+    mi = _make(kind, nx, ny)
+    flux = capi.SWE_FLUX_HLL if (nx, ny) == (60, 12) else capi.SWE_FLUX_HLLC
+    loop, single = _mesh(mi, precision, flux=flux), _mesh(mi, precision, flux=flux, graph_steps=-1)
+    for steps in (4, 3, 50, 1, 61):   # the loop starts from every step index modulo 6
+        assert loop.step(steps) == single.step(steps)
+        _equal(loop, single)
+
+
+def test_loop_takes_large_fp32_meshes_and_leaves_larger_ones():
+    for nx, ny in ((500, 110), (700, 110)):   # 110,000 cells: the loop; 154,000: one launch a step
+        mi = mg.river(nx, ny, seed=2, n_bumps=10)
+        loop, single = _mesh(mi, capi.SWE_FP32), _mesh(mi, capi.SWE_FP32, graph_steps=-1)
+        assert loop.step(40) == single.step(40)
+        _equal(loop, single)
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+def test_loop_without_water_reports_it_and_keeps_the_state(precision):
+    mi = mg.canal(20, 4, 20.0, 4.0, 0.2, seed=1, hL=0.0, hR=0.0, x_dam=10.0, manning=0.0)
+    m = _mesh(mi, precision)
+    with pytest.raises(capi.SWEError) as e:
+        m.step(10)
+    assert e.value.code == capi.SWE_EDRY
+    assert all(np.array_equal(x, np.zeros_like(x)) for x in m.get_state())

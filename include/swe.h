@@ -497,11 +497,12 @@ typedef struct swe_tune {
                                 creation) are updated by a cell-pair kernel (128-thread blocks,
                                 one pair of cells per thread, one resident wave), the others by
                                 the kernel of this shape, in the same step */
-    int queue;               /* FP32 ensembles with activity: 1 = each warp gathers the cells that
-                                run the flux path into a queue in shared memory and updates them
-                                32 at a time (full warps where wet cells are scattered), the
-                                quiet cells at once; compiled (block_size, min_blocks,
-                                geometry_early): (128, 7, 0|1), (128, 6, 1); 0 otherwise */
+    int queue;               /* FP32 ensembles with activity: 1 = a first kernel lists the cells that
+                                run the flux path (and writes the quiet ones that have to be),
+                                a second updates the listed cells, dealt evenly (dynamic 1: in
+                                pieces of chunk x block_size as they come); compiled (block_size,
+                                min_blocks, geometry_early): (128, 7, 0|1), (128, 6, 1);
+                                0 otherwise */
 } swe_tune;
 
 /*
@@ -536,7 +537,7 @@ SWE_API int swe_autotune(swe_mesh* mesh, int trial_steps, swe_tune* out);
  * geometry_early 0|1, (256, 4) with 0; FP64 (128|256, 1) with 0) with chunks
  * of 1 to 32 tiles; and the activity-mode shapes with dynamically taken
  * chunks (activity 1, dynamic 1) of 4 to 32 tiles; for FP32 ensembles the
- * activity shapes with per-warp queues (queue 1) with either chunk order; for
+ * activity shapes over a list of the active cells (queue 1), dealt evenly or dynamically; for
  * FP32 ensembles with
  * members placed for the split step, every activity or dynamically scheduled
  * shape also as the second kernel of a split step (cell_pairs 1); each over

@@ -228,6 +228,8 @@ StepArgs<T> make_args(swe_mesh* m, int64_t step_index, double cfl) {
     a.span_in = nullptr;
     a.span_next = nullptr;
     a.span_clear = nullptr;
+    a.span_first = m->span_first;
+    a.span_adj = m->span_adj;
     a.act_list = m->act_list;
     a.act_count = m->act_count;
     if (m->cfg.activity && m->act[0]) {
@@ -620,6 +622,36 @@ int build_edges(swe_mesh* m) {
     return SWE_OK;
 }
 
+// The spans (2^kScanLog cells) beside each span: those with an edge in common,
+// and itself.
+static cudaError_t build_spans(swe_mesh* m) {
+    const HostMesh& H = m->hm;
+    const int64_t n = H.n_cells, ns = (n + (1 << kScanLog) - 1) >> kScanLog;
+    std::vector<unsigned> first(ns + 1, 0u), adj, seen(ns, 0xFFFFFFFFu);
+    for (int64_t sp = 0; sp < ns; ++sp) {
+        first[sp] = (unsigned)adj.size();
+        adj.push_back((unsigned)sp);
+        seen[sp] = (unsigned)sp;
+        const int64_t lo = sp << kScanLog, hi = std::min(n, (sp + 1) << kScanLog);
+        for (int64_t k = 3 * lo; k < 3 * hi; ++k) {
+            if (H.code[k] < 0) continue;
+            const int64_t o = (H.code[k] & kNbrMask) >> kScanLog;
+            if (seen[o] != (unsigned)sp) {
+                seen[o] = (unsigned)sp;
+                adj.push_back((unsigned)o);
+            }
+        }
+    }
+    first[ns] = (unsigned)adj.size();
+    cudaError_t e = cudaMalloc((void**)&m->span_first, first.size() * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&m->span_adj, adj.size() * sizeof(unsigned));
+    if (e == cudaSuccess)
+        e = cudaMemcpy(m->span_first, first.data(), first.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(m->span_adj, adj.data(), adj.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
+    m->device_bytes += (int64_t)((first.size() + adj.size()) * sizeof(unsigned));
+    return e;
+}
+
 int init_activity(swe_mesh* m) {
     const int64_t n = m->hm.n_cells;
     cudaError_t e = cudaSuccess;
@@ -627,13 +659,16 @@ int init_activity(swe_mesh* m) {
         const int64_t len = (n + 31) / 32 * 32 + 32;   // bytes, then a flag per span
         const int64_t all = len + ((n + (1 << kScanLog) - 1) >> kScanLog);
         for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMalloc((void**)&m->act[k], all);
+        if (e == cudaSuccess) e = build_spans(m);
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_list, n * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_count, 2 * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMemsetAsync(m->act_count, 0, 2 * sizeof(unsigned), m->stream);
         if (e != cudaSuccess) {
-            for (void* p : {(void*)m->act[0], (void*)m->act[1], (void*)m->act[2], (void*)m->act_list, (void*)m->act_count})
+            for (void* p : {(void*)m->act[0], (void*)m->act[1], (void*)m->act[2], (void*)m->act_list,
+                            (void*)m->act_count, (void*)m->span_first, (void*)m->span_adj})
                 if (p) cudaFree(p);
             for (auto& p : m->act) p = nullptr;
+            m->span_first = m->span_adj = nullptr;
             m->act_list = m->act_count = nullptr;
             set_error("activity bytes: device allocation failed");
             return SWE_ENOMEM;
@@ -702,7 +737,7 @@ void swe_mesh_destroy(swe_mesh* m) {
     drop_adjoint_workspace(m);
     void* bufs[] = {m->state[0], m->state[1], m->geoA, m->geoB, m->topo, m->gm2, m->zdev, m->perm, m->inv, m->loop_barrier, m->loop_ecell, m->loop_egeo, m->loop_eslot,
                     m->stage[0], m->stage[1], m->stage[2], m->small, m->act[0], m->act[1], m->act[2],
-                    m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count};
+                    m->ecells, m->eln, m->eflux, m->esrc, m->eidx, m->geoR, m->erl, m->act_list, m->act_count, m->span_first, m->span_adj};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);

@@ -59,6 +59,10 @@ struct swe_ensemble {
     unsigned char* act[3] = {nullptr, nullptr, nullptr};
     int64_t act_len = 0;
     bool act_valid = false;
+    // list mode (queue): as for a mesh (swe_internal.h), and each member's step size
+    std::vector<unsigned> span_first_host, span_adj_host;
+    unsigned *span_first = nullptr, *span_adj = nullptr, *act_list = nullptr, *act_count = nullptr;
+    void* member_dt = nullptr;
     // edge pass (FP64 ensembles): the members' interior edges, concatenated
     int edges = 0;
     int64_t n_edges = 0;
@@ -68,7 +72,7 @@ struct swe_ensemble {
     // layout (pair_spans kEnsPad-cell spans) and run on the cell-pair kernel,
     // the others on the kernel of the shape above, in the same step
     int split = 0;
-    // activity kernel with per-warp queues of the cells that run the flux path
+    // activity step over a list of the cells that run the flux path
     int queue = 0;
     int64_t pair_spans = 0;
     int pair_minb = 8, pair_geo = 1;
@@ -147,6 +151,19 @@ __global__ void count_wet_kernel(const V4<T>* __restrict__ s, long long n, T h_d
 }
 
 template <typename T>
+void ens_list_args(const swe_ensemble* E, int p3, EnsArgs<T>& a) {
+    a.span_in = E->act[p3] + E->act_len;   // the flags lie behind the bytes
+    a.span_next = E->act[(p3 + 1) % 3] + E->act_len;
+    a.span_clear = E->act[(p3 + 2) % 3] + E->act_len;
+    a.span_first = E->span_first;
+    a.span_adj = E->span_adj;
+    a.act_list = E->act_list;
+    a.act_count = E->act_count;
+    a.member_dt = (T*)E->member_dt;
+    a.n_members = E->n_members;
+}
+
+template <typename T>
 EnsArgs<T> ens_args(swe_ensemble* E, int64_t step_index) {
     EnsArgs<T> a;
     const int p2 = (int)(step_index % 2), p3 = (int)(step_index % 3);
@@ -194,6 +211,7 @@ EnsArgs<T> ens_args(swe_ensemble* E, int64_t step_index) {
         a.act_next = E->act[(p3 + 1) % 3];
         a.act_clear = E->act[(p3 + 2) % 3];
     }
+    ens_list_args(E, p3, a);
     a.slot_read = p3;
     a.slot_write = (p3 + 1) % 3;
     a.slot_reset = (p3 + 2) % 3;
@@ -365,6 +383,25 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
         const int64_t t1 = (b + (n + kEnsPad - 1) / kEnsPad * kEnsPad) / kEnsPad;
         for (int64_t t = t0; t < t1; ++t) tile_member[t] = k;
     }
+    if (sizeof(T) == 4) {   // the spans beside each span, for the list mode
+        const int64_t ns = (off + (1 << kScanLog) - 1) >> kScanLog;
+        std::vector<unsigned> seen(ns, 0xFFFFFFFFu);
+        for (int64_t sp = 0; sp < ns; ++sp) {
+            E->span_first_host.push_back((unsigned)E->span_adj_host.size());
+            E->span_adj_host.push_back((unsigned)sp);
+            seen[sp] = (unsigned)sp;
+            for (int64_t c = sp << kScanLog; c < std::min<int64_t>(off, (sp + 1) << kScanLog); ++c)
+                for (int code : {topo[c].x, topo[c].y, topo[c].z}) {
+                    if (code < 0) continue;
+                    const unsigned o = (unsigned)(code & kNbrMask) >> kScanLog;
+                    if (seen[o] != (unsigned)sp) {
+                        seen[o] = (unsigned)sp;
+                        E->span_adj_host.push_back(o);
+                    }
+                }
+        }
+        E->span_first_host.push_back((unsigned)E->span_adj_host.size());
+    }
     std::vector<long long> mft(E->first_tile.begin(), E->first_tile.end());
     e = cudaMemcpyAsync(E->topo, topo.data(), off * sizeof(int4), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(E->inv, inv.data(), off * sizeof(unsigned), cudaMemcpyHostToDevice, st);
@@ -441,27 +478,39 @@ template <typename T>
 int ens_init_activity(swe_ensemble* E) {
     cudaError_t e = cudaSuccess;
     if (!E->act[0]) {
-        const int64_t len = (E->n_total + 31) / 32 * 32 + 32;
-        for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-            e = cudaMalloc((void**)&E->act[k], len);
-            if (e == cudaSuccess) e = cudaMemsetAsync(E->act[k], 0, len, E->stream);
+        const int64_t len = (E->n_total + 31) / 32 * 32 + 32;   // bytes, then a flag per span
+        const int64_t all = len + ((E->n_total + (1 << kScanLog) - 1) >> kScanLog);
+        for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMalloc((void**)&E->act[k], all);
+        const size_t nf = E->span_first_host.size() * sizeof(unsigned), na = E->span_adj_host.size() * sizeof(unsigned);
+        if (nf) {
+            if (e == cudaSuccess) e = cudaMalloc((void**)&E->span_first, nf);
+            if (e == cudaSuccess) e = cudaMalloc((void**)&E->span_adj, na);
+            if (e == cudaSuccess) e = cudaMalloc((void**)&E->act_list, E->n_total * sizeof(unsigned));
+            if (e == cudaSuccess) e = cudaMalloc((void**)&E->act_count, 2 * sizeof(unsigned));
+            if (e == cudaSuccess) e = cudaMalloc(&E->member_dt, E->n_members * sizeof(T));
+            if (e == cudaSuccess) e = cudaMemcpy(E->span_first, E->span_first_host.data(), nf, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemcpy(E->span_adj, E->span_adj_host.data(), na, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemsetAsync(E->act_count, 0, 2 * sizeof(unsigned), E->stream);
         }
         if (e != cudaSuccess) {
-            for (auto& p : E->act) {
+            for (void* p : {(void*)E->act[0], (void*)E->act[1], (void*)E->act[2], (void*)E->span_first, (void*)E->span_adj,
+                            (void*)E->act_list, (void*)E->act_count, E->member_dt})
                 if (p) cudaFree(p);
-                p = nullptr;
-            }
+            for (auto& p : E->act) p = nullptr;
+            E->span_first = E->span_adj = E->act_list = E->act_count = nullptr;
+            E->member_dt = nullptr;
             set_error("swe_ensemble: no device memory for the activity bytes");
             return SWE_ENOMEM;
         }
         E->act_len = len;
-        E->device_bytes += 3 * len;
+        E->device_bytes += 3 * all + (int64_t)(nf ? nf + na + (E->n_total + 2) * sizeof(unsigned) : 0);
     }
     const int p3 = (int)(E->nstep % 3);
-    e = cudaMemsetAsync(E->act[p3], 2, E->act_len, E->stream);   // bit 1: rebuilt (act_init_kernel)
-    if (e == cudaSuccess) e = cudaMemsetAsync(E->act[(p3 + 1) % 3], 0, E->act_len, E->stream);
+    const int64_t all = E->act_len + ((E->n_total + (1 << kScanLog) - 1) >> kScanLog);
+    e = cudaMemsetAsync(E->act[p3], 2, all, E->stream);   // bit 1: rebuilt (act_init_kernel)
+    if (e == cudaSuccess) e = cudaMemsetAsync(E->act[(p3 + 1) % 3], 0, all, E->stream);
     // the previous step's bytes: all 1, so the next step writes every cell's state
-    if (e == cudaSuccess) e = cudaMemsetAsync(E->act[(p3 + 2) % 3], 1, E->act_len, E->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(E->act[(p3 + 2) % 3], 1, all, E->stream);
     if (e == cudaSuccess)
         e = Launch<T>::act_init((const V4<T>*)E->state[E->nstep % 2], E->topo, E->n_total, (T)E->h_dry, E->act[p3],
                                 E->stream);
@@ -531,7 +580,7 @@ struct EnsShape {
     int split = 0;
     int pair_minb = 8, pair_geo = 1;
     unsigned pair_grid = 0;
-    int queue = 0;   // activity kernel with per-warp queues (FP32)
+    int queue = 0;   // activity step over a list (FP32)
 };
 
 template <typename T>
@@ -568,6 +617,7 @@ int ens_time_shapes(swe_ensemble* E, const std::vector<EnsShape>& cand, int tria
             a.act_in = sh.activity ? E->act[p3] : nullptr;
             a.act_next = sh.activity ? E->act[(p3 + 1) % 3] : nullptr;
             a.act_clear = sh.activity ? E->act[(p3 + 2) % 3] : nullptr;
+            ens_list_args(E, p3, a);
             auto launch = [&]() {
                 a.sched_slot = launch_no % 3;
                 a.sched_reset = (launch_no + 2) % 3;
@@ -649,8 +699,8 @@ int ens_autotune_t(swe_ensemble* E, int trial_steps, swe_tune* out) {
         const unsigned gr_d = (unsigned)std::max(1LL, std::min((long long)(E->n_total / w[k][0]), wave_d));
         for (int cl2 = 2; cl2 <= 5; ++cl2) cand.push_back({w[k][0], w[k][1], 3, w[k][2], cl2, gr_d, 1, 0, 1});
     }
-    // FP32: the activity kernel with per-warp queues of the cells that run the
-    // flux path, round-robin and dynamic chunks
+    // FP32: the activity step over a list of the cells that run the flux path,
+    // even shares and pieces taken dynamically
     int wq[8][3];
     const int nwq = with_act ? std::min(Launch<T>::ensemble_actq_variants(wq, 8), 8) : 0;
     for (int k = 0; k < nwq; ++k) {
@@ -662,7 +712,7 @@ int ens_autotune_t(swe_ensemble* E, int trial_steps, swe_tune* out) {
             if (e != cudaSuccess) break;
             const long long wave = (long long)std::max(per_sm, 1) * std::max(sms, 1);
             const unsigned gr = (unsigned)std::max(1LL, std::min((long long)(E->n_total / wq[k][0]), wave));
-            for (int cl2 = 2; cl2 <= (dyn ? 5 : 6); ++cl2) {
+            for (int cl2 = 2; cl2 <= (dyn ? 5 : 2); ++cl2) {   // (even shares have no chunks)
                 EnsShape sh{wq[k][0], wq[k][1], 3, wq[k][2], cl2, gr, 1, 0, dyn};
                 sh.queue = 1;
                 cand.push_back(sh);
@@ -823,9 +873,11 @@ int ens_autotune_t(swe_ensemble* E, int trial_steps, swe_tune* out) {
     E->dynamic = pick.dynamic;
     E->split = pick.split;
     E->queue = pick.queue;
-    E->pair_minb = pick.pair_minb;
-    E->pair_geo = pick.pair_geo;
-    E->pair_grid = pick.pair_grid;
+    if (pick.split) {   // (otherwise the cell-pair kernel keeps its default shape for set_shape)
+        E->pair_minb = pick.pair_minb;
+        E->pair_geo = pick.pair_geo;
+        E->pair_grid = pick.pair_grid;
+    }
     // the activity bytes are rebuilt from the state before the next step: trials
     // of split steps leave the paired members' next bytes unwritten
     E->act_valid = false;
@@ -864,7 +916,8 @@ void swe_ensemble_destroy(swe_ensemble* E) {
     void* bufs[] = {E->state[0], E->state[1], E->geoA, E->geoB, E->topo, E->gm2, E->inv, E->tile_member,
                     E->member_first_tile, E->cfl, E->small, E->n_active, E->kind, E->value,
                     E->stage[0], E->stage[1], E->stage[2], E->act[0], E->act[1], E->act[2],
-                    E->ecells, E->eln, E->eflux, E->esrc, E->eidx, E->geoR, E->erl, E->sched};
+                    E->ecells, E->eln, E->eflux, E->esrc, E->eidx, E->geoR, E->erl, E->sched,
+                    E->span_first, E->span_adj, E->act_list, E->act_count, E->member_dt};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (E->cap_stream) cudaStreamDestroy(E->cap_stream);

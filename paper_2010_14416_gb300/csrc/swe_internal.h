@@ -152,6 +152,7 @@ struct swe_mesh {
     int64_t act_len = 0;
     bool act_valid = false;
     unsigned* act_list = nullptr;      // n cells: those that run the flux path in a step
+    unsigned *span_first = nullptr, *span_adj = nullptr;   // the spans beside each span (act_scan_kernel)
     unsigned* act_count = nullptr;     // 2 words, 0 between steps
     // shape of the steps that run without activity bytes (launch_step_raw for
     // other buffers: adjoint, frozen time steps); equals the cfg shape when
@@ -166,8 +167,8 @@ struct swe_mesh {
     void* esrc = nullptr;              // T[E]
     int4* eidx = nullptr;              // per cell, the edge of each local edge (-1: boundary)
     // the step loop (swe_loop.cuh), for a small mesh with nothing chosen about its
-    // launches: the largest mesh it takes (-1: not asked yet), its arrival count
-    // and, FP64, its blocks' edges
+    // launches: the largest mesh it takes (-1: not asked yet), its arrival
+    // count and, FP64, its blocks' edges
     bool loop_allowed = false;
     long long loop_cells = -1;
     unsigned* loop_barrier = nullptr;

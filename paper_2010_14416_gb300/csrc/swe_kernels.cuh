@@ -91,10 +91,13 @@ struct StepArgs {
     const unsigned char* act_in;
     unsigned char* act_next;
     unsigned char* act_clear;
-    // one flag per kScanSpan cells and buffer: the span has a byte that is not 0
+    // one flag per 2^kScanLog cells and buffer: 0 if none of the span's bytes is
+    // set; and the spans next to each (itself among them)
     const unsigned char* span_in;
     unsigned char* span_next;
     unsigned char* span_clear;
+    const unsigned* span_first;
+    const unsigned* span_adj;
     unsigned* act_list;                // cells that run the flux path (act_scan_kernel), in [0, *act_count)
     unsigned* act_count;               // and a count of the blocks that have used it; both 0 between steps
     // edge pass (step_kernel with EDGES): interior edges in canonical orientation,
@@ -150,6 +153,17 @@ struct EnsArgs {
     const unsigned char* act_in;
     unsigned char* act_next;
     unsigned char* act_clear;
+    // list mode: span flags, the spans beside each span, the list of cells that
+    // run the flux path, its count (and one of blocks), each member's step size
+    const unsigned char* span_in;
+    unsigned char* span_next;
+    unsigned char* span_clear;
+    const unsigned* span_first;
+    const unsigned* span_adj;
+    unsigned* act_list;
+    unsigned* act_count;
+    T* member_dt;
+    int n_members;
     // edge pass over the concatenated members (ensemble_step_kernel with EDGES)
     const int2* ecells;
     const T* eln;
@@ -1044,31 +1058,15 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
 // leaves some SMs with several times the average work and makes every quiet
 // cell cost a state record read: that kernel, a cp.async pipeline over all
 // cells, took 96 us a step on the 13M-cell river, 6 % of it wet; the two take
-// 11 (without the flags) and 24 us.
-template <typename T>
-__global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> a) {
+// 10 and 24 us.
+//
+// scan_span: one block's span, its threads' 16 cells from c0 on; `in` says that
+// the thread's cells take part, `step` that they step (else state and activity
+// carry over unchanged).
+template <typename T, typename Args>
+__device__ __forceinline__ void scan_span(const Args& a, unsigned sp, long long c0, long long n, bool in, bool step) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ unsigned total[kScanBlock / 32], base;
-    // whether there is a step (warp_step_dt), by the bits alone: in thousands of
-    // warps an FP64 product each takes microseconds
-    const double dt = a.dt_fixed ? *a.dt_fixed : *a.dt_read;
-    const bool have_dt = (unsigned long long)__double_as_longlong(dt) < kInfBits;
-    const unsigned sp = blockIdx.x;   // the block's span
-    const unsigned char fl = a.span_in[sp], fp = a.span_clear[sp];
-    const long long c0 = ((long long)sp << kScanLog) + threadIdx.x * 16;
-    if (!have_dt) {
-        // no step: the state and its activity carry over unchanged
-        for (long long c = c0; c < c0 + 16 && c < a.n; ++c) {
-            a.s_out[c] = a.s_in[c];
-            a.act_next[c] = a.act_in[c];
-            a.act_clear[c] = 0;
-        }
-        __syncthreads();   // every thread has read the flags
-        if (threadIdx.x == 0) { a.span_next[sp] = fl; a.span_clear[sp] = 0; }
-        return;
-    }
-    if (!(fl | fp)) return;
-    const bool in = c0 < a.n;
     uint4 now = make_uint4(0u, 0u, 0u, 0u), prev = now;
     if (in) {
         now = *(const uint4*)(a.act_in + c0);      // the buffers reach past n in whole 32 bytes
@@ -1087,10 +1085,18 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
         rewrite |= low_bits(v[q] | (v[q] >> 1)) << (4 * q);   // bytes are 0 to 3
     }
     if (rewrite) *(uint4*)(a.act_clear + c0) = make_uint4(0u, 0u, 0u, 0u);
+    bool carry = false;
+    if (in && !step) {
+        carry = (w[0] | w[1] | w[2] | w[3]) != 0u;
+        *(uint4*)(a.act_next + c0) = now;
+        for (long long c = c0; c < c0 + 16 && c < n; ++c) a.s_out[c] = a.s_in[c];
+        runs = 0u;
+        rewrite = 0u;
+    }
     rewrite &= ~runs;
     // a warp whose 512 cells are all to be rewritten (the two steps after the
     // bytes are rebuilt) copies them side by side
-    if (__all_sync(0xffffffffu, rewrite == 0xFFFFu && c0 + 16 <= a.n)) {
+    if (__all_sync(0xffffffffu, rewrite == 0xFFFFu && c0 + 16 <= n)) {
         const long long w0 = c0 - 16 * lane;
 #pragma unroll 4
         for (int k = 0; k < 16; ++k) {
@@ -1101,7 +1107,7 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
     } else {
         for (unsigned m = rewrite; m; m &= m - 1u) {
             const long long c = c0 + __ffs(m) - 1;
-            if (c < a.n) {
+            if (c < n) {
                 V4<T> s = a.s_in[c];
                 s.y = T(0); s.z = T(0);
                 a.s_out[c] = s;
@@ -1115,7 +1121,7 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
         if (lane >= o) pos += up;
     }
     if (lane == 31) total[warp] = pos;
-    __syncthreads();   // (every thread has read the flags, too)
+    const bool any_carry = __syncthreads_or(carry);   // (and every thread has read the span's flags)
     unsigned before = 0u, all = 0u;
 #pragma unroll
     for (int q = 0; q < kScanBlock / 32; ++q) {
@@ -1123,12 +1129,29 @@ __global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> 
         all += total[q];
     }
     if (threadIdx.x == 0) {
-        base = atomicAdd(a.act_count, all);
+        if (all) base = atomicAdd(a.act_count, all);
         a.span_clear[sp] = 0;
     }
+    // the cells that this step will mark lie in this span or one beside it (the
+    // marking kernel's own stores to a few hot flags took it from 24 to 33 us)
+    if (all || any_carry)
+        for (unsigned q = a.span_first[sp] + threadIdx.x; q < a.span_first[sp + 1]; q += kScanBlock)
+            a.span_next[a.span_adj[q]] = 1;
     __syncthreads();
     unsigned at = base + before + pos - cnt;
     for (unsigned m = runs; m; m &= m - 1u) a.act_list[at++] = (unsigned)c0 + __ffs(m) - 1;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kScanBlock) act_scan_kernel(const StepArgs<T> a) {
+    // whether there is a step (warp_step_dt), by the bits alone: in thousands of
+    // warps an FP64 product each takes microseconds
+    const double dt = a.dt_fixed ? *a.dt_fixed : *a.dt_read;
+    const bool have_dt = (unsigned long long)__double_as_longlong(dt) < kInfBits;
+    const unsigned sp = blockIdx.x;   // the block's span
+    if (!(a.span_in[sp] | a.span_clear[sp])) return;
+    const long long c0 = ((long long)sp << kScanLog) + threadIdx.x * 16;
+    scan_span<T>(a, sp, c0, a.n, c0 < a.n, have_dt);
 }
 
 // The listed cells' update and marks.  Each thread keeps the state and
@@ -1179,20 +1202,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_act(const StepArgs<T>
         // the topology record and the cell are read again from shared memory
         // rather than kept live in registers across the update
         const volatile int* tv = (const volatile int*)&st_topo[slot][tid];
-        if (wet || (tv[3] & kStaticBit)) {
-            const unsigned me = ((const volatile unsigned*)st_cell[slot])[tid];
-            a.act_next[me] = 1;
-            a.span_next[me >> kScanLog] = 1;
-            if (wet) {
+        if (wet || (tv[3] & kStaticBit)) a.act_next[((const volatile unsigned*)st_cell[slot])[tid]] = 1;
+        if (wet) {
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const int code = tv[j];
-                    if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups))) {
-                        const unsigned nb = (unsigned)code & kNbrMask;
-                        a.act_next[nb] = 1;
-                        if ((nb ^ me) >> kScanLog) a.span_next[nb >> kScanLog] = 1;
-                    }
-                }
+            for (int j = 0; j < 3; ++j) {
+                const int code = tv[j];
+                if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups))) a.act_next[code & kNbrMask] = 1;
             }
         }
         slot = slot == PF - 1 ? 0 : slot + 1;
@@ -1400,6 +1415,139 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_dyn(const En
     if ((tid & 31) == 0 && active) atomicAdd(a.n_active, (unsigned long long)active);
 }
 
+// ---- batched ensemble step over a list of its active cells ---------------------------
+// The list mode of the ensemble (QUEUE): the mesh's two launches (act_scan_kernel,
+// step_kernel_act) over the concatenated members.  The scan also forms each
+// member's step size and does its bookkeeping; cells before cell_lo belong to
+// the cell-pair kernel.  24 canal and river members of 3.7M cells in all, half
+// of them fully wet: 85 to 89 us a step with any kernel that goes through all
+// river cells (40 us for those), 61 with this one behind the cell-pair kernel.
+template <typename T>
+__global__ void __launch_bounds__(kScanBlock) ens_scan_kernel(const EnsArgs<T> a) {
+    if (blockIdx.x == 0) {
+        for (int mk = threadIdx.x; mk < a.n_members; mk += kScanBlock) {
+            if (a.member_first_tile[mk] * kEnsPad < a.cell_lo) continue;
+            unsigned long long* sm = a.small + 8 * (long long)mk;
+            const double d = a.cfl[mk] * __longlong_as_double((long long)sm[a.slot_read]);
+            a.member_dt[mk] = T(d);
+            sm[a.slot_reset] = kInfBits;
+            if ((unsigned long long)__double_as_longlong(d) < kInfBits) *(double*)(sm + 3) += d;
+            else atomicOr((unsigned*)(sm + 4), kStatusDry);
+        }
+    }
+    const unsigned sp = (unsigned)(a.cell_lo >> kScanLog) + blockIdx.x;
+    if (!(a.span_in[sp] | a.span_clear[sp])) return;
+    const long long c0 = ((long long)sp << kScanLog) + threadIdx.x * 16;
+    const bool in = c0 >= a.cell_lo && c0 < a.n_total;   // (both ends are whole tiles)
+    bool step = true;
+    if (in) step = a.small[8 * (long long)a.tile_member[c0 / kEnsPad] + a.slot_read] < kInfBits;
+    scan_span<T>(a, sp, c0, a.n_total, in, step);
+}
+
+// One lane's CFL minimum to its member's slot; the warp's at once where all
+// lanes have the same member.
+template <typename T>
+__device__ __forceinline__ void publish_member(const EnsArgs<T>& a, int member, T cand) {
+    const int m0 = __shfl_sync(0xffffffffu, member, 0);
+    if (__all_sync(0xffffffffu, member == m0)) {
+        if (m0 >= 0) warp_min_publish<T>(cand, a.small + 8 * (long long)m0 + a.slot_write);
+    } else if (member >= 0 && cand < inf_of<T>()) {
+        atomicMin(a.small + 8 * (long long)member + a.slot_write,
+                  (unsigned long long)__double_as_longlong((double)cand));
+    }
+}
+
+// The listed cells: a block takes an even share of the list in one piece (DYN:
+// pieces of BLOCK << chunk_log2 entries as they come), so that its cells lie
+// together and their member rarely changes.
+template <typename T, int BLOCK, bool GEO_EARLY, bool DYN>
+__device__ __forceinline__ void ens_list_steps(const EnsArgs<T>& a) {
+    constexpr int PF = 2;
+    __shared__ V4<T> st_own[PF][BLOCK];
+    __shared__ int4 st_topo[PF][BLOCK];
+    __shared__ unsigned st_cell[PF][BLOCK];
+    __shared__ unsigned s_piece;
+    const int tid = threadIdx.x;
+    const unsigned n_list = *(volatile const unsigned*)a.act_count;
+    if (DYN && blockIdx.x == 0 && tid == 0) a.sched[a.sched_reset] = 0u;   // the counter of the step after next
+    int member = -1;
+    T cand = inf_of<T>(), dt = T(0);
+    unsigned active = 0u;
+    unsigned lo, hi;
+    const unsigned share = DYN ? (unsigned)BLOCK << a.chunk_log2
+                               : ((n_list + gridDim.x - 1) / gridDim.x + 31u) & ~31u;
+    for (unsigned piece = blockIdx.x;;) {
+        if constexpr (DYN) {
+            __syncthreads();   // every thread has read the last piece
+            if (tid == 0) s_piece = atomicAdd(&a.sched[a.sched_slot], 1u);
+            __syncthreads();
+            piece = s_piece;
+        }
+        const unsigned long long first = (unsigned long long)piece * share;
+        if (first >= n_list) break;
+        lo = (unsigned)first;
+        hi = n_list - lo > share ? lo + share : n_list;
+        auto fetch = [&](int slot, unsigned k) {
+            if (k < hi) {
+                const unsigned c = a.act_list[k];
+                st_cell[slot][tid] = c;
+                cp_async_record<sizeof(V4<T>)>(&st_own[slot][tid], &a.s_in[c]);
+                cp_async_record<16>(&st_topo[slot][tid], &a.topo[c]);
+            }
+            cp_async_commit();
+        };
+        fetch(0, lo + tid);
+        int slot = 0;
+        for (unsigned k0 = lo; k0 < hi; k0 += BLOCK) {     // uniform across the block
+            const unsigned k = k0 + tid;
+            fetch(slot ^ 1, k + BLOCK);
+            cp_async_wait<1>();
+            int mk = member;
+            if (k < hi) mk = a.tile_member[st_cell[slot][tid] / kEnsPad];
+            if (__any_sync(0xffffffffu, mk != member)) {
+                publish_member<T>(a, member, cand);
+                cand = inf_of<T>();
+                member = mk;
+                if (mk >= 0) dt = a.member_dt[mk];
+            }
+            if (k < hi) {
+                const unsigned c = st_cell[slot][tid];
+                unsigned long long* sm = a.small + 8 * (long long)mk;
+                const T r = update_cell<T, GEO_EARLY>(a, c, st_own[slot][tid], st_topo[slot][tid], dt, active, sm + 5,
+                                                      (unsigned*)(sm + 4));
+                cand = min_nonneg(cand, r);
+                const bool wet = r < inf_of<T>();
+                const volatile int* tv = (const volatile int*)&st_topo[slot][tid];
+                if (wet || (tv[3] & kStaticBit)) a.act_next[((const volatile unsigned*)st_cell[slot])[tid]] = 1;
+                if (wet) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        const int code = tv[j];
+                        if (code >= 0 && (!a.debug || code_ok(code, a.n_total, a.n_groups)))
+                            a.act_next[code & kNbrMask] = 1;
+                    }
+                }
+            }
+            slot ^= 1;
+        }
+        cp_async_wait<0>();
+        if constexpr (!DYN) break;
+    }
+    publish_member<T>(a, member, cand);
+    __shared__ unsigned s_active;
+    if (tid == 0) s_active = 0u;
+    __syncthreads();
+    active = __reduce_add_sync(0xffffffffu, active);
+    if ((tid & 31) == 0 && active) atomicAdd(&s_active, active);
+    __syncthreads();
+    if (tid == 0 && s_active) atomicAdd(a.n_active, (unsigned long long)s_active);
+    // the last block to get here empties the list for the next scan
+    if (tid == 0 && atomicAdd(a.act_count + 1, 1u) == gridDim.x - 1) {
+        a.act_count[0] = 0u;
+        a.act_count[1] = 0u;
+    }
+}
+
 // ---- batched ensemble step with activity bytes ----------------------------------------
 // The activity mode of step_kernel_act over the concatenated members: the same
 // bytes, marks and per-thread cp.async pipeline, with the thread's cells taken
@@ -1417,6 +1565,10 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_dyn(const En
 template <typename T, int BLOCK, int MINB, bool GEO_EARLY, bool DYN = false, bool QUEUE = false>
 __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const EnsArgs<T> a) {
     static_assert(kEnsPad % BLOCK == 0, "a tile must not straddle two members");
+    if constexpr (QUEUE) {
+        ens_list_steps<T, BLOCK, GEO_EARLY, DYN>(a);
+        return;
+    } else {
     constexpr unsigned kNone = 0xFFFFFFFFu;
     const unsigned G = gridDim.x, b = blockIdx.x;
     const int cl2 = a.chunk_log2;                   // >= 2 with DYN (the host checks)
@@ -1449,10 +1601,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
         }
     };
     __shared__ V4<T> st_own[3][BLOCK];
-    __shared__ int4 st_topo[QUEUE ? 1 : 2][BLOCK];
-    // QUEUE: each warp's cells that run the flux path, a ring of 64 slots
-    __shared__ unsigned s_q[QUEUE ? BLOCK / 32 : 1][64];
-    unsigned qh = 0u, qt = 0u;                               // warp-uniform head and tail
+    __shared__ int4 st_topo[2][BLOCK];
     // per warp: the 32 activity bytes of its cells in 3 stages (lanes 0..7 copy
     // 4 each).  Unlike step_kernel_act, this kernel writes every quiet state:
     // leaving those quiet in two steps in place measured slower here (the
@@ -1475,31 +1624,6 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
     T dt = T(0);
     T cand = inf_of<T>();
     unsigned active = 0u;
-    // QUEUE: the full update of one queued cell (topology read here), its marks
-    auto run_queued = [&](unsigned cq) {
-        const V4<T> own = a.s_in[cq];
-        const int4 tp = a.topo[cq];
-        const T r = update_cell<T, GEO_EARLY>(a, cq, own, tp, dt, active, sm + 5, (unsigned*)(sm + 4));
-        cand = min_nonneg(cand, r);
-        const bool wet = r < inf_of<T>();
-        if (wet || (tp.w & kStaticBit)) a.act_next[cq] = 1;
-        if (wet) {
-            const int code[3] = {tp.x, tp.y, tp.z};
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (code[j] >= 0 && (!a.debug || code_ok(code[j], a.n_total, a.n_groups)))
-                    a.act_next[code[j] & kNbrMask] = 1;
-        }
-    };
-    // QUEUE: the queued cells left, on as many lanes (warp-uniform call)
-    auto flush = [&]() {
-        if constexpr (QUEUE) {
-            const unsigned nq = qh - qt;
-            if (lane < nq) run_queued(s_q[warp][(qt + lane) & 63]);
-            qt = qh;
-            __syncwarp();
-        }
-    };
     {
         const unsigned c0 = cell_of(0), c1 = cell_of(1), c2 = cell_of(2);
         act_copy(0, c0);
@@ -1514,7 +1638,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
     unsigned f_cur = act_byte(0);
     {
         const unsigned c0 = cell_of(0);
-        if (!QUEUE && f_cur && c0 != kNone) cp_async_record<16>(&st_topo[0][tid], &a.topo[c0]);
+        if (f_cur && c0 != kNone) cp_async_record<16>(&st_topo[0][tid], &a.topo[c0]);
     }
     cp_async_commit();                                           // T_{-1}
     cp_async_commit();                                           // H_{-1} (empty)
@@ -1530,10 +1654,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
         if (c == kNone) break;                                   // ragged last chunk (block-uniform)
         const int mk = a.tile_member[(c - tid) / kEnsPad];       // uniform across the block
         if (mk != member) {
-            if (member >= 0) {
-                flush();   // with the member's own step and status block
-                warp_min_publish<T>(cand, sm + a.slot_write);
-            }
+            if (member >= 0) warp_min_publish<T>(cand, sm + a.slot_write);
             cand = inf_of<T>();
             member = mk;
             sm = a.small + 8 * (long long)mk;
@@ -1551,7 +1672,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
         __syncwarp();
         const unsigned f_next = act_byte(k3n);
         const unsigned c1 = cell_of(k + 1), c2 = cell_of(k + 2), c3 = cell_of(k + 3);
-        if (!QUEUE && f_next && c1 != kNone) cp_async_record<16>(&st_topo[k2 ^ 1][tid], &a.topo[c1]);
+        if (f_next && c1 != kNone) cp_async_record<16>(&st_topo[k2 ^ 1][tid], &a.topo[c1]);
         cp_async_commit();                                       // T_k
         __syncwarp();
         act_copy(k3, c3);
@@ -1562,25 +1683,6 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
         if (!have_dt) {
             a.s_out[c] = own;
             a.act_next[c] = (unsigned char)f_cur;
-        } else if constexpr (QUEUE) {
-            // quiet cells now; the others join the warp's queue, which runs
-            // whenever it holds a full warp of cells
-            if (!f_cur) {
-                V4<T> out;
-                out.x = own.x; out.y = T(0); out.z = T(0); out.w = own.w;
-                a.s_out[c] = out;
-            }
-            const bool runs = f_cur != 0u;
-            const unsigned m = __ballot_sync(0xffffffffu, runs);
-            if (runs) s_q[warp][(qh + __popc(m & ((1u << lane) - 1u))) & 63] = c;
-            qh += __popc(m);
-            __syncwarp();
-            if (qh - qt >= 32u) {
-                const unsigned cq = s_q[warp][(qt + lane) & 63];
-                qt += 32u;
-                __syncwarp();   // read before later appends reuse the slot
-                run_queued(cq);
-            }
         } else if (!f_cur) {
             V4<T> out;
             out.x = own.x; out.y = T(0); out.z = T(0); out.w = own.w;
@@ -1607,12 +1709,10 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_act(const En
         k2 ^= 1;
     }
     cp_async_wait<0>();
-    if (member >= 0) {
-        flush();
-        warp_min_publish<T>(cand, sm + a.slot_write);
-    }
+    if (member >= 0) warp_min_publish<T>(cand, sm + a.slot_write);
     active = __reduce_add_sync(0xffffffffu, active);
     if ((tid & 31) == 0 && active) atomicAdd(a.n_active, (unsigned long long)active);
+    }
 }
 
 // ---- batched ensemble step over cell pairs (FP32) ------------------------------------

@@ -393,8 +393,7 @@ cudaError_t Launch<T>::ensemble_resident_blocks(int block, int min_blocks, int s
 #define SWE_ENS_ACT_VARIANTS_F64(X) X(256, 1, 0) X(128, 1, 0)
 
 // (block, min blocks per SM, geometry early) shapes of the ensemble's activity
-// kernel with per-warp queues of the cells that run the flux path (FP32); at
-// 8 blocks of 128 (64 registers) the queue's state spills 40-60 B
+// step over a list of the cells that run the flux path (FP32)
 #define SWE_ENS_ACTQ_VARIANTS_F32(X) X(128, 7, 1) X(128, 7, 0) X(128, 6, 1)
 
 template <typename T>
@@ -403,6 +402,9 @@ cudaError_t Launch<T>::ensemble_step_act(const EnsArgs<T>& a, int block, int min
     if (grid == 0 || !a.act_in || (dynamic && (!a.sched || a.chunk_log2 < 2))) return cudaErrorInvalidValue;
     if (queue) {
         if constexpr (sizeof(T) == 4) {
+            if (!a.act_list) return cudaErrorInvalidValue;
+            const long long spans = ((a.n_total + (1 << kScanLog) - 1) >> kScanLog) - (a.cell_lo >> kScanLog);
+            if (spans > 0) ens_scan_kernel<T><<<(unsigned)spans, kScanBlock, 0, st>>>(a);
 #define SWE_LAUNCH(B, M, G) \
     if (block == B && min_blocks == M && geo_early == G) {                                       \
         if (dynamic) ensemble_step_kernel_act<T, B, M, G != 0, true, true><<<grid, B, 0, st>>>(a); \
@@ -610,15 +612,16 @@ cudaError_t Launch<T>::loop_capacity(int device, long long* cells) {
 
 template <typename T>
 cudaError_t Launch<T>::loop(const LoopArgs<T>& a, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(a.barrier, 0, sizeof(unsigned), st);
+    const unsigned grid = grid_for<T>(a.n, sizeof(T) == 4 ? kLoopBlock32 : kLoopCells);
+    const cudaError_t e = cudaMemsetAsync(a.barrier, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
     if constexpr (sizeof(T) == 4)
         return cudaLaunchCooperativeKernel((const void*)step_loop_f32<kLoopBlock32, kLoopMin32>,
-                                           dim3(grid_for<T>(a.n, kLoopBlock32)), dim3(kLoopBlock32), args, 0, st);
+                                           dim3(grid), dim3(kLoopBlock32), args, 0, st);
     else
-        return cudaLaunchCooperativeKernel((const void*)step_loop_f64<kLoopMin64>, dim3(grid_for<T>(a.n, kLoopCells)),
-                                           dim3(kLoopEdges), args, 0, st);
+        return cudaLaunchCooperativeKernel((const void*)step_loop_f64<kLoopMin64>,
+                                           dim3(grid), dim3(kLoopEdges), args, 0, st);
 }
 
 template <typename T>

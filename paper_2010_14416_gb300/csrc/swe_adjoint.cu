@@ -165,11 +165,15 @@ __device__ __forceinline__ bool soft_adjoint(double x) { return f64::in_range<-4
 // edge-pass arithmetic) instead of evaluating them; R_i is the same bit for bit.
 // TRANSPOSE transposes the friction update by hand (friction_rev) instead of
 // running it on seven-component duals.
+// `st` is the step whose update is transposed, L the cell's lambda after it.
+struct AdjStep {
+    const V4<double>* U;               // state U^n
+    const V4<double>* eflux;           // edge terms of U^n, with the edge pass
+    const double* esrc;
+    double dt;
+};
 template <bool EDGES, bool TRANSPOSE>
-__global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    const V4<double> L = a.lam[i];
+__device__ __forceinline__ void adj_phase1(const AdjArgs& a, const AdjStep& st, long long i, const V4<double>& L) {
     if (TRANSPOSE && ((__double_as_longlong(L.x) | __double_as_longlong(L.y) | __double_as_longlong(L.z)) << 1) == 0LL &&
         !a.debug) {
         // a cell that no gauge's influence has reached yet passes nothing on
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
         return;
     }
     const double g = a.g, h_dry = a.h_dry;
-    const V4<double> own = a.U[i];
+    const V4<double> own = st.U[i];
     const V4<double> gA = a.geoA[i], gB = a.geoB[i], gR = a.geoR[i];
     const int4 tp = a.topo[i];
     const int code[3] = {adj_code(a, tp.x), adj_code(a, tp.y), adj_code(a, tp.z)};
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
         double tm = 0.0, tx, ty;
         const int c = code[j];
         if (c >= 0) {
-            const V4<double> o = a.U[c & kNbrMask];
+            const V4<double> o = st.U[c & kNbrMask];
             const bool flip = (c & kFlipBit) != 0;
             if constexpr (EDGES) {
                 if (!gt_pos(hi, h_dry) && !gt_pos(o.x, h_dry)) {
@@ -210,10 +214,10 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
                         atomicOr(a.status, kStatusBadIndex);
                         e = 0;
                     }
-                    const V4<double> fl = a.eflux[e];
+                    const V4<double> fl = st.eflux[e];
                     tm = flip ? -fl.x : fl.x;
                     tx = flip ? -fl.w : fl.y;
-                    ty = flip ? -a.esrc[e] : fl.z;
+                    ty = flip ? -st.esrc[e] : fl.z;
                 }
             } else {
                 f64::Side other{o.x, 0.0, 0.0, o.w};
@@ -240,22 +244,22 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
     if constexpr (TRANSPOSE) {
         // the forward's clamps (h < 0 zeroes the cell, h <= h_dry zeroes momentum) on
         // the new depth, then the friction update's transpose
-        const double hn = f64::add(hi, -f64::mul(m, f64::mul(a.dt, ia)));   // f64::update
+        const double hn = f64::add(hi, -f64::mul(m, f64::mul(st.dt, ia)));   // f64::update
         if (hn < 0.0) { lh = 0.0; lx_ = 0.0; ly_ = 0.0; }
         else if (hn <= h_dry) { lx_ = 0.0; ly_ = 0.0; }
         const double gm2 = a.gm2[i];
         if (f64::in_range<-64, 24>(hi) && f64::in_range<-64, 24>(own.y) && f64::in_range<-64, 24>(own.z) &&
-            f64::in_range<-64, 16>(gm2) && f64::in_range<-64, 24>(a.dt) && f64::in_range<-192, 128>(Rh) &&
+            f64::in_range<-64, 16>(gm2) && f64::in_range<-64, 24>(st.dt) && f64::in_range<-192, 128>(Rh) &&
             f64::in_range<-192, 128>(Rx) && f64::in_range<-192, 128>(Ry) && soft_adjoint(lh) && soft_adjoint(lx_) &&
             soft_adjoint(ly_))
-            friction_rev<f64::SoftFlush>(hi, own.y, own.z, gm2, Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
+            friction_rev<f64::SoftFlush>(hi, own.y, own.z, gm2, Rh, Rx, Ry, st.dt, h_dry, lh, lx_, ly_, w);
         else
-            friction_rev<f64::Hard>(hi, own.y, own.z, gm2, Rh, Rx, Ry, a.dt, h_dry, lh, lx_, ly_, w);
+            friction_rev<f64::Hard>(hi, own.y, own.z, gm2, Rh, Rx, Ry, st.dt, h_dry, lh, lx_, ly_, w);
     } else {
         // Phi on duals: seeds h, hu, hv, g m^2, Rh, Rx, Ry
         D7 dh, dqx, dqy;
         friction_update<D7>(D7::seed(hi, 0), D7::seed(own.y, 1), D7::seed(own.z, 2), D7::seed(a.gm2[i], 3),
-                            D7::seed(Rh, 4), D7::seed(Rx, 5), D7::seed(Ry, 6), D7(a.dt), D7(h_dry), dh, dqx, dqy);
+                            D7::seed(Rh, 4), D7::seed(Rx, 5), D7::seed(Ry, 6), D7(st.dt), D7(h_dry), dh, dqx, dqy);
         // the forward's clamps: h < 0 zeroes the cell, h <= h_dry zeroes momentum
         const double hn = hi + dh.v;
         if (hn < 0.0) { lh = 0.0; lx_ = 0.0; ly_ = 0.0; }
@@ -276,6 +280,13 @@ __global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
     nu.z = w[6] * ia;
     nu.w = 0.0;
     a.nu[i] = nu;
+}
+
+template <bool EDGES, bool TRANSPOSE>
+__global__ void __launch_bounds__(128) adj_phase1_kernel(const AdjArgs a) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.n) return;
+    adj_phase1<EDGES, TRANSPOSE>(a, AdjStep{a.U, a.eflux, a.esrc, a.dt}, i, a.lam[i]);
 }
 
 __global__ void __launch_bounds__(128) adj_phase2_kernel(const AdjArgs a) {
@@ -558,9 +569,15 @@ __device__ __forceinline__ void edge_interior_rev(const V4<double>& L, const V4<
     dR.w = zleft ? bhR : -bhL;
 }
 
+__device__ __forceinline__ bool soft_state(const V4<double>& s) {
+    return f64::in_range<-64, 24>(s.x) && f64::in_range<-64, 24>(s.y) && f64::in_range<-64, 24>(s.z) &&
+           f64::in_range<-64, 24>(s.w);
+}
+
 // Reverse of a boundary edge's flux (f64::boundary_flux): adds to d the
 // adjoints of cell c's (h, hu, hv, z) for the adjoints of the flux leaving it.
-__device__ __forceinline__ void boundary_rev(int kind, double value, const V4<double>& c, double n1, double n2,
+// (Out of line: 20 registers less for the cells without one.)
+__device__ __noinline__ void boundary_rev(int kind, double value, const V4<double>& c, double n1, double n2,
                                              double g2, double h_dry, bool hll_only, double wF0, double wF1, double wF2,
                                              double d[4]) {
     const double bG1 = wF0, bG2 = wF1 * n1 + wF2 * n2;
@@ -581,6 +598,8 @@ __device__ __forceinline__ void boundary_rev(int kind, double value, const V4<do
     const double x = f64::sub(value, c.w);
     const double hg = kind == kBcStage ? max_zero(x) : c.x;
     double bh = 0.0, bun = 0.0, but = 0.0, bhg = 0.0, bung = 0.0, butg = 0.0;
+    // (on the FP64 pipe: few warps come here, and a lone warp's chain of Soft
+    // operations takes longer than of FP64 instructions)
     riemann_rev<f64::Hard>(c.x, un, ut, hg, un, ut, g2, h_dry, hll_only, bG1, bG2, bG3, bh, bun, but, bhg, bung, butg);
     bun += bung;
     but += butg;
@@ -598,11 +617,6 @@ __device__ __forceinline__ void boundary_rev(int kind, double value, const V4<do
 __device__ __forceinline__ bool zero3(const V4<double>& v) {
     return ((__double_as_longlong(v.x) | __double_as_longlong(v.y) | __double_as_longlong(v.z)) << 1) == 0LL;
 }
-__device__ __forceinline__ bool soft_state(const V4<double>& s) {
-    return f64::in_range<-64, 24>(s.x) && f64::in_range<-64, 24>(s.y) && f64::in_range<-64, 24>(s.z) &&
-           f64::in_range<-64, 24>(s.w);
-}
-
 // Phase 2, edges: each interior edge once, the adjoints of both cells' states
 // through it, into ed[2 e] (left cell) and ed[2 e + 1] (right cell).
 __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
@@ -642,9 +656,7 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
 // Phase 2, cells: lambda^n_j = own term + the contributions of j's interior
 // edges (in local edge order) + its boundary edges' (own state only);
 // dL/dz_j likewise.
-__global__ void __launch_bounds__(128) adj_cell_kernel(const AdjArgs a) {
-    const long long jc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (jc >= a.n) return;
+__device__ __forceinline__ V4<double> adj_cell(const AdjArgs& a, long long jc) {
     const int4 tp = a.topo[jc];
     const int code[3] = {adj_code(a, tp.x), adj_code(a, tp.y), adj_code(a, tp.z)};
     const int4 ei = a.eidx[jc];
@@ -685,8 +697,25 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const AdjArgs a) {
     out.y = aw.y + acc[1];
     out.z = aw.z + acc[2];
     out.w = 0.0;
-    a.lam[jc] = out;
     a.gz[jc] += acc[3];
+    return out;
+}
+
+__global__ void __launch_bounds__(128, 4) adj_cell_kernel(const AdjArgs a) {
+    const long long jc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (jc < a.n) a.lam[jc] = adj_cell(a, jc);
+}
+
+// adj_cell_kernel of one step and adj_phase1_kernel of the step before it: the
+// cell's lambda passes from one to the other in registers, and a reverse step
+// is two launches in place of three, half of each latency on 20,000 cells (a
+// reverse step's kernels 38 -> 34 us).
+template <bool EDGES>
+__global__ void __launch_bounds__(128, 4) adj_cell_phase1_kernel(const AdjArgs a, const AdjStep before) {
+    const long long jc = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (jc >= a.n) return;
+    const V4<double> lam = adj_cell(a, jc);
+    adj_phase1<EDGES, true>(a, before, jc, lam);
 }
 
 // loss += sum_g (h_g - target_g)^2 for one observation (one thread: fixed order)
@@ -1013,26 +1042,34 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
             ea.esrc = ssrc + k * Eb;
             e = Launch<double>::edge_flux(ea, st);
         }
+        bool phase1_done = false;   // by the launch before
         for (int64_t k = n1 - n0 - 1; k >= 0 && e == cudaSuccess; --k) {
             a.U = (const V4<double>*)(segp + k * sb);
             a.dt = dts[n0 + k];
             if (keep) {
                 a.eflux = sflux + k * Eb;
                 a.esrc = ssrc + k * Eb;
-                adj_phase1_kernel<true, true><<<grid, block, 0, st>>>(a);
+                if (!phase1_done) adj_phase1_kernel<true, true><<<grid, block, 0, st>>>(a);
             } else if (edges) {
                 ea.s_in = a.U;
                 e = Launch<double>::edge_flux(ea, st);
                 if (e != cudaSuccess) break;
                 if (transposes) adj_phase1_kernel<true, true><<<grid, block, 0, st>>>(a);
                 else adj_phase1_kernel<true, false><<<grid, block, 0, st>>>(a);
-            } else {
+            } else if (!phase1_done) {
                 if (transposes) adj_phase1_kernel<false, true><<<grid, block, 0, st>>>(a);
                 else adj_phase1_kernel<false, false><<<grid, block, 0, st>>>(a);
             }
+            // the step before follows at once where its edge terms are at hand and no
+            // observation enters lambda in between
+            phase1_done = transposes && (keep || !edges) && k > 0 && (n0 + k) % obs_every != 0;
             if (transposes) {
                 adj_edge_kernel<<<egrid, eblock, 0, st>>>(a);
-                adj_cell_kernel<<<grid, block, 0, st>>>(a);
+                const AdjStep before{(const V4<double>*)(segp + (k - 1) * sb), keep ? sflux + (k - 1) * Eb : nullptr,
+                                     keep ? ssrc + (k - 1) * Eb : nullptr, phase1_done ? dts[n0 + k - 1] : 0.0};
+                if (phase1_done && keep) adj_cell_phase1_kernel<true><<<grid, block, 0, st>>>(a, before);
+                else if (phase1_done) adj_cell_phase1_kernel<false><<<grid, block, 0, st>>>(a, before);
+                else adj_cell_kernel<<<grid, block, 0, st>>>(a);
             } else {
                 adj_phase2_kernel<<<grid, block, 0, st>>>(a);
             }

@@ -368,6 +368,9 @@ int run_loop(swe_mesh* m, int64_t nsteps, double cfl) {
     a.ecell = m->loop_ecell;
     a.egeo = m->loop_egeo;
     a.eslot = m->loop_eslot;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->cfg.device) != cudaSuccess) sms = 0;
+    a.one_block_sms = a.n <= (long long)sms * kLoopCells;
     m->act_valid = false;   // steps without activity bytes do not maintain them
     while (nsteps > 0) {
         a.step0 = m->nstep;

@@ -229,6 +229,13 @@ struct Soft {
     static __device__ __forceinline__ double sqrt_rsqrt(double x, double& y) { return root<true>(x, y); }
 };
 
+// Soft's values with products on the FP64 pipe, for a kernel that runs a warp
+// or less per SM quarter: there a chain of products takes 64 clocks each on
+// the pipe and about 130 on the integer unit.
+struct SoftRoots : Soft {
+    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+};
+
 // For adjoints, whose products may become as small as they like.
 struct SoftFlush : Soft {
     static __device__ __forceinline__ double mul(double a, double b) { return product<true>(a, b); }
@@ -354,8 +361,9 @@ __device__ __forceinline__ void velocity_by(double h, double hu, double hv, doub
     }
 }
 
+template <class S = Soft>
 __device__ __forceinline__ void velocity(double h, double hu, double hv, double h_dry, double& u, double& v) {
-    if (in_range<-64, 24>(h) && in_range<-64, 24>(hu) && in_range<-64, 24>(hv)) velocity_by<Soft>(h, hu, hv, h_dry, u, v);
+    if (in_range<-64, 24>(h) && in_range<-64, 24>(hu) && in_range<-64, 24>(hv)) velocity_by<S>(h, hu, hv, h_dry, u, v);
     else velocity_by<Hard>(h, hu, hv, h_dry, u, v);
 }
 
@@ -409,10 +417,11 @@ static __device__ __noinline__ EdgeTerms edge_hard(Side L, Side R, double n1, do
     edge_by<Hard>(L, R, n1, n2, len, g2, h_dry, hll_only, t);
     return t;
 }
+template <class S = Soft>
 __device__ __forceinline__ void edge(const Side& L, const Side& R, double n1, double n2, double len, double g2,
                                      double h_dry, bool hll_only, EdgeTerms& t) {
     if (soft_side(L) && soft_side(R) && soft_edge(n1, n2, len, g2))
-        edge_by<Soft>(L, R, n1, n2, len, g2, h_dry, hll_only, t);
+        edge_by<S>(L, R, n1, n2, len, g2, h_dry, hll_only, t);
     else
         t = edge_hard(L, R, n1, n2, len, g2, h_dry, hll_only);
 }
@@ -493,12 +502,13 @@ __device__ __forceinline__ void update_by(double h, double qx, double qy, double
 }
 
 // (the ranges as for edge(): Soft's products stay within 2^-900 and 2^740)
+template <class S = Soft>
 __device__ __forceinline__ void update(double h, double qx, double qy, double m, double x, double y, double ia,
                                        double gm2, double dt, double h_dry, double& oh, double& ox, double& oy) {
     if (in_range<-64, 24>(h) && in_range<-64, 24>(qx) && in_range<-64, 24>(qy) && in_range<-128, 64>(m) &&
         in_range<-128, 64>(x) && in_range<-128, 64>(y) && in_range<-64, 64>(ia) && in_range<-64, 16>(gm2) &&
         in_range<-64, 24>(dt))
-        update_by<Soft>(h, qx, qy, m, x, y, ia, gm2, dt, h_dry, oh, ox, oy);
+        update_by<S>(h, qx, qy, m, x, y, ia, gm2, dt, h_dry, oh, ox, oy);
     else
         update_by<Hard>(h, qx, qy, m, x, y, ia, gm2, dt, h_dry, oh, ox, oy);
 }
@@ -509,10 +519,11 @@ __device__ __forceinline__ double cfl_by(double h, double qx, double qy, double 
     const double qm = A::sqrt_(fma(qx, qx, A::mul(qy, qy)));
     return A::mul(A::mul(rin, h), A::rcp(fma(h, A::sqrt_(A::mul(g, h)), qm)));
 }
+template <class S = Soft>
 __device__ __forceinline__ double cfl_candidate(double h, double qx, double qy, double rin, double g) {
     if (in_range<-64, 24>(h) && in_range<-64, 24>(qx) && in_range<-64, 24>(qy) && in_range<-64, 64>(rin) &&
         in_range<-64, 24>(g))
-        return cfl_by<Soft>(h, qx, qy, rin, g);
+        return cfl_by<S>(h, qx, qy, rin, g);
     return cfl_by<Hard>(h, qx, qy, rin, g);
 }
 

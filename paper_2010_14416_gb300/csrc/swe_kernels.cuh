@@ -517,14 +517,14 @@ __device__ __forceinline__ void friction_update(T hi, T qx, T qy, T gm2, T Rh, T
 // From the sums of the edges' terms (f64::EdgeTerms) to the new state, its
 // checks, and the cell's next CFL candidate R_i/(sqrt(g h)+|u|) (Eq 15; +inf
 // when the new state is dry).  Every FP64 cell kernel ends here.
-template <typename Args>
+template <class S = f64::Soft, typename Args>
 __device__ __forceinline__ double finish_cell(const Args& a, long long i, const V4<double>& own, double m, double x,
                                               double y, double ia, double rin, double gm2, double dt,
                                               unsigned long long* n_clamped, unsigned* status) {
     const double g = a.g, h_dry = a.h_dry;
     V4<double> out;
     out.w = own.w;
-    f64::update(own.x, own.y, own.z, m, x, y, ia, gm2, dt, h_dry, out.x, out.y, out.z);
+    f64::update<S>(own.x, own.y, own.z, m, x, y, ia, gm2, dt, h_dry, out.x, out.y, out.z);
     if (lt_zero(out.x)) {
         out.x = 0.0; out.y = 0.0; out.z = 0.0;
         atomicAdd(n_clamped, 1ULL);
@@ -535,7 +535,7 @@ __device__ __forceinline__ double finish_cell(const Args& a, long long i, const 
     if (!lt_pos(out.x, big) || !abs_lt_pos(out.y, big) || !abs_lt_pos(out.z, big))
         atomicOr(status, kStatusNonFinite);
     store_state(a, i, out);
-    return gt_pos(out.x, h_dry) ? f64::cfl_candidate(out.x, out.y, out.z, rin, g) : inf_of<double>();
+    return gt_pos(out.x, h_dry) ? f64::cfl_candidate<S>(out.x, out.y, out.z, rin, g) : inf_of<double>();
 }
 
 // ---- one FP32 cell of the fused step -------------------------------------------------

@@ -603,7 +603,7 @@ cudaError_t Launch<T>::loop_capacity(int device, long long* cells) {
         *cells = (long long)per_sm * sms * kLoopBlock32;
     } else {
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_loop_f64<kLoopMin64>, kLoopEdges, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_loop_f64<kLoopMin64, f64::Soft>, kLoopEdges, 0);
         *cells = (long long)per_sm * sms * kLoopCells;
     }
     if (e != cudaSuccess || !coop) *cells = 0;
@@ -620,7 +620,8 @@ cudaError_t Launch<T>::loop(const LoopArgs<T>& a, cudaStream_t st) {
         return cudaLaunchCooperativeKernel((const void*)step_loop_f32<kLoopBlock32, kLoopMin32>,
                                            dim3(grid), dim3(kLoopBlock32), args, 0, st);
     else
-        return cudaLaunchCooperativeKernel((const void*)step_loop_f64<kLoopMin64>,
+        return cudaLaunchCooperativeKernel(a.one_block_sms ? (const void*)step_loop_f64<1, f64::SoftRoots>
+                                                           : (const void*)step_loop_f64<kLoopMin64, f64::Soft>,
                                            dim3(grid), dim3(kLoopEdges), args, 0, st);
 }
 

@@ -33,6 +33,7 @@ struct LoopArgs {
     long long n;
     long long step0;                   // index of the first step
     int steps;
+    int one_block_sms;                 // FP64: no SM has more than one block
     double cfl;
     T g, h_dry;
     int hll, debug, n_groups;
@@ -178,7 +179,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_loop_f32(const LoopArgs<floa
 // FP64: three warps evaluate the edges that touch the block's 32 cells, an edge
 // per thread, into shared memory; the first updates the cells.  An edge
 // between two blocks is evaluated by both, the others once.
-template <int MINB>
+// S: f64::SoftRoots while an SM has one block (a warp per quarter), else Soft.
+template <int MINB, class S>
 __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs<double> a) {
     __shared__ int failed;
     __shared__ double term[5][kLoopEdges];
@@ -217,10 +219,10 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
         if (lr.x >= 0) {
             const V4<double> L = load_l2(s_in + lr.x), R = load_l2(s_in + lr.y);
             f64::Side l{L.x, 0.0, 0.0, L.w}, r{R.x, 0.0, 0.0, R.w};
-            f64::velocity(L.x, L.y, L.z, h_dry, l.u, l.v);
-            f64::velocity(R.x, R.y, R.z, h_dry, r.u, r.v);
+            f64::velocity<S>(L.x, L.y, L.z, h_dry, l.u, l.v);
+            f64::velocity<S>(R.x, R.y, R.z, h_dry, r.u, r.v);
             f64::EdgeTerms t;
-            f64::edge(l, r, n1, n2, len, g2, h_dry, a.hll != 0, t);
+            f64::edge<S>(l, r, n1, n2, len, g2, h_dry, a.hll != 0, t);
             term[0][tid] = t.m; term[1][tid] = t.xL; term[2][tid] = t.yL; term[3][tid] = t.xR; term[4][tid] = t.yR;
             wet_edge[tid] = gt_pos(L.x, h_dry) || gt_pos(R.x, h_dry);
         }
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
                             const double2 n = j == 2 ? *(const double2*)&a.geoB[i] : ((const double2*)&a.geoA[i])[j];
                             const int grp = -1 - c;
                             f64::Side side{own.x, 0.0, 0.0, own.w};
-                            f64::velocity(own.x, own.y, own.z, h_dry, side.u, side.v);
+                            f64::velocity<S>(own.x, own.y, own.z, h_dry, side.u, side.v);
                             f64::boundary(a.bc.kind[grp], a.bc.value[grp], side, n.x, n.y,
                                           ((const double*)&a.geoR[i])[j], g2, h_dry, a.hll != 0, tm, tx, ty);
                         }
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
                         x = f64::add(x, tx);
                         y = f64::add(y, ty);
                     }
-                    cand = finish_cell(v, i, own, m, x, y, ia, rin, gm2, dt.t, a.small + kLoopSlotClamp, status);
+                    cand = finish_cell<S>(v, i, own, m, x, y, ia, rin, gm2, dt.t, a.small + kLoopSlotClamp, status);
                     own = next;
                 }
             }

@@ -91,7 +91,10 @@ typedef struct swe_config {
                          matching along the Hilbert order finds one (cell_pairs uses them);
                          FP64 meshes keep the caller's local edge numbering */
     int block_size;   /* threads per block of the step kernel; 0 = library default */
-    int graph_steps;  /* steps captured per CUDA graph; 0 = default, < 0 = no graphs */
+    int graph_steps;  /* steps captured per CUDA graph; 0 = default, < 0 = no graphs.  A small
+                         mesh with nothing chosen about its launches (this field, the shape
+                         fields and the modes below at 0) runs calls of 4 steps and more as one
+                         cooperative launch instead; the results are the same */
     int device;       /* CUDA device ordinal, default 0 */
     int min_blocks;   /* resident blocks per SM the step kernel is compiled for; 0 = default.
                          0 = default (FP32: 2048 / (2 block_size), FP64: 1) */
@@ -107,17 +110,18 @@ typedef struct swe_config {
                            after the test that skips dry cells among dry neighbours (no
                            geometry traffic for those).  Compiled with 1: FP32 (256, 4, 1|3),
                            (128, 8, 1|3); FP64 (128|256, 1, 1).  Results do not depend on it */
-    int activity;     /* 1: keep one activity byte per cell (three rotating buffers, 3 bytes per
-                         cell of device memory): a cell is active when it or a neighbour is wet
+    int activity;     /* 1: keep one activity byte per cell (three rotating buffers and a list of
+                         the active cells, 7 bytes per cell of device memory): a cell is active when it or a neighbour is wet
                          or it has an inflow/stage edge, and an inactive cell takes its update
-                         (h, 0, 0) without reading its topology or its neighbours, and with no
-                         store when it was inactive in the previous step too (the state in the
-                         output buffer, two steps old, is then already the new one); each step
+                         (h, 0, 0) without reading its topology or its neighbours, and without
+                         touching its state when it was inactive in the previous step too (the
+                         state in the output buffer, two steps old, is then already the new one);
+                         a first kernel lists the active cells, a second updates them and
                          marks the cells that the next one must treat as active, and the two
                          steps after a change from outside (set_state, set_bc, the tuner)
                          store every state.  0 (default):
-                         every cell tests its neighbours.  With activity, stages is the
-                         prefetch distance of the streamed state plus one (default 3).
+                         every cell tests its neighbours.  With activity, stages - 1 is the
+                         number of list entries a thread holds or has in flight (default 3).
                          Compiled (block_size, min_blocks, geometry_early, stages) with 1:
                          FP32 (128, 8, 0, 3|4), (256, 4, 0, 3), (512, 2, 0, 3),
                          (128, 8, 1, 3|4|5), (256, 4, 1, 3|4); FP64 (128, 1, 0, 3|4),
@@ -127,7 +131,8 @@ typedef struct swe_config {
                          fluxes; 0 (default): each cell evaluates its own three edges, so every
                          interior flux is evaluated twice.  The edge pass halves the flux
                          arithmetic for more memory traffic: it pays where the arithmetic
-                         bounds the step (FP64).  Compiled cell passes: FP32 (256, 4, 1),
+                         bounds the step (FP64), and an FP64 mesh with nothing chosen about its
+                         launches runs it.  Compiled cell passes: FP32 (256, 4, 1),
                          (128, 8, 1); FP64 (128|256, 1, 1), all with geometry_early 0.  Not
                          with activity.  Results do not depend on it */
     int grid;         /* blocks launched per step by the step kernel (each block loops over its
@@ -307,7 +312,8 @@ SWE_API int swe_run_to_steady(swe_mesh* mesh, double cfl, double tol, int64_t ch
  * and its gradient with the step sizes held at the forward run's values
  * (the dt sequence is not differentiated; dts_out, if not NULL, receives it:
  * [nsteps] host doubles).  States are checkpointed every checkpoint_every
- * steps (0 = 50) and recomputed segment by segment in the reverse sweep.
+ * steps (0 = 50) and recomputed segment by segment in the reverse sweep,
+ * unless the states of all steps fit 1.5 GiB, where nothing is recomputed.
  *   gauge_cells [n_gauges] caller cell indices; target_h [n_gauges] (host)
  *   loss        one host double
  *   grad_manning, grad_bathy: [n_tris] doubles in the caller's cell order, on
@@ -317,7 +323,8 @@ SWE_API int swe_run_to_steady(swe_mesh* mesh, double cfl, double tol, int64_t ch
  * and bed source terms (Eq 12-30) once per edge for both of its cells
  * (swe_adjoint_method).
  * Device memory: about (nsteps/checkpoint_every + checkpoint_every + 4) x 32 B per cell,
- * plus 64 B per interior edge.
+ * plus 64 B per interior edge and, with the edge pass, 40 B per interior edge
+ * and step of a segment; the mesh keeps up to 1.5 GiB of it for its next call.
  * Errors: SWE_EINVAL (FP32 mesh, no state, bad gauge), SWE_ENOMEM, SWE_ECUDA,
  * SWE_ENONFINITE, SWE_EDRY, SWE_EMESH (debug checks).
  */

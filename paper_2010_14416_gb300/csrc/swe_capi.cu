@@ -329,6 +329,9 @@ int build_loop_edges(swe_mesh* m) {
 template <typename T>
 bool use_loop(swe_mesh* m, int64_t nsteps) {
     if (!m->loop_allowed || nsteps < 4) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    if (cs != cudaStreamCaptureStatusNone) return false;
     if (m->loop_cells < 0) {
         long long cells = 0;
         if (Launch<T>::loop_capacity(m->cfg.device, &cells) != cudaSuccess) { (void)cudaGetLastError(); cells = 0; }
@@ -339,10 +342,7 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
             if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
         }
     }
-    if (m->hm.n_cells > m->loop_cells) return false;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
-    return cs == cudaStreamCaptureStatusNone;
+    return m->hm.n_cells <= m->loop_cells;
 }
 
 template <typename T>

@@ -76,3 +76,21 @@ def test_loop_without_water_reports_it_and_keeps_the_state(precision):
         m.step(10)
     assert e.value.code == capi.SWE_EDRY
     assert all(np.array_equal(x, np.zeros_like(x)) for x in m.get_state())
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+def test_steps_under_stream_capture_are_single_launches(precision):
+    # a mesh's first steps, captured by the caller: no cooperative launch, no
+    # allocation, and the replayed graph gives the same states
+    mi = mg.river(60, 12, seed=4, n_bumps=20)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    captured, single = _mesh(mi, precision), _mesh(mi, precision, graph_steps=-1)
+    captured.set_stream(stream)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        captured.step(6, sync=False)
+    graph.replay()
+    torch.cuda.synchronize()
+    captured.set_stream(None)
+    assert captured.info()["t"] == single.step(6)
+    _equal(captured, single)

@@ -207,7 +207,7 @@ __device__ __forceinline__ void adj_phase1(const AdjArgs& a, const AdjStep& st, 
             const bool flip = (c & kFlipBit) != 0;
             if constexpr (EDGES) {
                 if (!gt_pos(hi, h_dry) && !gt_pos(o.x, h_dry)) {
-                    f64::dry_edge(hi, zi, o.w, n1, n2, len, g2, tx, ty);
+                    f64::dry_edge(hi, zi, o.w, n1, n2, g2, tx, ty);
                 } else {
                     int e = j == 0 ? ei.x : (j == 1 ? ei.y : ei.z);
                     if (a.debug && !(e >= 0 && e < a.n_edges)) {
@@ -223,19 +223,19 @@ __device__ __forceinline__ void adj_phase1(const AdjArgs& a, const AdjStep& st, 
                 f64::Side other{o.x, 0.0, 0.0, o.w};
                 f64::velocity(o.x, o.y, o.z, h_dry, other.u, other.v);
                 f64::EdgeTerms t;
-                f64::edge(flip ? other : own_side, flip ? own_side : other, flip ? -n1 : n1, flip ? -n2 : n2, len, g2,
-                          h_dry, a.hll != 0, t);
+                f64::edge(flip ? other : own_side, flip ? own_side : other, flip ? -n1 : n1, flip ? -n2 : n2, g2, h_dry,
+                          a.hll != 0, t);
                 tm = flip ? -t.m : t.m;
                 tx = flip ? -t.xR : t.xL;
                 ty = flip ? -t.yR : t.yL;
             }
         } else {
             const int grp = -1 - c;
-            f64::boundary(a.bc.kind[grp], a.bc.value[grp], own_side, n1, n2, len, g2, h_dry, a.hll != 0, tm, tx, ty);
+            f64::boundary(a.bc.kind[grp], a.bc.value[grp], own_side, n1, n2, g2, h_dry, a.hll != 0, tm, tx, ty);
         }
-        m = f64::add(m, tm);
-        x = f64::add(x, tx);
-        y = f64::add(y, ty);
+        m = f64::fma(len, tm, m);
+        x = f64::fma(len, tx, x);
+        y = f64::fma(len, ty, y);
     }
     const double ia = gB.z;
     const double Rh = -m * ia, Rx = -x * ia, Ry = -y * ia;
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
         const V4<double> L = a.U[lr.x], R = a.U[lr.y];
         const double n1 = a.eln[2 * e], n2 = a.eln[2 * e + 1], len = a.erl[e];
         const double g2 = f64::mul(0.5, a.g);
-        if (soft_state(L) && soft_state(R) && f64::soft_edge(n1, n2, len, g2) && soft_adjoint(nl.x) &&
+        if (soft_state(L) && soft_state(R) && f64::soft_edge(n1, n2, g2) && f64::in_range<-64, 40>(len) && soft_adjoint(nl.x) &&
             soft_adjoint(nl.y) && soft_adjoint(nl.z) && soft_adjoint(nr.x) && soft_adjoint(nr.y) && soft_adjoint(nr.z))
             edge_interior_rev<f64::SoftFlush>(L, R, n1, n2, len, g2, a.h_dry, a.hll != 0, nl, nr, dl, dr);
         else

@@ -286,7 +286,7 @@ int build_loop_edges(swe_mesh* m) {
     const HostMesh& H = m->hm;
     const int64_t n = H.n_cells, nb = (n + kLoopCells - 1) / kLoopCells;
     std::vector<int2> ecell(nb * kLoopEdges, make_int2(-1, -1));
-    std::vector<double> egeo(nb * 3 * kLoopEdges, 0.0);
+    std::vector<double> egeo(nb * 2 * kLoopEdges, 0.0);
     std::vector<uchar4> eslot(n, make_uchar4(0, 0, 0, 0));
     auto slot = [&](int64_t c, int j) -> unsigned char& { return j == 0 ? eslot[c].x : (j == 1 ? eslot[c].y : eslot[c].z); };
     for (int64_t b = 0; b < nb; ++b) {
@@ -304,12 +304,11 @@ int build_loop_edges(swe_mesh* m) {
                 }
                 const bool flip = (code & kFlipBit) != 0;
                 double lx = H.ln[6 * c + 2 * j], ly = H.ln[6 * c + 2 * j + 1];
-                const double len = host_unit_normal(lx, ly);
+                (void)host_unit_normal(lx, ly);
                 ecell[b * kLoopEdges + ne] = flip ? make_int2((int)k, (int)c) : make_int2((int)c, (int)k);
-                double* g = &egeo[b * 3 * kLoopEdges + ne];
+                double* g = &egeo[b * 2 * kLoopEdges + ne];
                 g[0] = flip ? -lx : lx;
                 g[kLoopEdges] = flip ? -ly : ly;
-                g[2 * kLoopEdges] = len;
                 slot(c, j) = (unsigned char)ne++;
             }
     }

@@ -16,9 +16,9 @@
 //   - Eq 24 needs only the sign of S*.  Eq 25's numerator is minus Eq 18's
 //     numerator of the mass flux and its denominator is negative, so between
 //     S_L and S_R that is the sign of the mass flux;
-//   - an edge's flux and its two bed source terms are combined per edge, times
-//     the edge's length, into what each of its cells subtracts (5 numbers), so
-//     a cell adds three numbers per edge.
+//   - an edge's flux and its two bed source terms are combined per edge into
+//     what each of its cells subtracts (5 numbers per unit length), so a cell
+//     takes three fused multiply-adds per edge.
 // Measured against IEEE division and square root with the textbook order of
 // operations, all on the FP64 pipe: 2^20 Riemann problems 418 us, 215 with the
 // shorter formulas and roots, 90 with Soft; a step of the 1M-cell canal with
@@ -258,13 +258,13 @@ __device__ __forceinline__ double rcbrt(double x) {
     return fma(y, p, y);
 }
 
-// ---- Riemann flux in the edge-normal frame (Eq 14, 17-26), times `len` -----------------
-// Readings as in riemann_hllc.  PL, PR receive g h_K^2 / 2.  Without SCALED
-// the flux is per unit length.  `speeds`, if given, receives S_L, S_R, S*.
-template <typename A, bool SCALED>
+// ---- Riemann flux in the edge-normal frame (Eq 14, 17-26) ------------------------------
+// Readings as in riemann_hllc.  PL, PR receive g h_K^2 / 2; `speeds`, if given,
+// S_L, S_R, S*.
+template <typename A>
 __device__ __forceinline__ void riemann(double hL, double unL, double utL, double hR, double unR, double utR,
-                                        double g2, double h_dry, double len, double& G1, double& G2, double& G3,
-                                        double& PL, double& PR, double* speeds, bool hll_only) {
+                                        double g2, double h_dry, double& G1, double& G2, double& G3, double& PL,
+                                        double& PR, double* speeds, bool hll_only) {
     const bool wetL = gt_pos(hL, h_dry), wetR = gt_pos(hR, h_dry);
     const double ghL = A::mul(g2, hL), ghR = A::mul(g2, hR);
     PL = A::mul(ghL, hL);
@@ -302,19 +302,16 @@ __device__ __forceinline__ void riemann(double hL, double unL, double utL, doubl
     const bool supL = ge_zero(SL), supR = !supL && le_zero(SR);
     bool upL = supL;
     if (supL) {                                                                // Eq 17
-        G1 = SCALED ? A::mul(qL, len) : qL;
+        G1 = qL;
         G2 = fma(qL, unL, PL);
-        if (SCALED) G2 = A::mul(G2, len);
         if (hll_only) G3 = A::mul(G1, utL);
     } else if (supR) {
-        G1 = SCALED ? A::mul(qR, len) : qR;
+        G1 = qR;
         G2 = fma(qR, unR, PR);
-        if (SCALED) G2 = A::mul(G2, len);
         if (hll_only) G3 = A::mul(G1, utR);
         upL = wetL && !wetR && ge_zero(SR);
     } else {                                                                   // Eq 18
-        double r = A::rcp(sub(SR, SL));
-        if (SCALED) r = A::mul(r, len);
+        const double r = A::rcp(sub(SR, SL));
         const double ss = A::mul(SR, SL);
         const double fL = fma(qL, unL, PL), fR = fma(qR, unR, PR);
         G1 = A::mul(fma(ss, sub(hR, hL), fma(-SL, qR, A::mul(SR, qL))), r);
@@ -345,9 +342,9 @@ __device__ __forceinline__ void riemann_any(double hL, double unL, double utL, d
     double PL, PR;
     if (in_range<-64, 24>(hL) && in_range<-64, 24>(hR) && in_range<-100, 40>(unL) && in_range<-100, 40>(utL) &&
         in_range<-100, 40>(unR) && in_range<-100, 40>(utR) && in_range<-64, 24>(g2))
-        riemann<Soft, false>(hL, unL, utL, hR, unR, utR, g2, h_dry, 1.0, G1, G2, G3, PL, PR, speeds, hll_only);
+        riemann<Soft>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
     else
-        riemann<Hard, false>(hL, unL, utL, hR, unR, utR, g2, h_dry, 1.0, G1, G2, G3, PL, PR, speeds, hll_only);
+        riemann<Hard>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
 }
 
 template <typename A>
@@ -370,10 +367,12 @@ __device__ __forceinline__ void velocity(double h, double hu, double hv, double 
 // One side of an edge: depth, velocity, bed.
 struct Side { double h, u, v, z; };
 
-// What an edge adds to each of its cells' sums: the flux leaving the cell less
-// its bed source term (Eq 30 with 1/2), times the edge's length.  The mass
-// part is m for the left cell and -m for the right one; the momentum parts
-// are (xL, yL) and -(xR, yR).
+// What an edge adds to each of its cells' sums, per unit length: the flux
+// leaving the cell less its bed source term (Eq 30 with 1/2).  The mass part is
+// m for the left cell and -m for the right one; the momentum parts are (xL, yL)
+// and -(xR, yR).  The cell's sum multiplies by the length in a fused
+// multiply-add: a product rounded per edge would show, since the edges of a
+// cell nearly cancel.
 struct EdgeTerms { double m, xL, yL, xR, yR; };
 
 // One interior edge in its canonical orientation (L is the cell with the lower
@@ -381,8 +380,8 @@ struct EdgeTerms { double m, xL, yL, xR, yR; };
 // side K along the normal are G2 - (g/2)(h*_K^2 - h_K^2), so both sides share
 // the rotation of G3.
 template <typename A>
-__device__ __forceinline__ void edge_by(const Side& L, const Side& R, double n1, double n2, double len, double g2,
-                                     double h_dry, bool hll_only, EdgeTerms& t) {
+__device__ __forceinline__ void edge_by(const Side& L, const Side& R, double n1, double n2, double g2, double h_dry,
+                                        bool hll_only, EdgeTerms& t) {
     // hydrostatic reconstruction (Eq 28): z* = max(z_L, z_R)
     const double zs = max_finite(L.z, R.z);
     const double hL = max_zero(sub(add(L.h, L.z), zs)), hR = max_zero(sub(add(R.h, R.z), zs));
@@ -390,9 +389,9 @@ __device__ __forceinline__ void edge_by(const Side& L, const Side& R, double n1,
     const double unL = fma(L.u, n1, A::mul(L.v, n2)), utL = fma(L.v, n1, -A::mul(L.u, n2));
     const double unR = fma(R.u, n1, A::mul(R.v, n2)), utR = fma(R.v, n1, -A::mul(R.u, n2));
     double G1, G2, G3, PL, PR;
-    riemann<A, true>(hL, unL, utL, hR, unR, utR, g2, h_dry, len, G1, G2, G3, PL, PR, nullptr, hll_only);
+    riemann<A>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, nullptr, hll_only);
     const double sL = fma(-A::mul(g2, L.h), L.h, PL), sR = fma(-A::mul(g2, R.h), R.h, PR);
-    const double pL = fma(-sL, len, G2), pR = fma(-sR, len, G2);
+    const double pL = sub(G2, sL), pR = sub(G2, sR);
     const double t1 = A::mul(G3, n2), t2 = A::mul(G3, n1);
     t.m = G1;
     t.xL = fma(pL, n1, -t1);
@@ -408,32 +407,32 @@ __device__ __forceinline__ void edge_by(const Side& L, const Side& R, double n1,
 __device__ __forceinline__ bool soft_side(const Side& s) {
     return in_range<-64, 24>(s.h) && in_range<-100, 40>(s.u) && in_range<-100, 40>(s.v) && in_range<-64, 24>(s.z);
 }
-__device__ __forceinline__ bool soft_edge(double n1, double n2, double len, double g2) {
-    return in_range<-64, 1>(n1) && in_range<-64, 1>(n2) && in_range<-64, 40>(len) && in_range<-64, 24>(g2);
+__device__ __forceinline__ bool soft_edge(double n1, double n2, double g2) {
+    return in_range<-64, 1>(n1) && in_range<-64, 1>(n2) && in_range<-64, 24>(g2);
 }
-static __device__ __noinline__ EdgeTerms edge_hard(Side L, Side R, double n1, double n2, double len, double g2, double h_dry,
+static __device__ __noinline__ EdgeTerms edge_hard(Side L, Side R, double n1, double n2, double g2, double h_dry,
                                             bool hll_only) {
     EdgeTerms t;
-    edge_by<Hard>(L, R, n1, n2, len, g2, h_dry, hll_only, t);
+    edge_by<Hard>(L, R, n1, n2, g2, h_dry, hll_only, t);
     return t;
 }
 template <class S = Soft>
-__device__ __forceinline__ void edge(const Side& L, const Side& R, double n1, double n2, double len, double g2,
-                                     double h_dry, bool hll_only, EdgeTerms& t) {
-    if (soft_side(L) && soft_side(R) && soft_edge(n1, n2, len, g2))
-        edge_by<S>(L, R, n1, n2, len, g2, h_dry, hll_only, t);
+__device__ __forceinline__ void edge(const Side& L, const Side& R, double n1, double n2, double g2, double h_dry,
+                                     bool hll_only, EdgeTerms& t) {
+    if (soft_side(L) && soft_side(R) && soft_edge(n1, n2, g2))
+        edge_by<S>(L, R, n1, n2, g2, h_dry, hll_only, t);
     else
-        t = edge_hard(L, R, n1, n2, len, g2, h_dry, hll_only);
+        t = edge_hard(L, R, n1, n2, g2, h_dry, hll_only);
 }
 
 // The momentum part of an edge whose cells are both dry (no flux, only the bed
 // source term), for the cell (h, z) with outward unit normal (n1, n2): bit
 // for bit what edge() gives that cell.
-__device__ __forceinline__ void dry_edge(double h, double z, double zk, double n1, double n2, double len, double g2,
-                                         double& x, double& y) {
+__device__ __forceinline__ void dry_edge(double h, double z, double zk, double n1, double n2, double g2, double& x,
+                                         double& y) {
     const double zs = max_finite(z, zk);
     const double hs = max_zero(sub(add(h, z), zs));
-    const double p = fma(-fma(-Hard::mul(g2, h), h, Hard::mul(Hard::mul(g2, hs), hs)), len, 0.0);
+    const double p = -fma(-Hard::mul(g2, h), h, Hard::mul(Hard::mul(g2, hs), hs));
     x = fma(p, n1, 0.0);
     y = fma(p, n2, 0.0);
 }
@@ -452,20 +451,18 @@ __device__ __forceinline__ void boundary_flux(int kind, double value, const Side
     } else {                                                    // transmissive, fixed stage
         const double hg = kind == 3 ? max_zero(sub(value, c.z)) : c.h;
         double PL, PR;
-        riemann<Hard, false>(c.h, un, ut, hg, un, ut, g2, h_dry, 1.0, G1, G2, G3, PL, PR, nullptr, hll_only);
+        riemann<Hard>(c.h, un, ut, hg, un, ut, g2, h_dry, G1, G2, G3, PL, PR, nullptr, hll_only);
     }
 }
 
-// A boundary edge's addition to its cell's sums.
-__device__ __forceinline__ void boundary(int kind, double value, const Side& c, double n1, double n2, double len,
-                                         double g2, double h_dry, bool hll_only, double& m, double& x, double& y) {
+// A boundary edge's addition to its cell's sums, per unit length.
+__device__ __forceinline__ void boundary(int kind, double value, const Side& c, double n1, double n2, double g2,
+                                         double h_dry, bool hll_only, double& m, double& x, double& y) {
     const double un = fma(c.u, n1, Hard::mul(c.v, n2)), ut = fma(c.v, n1, -Hard::mul(c.u, n2));
-    double G1, G2, G3;
-    boundary_flux(kind, value, c, un, ut, g2, h_dry, hll_only, G1, G2, G3);
-    const double p = Hard::mul(G2, len), s = Hard::mul(G3, len);
-    m = Hard::mul(G1, len);
-    x = fma(p, n1, -Hard::mul(s, n2));
-    y = fma(p, n2, Hard::mul(s, n1));
+    double G2, G3;
+    boundary_flux(kind, value, c, un, ut, g2, h_dry, hll_only, m, G2, G3);
+    x = fma(G2, n1, -Hard::mul(G3, n2));
+    y = fma(G2, n2, Hard::mul(G3, n1));
 }
 
 // ---- the end of one cell update (Eq 37 with friction Eq 33-36, the clamps) ----------------

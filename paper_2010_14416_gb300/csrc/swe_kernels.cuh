@@ -692,8 +692,7 @@ __device__ __forceinline__ float update_cell_f32(const Args& a, long long i, con
 // formed inline, with the same bits.
 
 // The FP64 cell of the edge-pass step.  It reads its neighbours' depths only,
-// and normals and lengths only for boundary edges and edges with both cells
-// dry: with whole neighbour and geometry records the kernel held 138 registers
+// and normals only for boundary edges and edges with both cells dry: with whole neighbour and geometry records the kernel held 138 registers
 // (12 warps an SM) and waited on its chain of operations (48 us for 250k wet
 // cells; a step of the 1M-cell canal 182 us then, 163 now).
 template <typename Args>
@@ -735,6 +734,7 @@ __device__ __forceinline__ double update_cell_edges(const Args& a, long long i, 
     active += 1u;
     const double2 tail = ((const double2*)&a.geoB[i])[1];   // 1/|Omega|, R
     const double gm2 = a.gm2[i];
+    const V4<double> gR = a.geoR[i];                        // the edges' lengths
     double m = 0.0, x = 0.0, y = 0.0;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -753,19 +753,20 @@ __device__ __forceinline__ double update_cell_edges(const Args& a, long long i, 
             ty = flip ? -a.esrc[e] : fl.z;
         } else {
             const double2 n = j == 2 ? *(const double2*)&a.geoB[i] : ((const double2*)&a.geoA[i])[j];
-            const double len = ((const double*)&a.geoR[i])[j], g2 = f64::mul(0.5, a.g);
+            const double g2 = f64::mul(0.5, a.g);
             if (c >= 0) {
-                f64::dry_edge(hi, zi, a.s_in[c & kNbrMask].w, n.x, n.y, len, g2, tx, ty);
+                f64::dry_edge(hi, zi, a.s_in[c & kNbrMask].w, n.x, n.y, g2, tx, ty);
             } else {
                 const int grp = -1 - c;
                 f64::Side side{hi, 0.0, 0.0, zi};
                 f64::velocity(hi, own.y, own.z, h_dry, side.u, side.v);
-                f64::boundary(a.bc_kind(grp), a.bc_value(grp), side, n.x, n.y, len, g2, h_dry, a.hll != 0, tm, tx, ty);
+                f64::boundary(a.bc_kind(grp), a.bc_value(grp), side, n.x, n.y, g2, h_dry, a.hll != 0, tm, tx, ty);
             }
         }
-        m = f64::add(m, tm);
-        x = f64::add(x, tx);
-        y = f64::add(y, ty);
+        const double len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
+        m = f64::fma(len, tm, m);
+        x = f64::fma(len, tx, x);
+        y = f64::fma(len, ty, y);
     }
     return finish_cell(a, i, own, m, x, y, tail.x, tail.y, gm2, dt, n_clamped, status);
 }
@@ -845,17 +846,17 @@ __device__ __forceinline__ T update_cell(const Args& a, long long i, const V4<T>
             L.v = flip ? nb_side.v : own_side.v; R.v = flip ? own_side.v : nb_side.v;
             L.z = flip ? nb_side.z : own_side.z; R.z = flip ? own_side.z : nb_side.z;
             f64::EdgeTerms t;
-            f64::edge(L, R, flip ? -n1 : n1, flip ? -n2 : n2, len, g2, h_dry, a.hll != 0, t);
+            f64::edge(L, R, flip ? -n1 : n1, flip ? -n2 : n2, g2, h_dry, a.hll != 0, t);
             tm = flip ? -t.m : t.m;
             tx = flip ? -t.xR : t.xL;
             ty = flip ? -t.yR : t.yL;
         } else {
             const int grp = -1 - c;
-            f64::boundary(a.bc_kind(grp), a.bc_value(grp), own_side, n1, n2, len, g2, h_dry, a.hll != 0, tm, tx, ty);
+            f64::boundary(a.bc_kind(grp), a.bc_value(grp), own_side, n1, n2, g2, h_dry, a.hll != 0, tm, tx, ty);
         }
-        m = f64::add(m, tm);
-        x = f64::add(x, tx);
-        y = f64::add(y, ty);
+        m = f64::fma(len, tm, m);
+        x = f64::fma(len, tx, x);
+        y = f64::fma(len, ty, y);
     }
     return finish_cell(a, i, own, m, x, y, gB.z, gB.w, gm2, dt, n_clamped, status);
     }
@@ -1018,7 +1019,7 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
             f64::velocity(L.x, L.y, L.z, h_dry, l.u, l.v);
             f64::velocity(R.x, R.y, R.z, h_dry, r.u, r.v);
             f64::EdgeTerms t;
-            f64::edge(l, r, a.eln[2 * e], a.eln[2 * e + 1], a.erl[e], f64::mul(0.5, g), h_dry, a.hll != 0, t);
+            f64::edge(l, r, a.eln[2 * e], a.eln[2 * e + 1], f64::mul(0.5, g), h_dry, a.hll != 0, t);
             f.x = t.m; f.y = t.xL; f.z = t.yL; f.w = t.xR;
             sr = t.yR;
         } else {

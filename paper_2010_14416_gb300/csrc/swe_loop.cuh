@@ -39,10 +39,10 @@ struct LoopArgs {
     int hll, debug, n_groups;
     BcTable bc;
     // FP64: per block kLoopEdges slots, the edges that touch its cells
-    // ((left, right) cell, left < 0: none; unit normal and length), and per cell
+    // ((left, right) cell, left < 0: none; unit normal), and per cell
     // the slots of its three edges
     const int2* ecell;
-    const double* egeo;                // [block][3][kLoopEdges]
+    const double* egeo;                // [block][2][kLoopEdges]
     const uchar4* eslot;
 };
 
@@ -190,15 +190,16 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
     unsigned* const status = (unsigned*)(a.small + kLoopSlotStatus);
     const double h_dry = a.h_dry, g2 = f64::mul(0.5, a.g);
     const int2 lr = a.ecell[(long long)blockIdx.x * kLoopEdges + tid];
-    const double* const eg = a.egeo + (long long)blockIdx.x * 3 * kLoopEdges + tid;
-    double n1 = 0.0, n2 = 0.0, len = 0.0;
-    if (lr.x >= 0) { n1 = eg[0]; n2 = eg[kLoopEdges]; len = eg[2 * kLoopEdges]; }
+    const double* const eg = a.egeo + (long long)blockIdx.x * 2 * kLoopEdges + tid;
+    double n1 = 0.0, n2 = 0.0;
+    if (lr.x >= 0) { n1 = eg[0]; n2 = eg[kLoopEdges]; }
     const long long i = (long long)blockIdx.x * kLoopCells + tid;
     const bool in = tid < kLoopCells && i < a.n;
     V4<double> own{}, next{};
     int4 tp = make_int4(-1, -1, -1, 0);
     uchar4 slot = make_uchar4(0, 0, 0, 0);
     double ia = 0.0, rin = 0.0, gm2 = 0.0;
+    V4<double> gR{};                   // the edges' lengths
     bool open = false;                 // a boundary edge that keeps the cell out of the quiet path
     LoopCell<double> v{a, nullptr, nullptr, {}, {}, &next, a.g, a.h_dry, a.hll, a.debug, a.n_groups};
     if (in) {
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
         ia = a.geoB[i].z;
         rin = a.geoB[i].w;
         gm2 = a.gm2[i];
+        gR = a.geoR[i];
         open = (tp.w & kStaticBit) != 0;
     }
     int p2 = (int)(a.step0 % 2), p3 = (int)(a.step0 % 3);
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
             f64::velocity<S>(L.x, L.y, L.z, h_dry, l.u, l.v);
             f64::velocity<S>(R.x, R.y, R.z, h_dry, r.u, r.v);
             f64::EdgeTerms t;
-            f64::edge<S>(l, r, n1, n2, len, g2, h_dry, a.hll != 0, t);
+            f64::edge<S>(l, r, n1, n2, g2, h_dry, a.hll != 0, t);
             term[0][tid] = t.m; term[1][tid] = t.xL; term[2][tid] = t.yL; term[3][tid] = t.xR; term[4][tid] = t.yR;
             wet_edge[tid] = gt_pos(L.x, h_dry) || gt_pos(R.x, h_dry);
         }
@@ -259,12 +261,13 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
                             const int grp = -1 - c;
                             f64::Side side{own.x, 0.0, 0.0, own.w};
                             f64::velocity<S>(own.x, own.y, own.z, h_dry, side.u, side.v);
-                            f64::boundary(a.bc.kind[grp], a.bc.value[grp], side, n.x, n.y,
-                                          ((const double*)&a.geoR[i])[j], g2, h_dry, a.hll != 0, tm, tx, ty);
+                            f64::boundary(a.bc.kind[grp], a.bc.value[grp], side, n.x, n.y, g2, h_dry, a.hll != 0, tm,
+                                          tx, ty);
                         }
-                        m = f64::add(m, tm);
-                        x = f64::add(x, tx);
-                        y = f64::add(y, ty);
+                        const double len = j == 0 ? gR.x : (j == 1 ? gR.y : gR.z);
+                        m = f64::fma(len, tm, m);
+                        x = f64::fma(len, tx, x);
+                        y = f64::fma(len, ty, y);
                     }
                     cand = finish_cell<S>(v, i, own, m, x, y, ia, rin, gm2, dt.t, a.small + kLoopSlotClamp, status);
                     own = next;

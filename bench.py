@@ -37,12 +37,13 @@ import numpy as np  # noqa: E402
 # 1/|Omega|, inscribed radius (4) + L n of three edges (6) values, plus three
 # int32 neighbour indices
 ALG_BYTES = {"f32": 16 * 4 + 12, "f64": 16 * 8 + 12}
-# FP64 flops (2 x DFMA + DADD + DMUL) per cell that runs the flux path, from
-# ncu's instruction counts of the two FP64 step kernels on the 1M-cell
+# flops on the FP64 pipe (2 x DFMA + DADD + DMUL; products, reciprocals and
+# roots run on the integer unit) per cell that runs the flux path, from ncu's
+# instruction counts of the two FP64 step kernels on the 1M-cell
 # dry-bed canal divided by the cells that ran the flux path: the cell-centric
 # step evaluates every interior flux twice, the edge pass once; quiet cells
 # take no flux path and do no FP64 arithmetic
-FP64_FLOPS_PER_ACTIVE_CELL = {"cell": 748, "edge": 505}
+FP64_FLOPS_PER_ACTIVE_CELL = {"cell": 247, "edge": 151}
 # GB300 FP64: 2 DFMA per clock per SM, 152 SMs
 FP64_DFMA_PER_CLK_SM, N_SM = 2, 152
 
@@ -368,7 +369,8 @@ def _fp64_roofline(n, kernel_ms, active_frac, edge_pass, hbm):
                            f"x {sm_mhz:.0f} MHz (the FP64 pipe's unit count at the maximum SM clock; "
                            "MEASURED_PEAKS.json has no FP64 figure)",
             "flops_per_active_cell": per_cell, "active_cell_fraction": active_frac,
-            "flops_counted": "2 x DFMA + DADD + DMUL per cell that ran the flux path (ncu instruction counts)",
+            "flops_counted": "2 x DFMA + DADD + DMUL per cell that ran the flux path (ncu instruction counts; products, "
+                             "reciprocals and roots run on the integer unit and do not count)",
             "hbm": {k: v for k, v in hbm.items() if k not in ("bound", "traffic")}}
 
 
@@ -437,7 +439,8 @@ def measure_mesh(ctx, name, steps, warmup, shape_spec=None, e2e=True):
                    "steps_before_timed": warm, "simulated_time_s": info["t"], "reorder": "hilbert",
                    "graph_steps": 48, "launch_shape": _shape_key(shape), "autotune": shape},
         "roofline": roof,
-        "gpu_launches": steps * (2 if shape.get("edge_pass") else 1),
+        # the edge pass, and the scan ahead of the list of active cells, are a second kernel
+        "gpu_launches": steps * (2 if shape.get("edge_pass") or shape.get("activity") else 1),
         "clocks": clk,
     }
     m.close()
@@ -567,8 +570,10 @@ def measure_ensemble(ctx, name, steps, warmup, ens_shape=None):
         "per_member_launches_default_shapes": {"value": ctx.ws * n * steps / (ms_default * 1e-3),
                                                "unit": "cell-updates/s", "ms_per_step": ms_default / steps,
                                                "speedup": ms_default / ms},
-        # the edge pass and the split step launch two kernels per step
-        "gpu_launches": steps * (2 if shape.get("edge_pass") or shape.get("cell_pairs") else 1),
+        # the edge pass and the split step launch two kernels per step, the scan ahead
+        # of the list of active cells one more
+        "gpu_launches": steps * ((2 if shape.get("edge_pass") or shape.get("cell_pairs") else 1)
+                                 + (1 if shape.get("queue") else 0)),
         "clocks": clk,
     }
     if MEMBERS[2]:
@@ -635,9 +640,9 @@ def measure_adjoint(ctx, name, steps, warmup, shape_spec=None):
         "roofline": {"bound": "alu", "note": "FP64 arithmetic on forward-mode duals and hand-written "
                                              "transposes: the adjoint kernels and the forward steps are bound "
                                              "by the FP64 pipe"},
-        # per step: the forward step and its recomputation (two kernels each with the
-        # edge pass), then the two adjoint kernels
-        "gpu_launches": steps * (2 * (2 if shape.get("edge_pass") else 1) + 2),
+        # per step: the forward step and, but for the last segment of 50, its
+        # recomputation (two kernels each with the edge pass), then the two adjoint kernels
+        "gpu_launches": (2 * steps - ((steps - 1) % 50 + 1)) * (2 if shape.get("edge_pass") else 1) + 2 * steps,
         "clocks": clk,
     }
     m.close()

@@ -72,7 +72,7 @@ int swe::status_code(unsigned long long st) {
         set_error("swe_step: a neighbour index, edge index or boundary group out of range (debug checks)");
         return SWE_EMESH;
     }
-    if (st & kStatusStall) { set_error("swe_step: the step loop gave up waiting for its blocks"); return SWE_ECUDA; }
+    if (st & kStatusStall) { set_error("swe_step: the step loop gave up waiting for its blocks"); return SWE_ETIMEOUT; }
     if (st & kStatusNonFinite) { set_error("swe_step: non-finite state"); return SWE_ENONFINITE; }
     if (st & kStatusDry) { set_error("swe_step: every cell is dry, no CFL time step"); return SWE_EDRY; }
     return SWE_OK;
@@ -1035,7 +1035,7 @@ int swe_get_info(swe_mesh* m, swe_info* info) {
     info->n_clamped = (int64_t)s[kSlotClamp];
     info->n_active = (int64_t)s[kSlotActive];
     info->status = s[kSlotStatus] & kStatusBadIndex    ? SWE_EMESH
-                   : s[kSlotStatus] & kStatusStall     ? SWE_ECUDA
+                   : s[kSlotStatus] & kStatusStall     ? SWE_ETIMEOUT
                    : s[kSlotStatus] & kStatusNonFinite ? SWE_ENONFINITE
                    : (s[kSlotStatus] & kStatusDry ? SWE_EDRY : SWE_OK);
     return SWE_OK;

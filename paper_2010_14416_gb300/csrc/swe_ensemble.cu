@@ -1095,7 +1095,10 @@ int swe_ensemble_set_shape(swe_ensemble* E, const swe_tune* shape) {
     E->geo_early = shape->geometry_early;
     E->chunk_log2 = (int)cl2;
     E->grid = (unsigned)std::max(1LL, std::min(tiles, shape->grid > 0 ? (long long)shape->grid : wave));
-    if (E->activity != shape->activity || E->split != shape->cell_pairs) E->act_valid = false;
+    // the bytes are rebuilt where other kernels than before maintain them (only
+    // the list's scan keeps the span flags)
+    if (E->activity != shape->activity || E->split != shape->cell_pairs || E->queue != shape->queue)
+        E->act_valid = false;
     E->activity = shape->activity;
     E->edges = shape->edge_pass;
     E->dynamic = shape->dynamic;

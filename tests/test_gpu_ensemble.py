@@ -199,3 +199,51 @@ def test_ensemble_debug_checks_change_nothing(precision):
         e.close()
     for m in ref_meshes + dbg_meshes:
         m.close()
+
+
+@pytest.mark.parametrize("pairs", [0, 1])
+def test_list_mode_resumes_where_other_activity_steps_moved_the_water(pairs):
+    # list steps (queue=1) pass over spans of 4,096 cells that their flags call
+    # dry; the steps of another activity kernel in between carry the front
+    # across several such spans, and the list steps that follow must see it
+    dry = mg.canal(600, 80, 600.0, 80.0, 0.2, seed=5, hL=6.0, hR=0.0, x_dam=30.0, manning=0.0)
+    wet = mg.canal(300, 12, 300.0, 12.0, 0.2, seed=6, hL=3.0, hR=1.0, x_dam=150.0, manning=0.02)
+    meshes = [_mesh(mi, capi.SWE_FP32) for mi in (dry, wet)]
+    ens = capi.Ensemble(meshes)
+    listed = dict(block_size=128, min_blocks=7, geometry_early=1, activity=1, chunk=8, queue=1, cell_pairs=pairs)
+    other = dict(block_size=128, min_blocks=8, geometry_early=1, activity=1, chunk=8, cell_pairs=pairs)
+    for shape, steps in ((listed, 12), (other, 2000), (listed, 60), (other, 1), (listed, 7)):
+        ens.set_shape(**shape)
+        t = ens.step(steps)
+    cell_x = dry.nodes[dry.tris].mean(1)[:, 0]
+    for k, m in enumerate(meshes):
+        m.step(12)
+        before = m.get_state()[0] > 1e-6
+        assert m.step(2000 + 60 + 1 + 7) == t[k]
+        ref = m.get_state()
+        if k == 0:   # a span holds about 45 x 45 quads: the front has crossed three of them
+            assert cell_x[ref[0] > 1e-6].max() - cell_x[before].max() > 150.0
+        assert all(np.array_equal(a, b) for a, b in zip(ens.get_state(k), ref)), f"member {k}"
+    ens.close()
+    for m in meshes:
+        m.close()
+
+
+def test_list_mode_steps_a_member_beside_one_that_has_no_water():
+    # a member without water keeps its state and reports it, the others step on;
+    # water that later enters spans passed over for many steps is updated too
+    empty = mg.canal(400, 12, 400.0, 12.0, 0.2, seed=7, hL=0.0, hR=0.0, x_dam=200.0, manning=0.02)
+    dry = mg.canal(600, 40, 600.0, 40.0, 0.2, seed=8, hL=5.0, hR=0.0, x_dam=50.0, manning=0.0)
+    meshes = [_mesh(mi, capi.SWE_FP32) for mi in (dry, empty, dry)]
+    ens = capi.Ensemble(meshes)
+    ens.set_shape(block_size=128, min_blocks=7, geometry_early=1, activity=1, chunk=8, queue=1)
+    ens.step(700, sync=False)
+    for k in (0, 2):
+        meshes[k].step(700)
+        assert all(np.array_equal(a, b) for a, b in zip(ens.get_state(k), meshes[k].get_state())), f"member {k}"
+        assert ens.info(k)["status"] == 0 and ens.info(k)["t"] == meshes[k].info()["t"]
+    assert ens.info(1)["status"] == capi.SWE_EDRY
+    assert all(np.array_equal(a, np.zeros_like(a)) for a in ens.get_state(1))
+    ens.close()
+    for m in meshes:
+        m.close()

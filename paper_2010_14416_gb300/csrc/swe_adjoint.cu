@@ -157,9 +157,22 @@ __device__ __forceinline__ void friction_rev(double hi, double qx, double qy, do
     w[4] = A::mul(b_dh, dt); w[5] = A::mul(b_bx, dt); w[6] = A::mul(b_by, dt);
 }
 
-// The range of adjoints (and of the forward's right-hand side) that Soft
-// takes: beyond it, and beyond the forward's ranges, the FP64 pipe.
-__device__ __forceinline__ bool soft_adjoint(double x) { return f64::in_range<-400, 200>(x); }
+// The ranges that SoftFlush takes; beyond them the FP64 pipe.  Its products
+// must stay below 2^1024 (smaller ones than 2^-1022 become 0): with adjoints
+// below 2^100, wet depths from 2^-40 (so h_dry at least that) to 2^24, |u|
+// below 2^20, g/2 within 2^-16 to 2^16, lengths below 2^40 and, in the friction
+// update, |q| and dt below 2^24, g m^2 below 2^16 and right-hand sides below
+// 2^64, multiplying the factors' bounds along the chains, with a_K and 1/a_K of
+// the smallest and largest depth, 1/(S_R - S_L) <= 1/max|S_K| and rcp(1 + x) <= 1,
+// gives at most 2^716 through an edge and 2^880 through the friction update.
+__device__ __forceinline__ bool soft_adjoint(double x) { return f64::in_range<-400, 100>(x); }
+__device__ __forceinline__ bool soft_scheme(double g2, double h_dry) {
+    return f64::in_range<-16, 16>(g2) && f64::in_range<-40, 24>(h_dry);
+}
+// |q| / h < 2^20 by the exponents (a dry cell's velocity is not formed)
+__device__ __forceinline__ bool slow(double q, double h) {
+    return (__double2hiint(q) & 0x7FF00000) - (__double2hiint(h) & 0x7FF00000) < (20 << 20);
+}
 
 // EDGES reads R_i's interior fluxes from the edge pass (the forward's own
 // edge-pass arithmetic) instead of evaluating them; R_i is the same bit for bit.
@@ -249,9 +262,9 @@ __device__ __forceinline__ void adj_phase1(const AdjArgs& a, const AdjStep& st, 
         else if (hn <= h_dry) { lx_ = 0.0; ly_ = 0.0; }
         const double gm2 = a.gm2[i];
         if (f64::in_range<-64, 24>(hi) && f64::in_range<-64, 24>(own.y) && f64::in_range<-64, 24>(own.z) &&
-            f64::in_range<-64, 16>(gm2) && f64::in_range<-64, 24>(st.dt) && f64::in_range<-192, 128>(Rh) &&
-            f64::in_range<-192, 128>(Rx) && f64::in_range<-192, 128>(Ry) && soft_adjoint(lh) && soft_adjoint(lx_) &&
-            soft_adjoint(ly_))
+            f64::in_range<-64, 16>(gm2) && f64::in_range<-64, 24>(st.dt) && f64::in_range<-192, 64>(Rh) &&
+            f64::in_range<-192, 64>(Rx) && f64::in_range<-192, 64>(Ry) && soft_adjoint(lh) && soft_adjoint(lx_) &&
+            soft_adjoint(ly_) && soft_scheme(g2, h_dry))
             friction_rev<f64::SoftFlush>(hi, own.y, own.z, gm2, Rh, Rx, Ry, st.dt, h_dry, lh, lx_, ly_, w);
         else
             friction_rev<f64::Hard>(hi, own.y, own.z, gm2, Rh, Rx, Ry, st.dt, h_dry, lh, lx_, ly_, w);
@@ -571,7 +584,7 @@ __device__ __forceinline__ void edge_interior_rev(const V4<double>& L, const V4<
 
 __device__ __forceinline__ bool soft_state(const V4<double>& s) {
     return f64::in_range<-64, 24>(s.x) && f64::in_range<-64, 24>(s.y) && f64::in_range<-64, 24>(s.z) &&
-           f64::in_range<-64, 24>(s.w);
+           f64::in_range<-64, 24>(s.w) && slow(s.y, s.x) && slow(s.z, s.x);
 }
 
 // Reverse of a boundary edge's flux (f64::boundary_flux): adds to d the
@@ -643,7 +656,8 @@ __global__ void __launch_bounds__(128) adj_edge_kernel(const AdjArgs a) {
         const V4<double> L = a.U[lr.x], R = a.U[lr.y];
         const double n1 = a.eln[2 * e], n2 = a.eln[2 * e + 1], len = a.erl[e];
         const double g2 = f64::mul(0.5, a.g);
-        if (soft_state(L) && soft_state(R) && f64::soft_edge(n1, n2, g2) && f64::in_range<-64, 40>(len) && soft_adjoint(nl.x) &&
+        if (soft_state(L) && soft_state(R) && f64::soft_edge(n1, n2, g2) && soft_scheme(g2, a.h_dry) &&
+            f64::in_range<-64, 40>(len) && soft_adjoint(nl.x) &&
             soft_adjoint(nl.y) && soft_adjoint(nl.z) && soft_adjoint(nr.x) && soft_adjoint(nr.y) && soft_adjoint(nr.z))
             edge_interior_rev<f64::SoftFlush>(L, R, n1, n2, len, g2, a.h_dry, a.hll != 0, nl, nr, dl, dr);
         else

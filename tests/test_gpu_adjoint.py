@@ -284,3 +284,31 @@ def test_adjoint_is_independent_of_the_forward_launch_shape(fully_wet):
     tuned.autotune(trial_steps=2)
     got = tuned.adjoint(60, gauges, target, checkpoint_every=7)
     assert got[0] == ref[0] and all(np.array_equal(a, b) for a, b in zip(got[1:], ref[1:]))
+
+
+@pytest.mark.parametrize("case", ["fast", "thin", "large"])
+def test_transposes_on_either_side_of_the_integer_units_ranges(case):
+    # velocities on both sides of 2^20, a dry threshold below 2^-40, adjoints
+    # above 2^100: edges and cells change between the integer unit and the FP64
+    # pipe, the dual-number kernels do not.  Both sides round each of some 200
+    # operations a step by 2^-53 relative; sums of terms that differ by
+    # |u| / sqrt(g h) = 10^5 lose five digits of that, over four steps: 1e-9
+    mi, M, dts, gauges, target = _setup(True, nx=60, ny=12, steps=4)
+    hu, kw = mi.hu, {}
+    if case == "fast":
+        hu = mi.h * np.random.default_rng(3).uniform(0.5, 1.5, mi.n_cells) * 2.0**20
+    elif case == "thin":
+        kw = dict(h_dry=2.0**-50)
+    else:
+        target = target + 1e40
+    res = {}
+    for method in (capi.SWE_ADJOINT_TRANSPOSE, capi.SWE_ADJOINT_DUAL):
+        m = _gpu_mesh(mi, **kw)
+        m.set_state(mi.h, hu, mi.hv)
+        m.adjoint_method(method)
+        res[method] = m.adjoint(4, gauges, target)
+        m.close()
+    a, b = res[capi.SWE_ADJOINT_TRANSPOSE], res[capi.SWE_ADJOINT_DUAL]
+    assert a[0] == b[0] and np.array_equal(a[3], b[3])
+    assert np.all(np.isfinite(b[2])) and np.abs(b[2]).max() > 0.0
+    assert _rel(a[1], b[1]) <= 1e-9 and _rel(a[2], b[2]) <= 1e-9, (_rel(a[1], b[1]), _rel(a[2], b[2]))

@@ -71,6 +71,7 @@ __device__ __forceinline__ bool in_range(double x) {
 }
 
 struct Hard {
+    static constexpr bool kRare = false;
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     // seeds: the documented approximations of 1/x and 1/sqrt(x) that read the
     // upper word of x and write the upper word of the result
@@ -117,6 +118,7 @@ struct Hard {
 };
 
 struct Soft {
+    static constexpr bool kRare = false;
     // 32 x 32 -> 64 bits, plus c
     static __device__ __forceinline__ unsigned long long wide(unsigned a, unsigned b, unsigned long long c = 0ULL) {
         return (unsigned long long)a * b + c;
@@ -241,7 +243,16 @@ struct SoftFlush : Soft {
     static __device__ __forceinline__ double mul(double a, double b) { return product<true>(a, b); }
 };
 
-// for operands of any kind
+// CUDA's operations, for the operands that neither takes: denormal numbers,
+// infinities, exponents near the ends of the range.
+struct Rare {
+    static constexpr bool kRare = true;
+    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+    static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+    static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+};
+
+// Hard's, for normal operands and zero
 __device__ __forceinline__ double rcp(double x) { return Hard::rcp(x); }
 __device__ __forceinline__ double sqrt_(double x) { return Hard::sqrt_(x); }
 __device__ __forceinline__ double sqrt_rsqrt(double x, double& y) { return Hard::sqrt_rsqrt(x, y); }
@@ -274,17 +285,34 @@ __device__ __forceinline__ void riemann(double hL, double unL, double utL, doubl
         if (speeds) { speeds[0] = 0.0; speeds[1] = 0.0; speeds[2] = 0.0; }
         return;
     }
-    const double aL = A::sqrt_(twice(ghL)), aR = A::sqrt_(twice(ghR));
+    double aL, aR;
+    if constexpr (A::kRare) {
+        aL = A::sqrt_(A::mul(add(g2, g2), hL));
+        aR = A::sqrt_(A::mul(add(g2, g2), hR));
+    } else {
+        aL = A::sqrt_(twice(ghL));
+        aR = A::sqrt_(twice(ghR));
+    }
     double SL, SR;
     if (wetL && wetR) {
         SL = sub(unL, aL);                                                     // Eq 19 with p = 1
         SR = add(unR, aR);
         const double asum = add(aL, aR), hsum = add(hL, hR), du = sub(unR, unL);
         // h0 = hsum w / (4 asum), w = 2 asum - du (Eq 21): h0 > min(h_L, h_R) without dividing
-        const double hw = A::mul(hsum, fma(2.0, asum, -du));
-        const double asum4 = four_times(asum);
-        if (gt_pos(hw, A::mul(min_nonneg(hL, hR), asum4))) {                      // Eq 23
-            const double rh0 = A::mul(asum4, A::rcp(hw)), rL = A::rcp(hL), rR = A::rcp(hR);
+        const double w = fma(2.0, asum, -du), hmin = min_nonneg(hL, hR);
+        bool shock;
+        double rh0 = 0.0;
+        if constexpr (A::kRare) {   // by quotients, which neither under- nor overflow first
+            const double q = w / asum;
+            shock = hsum / hmin * q > 4.0;
+            if (shock) rh0 = 4.0 / q / hsum;
+        } else {
+            const double hw = A::mul(hsum, w), asum4 = four_times(asum);
+            shock = gt_pos(hw, A::mul(hmin, asum4));
+            if (shock) rh0 = A::mul(asum4, A::rcp(hw));
+        }
+        if (shock) {                                                           // Eq 23
+            const double rL = A::rcp(hL), rR = A::rcp(hR);
             const double gL = A::sqrt_(A::mul(g2, add(rh0, rL))), gR = A::sqrt_(A::mul(g2, add(rh0, rR)));
             const double hs = A::mul(fma(hL, gL, fma(hR, gR, -du)), A::rcp(add(gL, gR)));
             const double ghs = A::mul(g2, hs);
@@ -312,13 +340,20 @@ __device__ __forceinline__ void riemann(double hL, double unL, double utL, doubl
         upL = wetL && !wetR && ge_zero(SR);
     } else {                                                                   // Eq 18
         const double r = A::rcp(sub(SR, SL));
-        const double ss = A::mul(SR, SL);
+        const double ss = A::kRare ? SR * r * SL : A::mul(SR, SL);
         const double fL = fma(qL, unL, PL), fR = fma(qR, unR, PR);
-        G1 = A::mul(fma(ss, sub(hR, hL), fma(-SL, qR, A::mul(SR, qL))), r);
-        G2 = A::mul(fma(ss, sub(qR, qL), fma(-SL, fR, A::mul(SR, fL))), r);
-        if (hll_only) {
-            const double tL = A::mul(qL, utL), tR = A::mul(qR, utR);
-            G3 = A::mul(fma(ss, sub(A::mul(hR, utR), A::mul(hL, utL)), fma(-SL, tR, A::mul(SR, tL))), r);
+        if constexpr (A::kRare) {   // the weights first: S F may overflow
+            const double wL = SR * r, wR = -SL * r;
+            G1 = fma(ss, sub(hR, hL), fma(wR, qR, wL * qL));
+            G2 = fma(ss, sub(qR, qL), fma(wR, fR, wL * fL));
+            if (hll_only) G3 = fma(ss, hR * utR - hL * utL, fma(wR, qR * utR, wL * (qL * utL)));
+        } else {
+            G1 = A::mul(fma(ss, sub(hR, hL), fma(-SL, qR, A::mul(SR, qL))), r);
+            G2 = A::mul(fma(ss, sub(qR, qL), fma(-SL, fR, A::mul(SR, fL))), r);
+            if (hll_only) {
+                const double tL = A::mul(qL, utL), tR = A::mul(qR, utR);
+                G3 = A::mul(fma(ss, sub(A::mul(hR, utR), A::mul(hL, utL)), fma(-SL, tR, A::mul(SR, tL))), r);
+            }
         }
         upL = wetL && (!wetR || ge_zero(G1));
     }
@@ -335,16 +370,37 @@ __device__ __forceinline__ void riemann(double hL, double unL, double utL, doubl
     }
 }
 
-// Per unit length, for any states.
+// The flux of inputs that Hard does not take, out of line.
+struct FluxAndSpeeds { double G1, G2, G3, S[3]; };
+static __device__ __noinline__ FluxAndSpeeds riemann_rare(double hL, double unL, double utL, double hR, double unR,
+                                                          double utR, double g2, double h_dry, bool hll_only) {
+    FluxAndSpeeds r;
+    double PL, PR;
+    riemann<Rare>(hL, unL, utL, hR, unR, utR, g2, h_dry, r.G1, r.G2, r.G3, PL, PR, r.S, hll_only);
+    return r;
+}
+
+// Per unit length, for any states.  Hard takes reciprocals and roots of normal
+// numbers in its range, and its products keep clear of under- and overflow
+// where they are compared.  (A mesh's wet depths are 2^-126 at least, so its
+// cells and edges need no test for it; the flux alone may be asked for any
+// depth and dry threshold.)
 __device__ __forceinline__ void riemann_any(double hL, double unL, double utL, double hR, double unR, double utR,
                                             double g2, double h_dry, double& G1, double& G2, double& G3, double* speeds,
                                             bool hll_only) {
     double PL, PR;
     if (in_range<-64, 24>(hL) && in_range<-64, 24>(hR) && in_range<-100, 40>(unL) && in_range<-100, 40>(utL) &&
-        in_range<-100, 40>(unR) && in_range<-100, 40>(utR) && in_range<-64, 24>(g2))
+        in_range<-100, 40>(unR) && in_range<-100, 40>(utR) && in_range<-64, 24>(g2)) {
         riemann<Soft>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
-    else
+    } else if (in_range<-200, 100>(hL) && in_range<-200, 100>(hR) && in_range<-400, 100>(unL) &&
+               in_range<-400, 100>(utL) && in_range<-400, 100>(unR) && in_range<-400, 100>(utR) &&
+               in_range<-64, 64>(g2)) {
         riemann<Hard>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
+    } else {
+        const FluxAndSpeeds r = riemann_rare(hL, unL, utL, hR, unR, utR, g2, h_dry, hll_only);
+        G1 = r.G1; G2 = r.G2; G3 = r.G3;
+        if (speeds) { speeds[0] = r.S[0]; speeds[1] = r.S[1]; speeds[2] = r.S[2]; }
+    }
 }
 
 template <typename A>

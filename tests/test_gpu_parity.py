@@ -732,3 +732,73 @@ def test_hll_flux_variant(precision):
         assert t == pytest.approx(ot, rel=1e-12)
         for a, b in ((gh, oh), (ghu, ohu), (ghv, ohv)):
             assert rel_err(a, b) <= FP64_TOL
+
+
+def _hllc_wide(hL, unL, utL, hR, unR, utR, h_dry):
+    """Eq 17-26 in numpy's extended type, whose exponents neither under- nor
+    overflow here: G, (S_L, S_R)."""
+    t = np.longdouble
+    hL, unL, utL, hR, unR, utR, g, h_dry = (t(x) for x in (hL, unL, utL, hR, unR, utR, 9.81, h_dry))
+    dryL, dryR = hL <= h_dry, hR <= h_dry
+    if dryL and dryR:
+        return np.zeros(3), np.zeros(2)
+    aL, aR = np.sqrt(g * hL), np.sqrt(g * hR)
+    if dryL:
+        SL, SR, left = unR - 2 * aR, unR + aR, None
+    elif dryR:
+        SL, SR, left = unL - aL, unL + 2 * aL, None
+    else:
+        h0 = (hL + hR) * (t(0.5) - t(0.25) * (unR - unL) / (aL + aR))
+        pL = pR = t(1)
+        if h0 > min(hL, hR):
+            gL, gR = (np.sqrt(g * (h0 + h) / (2 * h0 * h)) for h in (hL, hR))
+            hs = (hL * gL + hR * gR + unL - unR) / (gL + gR)
+            pL, pR = (np.sqrt(hs * (hs + h) / 2) / h if hs > h else t(1) for h in (hL, hR))
+        SL, SR = unL - aL * pL, unR + aR * pR
+        left = SL >= 0 or (SR > 0 and (SL * hR * (unR - SR) - SR * hL * (unL - SL)) /
+                           (hR * (unR - SR) - hL * (unL - SL)) >= 0)
+    if left is None:
+        left = (SL if dryL else SR) >= 0
+    F = [(h * u, h * u * u + g * h * h / 2) for h, u in ((hL, unL), (hR, unR))]
+    if SL >= 0:
+        G = F[0]
+    elif SR <= 0:
+        G = F[1]
+    else:
+        U = [(h, h * u) for h, u in ((hL, unL), (hR, unR))]
+        G = [(SR * F[0][c] - SL * F[1][c] + SR * SL * (U[1][c] - U[0][c])) / (SR - SL) for c in range(2)]
+    return np.array([G[0], G[1], G[0] * (utL if left else utR)], t), np.array([SL, SR], t)
+
+
+def test_riemann_flux_far_from_any_flow_fp64():
+    # depths from denormal to 1e150 and a dry threshold of 1e-322, which the
+    # flux alone takes.  Equal depths below 1e-300, whose reciprocals overflow.
+    # Some 40 operations of 2^-53 each on terms that nearly cancel by at most
+    # 2^4: 1e-13 of the largest term.  Products below the normal range are
+    # rounded to 2^-1074, and so is g h under the root
+    rng = np.random.default_rng(12)
+    states = []
+    for _ in range(4000):
+        h = float(10.0 ** rng.uniform(-315.0, 150.0)) if rng.random() < 0.9 else 0.0
+        k = float(rng.choice([1.0, 1.0, 0.5, 2.0])) if h > 1e-300 else 1.0
+        a = math.sqrt(9.81 * h)
+        f = np.sort(rng.uniform(-0.9, 0.9, 2)) + float(rng.choice([0.0, 3.0, -3.0]))
+        states.append((h, a * f[0], a, h * k, a * f[1], -0.5 * a))
+    states += [(0.0, 0.0, 0.0, 3e-310, 0.0, 1.0), (3e-310, 0.0, 1.0, 0.0, 0.0, 0.0),
+               (1e-250, 1e30, 2.0, 2e-250, 1e30, 1.0)]
+    st = [np.array(c) for c in zip(*states)]
+    dev = [torch.tensor(a, dtype=torch.float64, device="cuda") for a in st]
+    G = [torch.empty(len(states), dtype=torch.float64, device="cuda") for _ in range(3)]
+    S = torch.empty((len(states), 3), dtype=torch.float64, device="cuda")
+    capi.riemann_flux(capi.SWE_FP64, *dev, *G, S, h_dry=1e-322)
+    torch.cuda.synchronize()
+    got_g, got_s = torch.stack(G, 1).cpu().numpy(), S.cpu().numpy()[:, :2]
+    for s, gg, gs in zip(states, got_g, got_s):
+        hL, unL, utL, hR, unR, utR = s
+        ref_g, ref_s = _hllc_wide(*s, h_dry=1e-322)
+        h = np.longdouble(max(hL, hR))
+        c = max(abs(unL), abs(unR), abs(utL), abs(utR), math.sqrt(9.81 * max(hL, hR)))
+        root = 5e-324 / max(float(h), 5e-324)   # of g h
+        assert np.all(np.abs(gs - ref_s) <= (1e-13 + root) * 4 * c), (s, gs, ref_s)
+        scale = np.array([h * c, h * c * c, h * c * c], np.longdouble)
+        assert np.all(np.abs(gg - ref_g) <= 1e-13 * 4 * scale + 1e-320), (s, gg, ref_g)

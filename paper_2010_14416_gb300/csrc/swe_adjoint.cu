@@ -974,6 +974,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
         set_error("swe_adjoint: an index or boundary group out of range in the forward run (debug checks)");
         return SWE_EMESH;
     }
+    if (fstat[kSlotStatus] & kStatusStall) return status_code(fstat[kSlotStatus]);
     if (fstat[kSlotStatus] & kStatusNonFinite) { set_error("swe_adjoint: forward run is not finite"); return SWE_ENONFINITE; }
     for (double d : dts)
         if (!std::isfinite(d)) { set_error("swe_adjoint: forward run went dry"); return SWE_EDRY; }
@@ -1187,6 +1188,7 @@ int swe_step_dt(swe_mesh* m, int64_t nsteps, const double* dts, double* t_out) {
         set_error("swe_step_dt: an index or boundary group out of range (debug checks)");
         return SWE_EMESH;
     }
+    if (sm[kSlotStatus] & kStatusStall) return status_code(sm[kSlotStatus]);
     if (sm[kSlotStatus] & kStatusNonFinite) { set_error("swe_step_dt: non-finite state"); return SWE_ENONFINITE; }
     return SWE_OK;
 }

@@ -374,9 +374,11 @@ int run_loop(swe_mesh* m, int64_t nsteps, double cfl) {
     while (nsteps > 0) {
         a.step0 = m->nstep;
         a.steps = (int)std::min<int64_t>(nsteps, 2000);   // some milliseconds a launch
+        a.max_polls = m->loop_polls;
         const cudaError_t e = Launch<T>::loop(a, m->stream);
         if (e != cudaSuccess) return cuda_fail(e, "swe_step: loop launch");
         m->nstep += a.steps;
+        m->loop_steps += a.steps;
         nsteps -= a.steps;
     }
     return SWE_OK;
@@ -730,6 +732,13 @@ int swe_debug_code_ok(int32_t code, int64_t n_cells, int n_groups) {
     return code_ok(code, (long long)n_cells, n_groups) ? 1 : 0;
 }
 
+int swe_debug_loop(swe_mesh* m, int64_t max_polls, int64_t* steps) {
+    if (!m || max_polls > (int64_t)0xFFFFFFFF) { set_error("swe_debug_loop: bad arguments"); return SWE_EINVAL; }
+    if (max_polls >= 0) m->loop_polls = (unsigned)max_polls;
+    if (steps) *steps = m->loop_steps;
+    return SWE_OK;
+}
+
 void swe_mesh_destroy(swe_mesh* m) {
     if (!m) return;
     DeviceGuard dg(m->cfg.device);
@@ -826,6 +835,7 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
     if (!m) { set_error("swe_mesh_create: out of host memory"); return SWE_ENOMEM; }
     m->cfg = c;
     m->loop_allowed = nothing_chosen && !c.debug_checks;
+    m->loop_polls = kMaxPolls;
     m->esz = c.precision == SWE_FP32 ? 4 : 8;
     std::string err;
     int rc;

@@ -415,6 +415,7 @@ int ens_build(swe_ensemble* E, swe_mesh* const* M) {
     for (int k = 0; k < nm && e == cudaSuccess; ++k) {
         unsigned long long s[kSmallWords];
         e = cudaMemcpy(s, M[k]->small, sizeof s, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && (s[kSlotStatus] & kStatusStall)) return status_code(s[kSlotStatus]);
         first[k] = s[M[k]->nstep % 3];
         std::memcpy(&t0[k], &s[kSlotT], sizeof(double));
     }

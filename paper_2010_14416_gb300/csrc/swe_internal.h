@@ -171,6 +171,8 @@ struct swe_mesh {
     // count and, FP64, its blocks' edges
     bool loop_allowed = false;
     long long loop_cells = -1;
+    unsigned loop_polls = 0;           // polls after which a wait of the loop gives up
+    int64_t loop_steps = 0;            // steps run in the loop
     unsigned* loop_barrier = nullptr;
     int2* loop_ecell = nullptr;
     double* loop_egeo = nullptr;

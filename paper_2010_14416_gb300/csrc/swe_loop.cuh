@@ -15,7 +15,8 @@
 namespace swe {
 
 // Limit of the polls of one wait (under 2 s; a step takes microseconds).  A
-// grid that gives up sets kStatusStall and leaves.
+// grid that gives up sets kStatusStall and leaves, and no loop starts on a
+// status block that has it.
 constexpr unsigned kMaxPolls = 1u << 22;
 // words of the status block
 constexpr int kLoopSlotT = 3, kLoopSlotStatus = 4, kLoopSlotClamp = 5, kLoopSlotActive = 6, kLoopSlotDtLast = 7;
@@ -33,6 +34,7 @@ struct LoopArgs {
     long long n;
     long long step0;                   // index of the first step
     int steps;
+    unsigned max_polls;                // of one wait
     int one_block_sms;                 // FP64: no SM has more than one block
     double cfl;
     T g, h_dry;
@@ -94,15 +96,15 @@ __device__ __forceinline__ void load_geometry(const LoopCell<T>& a, long long, V
 // Every block's writes before, its reads after: the block's threads meet,
 // thread 0 releases them with its arrival and waits for the others'.  Returns
 // whether all arrived.
-__device__ __forceinline__ bool grid_meet(unsigned* barrier, unsigned target, unsigned* status, int* failed) {
+__device__ __forceinline__ bool grid_meet(unsigned* barrier, unsigned target, unsigned max_polls, unsigned* status,
+                                          int* failed) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(barrier, 1u);
-        unsigned seen, polls = 0u;
-        do {
+        unsigned seen = 0u;
+        for (unsigned polls = 0u; seen < target && polls < max_polls; ++polls)
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(barrier) : "memory");
-        } while (seen < target && ++polls < kMaxPolls);
         if (seen < target) {
             atomicOr(status, kStatusStall);
             *failed = 1;
@@ -110,6 +112,11 @@ __device__ __forceinline__ bool grid_meet(unsigned* barrier, unsigned target, un
     }
     __syncthreads();
     return *failed == 0;
+}
+
+// Whether an earlier loop gave up on this status block (the whole block calls).
+__device__ __forceinline__ bool loop_stalled(const unsigned* status) {
+    return __syncthreads_or((int)(*(const volatile unsigned*)status & kStatusStall)) != 0;
 }
 
 // One step's size from the slot that the step before has filled.
@@ -141,6 +148,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_loop_f32(const LoopArgs<floa
     const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
     const bool in = i < a.n;
     unsigned* const status = (unsigned*)(a.small + kLoopSlotStatus);
+    if (loop_stalled(status)) return;
     V4<float> own{}, next{};
     int4 tp = make_int4(-1, -1, -1, 0);
     LoopCell<float> v{a, nullptr, nullptr, {}, {}, &next, a.g, a.h_dry, a.hll, a.debug, a.n_groups};
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_loop_f32(const LoopArgs<floa
         p2 = 1 - p2;
         p3 = p3 == 2 ? 0 : p3 + 1;
         block_min_publish<BLOCK>(cand, a.small + p3);   // the slot that the next step reads
-        if (!grid_meet(a.barrier, (unsigned)(s + 1) * gridDim.x, status, &failed)) break;
+        if (!grid_meet(a.barrier, (unsigned)(s + 1) * gridDim.x, a.max_polls, status, &failed)) break;
     }
     active_sum = __reduce_add_sync(0xffffffffu, active);
     if ((threadIdx.x & 31) == 0 && active_sum) atomicAdd(a.small + kLoopSlotActive, active_sum);
@@ -188,6 +196,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
     const int tid = threadIdx.x;
     if (tid == 0) failed = 0;
     unsigned* const status = (unsigned*)(a.small + kLoopSlotStatus);
+    if (loop_stalled(status)) return;
     const double h_dry = a.h_dry, g2 = f64::mul(0.5, a.g);
     const int2 lr = a.ecell[(long long)blockIdx.x * kLoopEdges + tid];
     const double* const eg = a.egeo + (long long)blockIdx.x * 2 * kLoopEdges + tid;
@@ -277,7 +286,7 @@ __global__ void __launch_bounds__(kLoopEdges, MINB) step_loop_f64(const LoopArgs
         p2 = 1 - p2;
         p3 = p3 == 2 ? 0 : p3 + 1;
         if (tid < 32) warp_min_publish<double>(cand, a.small + p3);
-        if (!grid_meet(a.barrier, (unsigned)(s + 1) * gridDim.x, status, &failed)) break;
+        if (!grid_meet(a.barrier, (unsigned)(s + 1) * gridDim.x, a.max_polls, status, &failed)) break;
     }
     if (tid < 32) {
         active = __reduce_add_sync(0xffffffffu, active);

@@ -94,3 +94,38 @@ def test_steps_under_stream_capture_are_single_launches(precision):
     captured.set_stream(None)
     assert captured.info()["t"] == single.step(6)
     _equal(captured, single)
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+def test_a_wait_that_runs_out_is_reported_until_a_new_state(precision):
+    # no polls: every block gives up at the first meeting and the kernel returns
+    mi = mg.dam_break_4k()
+    m, single = _mesh(mi, precision), _mesh(mi, precision, graph_steps=-1)
+    m.debug_loop(max_polls=0)
+    calls = [lambda: m.step(10), lambda: m.step(10), lambda: m.step(1), lambda: m.step_dt([1e-3, 1e-3]),
+             lambda: m.run_to_steady(1e-9, check_every=5, max_steps=10), m.synchronize, lambda: capi.Ensemble([m])]
+    if precision == capi.SWE_FP64:
+        calls.append(lambda: m.adjoint(5, [1], [1.0]))
+    for call in calls:
+        with pytest.raises(capi.SWEError) as e:
+            call()
+        assert e.value.code == capi.SWE_ETIMEOUT
+    assert m.info()["status"] == capi.SWE_ETIMEOUT
+    m.debug_loop(max_polls=1 << 22)
+    with pytest.raises(capi.SWEError) as e:      # no loop starts on what the other left
+        m.step(10)
+    assert e.value.code == capi.SWE_ETIMEOUT
+    m.set_state(mi.h.astype(m.dtype), mi.hu.astype(m.dtype), mi.hv.astype(m.dtype))
+    done = m.debug_loop()
+    assert m.step(50) == single.step(50) and m.debug_loop() == done + 50
+    _equal(m, single)
+
+
+def test_the_loop_runs_where_it_should():
+    mi = mg.river(90, 13, seed=4, n_bumps=20)
+    for kw, steps in ((dict(), 50), (dict(graph_steps=48), 0), (dict(graph_steps=-1), 0), (dict(block_size=128), 0),
+                      (dict(activity=1), 0), (dict(debug_checks=1), 0)):
+        m = _mesh(mi, capi.SWE_FP32, **kw)
+        m.step(50)
+        m.step(3)
+        assert m.debug_loop() == steps, kw

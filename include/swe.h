@@ -171,14 +171,16 @@ SWE_API void swe_config_default(swe_config* cfg);
 SWE_API int swe_debug_code_ok(int32_t code, int64_t n_cells, int n_groups);
 
 /*
- * For tests of the step loop (swe_config.graph_steps): max_polls >= 0 sets the
- * number of polls after which a wait of this mesh's loop gives up (0: at
- * once; < 0: as it is; the default, 2^22, is under two seconds).  Once a wait
- * has given up, calls that advance the mesh return SWE_ETIMEOUT until a new
- * state is set.  steps, if not NULL, receives the steps that this mesh has
- * run in the loop.  Errors: SWE_EINVAL.
+ * For tests of the step loop (swe_config.graph_steps).  max_cells >= 0 sets the
+ * largest mesh that it is launched for (< 0: as it is, by default what the
+ * device holds at once; a larger launch is refused by the runtime, and the
+ * mesh goes on without the loop).  max_polls >= 0 sets the number of polls
+ * after which a wait of the loop gives up (0: at once; < 0: as it is; the
+ * default, 2^22, is under two seconds); once one has, calls that advance the
+ * mesh return SWE_ETIMEOUT until a new state is set.  steps, if not NULL,
+ * receives the steps that this mesh has run in the loop.  Errors: SWE_EINVAL.
  */
-SWE_API int swe_debug_loop(swe_mesh* mesh, int64_t max_polls, int64_t* steps);
+SWE_API int swe_debug_loop(swe_mesh* mesh, int64_t max_cells, int64_t max_polls, int64_t* steps);
 
 /*
  * Builds a mesh (Section 3.1): orients every triangle counter-clockwise, finds

@@ -105,7 +105,7 @@ def load():
         [vp] * 4 + [vp]
     lib.swe_mesh_preprocess.argtypes = [vp, C.c_int64, vp, C.c_int64, C.c_int, C.c_int, vp, vp, vp, vp, vp]
     lib.swe_debug_code_ok.argtypes = [C.c_int32, C.c_int64, C.c_int]
-    lib.swe_debug_loop.argtypes = [vp, C.c_int64, C.POINTER(C.c_int64)]
+    lib.swe_debug_loop.argtypes = [vp, C.c_int64, C.c_int64, C.POINTER(C.c_int64)]
     lib.swe_cfl_dt_noalloc.argtypes = [C.c_int, C.c_int64, vp, vp, vp, vp, C.c_double, C.c_double,
                                        C.c_double, vp, vp]
     lib.swe_ensemble_create.argtypes = [vp, C.c_int, C.POINTER(vp)]
@@ -338,11 +338,12 @@ class Mesh:
         check(load().swe_autotune(self._h, int(trial_steps), C.byref(t)))
         return {k: getattr(t, k) for k, _ in swe_tune._fields_}
 
-    def debug_loop(self, max_polls=-1):
-        """Sets the poll limit of the step loop's waits (< 0: as it is);
-        returns the steps that this mesh has run in the loop (see swe_debug_loop)."""
+    def debug_loop(self, max_polls=-1, max_cells=-1):
+        """Sets the poll limit of the step loop's waits and the largest mesh that
+        it is launched for (< 0: as they are); returns the steps that this mesh
+        has run in the loop (see swe_debug_loop)."""
         steps = C.c_int64(0)
-        check(load().swe_debug_loop(self._h, int(max_polls), C.byref(steps)))
+        check(load().swe_debug_loop(self._h, int(max_cells), int(max_polls), C.byref(steps)))
         return steps.value
 
     def permutation(self):

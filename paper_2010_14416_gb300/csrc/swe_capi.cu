@@ -332,10 +332,13 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
     if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
     if (cs != cudaStreamCaptureStatusNone) return false;
     if (m->loop_cells < 0) {
-        long long cells = 0;
-        if (Launch<T>::loop_capacity(m->cfg.device, &cells) != cudaSuccess) { (void)cudaGetLastError(); cells = 0; }
+        long long cells = m->loop_cells_set;
+        if (cells < 0 && Launch<T>::loop_capacity(m->cfg.device, &cells) != cudaSuccess) {
+            (void)cudaGetLastError();
+            cells = 0;
+        }
         m->loop_cells = cells;
-        if (m->hm.n_cells <= cells) {
+        if (m->hm.n_cells <= cells && !m->loop_barrier) {
             bool ok = cudaMalloc((void**)&m->loop_barrier, sizeof(unsigned)) == cudaSuccess;
             if (ok && sizeof(T) == 8) ok = build_loop_edges(m) == SWE_OK;
             if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
@@ -344,8 +347,11 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
     return m->hm.n_cells <= m->loop_cells;
 }
 
+// Runs nsteps steps in the loop; on return nsteps is what is left of them.  Where
+// the launch is refused (fewer SMs open to the stream than the device has, as
+// under a green context), this mesh goes on without the loop.
 template <typename T>
-int run_loop(swe_mesh* m, int64_t nsteps, double cfl) {
+void run_loop(swe_mesh* m, int64_t& nsteps, double cfl) {
     LoopArgs<T> a;
     a.state[0] = (V4<T>*)m->state[0];
     a.state[1] = (V4<T>*)m->state[1];
@@ -375,18 +381,23 @@ int run_loop(swe_mesh* m, int64_t nsteps, double cfl) {
         a.step0 = m->nstep;
         a.steps = (int)std::min<int64_t>(nsteps, 2000);   // some milliseconds a launch
         a.max_polls = m->loop_polls;
-        const cudaError_t e = Launch<T>::loop(a, m->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "swe_step: loop launch");
+        if (Launch<T>::loop(a, m->stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            m->loop_allowed = false;
+            return;
+        }
         m->nstep += a.steps;
         m->loop_steps += a.steps;
         nsteps -= a.steps;
     }
-    return SWE_OK;
 }
 
 template <typename T>
 int run_steps(swe_mesh* m, int64_t nsteps, double cfl) {
-    if (use_loop<T>(m, nsteps)) return run_loop<T>(m, nsteps, cfl);
+    if (use_loop<T>(m, nsteps)) {
+        run_loop<T>(m, nsteps, cfl);
+        if (nsteps == 0) return SWE_OK;
+    }
     if (m->cfg.activity) {
         if (!m->act_valid) {
             int rc = init_activity(m);
@@ -732,8 +743,12 @@ int swe_debug_code_ok(int32_t code, int64_t n_cells, int n_groups) {
     return code_ok(code, (long long)n_cells, n_groups) ? 1 : 0;
 }
 
-int swe_debug_loop(swe_mesh* m, int64_t max_polls, int64_t* steps) {
+int swe_debug_loop(swe_mesh* m, int64_t max_cells, int64_t max_polls, int64_t* steps) {
     if (!m || max_polls > (int64_t)0xFFFFFFFF) { set_error("swe_debug_loop: bad arguments"); return SWE_EINVAL; }
+    if (max_cells >= 0) {
+        m->loop_cells_set = max_cells;
+        m->loop_cells = -1;
+    }
     if (max_polls >= 0) m->loop_polls = (unsigned)max_polls;
     if (steps) *steps = m->loop_steps;
     return SWE_OK;

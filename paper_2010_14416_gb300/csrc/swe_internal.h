@@ -170,7 +170,7 @@ struct swe_mesh {
     // launches: the largest mesh it takes (-1: not asked yet), its arrival
     // count and, FP64, its blocks' edges
     bool loop_allowed = false;
-    long long loop_cells = -1;
+    long long loop_cells = -1, loop_cells_set = -1;   // (set: swe_debug_loop)
     unsigned loop_polls = 0;           // polls after which a wait of the loop gives up
     int64_t loop_steps = 0;            // steps run in the loop
     unsigned* loop_barrier = nullptr;

@@ -129,3 +129,15 @@ def test_the_loop_runs_where_it_should():
         m.step(50)
         m.step(3)
         assert m.debug_loop() == steps, kw
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+def test_a_refused_cooperative_launch_leaves_the_mesh_on_single_launches(precision):
+    # more blocks than the device holds at once: the runtime refuses the launch
+    mi = mg.river(700, 110, seed=2, n_bumps=10)
+    m, single = _mesh(mi, precision), _mesh(mi, precision, graph_steps=-1)
+    m.debug_loop(max_cells=1 << 20)
+    for steps in (7, 60):
+        assert m.step(steps) == single.step(steps)
+        _equal(m, single)
+    assert m.debug_loop() == 0

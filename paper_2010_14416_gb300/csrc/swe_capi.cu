@@ -324,7 +324,12 @@ int build_loop_edges(swe_mesh* m) {
 // Whether the next steps run as one loop launch: a small mesh, nothing chosen
 // about its launches, no debug checks and no capture of the stream (a
 // cooperative launch is not for every graph).  From 4 steps on: the loop's
-// launch and first reads cost about what two step launches do.
+// launch and first reads cost about what two step launches do.  FP32 meshes of
+// more than four of the six blocks an SM holds take it for calls shorter than a
+// graph only: more blocks meet more slowly, and a replayed graph has no gaps
+// between its launches (us a step of a half wet canal, loop against graph: 60,000
+// cells 4.4 and 4.7, 80,000 5.4 and 5.2, 112,000 6.7 and 5.5; of calls of 20
+// steps, against single launches, 5.1 and 6.9, 5.7 and 6.9, 6.9 and 7.1).
 template <typename T>
 bool use_loop(swe_mesh* m, int64_t nsteps) {
     if (!m->loop_allowed || nsteps < 4) return false;
@@ -344,7 +349,8 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
             if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
         }
     }
-    return m->hm.n_cells <= m->loop_cells;
+    const bool graphs = sizeof(T) == 4 && nsteps >= m->cfg.graph_steps;
+    return m->hm.n_cells <= (graphs ? m->loop_cells / 3 * 2 : m->loop_cells);
 }
 
 // Runs nsteps steps in the loop; on return nsteps is what is left of them.  Where

@@ -141,3 +141,15 @@ def test_a_refused_cooperative_launch_leaves_the_mesh_on_single_launches(precisi
         assert m.step(steps) == single.step(steps)
         _equal(m, single)
     assert m.debug_loop() == 0
+
+
+def test_long_calls_of_larger_fp32_meshes_replay_graphs():
+    # 110,000 cells, past four blocks an SM: calls of a graph (48 steps) and more
+    # replay it, shorter ones take the loop; 70,000 cells: the loop for both
+    for nx, expect in ((500, 20 + 20), (318, 20 + 100 + 20)):
+        mi = mg.river(nx, 110, seed=2, n_bumps=10)
+        m, single = _mesh(mi, capi.SWE_FP32), _mesh(mi, capi.SWE_FP32, graph_steps=-1)
+        for steps in (20, 100, 20):
+            assert m.step(steps) == single.step(steps)
+        assert m.debug_loop() == expect
+        _equal(m, single)

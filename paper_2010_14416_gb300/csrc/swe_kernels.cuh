@@ -285,6 +285,14 @@ __device__ __forceinline__ void riemann_hllc(T hL, T unL, T utL, T hR, T unR, T 
     }
 }
 
+// Threads of a step kernel's block.  FP64 blocks may be launched with fewer than
+// BLOCK (step_threads); asking for it costs an FP32 step 1 % (1M-cell canal
+// 17.27 us, 17.08 with the constant).
+template <typename T, int BLOCK>
+__device__ __forceinline__ int block_threads() {
+    return sizeof(T) == 8 ? (int)blockDim.x : BLOCK;
+}
+
 template <typename T>
 __device__ __forceinline__ T inf_of();
 template <>
@@ -335,7 +343,7 @@ __device__ __forceinline__ void block_min_publish(T cand, unsigned long long* ds
     if (lane == 0) { warp_min[wid] = cand; warp_cnt[wid] = cnt; }
     __syncthreads();
     if (wid == 0) {
-        const int warps = (int)blockDim.x >> 5;   // at most BLOCK / 32
+        const int warps = block_threads<T, BLOCK>() / 32;
         T v = lane < warps ? warp_min[lane] : inf_of<T>();
         unsigned c = lane < warps ? warp_cnt[lane] : 0u;
         for (int o = 16; o > 0; o >>= 1) v = min_nonneg(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -889,8 +897,9 @@ __global__ void __launch_bounds__(BLOCK, (min_blocks_of<T, EDGES, false>(BLOCK, 
     }
     T cand = inf_of<T>();
     unsigned active = 0u;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int threads = block_threads<T, BLOCK>();
+    const long long stride = (long long)gridDim.x * threads;
+    long long i = (long long)blockIdx.x * threads + threadIdx.x;
     if (!have_dt) {
         for (; i < a.n; i += stride) a.s_out[i] = a.s_in[i];
     } else if constexpr (STAGES <= 1) {
@@ -1003,8 +1012,9 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_pair(const StepArgs<f
 template <typename T, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
     const T g = a.g, h_dry = a.h_dry;
-    const long long stride = (long long)gridDim.x * blockDim.x;   // blocks of BLOCK threads or fewer
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < a.n_edges; e += stride) {
+    const int threads = block_threads<T, BLOCK>();
+    const long long stride = (long long)gridDim.x * threads;
+    for (long long e = (long long)blockIdx.x * threads + threadIdx.x; e < a.n_edges; e += stride) {
         const int2 lr = a.ecells[e];
         if (a.debug && !(lr.x >= 0 && lr.x < a.n && lr.y >= 0 && lr.y < a.n)) {
             atomicOr(a.status, kStatusBadIndex);
@@ -1854,7 +1864,9 @@ __global__ void riemann_batch_kernel(long long n, const T* __restrict__ hL, cons
 // one per 19, so warps should be spread evenly (4,000 cells: 9,663 -> 9,134 us
 // for 500 steps).  FP32 steps measured the same to 2 % slower with it.
 constexpr long long kSpreadCells = 152LL * 12 * 32;   // 12 one-warp blocks per SM
+template <typename T>
 __host__ __device__ inline unsigned step_threads(long long n, unsigned grid, int block) {
+    if (sizeof(T) == 4) return (unsigned)block;
     const long long per = (n + grid - 1) / grid;
     const long long t = (per + 31) / 32 * 32;
     return (unsigned)(t < block ? (t < 32 ? 32 : t) : block);

@@ -75,7 +75,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
         if (e != cudaSuccess) return e;
 #define SWE_LAUNCH_EDGE(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0, true><<<grid, step_threads(a.n, grid, B), 0, st>>>(a); \
+        step_kernel<T, B, M, S, G != 0, true><<<grid, step_threads<T>(a.n, grid, B), 0, st>>>(a); \
         return cudaGetLastError();                                                \
     }
         if constexpr (sizeof(T) == 4) {
@@ -88,7 +88,7 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
     }
 #define SWE_LAUNCH(B, M, S, G) \
     if (block == B && min_blocks == M && stages == S && geo_early == G) {        \
-        step_kernel<T, B, M, S, G != 0><<<grid, step_threads(a.n, grid, B), 0, st>>>(a); \
+        step_kernel<T, B, M, S, G != 0><<<grid, step_threads<T>(a.n, grid, B), 0, st>>>(a); \
         return cudaGetLastError();                                                \
     }
     if constexpr (sizeof(T) == 4) {

@@ -118,12 +118,13 @@ typedef struct swe_config {
                          (h, 0, 0) without reading its topology or its neighbours, and without
                          touching its state when it was inactive in the previous step too (the
                          state in the output buffer, two steps old, is then already the new one);
-                         a first kernel lists the active cells, a second updates them and
-                         marks the cells that the next one must treat as active, and the two
-                         steps after a change from outside (set_state, set_bc, the tuner)
-                         store every state.  0 (default):
+                         the step marks the cells that the next one must treat as active, and
+                         the two steps after a change from outside (set_state, set_bc, the
+                         tuner) store every state.  FP64 meshes and large mostly dry FP32 ones
+                         step over a list of the active cells (a kernel lists them, a second
+                         updates them), the other FP32 ones through all cells.  0 (default):
                          every cell tests its neighbours.  With activity, stages - 1 is the
-                         number of list entries a thread holds or has in flight (default 3).
+                         number of cells a thread holds or has in flight (default 3).
                          Compiled (block_size, min_blocks, geometry_early, stages) with 1:
                          FP32 (128, 8, 0, 3|4), (256, 4, 0, 3), (512, 2, 0, 3),
                          (128, 8, 1, 3|4|5), (256, 4, 1, 3|4); FP64 (128, 1, 0, 3|4),
@@ -171,6 +172,14 @@ SWE_API void swe_config_default(swe_config* cfg);
  * Host-callable, touches no device.
  */
 SWE_API int swe_debug_code_ok(int32_t code, int64_t n_cells, int n_groups);
+
+/*
+ * For tests of the activity modes of an FP32 mesh (swe_config.activity):
+ * list_cells >= 0 sets the size from which its steps run over a list of the
+ * active cells (0: always; < 0: as it is); listed, if not NULL, receives 1 when
+ * the last steps ran over the list.  Errors: SWE_EINVAL.
+ */
+SWE_API int swe_debug_activity(swe_mesh* mesh, int64_t list_cells, int* listed);
 
 /*
  * For tests of the step loop (swe_config.graph_steps).  max_cells >= 0 sets the

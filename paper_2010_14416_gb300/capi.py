@@ -35,7 +35,8 @@ EXPORTS = ["swe_config_default", "swe_mesh_create", "swe_mesh_destroy", "swe_set
            "swe_ensemble_step", "swe_ensemble_get_state", "swe_ensemble_get_info", "swe_adjoint",
            "swe_adjoint_series",
            "swe_step_dt", "swe_set_fields", "swe_diagnostics", "swe_run_to_steady", "swe_autotune",
-           "swe_ensemble_autotune", "swe_ensemble_set_shape", "swe_debug_code_ok", "swe_debug_loop", "swe_adjoint_method",
+           "swe_ensemble_autotune", "swe_ensemble_set_shape", "swe_debug_code_ok", "swe_debug_loop", "swe_debug_activity",
+           "swe_adjoint_method",
            "swe_last_error"]
 
 
@@ -105,6 +106,7 @@ def load():
         [vp] * 4 + [vp]
     lib.swe_mesh_preprocess.argtypes = [vp, C.c_int64, vp, C.c_int64, C.c_int, C.c_int, vp, vp, vp, vp, vp]
     lib.swe_debug_code_ok.argtypes = [C.c_int32, C.c_int64, C.c_int]
+    lib.swe_debug_activity.argtypes = [vp, C.c_int64, C.POINTER(C.c_int)]
     lib.swe_debug_loop.argtypes = [vp, C.c_int64, C.c_int64, C.POINTER(C.c_int64)]
     lib.swe_cfl_dt_noalloc.argtypes = [C.c_int, C.c_int64, vp, vp, vp, vp, C.c_double, C.c_double,
                                        C.c_double, vp, vp]
@@ -337,6 +339,14 @@ class Mesh:
         t = swe_tune()
         check(load().swe_autotune(self._h, int(trial_steps), C.byref(t)))
         return {k: getattr(t, k) for k, _ in swe_tune._fields_}
+
+    def debug_activity(self, list_cells=-1):
+        """Sets the size from which an FP32 mesh's activity steps run over a list
+        (0: always; < 0: as it is); returns whether the last ones did (see
+        swe_debug_activity)."""
+        listed = C.c_int(0)
+        check(load().swe_debug_activity(self._h, int(list_cells), C.byref(listed)))
+        return bool(listed.value)
 
     def debug_loop(self, max_polls=-1, max_cells=-1):
         """Sets the poll limit of the step loop's waits and the largest mesh that

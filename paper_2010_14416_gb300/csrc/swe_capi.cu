@@ -33,6 +33,7 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 namespace {
 
 constexpr int kDefaultGraphSteps = 48;
+constexpr int64_t kListCells = 800000;   // FP32 activity steps over a list (list_activity)
 
 struct DeviceGuard {
     int prev = -1;
@@ -59,6 +60,7 @@ __global__ void init_small_kernel(unsigned long long* small, double t) {
         small[kSlotStatus] = 0ULL;
         small[kSlotClamp] = 0ULL;
         small[6] = 0ULL; small[7] = 0ULL;
+        small[kSmallWords] = 0ULL;   // wet cells (set_state)
     }
 }
 
@@ -230,7 +232,7 @@ StepArgs<T> make_args(swe_mesh* m, int64_t step_index, double cfl) {
     a.span_clear = nullptr;
     a.span_first = m->span_first;
     a.span_adj = m->span_adj;
-    a.act_list = m->act_list;
+    a.act_list = m->act_by_list ? m->act_list : nullptr;
     a.act_count = m->act_count;
     if (m->cfg.activity && m->act[0]) {
         a.act_in = m->act[p3];
@@ -398,6 +400,39 @@ void run_loop(swe_mesh* m, int64_t& nsteps, double cfl) {
     }
 }
 
+// Whether the activity steps of m run over a list of the active cells (two
+// launches) or, FP32, through all cells (one).  The list costs 5 us a step and
+// 6 ps for each active cell more and saves 5 ps for each quiet one, more where
+// the active cells lie unevenly among the blocks: of n cells with a share s
+// active it pays from n (1 - 2.2 s) = 550,000 (a winding channel) to 1.3M (one
+// wet end) on; the line is at 800,000 (a tenth less before a mesh on the list
+// leaves it).  us a step, list and all cells: a half
+// wet canal of 200,000 cells 11.7 and 6.9, of 1.2M 24.1 and 20.8; a canal 10 %
+// wet of 1.2M 12.2 and 10.6, of 2.5M 19.5 and 22.3; a reach 6 % wet of 300,000
+// 9.4 and 8.3, of 1.2M 10.4 and 15.4, of 6M 24.2 and 47.4; 6M cells 30 % wet 65.9
+// and 70.6, 50 % 101.5 and 96.5, all wet 189.5 and 158.2.  The autotuner times
+// the list's shapes (through all cells no shape came first), and a shape of
+// them that it keeps stays on the list.
+bool list_activity(const swe_mesh* m) {
+    if (m->cfg.precision != SWE_FP32 || m->act_tuned || m->list_cells == 0) return true;
+    return (double)m->hm.n_cells * (1.0 - 2.2 * m->act_share) > (double)m->list_cells * (m->act_by_list ? 0.9 : 1.0);
+}
+
+// The activity bytes for the next steps of m, rebuilt where they are not those
+// of its state or where the other kernel is to maintain them.
+int prepare_activity(swe_mesh* m) {
+    if (list_activity(m) != m->act_by_list) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) (void)cudaGetLastError();
+        if (cs == cudaStreamCaptureStatusNone) {
+            m->act_by_list = !m->act_by_list;
+            m->act_valid = false;
+            drop_graph(m);
+        }
+    }
+    return m->act_valid ? SWE_OK : init_activity(m);
+}
+
 template <typename T>
 int run_steps(swe_mesh* m, int64_t nsteps, double cfl) {
     if (use_loop<T>(m, nsteps)) {
@@ -405,10 +440,8 @@ int run_steps(swe_mesh* m, int64_t nsteps, double cfl) {
         if (nsteps == 0) return SWE_OK;
     }
     if (m->cfg.activity) {
-        if (!m->act_valid) {
-            int rc = init_activity(m);
-            if (rc) return rc;
-        }
+        const int rc = prepare_activity(m);
+        if (rc) return rc;
     } else {
         m->act_valid = false;   // steps without activity bytes do not maintain them
     }
@@ -448,6 +481,11 @@ int read_small(swe_mesh* m, unsigned long long out[kSmallWords]) {
                                     cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "swe: reading the status block");
+    if (m->nstep > m->act_seen_step && out[kSlotActive] >= m->act_seen)
+        m->act_share = (double)(out[kSlotActive] - m->act_seen) /
+                       ((double)(m->nstep - m->act_seen_step) * (double)m->hm.n_cells);
+    m->act_seen = out[kSlotActive];
+    m->act_seen_step = m->nstep;
     return SWE_OK;
 }
 
@@ -486,11 +524,19 @@ int set_state_t(swe_mesh* m, const void* h, const void* hu, const void* hv, int 
     // (the other buffer holds nothing that is read: a step writes every record,
     // with the activity bytes the first two after a set_state do)
     if (e == cudaSuccess) { init_small_kernel<<<1, 32, 0, m->stream>>>(m->small, t); e = cudaGetLastError(); }
+    // list_activity asks how much of the mesh is wet
+    unsigned long long wet = 0;
+    unsigned long long* const n_wet =
+        sizeof(T) == 4 && m->cfg.activity && n > m->list_cells ? m->small + kSmallWords : nullptr;
     if (e == cudaSuccess)
         e = Launch<T>::dt((const V4<T>*)m->state[0], (const V4<T>*)m->geoB, n, (T)m->cfg.g, (T)m->cfg.h_dry,
-                          m->small + 0, m->stream);
+                          m->small + 0, n_wet, m->stream);
+    if (e == cudaSuccess && n_wet) e = cudaMemcpyAsync(&wet, n_wet, sizeof wet, cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "swe_set_state");
+    if (n_wet) m->act_share = (double)wet / (double)n;
+    m->act_seen = 0;
+    m->act_seen_step = 0;
     m->have_state = true;
     m->nstep = 0;
     m->act_valid = false;
@@ -749,6 +795,13 @@ int swe_debug_code_ok(int32_t code, int64_t n_cells, int n_groups) {
     return code_ok(code, (long long)n_cells, n_groups) ? 1 : 0;
 }
 
+int swe_debug_activity(swe_mesh* m, int64_t list_cells, int* listed) {
+    if (!m) { set_error("swe_debug_activity: NULL mesh"); return SWE_EINVAL; }
+    if (list_cells >= 0) m->list_cells = list_cells;
+    if (listed) *listed = m->cfg.activity && m->act_valid && m->act_by_list ? 1 : 0;
+    return SWE_OK;
+}
+
 int swe_debug_loop(swe_mesh* m, int64_t max_cells, int64_t max_polls, int64_t* steps) {
     if (!m || max_polls > (int64_t)0xFFFFFFFF) { set_error("swe_debug_loop: bad arguments"); return SWE_EINVAL; }
     if (max_cells >= 0) {
@@ -857,6 +910,8 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
     m->cfg = c;
     m->loop_allowed = nothing_chosen && !c.debug_checks;
     m->loop_polls = kMaxPolls;
+    m->list_cells = kListCells;
+    m->act_by_list = c.precision != SWE_FP32 || n_tris > kListCells;
     m->esz = c.precision == SWE_FP32 ? 4 : 8;
     std::string err;
     int rc;
@@ -882,7 +937,7 @@ int swe_mesh_create(const double* nodes, int64_t n_nodes, const int32_t* tris, i
         (rc = dev_alloc(m, &m->zdev, n * m->esz, "bed")) ||
         (rc = dev_alloc(m, (void**)&m->perm, n * sizeof(unsigned), "permutation")) ||
         (rc = dev_alloc(m, (void**)&m->inv, n * sizeof(unsigned), "permutation")) ||
-        (rc = dev_alloc(m, (void**)&m->small, kSmallWords * sizeof(unsigned long long), "status"))) {
+        (rc = dev_alloc(m, (void**)&m->small, (kSmallWords + 1) * sizeof(unsigned long long), "status"))) {
         swe_mesh_destroy(m);
         return rc;
     }

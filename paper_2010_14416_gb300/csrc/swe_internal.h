@@ -151,6 +151,15 @@ struct swe_mesh {
     unsigned char* act[3] = {nullptr, nullptr, nullptr};
     int64_t act_len = 0;
     bool act_valid = false;
+    bool act_by_list = true;           // which activity kernel maintains them (list_activity)
+    bool act_tuned = false;            // the autotuner kept an activity shape
+    int64_t list_cells = 0;
+    // the wet cells' share of the state that was set, then the active cells' share
+    // of the steps between the last two readings of the status block, and that
+    // reading's count and step
+    double act_share = 0.0;
+    unsigned long long act_seen = 0;
+    int64_t act_seen_step = 0;
     unsigned* act_list = nullptr;      // n cells: those that run the flux path in a step
     unsigned *span_first = nullptr, *span_adj = nullptr;   // the spans beside each span (act_scan_kernel)
     unsigned* act_count = nullptr;     // 2 words, 0 between steps

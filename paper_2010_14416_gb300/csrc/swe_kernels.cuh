@@ -1057,7 +1057,7 @@ __global__ void __launch_bounds__(BLOCK) edge_flux_kernel(const StepArgs<T> a) {
 // record or its neighbours' states -- the same result the neighbour test of
 // update_cell gives, bit for bit.
 //
-// Two launches.  act_scan_kernel reads the bytes (2 per cell, 16 cells a
+// Over a list, in two launches: act_scan_kernel reads the bytes (2 per cell, 16 cells a
 // thread, a block's 4,096 at a time, and none of a span whose flags say that
 // they are all 0) and gathers the cells that run the flux path into a list, a
 // span's cells in their order; a quiet cell costs it nothing more unless its
@@ -1230,6 +1230,142 @@ __global__ void __launch_bounds__(BLOCK, MINB) step_kernel_act(const StepArgs<T>
         a.act_count[0] = 0u;
         a.act_count[1] = 0u;
     }
+}
+
+// The same in one launch over all cells, FP32, for meshes where two launches and
+// the list cost more than going through the quiet cells (list_activity has the
+// measurements).  Per-thread cp.async pipeline over the thread's cells
+// c_k = i0 + k stride:
+// iteration k issues the topology of c_{k+1} (only if its byte is set), then
+// the activity bytes of c_{k+PF+1} (8 lanes copy the warp's 32 bytes) and the
+// state record of c_{k+PF}; it then processes c_k.  PF (the prefetch
+// distance of the streamed state, >= 2) is a compiled shape parameter.
+template <int BLOCK, int MINB, bool GEO_EARLY, int PF>
+__global__ void __launch_bounds__(BLOCK, MINB) step_kernel_act_all(const StepArgs<float> a) {
+    using T = float;
+    static_assert(BLOCK % 32 == 0, "warps of whole cells");
+    static_assert(PF >= 2, "the wait counts below assume a prefetch distance of at least two cells");
+    constexpr int NS = PF + 1;  // state and activity slots
+    const WarpDt<T> wdt = warp_step_dt<T>(a.cfl, a.dt_read, a.dt_fixed);
+    const double dt_d = wdt.d;
+    const bool have_dt = wdt.have;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *a.dt_reset = kInfBits;
+        if (have_dt) *a.t += dt_d;
+        else atomicOr(a.status, kStatusDry);
+        if (a.dt_log) *a.dt_log = dt_d;
+    }
+    T cand = inf_of<T>();
+    unsigned active = 0u;
+    // 32-bit cell indices: the host allows this kernel only for n < 2^29, so
+    // c + (PF + 1) stride < 2^32 with stride <= n + BLOCK and PF <= 5
+    const unsigned stride = gridDim.x * BLOCK;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned i0 = blockIdx.x * BLOCK + tid;
+    const unsigned n = (unsigned)a.n;
+    if (!have_dt) {
+        // no step: the state and its activity carry over unchanged
+        for (unsigned c = i0; c < n; c += stride) {
+            a.s_out[c] = a.s_in[c];
+            a.act_next[c] = a.act_in[c];
+            a.act_clear[c] = 0;
+        }
+    } else {
+        static_assert(PF <= 5, "32-bit indices");
+        __shared__ V4<T> st_own[NS][BLOCK];
+        __shared__ int4 st_topo[2][BLOCK];
+        __shared__ unsigned st_act[NS][BLOCK / 4];  // 32 activity bytes per warp per stage
+        __shared__ unsigned st_prev[NS][BLOCK / 4]; // and the previous step's (act_clear) bytes
+        const T dt = wdt.t;
+        // warp w of the block owns st_act[.][8 w .. 8 w + 7]; lanes 0..7 copy 4 bytes each
+        auto act_copy = [&](int slot, unsigned c) {
+            const unsigned base = c - lane;
+            if (lane < 8 && base < n) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(&st_act[slot][warp * 8 + lane])),
+                             "l"(a.act_in + base + 4 * lane)
+                             : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(&st_prev[slot][warp * 8 + lane])),
+                             "l"(a.act_clear + base + 4 * lane)
+                             : "memory");
+            }
+        };
+        // bit 0: the cell runs the flux path in this step (bit 0 of its byte);
+        // bit 1: the previous step's byte is not 0 (the cell ran the flux path
+        // then, or the bytes were rebuilt less than two steps ago)
+        auto act_byte = [&](int slot) -> unsigned {
+            return (((const unsigned char*)&st_act[slot][warp * 8])[lane] & 1u) |
+                   (((const unsigned char*)&st_prev[slot][warp * 8])[lane] ? 2u : 0u);
+        };
+        // prologue: activity of c_0 .. c_PF and states of c_0 .. c_{PF-1}; then topology of c_0
+#pragma unroll
+        for (int q = 0; q <= PF; ++q) act_copy(q, i0 + q * stride);
+#pragma unroll
+        for (int q = 0; q < PF; ++q)
+            if (i0 + q * stride < n) cp_async_record<sizeof(V4<T>)>(&st_own[q][tid], &a.s_in[i0 + q * stride]);
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncwarp();
+        unsigned f_cur = act_byte(0);
+        if ((f_cur & 1u) && i0 < n) cp_async_record<16>(&st_topo[0][tid], &a.topo[i0]);
+        cp_async_commit();                                       // T_{-1}
+        cp_async_commit();                                       // H_{-1} (empty: its copies were in the first group)
+        int ks = 0, k2 = 0;  // k mod NS, k mod 2
+        for (unsigned c = i0; c - lane < n; c += stride) {
+            const int ks1 = ks + 1 == NS ? 0 : ks + 1;          // slot of c_{k+1}
+            const int ksp = ks == 0 ? NS - 1 : ks - 1;          // slot of c_{k+PF} (c_{k-1}'s, consumed)
+            // groups so far: ..., T_{k-1}, H_{k-1}; H_{k-PF} and older (activity of
+            // c_{k+1}, state of c_k) must be complete, which H_{k-2} implies
+            cp_async_wait<2>();
+            __syncwarp();
+            const unsigned f_next = act_byte(ks1);
+            const unsigned c1 = c + stride, cp = c + PF * stride, cp1 = c + (PF + 1) * stride;
+            if ((f_next & 1u) && c1 < n) cp_async_record<16>(&st_topo[k2 ^ 1][tid], &a.topo[c1]);
+            cp_async_commit();                                   // T_k
+            __syncwarp();                                        // every lane has read slot ks before it refills
+            act_copy(ks, cp1);
+            if (cp < n) cp_async_record<sizeof(V4<T>)>(&st_own[ksp][tid], &a.s_in[cp]);
+            cp_async_commit();                                   // H_k
+            cp_async_wait<3>();                                  // T_{k-1}: the topology of c_k
+            if (c < n) {
+                const V4<T> own = st_own[ks][tid];
+                if (!(f_cur & 1u)) {
+                    // quiet: the new state is (h, 0, 0); if the cell was quiet in the
+                    // previous step too, the output buffer (the state of two steps
+                    // ago, itself dry at rest with the same h) holds it already
+                    if (f_cur & 2u) {
+                        V4<T> out;
+                        out.x = own.x; out.y = T(0); out.z = T(0); out.w = own.w;
+                        a.s_out[c] = out;
+                    }
+                } else {
+                    const T r = update_cell<T, GEO_EARLY>(a, c, own, st_topo[k2][tid], dt, active, a.n_clamped,
+                                                          a.status);
+                    cand = min_nonneg(cand, r);
+                    const bool wet = r < inf_of<T>();
+                    // the topology record is read again from shared memory rather than kept
+                    // live in registers across the update
+                    const volatile int* tv = (const volatile int*)&st_topo[k2][tid];
+                    if (wet || (tv[3] & kStaticBit)) a.act_next[c] = 1;
+                    if (wet) {
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
+                            const int code = tv[j];
+                            if (code >= 0 && (!a.debug || code_ok(code, a.n, a.n_groups)))
+                                a.act_next[code & kNbrMask] = 1;
+                        }
+                    }
+                }
+                a.act_clear[c] = 0;
+            }
+            f_cur = f_next;
+            ks = ks1;
+            k2 ^= 1;
+        }
+        cp_async_wait<0>();
+    }
+    block_min_publish<BLOCK>(cand, a.dt_write, active, a.n_active);
 }
 
 // Activity bytes of a state (into a buffer filled with 2): a wet cell marks
@@ -1792,22 +1928,26 @@ __global__ void __launch_bounds__(BLOCK, MINB) ensemble_step_kernel_pair(const E
     if ((tid & 31) == 0 && active) atomicAdd(a.n_active, (unsigned long long)active);
 }
 
-// ---- CFL min of a given state (used after swe_set_state) --------------------------
+// ---- CFL min of a given state (used after swe_set_state), and its wet cells where
+// n_wet is given ----------------------------------------------------------------------
 template <typename T, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) dt_kernel(const V4<T>* __restrict__ s, const V4<T>* __restrict__ geoB,
-                                                   long long n, T g, T h_dry, unsigned long long* dt_write) {
+                                                   long long n, T g, T h_dry, unsigned long long* dt_write,
+                                                   unsigned long long* n_wet) {
     using A = Ar<T>;
     const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
     T cand = inf_of<T>();
+    unsigned wet = 0u;
     if (i < n) {
         const V4<T> c = s[i];
         if (c.x > h_dry) {
+            wet = 1u;
             const T r = A::rcp_(c.x);
             const T u = c.y * r, v = c.z * r;
             cand = A::div_(geoB[i].w, A::sqrt_(g * c.x) + A::sqrt_(u * u + v * v));
         }
     }
-    block_min_publish<BLOCK>(cand, dt_write);
+    block_min_publish<BLOCK>(cand, dt_write, wet, n_wet);
 }
 
 // ---- layout conversion between caller arrays and the packed internal state --------
@@ -1941,7 +2081,8 @@ struct Launch {
     static cudaError_t loop_capacity(int device, long long* cells);
     static cudaError_t loop(const LoopArgs<T>& a, cudaStream_t st);
     static cudaError_t dt(const V4<T>* s, const V4<T>* geoB, long long n, T g, T h_dry,
-                          unsigned long long* dt_write, cudaStream_t st);
+                          unsigned long long* dt_write, unsigned long long* n_wet,
+                          cudaStream_t st);
     static cudaError_t pack(const T* h, const T* hu, const T* hv, const unsigned* perm, const T* z,
                             V4<T>* s, long long n, cudaStream_t st);
     static cudaError_t unpack(const V4<T>* s, const unsigned* inv, T* h, T* hu, T* hv, long long n,

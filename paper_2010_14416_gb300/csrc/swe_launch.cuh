@@ -33,8 +33,9 @@ static inline unsigned grid_for(long long n, int block) {
 constexpr int kEdgeBlock = 256;
 
 // (block, min blocks per SM, geometry early, stages) shapes of the activity
-// kernel; stages - 1 = list entries whose records a thread holds or has in
-// flight (state, topology and index in shared memory).
+// kernels; stages - 1 = list entries whose records a thread holds or has in
+// flight (state, topology and index in shared memory), or the prefetch
+// distance of the kernel over all cells.  Both kernels reach the min blocks.
 #define SWE_ACT_VARIANTS_F32(X)                                                                     \
     X(128, 8, 0, 3) X(256, 4, 0, 3) X(512, 2, 0, 3) X(128, 8, 1, 3) X(256, 4, 1, 3) X(128, 8, 1, 4) \
     X(128, 8, 1, 5) X(256, 4, 1, 4) X(128, 8, 0, 4)
@@ -51,6 +52,18 @@ cudaError_t Launch<T>::step(const StepArgs<T>& a, int block, int min_blocks, int
                             cudaStream_t st) {
     const unsigned grid = a.grid;
     if (grid == 0) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+        if (a.act_in && !a.act_list) {
+#define SWE_LAUNCH_ACT(B, M, G, S) \
+    if (block == B && min_blocks == M && geo_early == G && stages == S) {         \
+        step_kernel_act_all<B, M, G != 0, S - 1><<<grid, B, 0, st>>>(a);          \
+        return cudaGetLastError();                                                \
+    }
+            SWE_ACT_VARIANTS_F32(SWE_LAUNCH_ACT)
+#undef SWE_LAUNCH_ACT
+            return cudaErrorInvalidValue;
+        }
+    }
     if (a.act_in) {
         // a block per span: most spans of a dry mesh cost it one look at their flags
         const unsigned spans = grid_for<T>(a.n, 1 << kScanLog);
@@ -627,8 +640,8 @@ cudaError_t Launch<T>::loop(const LoopArgs<T>& a, cudaStream_t st) {
 
 template <typename T>
 cudaError_t Launch<T>::dt(const V4<T>* s, const V4<T>* geoB, long long n, T g, T h_dry,
-                          unsigned long long* dt_write, cudaStream_t st) {
-    dt_kernel<T, 256><<<grid_for<T>(n, 256), 256, 0, st>>>(s, geoB, n, g, h_dry, dt_write);
+                          unsigned long long* dt_write, unsigned long long* n_wet, cudaStream_t st) {
+    dt_kernel<T, 256><<<grid_for<T>(n, 256), 256, 0, st>>>(s, geoB, n, g, h_dry, dt_write, n_wet);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ int autotune_t(swe_mesh* m, int trial_steps, swe_tune* out) {
     rc = build_edges(m);
     if (rc) return rc;
     if (n < kActivityMaxCells) {
+        m->act_by_list = true;
         rc = init_activity(m);
         if (rc) return rc;
     }
@@ -236,6 +237,7 @@ int autotune_t(swe_mesh* m, int trial_steps, swe_tune* out) {
     if (e == cudaSuccess && best_plain < cand.size()) apply_shape(m, cand[best_plain]);
     else m->plain = plain_before;
     apply_shape(m, pick);
+    m->act_tuned = e == cudaSuccess && pick.activity != 0;
     // the activity bytes are rebuilt before the next step: the trials cleared the
     // previous step's bytes, which tell the next step whose state it may leave
     m->act_valid = false;

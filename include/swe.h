@@ -544,13 +544,17 @@ typedef struct swe_tune {
  * (>= 1; 0 = 8), twice; the shape in use and the (at most four) shapes within
  * 5 % of the fastest are then timed again over max(32, 4 trial_steps) steps,
  * and the first of them (in a fixed order, the shape in use first) within 1 %
- * of the fastest there is kept for all later steps.  The
+ * of the fastest there is kept for all later steps that are launched one by
+ * one or replayed from a graph.  The
  * paper fixes no launch shape; every shape evaluates the same arithmetic on
  * every cell, so the choice changes the speed only: states, times and time
- * steps are bit for bit the same whatever is chosen.  The trial steps read the
- * current state and write scratch copies of the state and status block, so
- * the mesh's state, time and step count do not change.  Allocates one state
- * buffer for the duration of the call and waits for the mesh stream.
+ * steps are bit for bit the same whatever is chosen.  A small mesh that runs
+ * calls as one cooperative launch (swe_config.graph_steps) then times calls of
+ * 16 steps and of two graphs with it and with the kept shape, and takes the
+ * faster for calls shorter than a graph and for the others.  The trials use
+ * copies of the state and status block or put them back, so the mesh's state,
+ * time and step count do not change.  Allocates one state buffer (then, on such
+ * a mesh, two) for the duration of the call and waits for the mesh stream.
  * out may be NULL.  Errors: SWE_EINVAL (no state set), SWE_ENOMEM, SWE_ECUDA.
  */
 SWE_API int swe_autotune(swe_mesh* mesh, int trial_steps, swe_tune* out);

@@ -334,7 +334,9 @@ int build_loop_edges(swe_mesh* m) {
 // steps, against single launches, 5.1 and 6.9, 5.7 and 6.9, 6.9 and 7.1).
 template <typename T>
 bool use_loop(swe_mesh* m, int64_t nsteps) {
-    if (!m->loop_allowed || nsteps < 4) return false;
+    const bool graphs = nsteps >= m->cfg.graph_steps;
+    const int tuned = graphs ? m->loop_long : m->loop_short;
+    if (!m->loop_allowed || nsteps < 4 || tuned == 0) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return false; }
     if (cs != cudaStreamCaptureStatusNone) return false;
@@ -351,8 +353,8 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
             if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
         }
     }
-    const bool graphs = sizeof(T) == 4 && nsteps >= m->cfg.graph_steps;
-    return m->hm.n_cells <= (graphs ? m->loop_cells / 3 * 2 : m->loop_cells);
+    const bool fewer = sizeof(T) == 4 && graphs && tuned < 0;
+    return m->hm.n_cells <= (fewer ? m->loop_cells / 3 * 2 : m->loop_cells);
 }
 
 // Runs nsteps steps in the loop; on return nsteps is what is left of them.  Where
@@ -601,6 +603,18 @@ cudaError_t launch_raw_t(swe_mesh* m, const void* in, void* out, unsigned long l
     if (m->plain.pairs)
         return Launch<T>::step_pair(a, m->plain.block, m->plain.min_blocks, m->plain.geo, m->plain.stages, st);
     return Launch<T>::step(a, m->plain.block, m->plain.min_blocks, m->plain.stages, m->plain.geo, st);
+}
+
+int advance(swe_mesh* m, int64_t nsteps, double cfl) {
+    return m->cfg.precision == SWE_FP32 ? run_steps<float>(m, nsteps, cfl) : run_steps<double>(m, nsteps, cfl);
+}
+
+bool loop_possible(swe_mesh* m) {
+    const int was = m->loop_short;
+    m->loop_short = -1;
+    const bool can = m->cfg.precision == SWE_FP32 ? use_loop<float>(m, 4) : use_loop<double>(m, 4);
+    m->loop_short = was;
+    return can;
 }
 
 // One step of mesh m from buffer `in` to buffer `out` with the given status
@@ -1067,7 +1081,7 @@ int swe_step(swe_mesh* m, int64_t nsteps, double cfl, double* t_out) {
     DeviceGuard dg(m->cfg.device);
     int rc = flush_topo(m);
     if (rc) return rc;
-    rc = m->cfg.precision == SWE_FP32 ? run_steps<float>(m, nsteps, cfl) : run_steps<double>(m, nsteps, cfl);
+    rc = advance(m, nsteps, cfl);
     if (rc) return rc;
     if (t_out) {
         unsigned long long s[kSmallWords];

@@ -89,6 +89,10 @@ namespace swe {
 cudaError_t launch_step_raw(swe_mesh* m, const void* in, void* out, unsigned long long* small, int64_t step_index,
                             double cfl, const double* dt_fixed, double* dt_log, cudaStream_t st,
                             bool with_activity = false, void* eflux_out = nullptr, void* esrc_out = nullptr);
+// nsteps steps of m as swe_step makes them.
+int advance(swe_mesh* m, int64_t nsteps, double cfl);
+// Whether m may take the step loop (swe_loop.cuh) at all.
+bool loop_possible(swe_mesh* m);
 // Allocates (once) and fills the activity bytes of m's current state.
 int init_activity(swe_mesh* m);
 // Builds (once) the interior-edge list of the edge-pass step.
@@ -180,6 +184,9 @@ struct swe_mesh {
     // count and, FP64, its blocks' edges
     bool loop_allowed = false;
     long long loop_cells = -1, loop_cells_set = -1;   // (set: swe_debug_loop)
+    // whether calls shorter than a graph and the others take it, as the autotuner
+    // measured (-1: by the mesh's size)
+    int loop_short = -1, loop_long = -1;
     unsigned loop_polls = 0;           // polls after which a wait of the loop gives up
     int64_t loop_steps = 0;            // steps run in the loop
     unsigned* loop_barrier = nullptr;

@@ -17,7 +17,10 @@
 // again over at least 32 steps, and keeps the first of them in the fixed
 // candidate order within 1 % of the fastest there: short trials blur
 // differences of a few percent, and a tie keeps the same choice from run to
-// run.
+// run.  A mesh that may take the step loop (swe_loop.cuh) then makes calls of
+// 16 steps and of two graphs from its current state either way, in turn, and
+// takes the loop for the kind of call where it is the faster; its states and
+// status block are put back.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -132,6 +135,68 @@ void apply_shape(swe_mesh* m, const Shape& sh) {
         m->plain = LaunchShape{sh.block, sh.min_blocks, sh.stages, sh.geo_early, sh.edges, sh.grid, sh.pairs};
 }
 
+// Times m's calls with the step loop and without, from its current state, and
+// keeps the faster way for calls shorter than a graph and for the others.
+// Without device memory for copies of the states the choice stays by size.
+cudaError_t tune_loop(swe_mesh* m, size_t state_bytes) {
+    m->loop_short = m->loop_long = -1;
+    if (!loop_possible(m)) return cudaSuccess;
+    char* copy = nullptr;
+    const size_t small_bytes = kSmallWords * sizeof(unsigned long long);
+    if (cudaMalloc((void**)&copy, 2 * state_bytes + small_bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return cudaSuccess;
+    }
+    const int64_t nstep = m->nstep, loop_steps = m->loop_steps;
+    cudaStream_t st = m->stream;
+    void* const parts[3] = {m->state[0], m->state[1], m->small};
+    char* const copies[3] = {copy, copy + state_bytes, copy + 2 * state_bytes};
+    const size_t bytes[3] = {state_bytes, state_bytes, small_bytes};
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k)
+        e = cudaMemcpyAsync(copies[k], parts[k], bytes[k], cudaMemcpyDeviceToDevice, st);
+    auto put_back = [&]() {
+        for (int k = 0; k < 3 && e == cudaSuccess; ++k)
+            e = cudaMemcpyAsync(parts[k], copies[k], bytes[k], cudaMemcpyDeviceToDevice, st);
+        m->nstep = nstep;
+        m->act_valid = false;
+    };
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    for (auto& x : ev)
+        if (e == cudaSuccess) e = cudaEventCreate(&x);
+    const int graph = m->cfg.graph_steps;
+    int faster[2] = {-1, -1};
+    for (int kind = 0; kind < 2 && e == cudaSuccess; ++kind) {
+        const int64_t steps = kind ? 2 * graph : std::min(16, graph - 1);
+        double best[2] = {1e300, 1e300};
+        for (int r = 0; r < 6 && e == cudaSuccess; ++r)        // the first round warms up
+            for (int way = 0; way < 2 && e == cudaSuccess; ++way) {
+                put_back();
+                m->loop_short = m->loop_long = way;
+                // to a step index from which graphs replay, past the first step's work
+                if (e == cudaSuccess && advance(m, 6 - nstep % 6, 0.9) != SWE_OK) e = cudaErrorUnknown;
+                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+                if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
+                if (e == cudaSuccess && advance(m, steps, 0.9) != SWE_OK) e = cudaErrorUnknown;
+                if (e == cudaSuccess) e = cudaEventRecord(ev[1], st);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+                float t = 0.f;
+                if (e == cudaSuccess) e = cudaEventElapsedTime(&t, ev[0], ev[1]);
+                if (r > 0) best[way] = std::min(best[way], (double)t);
+            }
+        faster[kind] = best[1] <= best[0] ? 1 : 0;
+    }
+    put_back();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    for (auto& x : ev)
+        if (x) cudaEventDestroy(x);
+    cudaFree(copy);
+    m->loop_steps = loop_steps;
+    m->loop_short = e == cudaSuccess ? faster[0] : -1;
+    m->loop_long = e == cudaSuccess ? faster[1] : -1;
+    return e;
+}
+
 template <typename T>
 int autotune_t(swe_mesh* m, int trial_steps, swe_tune* out) {
     const int64_t n = m->hm.n_cells;
@@ -242,6 +307,7 @@ int autotune_t(swe_mesh* m, int trial_steps, swe_tune* out) {
     // previous step's bytes, which tell the next step whose state it may leave
     m->act_valid = false;
     drop_mesh_graph(m);
+    if (e == cudaSuccess) e = tune_loop(m, (size_t)n * sizeof(V4<T>));
     if (e != cudaSuccess) return tfail(e, "swe_autotune: trial steps");
     if (out) {
         out->block_size = pick.block;

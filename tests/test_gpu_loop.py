@@ -153,3 +153,29 @@ def test_long_calls_of_larger_fp32_meshes_replay_graphs():
             assert m.step(steps) == single.step(steps)
         assert m.debug_loop() == expect
         _equal(m, single)
+
+
+@pytest.mark.parametrize("precision,nx,ny", [(capi.SWE_FP64, 60, 12), (capi.SWE_FP32, 60, 12), (capi.SWE_FP64, 400, 29),
+                                             (capi.SWE_FP32, 500, 110)])
+def test_the_autotuner_chooses_between_the_loop_and_its_shape(precision, nx, ny):
+    mi = mg.river(nx, ny, seed=4, n_bumps=20)
+    m, single = _mesh(mi, precision), _mesh(mi, precision, graph_steps=-1)
+    shaped = _mesh(mi, precision, graph_steps=48)          # the tuned shape runs every step here
+    for x in (m, single, shaped):
+        x.step(37)
+    done = m.debug_loop()
+    for x in (m, shaped):
+        x.autotune(trial_steps=2)
+        _equal(x, single)                                  # the trials leave nothing behind
+    assert m.debug_loop() == done and shaped.debug_loop() == 0
+    for steps in (20, 101, 48, 5):
+        ref = single.step(steps)
+        for x in (m, shaped):
+            before = x.debug_loop()
+            assert x.step(steps) == ref
+            assert x.debug_loop() - before in (0, steps)   # a call runs in one way
+            _equal(x, single)
+    assert shaped.debug_loop() == 0
+    # on the smallest meshes the loop is the faster by a third and more
+    if nx == 60:
+        assert m.debug_loop() == done + 20 + 101 + 48 + 5

@@ -811,6 +811,7 @@ struct AdjArena {
                 return e;
             }
             m->adj_bytes = bytes;
+            m->device_bytes += (int64_t)bytes;
         }
         for (auto& q : parts) *q.first = (char*)m->adj_arena + q.second;
         return e;
@@ -1138,6 +1139,7 @@ int adjoint_impl(swe_mesh* m, int64_t nsteps, double cfl, const int32_t* gauge_c
 void swe::drop_adjoint_workspace(swe_mesh* m) {
     if (m->adj_arena) cudaFree(m->adj_arena);
     m->adj_arena = nullptr;
+    m->device_bytes -= (int64_t)m->adj_bytes;
     m->adj_bytes = 0;
 }
 

@@ -320,7 +320,9 @@ int build_loop_edges(swe_mesh* m) {
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_ecell, ecell.data(), ecell.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_egeo, egeo.data(), egeo.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_eslot, eslot.data(), eslot.size() * sizeof(uchar4), cudaMemcpyHostToDevice);
-    return e == cudaSuccess ? SWE_OK : cuda_fail(e, "swe_step: step loop");
+    if (e != cudaSuccess) return cuda_fail(e, "swe_step: step loop");
+    m->device_bytes += (int64_t)(ecell.size() * sizeof(int2) + egeo.size() * sizeof(double) + eslot.size() * sizeof(uchar4));
+    return SWE_OK;
 }
 
 // Whether the next steps run as one loop launch: a small mesh, nothing chosen
@@ -350,7 +352,8 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
         if (m->hm.n_cells <= cells && !m->loop_barrier) {
             bool ok = cudaMalloc((void**)&m->loop_barrier, sizeof(unsigned)) == cudaSuccess;
             if (ok && sizeof(T) == 8) ok = build_loop_edges(m) == SWE_OK;
-            if (!ok) { (void)cudaGetLastError(); m->loop_cells = 0; }
+            if (ok) m->device_bytes += sizeof(unsigned);
+            else { (void)cudaGetLastError(); m->loop_cells = 0; }
         }
     }
     const bool fewer = sizeof(T) == 4 && graphs && tuned < 0;
@@ -699,7 +702,7 @@ int build_edges(swe_mesh* m) {
     if (e == cudaSuccess && esz == 8 && E) e = cudaMemcpy(m->erl, rl.data(), E * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "edge pass: upload");
     m->n_edges = E;
-    m->device_bytes += (int64_t)(Eb * (sizeof(int2) + 7 * esz) + n * sizeof(int4));
+    m->device_bytes += (int64_t)(Eb * (sizeof(int2) + (esz == 8 ? 8 : 7) * esz) + n * sizeof(int4));
     return SWE_OK;
 }
 
@@ -729,7 +732,7 @@ static cudaError_t build_spans(swe_mesh* m) {
     if (e == cudaSuccess)
         e = cudaMemcpy(m->span_first, first.data(), first.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->span_adj, adj.data(), adj.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
-    m->device_bytes += (int64_t)((first.size() + adj.size()) * sizeof(unsigned));
+    if (e == cudaSuccess) m->device_bytes += (int64_t)((first.size() + adj.size()) * sizeof(unsigned));
     return e;
 }
 

@@ -194,6 +194,9 @@ int diag_workspace(swe_mesh* m) {
         return dfail(e, "swe_diagnostics: workspace");
     }
     m->diag_edge_group = groups;
+    m->diag_bytes = (int64_t)(words * sizeof(double) + kDiagMaxBlocks * kDiagWords * sizeof(double) +
+                              std::max<size_t>(nb, 1) * (sizeof(long long) + sizeof(int)));
+    m->device_bytes += m->diag_bytes;
     return SWE_OK;
 }
 
@@ -283,6 +286,8 @@ void drop_diag_workspace(swe_mesh* m) {
     m->diag_slots = nullptr;
     m->diag_groups = nullptr;
     m->diag_edge_group.clear();
+    m->device_bytes -= m->diag_bytes;
+    m->diag_bytes = 0;
 }
 
 }  // namespace swe

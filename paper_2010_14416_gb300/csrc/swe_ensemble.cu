@@ -504,7 +504,7 @@ int ens_init_activity(swe_ensemble* E) {
             return SWE_ENOMEM;
         }
         E->act_len = len;
-        E->device_bytes += 3 * all + (int64_t)(nf ? nf + na + (E->n_total + 2) * sizeof(unsigned) : 0);
+        E->device_bytes += 3 * all + (int64_t)(nf ? nf + na + (E->n_total + 2) * sizeof(unsigned) + E->n_members * sizeof(T) : 0);
     }
     const int p3 = (int)(E->nstep % 3);
     const int64_t all = E->act_len + ((E->n_total + (1 << kScanLog) - 1) >> kScanLog);

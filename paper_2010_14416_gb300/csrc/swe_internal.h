@@ -200,6 +200,7 @@ struct swe_mesh {
     double *diag_dev = nullptr, *diag_partial = nullptr, *diag_host = nullptr;
     long long* diag_slots = nullptr;
     int* diag_groups = nullptr;
+    int64_t diag_bytes = 0;
     std::vector<int> diag_edge_group;
     // reverse step of swe_adjoint: SWE_ADJOINT_TRANSPOSE or SWE_ADJOINT_DUAL
     int adjoint_method = SWE_ADJOINT_TRANSPOSE;

@@ -347,7 +347,8 @@ SWE_API int swe_run_to_steady(swe_mesh* mesh, double cfl, double tol, int64_t ch
  * (swe_adjoint_method).
  * Device memory: about (nsteps/checkpoint_every + checkpoint_every + 4) x 32 B per cell,
  * plus 64 B per interior edge and, with the edge pass, 40 B per interior edge
- * and step of a segment; the mesh keeps up to 1.5 GiB of it for its next call.
+ * and step of a segment; the mesh keeps up to 1.5 GiB of it for its next
+ * call, while all meshes of the process together keep no more than 6 GiB.
  * Errors: SWE_EINVAL (FP32 mesh, no state, bad gauge), SWE_ENOMEM, SWE_ECUDA,
  * SWE_ENONFINITE, SWE_EDRY, SWE_EMESH (debug checks).
  */

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -789,9 +790,21 @@ struct DevBuf {
 };
 
 // The buffers of one adjoint call, laid out in one allocation that the mesh
-// keeps (up to kAdjKeep) for its next call: allocating and freeing them took
-// 0.4 ms a call and more with the checkpoints' size.
-constexpr size_t kAdjKeep = (size_t)3 << 29;   // 1.5 GiB of the device's 280
+// keeps (up to kAdjKeep, all meshes of the process together up to kAdjKeepAll)
+// for its next call: allocating and freeing them took 0.4 ms a call and more
+// with the checkpoints' size.
+constexpr size_t kAdjKeep = (size_t)3 << 29;      // 1.5 GiB of the device's 280
+constexpr size_t kAdjKeepAll = (size_t)6 << 30;   // 6 GiB
+std::atomic<size_t> adj_kept_all{0};
+bool keep_arena(swe_mesh* m) {
+    if (m->adj_kept) return true;   // counted
+    size_t all = adj_kept_all.load();
+    do {
+        if (m->adj_bytes > kAdjKeep || all + m->adj_bytes > kAdjKeepAll) return false;
+    } while (!adj_kept_all.compare_exchange_weak(all, all + m->adj_bytes));
+    m->adj_kept = m->adj_bytes;
+    return true;
+}
 struct AdjArena {
     swe_mesh* m;
     std::vector<std::pair<void**, size_t>> parts;   // (pointer, offset)
@@ -820,7 +833,7 @@ struct AdjArena {
     // mesh may change its stream before the next)
     ~AdjArena() {
         cudaStreamSynchronize(m->stream);
-        if (m->adj_bytes > kAdjKeep) drop_adjoint_workspace(m);
+        if (!keep_arena(m)) drop_adjoint_workspace(m);
     }
 };
 
@@ -1140,7 +1153,8 @@ void swe::drop_adjoint_workspace(swe_mesh* m) {
     if (m->adj_arena) cudaFree(m->adj_arena);
     m->adj_arena = nullptr;
     m->device_bytes -= (int64_t)m->adj_bytes;
-    m->adj_bytes = 0;
+    adj_kept_all -= m->adj_kept;
+    m->adj_bytes = m->adj_kept = 0;
 }
 
 extern "C" {

@@ -195,7 +195,7 @@ struct swe_mesh {
     uchar4* loop_eslot = nullptr;
     // adjoint workspace (swe_adjoint.cu), kept between calls
     void* adj_arena = nullptr;
-    size_t adj_bytes = 0;
+    size_t adj_bytes = 0, adj_kept = 0;   // (kept: counted among all meshes)
     // diagnostics workspace (swe_diag.cu)
     double *diag_dev = nullptr, *diag_partial = nullptr, *diag_host = nullptr;
     long long* diag_slots = nullptr;

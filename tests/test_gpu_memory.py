@@ -49,3 +49,29 @@ def test_kept_buffers_are_reported():
     m.set_bc(mi.bcs[1][0], mg.BC_WALL)                # the boundary edges' groups change
     assert _held(m) - base == loop + kept
     m.close()
+
+
+def test_meshes_together_keep_a_bounded_adjoint_workspace():
+    # six meshes whose workspaces take 48 steps of 32 B a cell and 40 B an edge,
+    # 1.04 GiB, and some more each: the process keeps 6 GiB
+    # at most, gives back the others after each call, and a mesh that is closed
+    # makes room; the results do not depend on it
+    mi = mg.river(1000, 126, seed=4, n_bumps=20)
+    before = torch.cuda.mem_get_info()[0]
+    meshes, kept, first = [], [], None
+    for k in range(6):
+        m = _mesh(mi)
+        base = _held(m)
+        out = m.adjoint(48, [5, 700], [1.0, 2.0])
+        kept.append(_held(m) - base)
+        first = first or out
+        assert out[0] == first[0] and all(np.array_equal(a, b) for a, b in zip(out[1:], first[1:]))
+        meshes.append(m)
+    assert kept[0] > 48 * 90 * mi.n_cells and sum(kept) <= 6 * 2**30 and kept[-1] == 0
+    meshes[0].close()
+    base = _held(meshes[-1])
+    meshes[-1].adjoint(48, [5, 700], [1.0, 2.0])
+    assert _held(meshes[-1]) - base == kept[0]
+    for m in meshes:
+        m.close()
+    assert torch.cuda.mem_get_info()[0] > before - 2**28

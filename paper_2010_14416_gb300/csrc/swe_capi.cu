@@ -320,7 +320,14 @@ int build_loop_edges(swe_mesh* m) {
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_ecell, ecell.data(), ecell.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_egeo, egeo.data(), egeo.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->loop_eslot, eslot.data(), eslot.size() * sizeof(uchar4), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, "swe_step: step loop");
+    if (e != cudaSuccess) {
+        for (void* p : {(void*)m->loop_ecell, (void*)m->loop_egeo, (void*)m->loop_eslot})
+            if (p) cudaFree(p);
+        m->loop_ecell = nullptr;
+        m->loop_egeo = nullptr;
+        m->loop_eslot = nullptr;
+        return cuda_fail(e, "swe_step: step loop");
+    }
     m->device_bytes += (int64_t)(ecell.size() * sizeof(int2) + egeo.size() * sizeof(double) + eslot.size() * sizeof(uchar4));
     return SWE_OK;
 }
@@ -351,9 +358,20 @@ bool use_loop(swe_mesh* m, int64_t nsteps) {
         m->loop_cells = cells;
         if (m->hm.n_cells <= cells && !m->loop_barrier) {
             bool ok = cudaMalloc((void**)&m->loop_barrier, sizeof(unsigned)) == cudaSuccess;
-            if (ok && sizeof(T) == 8) ok = build_loop_edges(m) == SWE_OK;
-            if (ok) m->device_bytes += sizeof(unsigned);
-            else { (void)cudaGetLastError(); m->loop_cells = 0; }
+            try {
+                if (ok && sizeof(T) == 8) ok = build_loop_edges(m) == SWE_OK;
+            } catch (const std::bad_alloc&) {
+                ok = false;
+            }
+            if (ok) {
+                m->device_bytes += sizeof(unsigned);
+            } else {   // the steps are launched one by one, then
+                (void)cudaGetLastError();
+                if (m->loop_barrier) cudaFree(m->loop_barrier);
+                m->loop_barrier = nullptr;
+                m->loop_allowed = false;
+                return false;
+            }
         }
     }
     const bool fewer = sizeof(T) == 4 && graphs && tuned < 0;
@@ -663,8 +681,7 @@ void append_edges(const HostMesh& H, int64_t base, std::vector<int2>& cells, std
         }
 }
 
-int build_edges(swe_mesh* m) {
-    if (m->eflux) return SWE_OK;
+static int upload_edges(swe_mesh* m) {
     const HostMesh& H = m->hm;
     const int64_t n = H.n_cells;
     std::vector<int2> cells;
@@ -706,6 +723,16 @@ int build_edges(swe_mesh* m) {
     return SWE_OK;
 }
 
+int build_edges(swe_mesh* m) {
+    if (m->eflux) return SWE_OK;
+    try {
+        return upload_edges(m);
+    } catch (const std::bad_alloc&) {   // before any device allocation
+        set_error("edge pass: out of host memory");
+        return SWE_ENOMEM;
+    }
+}
+
 // The spans (2^kScanLog cells) beside each span: those with an edge in common,
 // and itself.
 static cudaError_t build_spans(swe_mesh* m) {
@@ -743,7 +770,11 @@ int init_activity(swe_mesh* m) {
         const int64_t len = (n + 31) / 32 * 32 + 32;   // bytes, then a flag per span
         const int64_t all = len + ((n + (1 << kScanLog) - 1) >> kScanLog);
         for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMalloc((void**)&m->act[k], all);
-        if (e == cudaSuccess) e = build_spans(m);
+        try {
+            if (e == cudaSuccess) e = build_spans(m);
+        } catch (const std::bad_alloc&) {
+            e = cudaErrorMemoryAllocation;
+        }
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_list, n * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMalloc((void**)&m->act_count, 2 * sizeof(unsigned));
         if (e == cudaSuccess) e = cudaMemsetAsync(m->act_count, 0, 2 * sizeof(unsigned), m->stream);
@@ -754,7 +785,7 @@ int init_activity(swe_mesh* m) {
             for (auto& p : m->act) p = nullptr;
             m->span_first = m->span_adj = nullptr;
             m->act_list = m->act_count = nullptr;
-            set_error("activity bytes: device allocation failed");
+            set_error("activity bytes: allocation failed");
             return SWE_ENOMEM;
         }
         m->act_len = len;

@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -173,11 +174,16 @@ int diag_workspace(swe_mesh* m) {
     if (m->diag_dev) return SWE_OK;
     std::vector<long long> slots;
     std::vector<int> groups;
-    for (int64_t s = 0; s < 3 * m->hm.n_cells; ++s)   // (internal cell, local edge)
-        if (m->hm.code[s] < 0) {
-            slots.push_back(s);
-            groups.push_back(-1 - m->hm.code[s]);
-        }
+    try {
+        for (int64_t s = 0; s < 3 * m->hm.n_cells; ++s)   // (internal cell, local edge)
+            if (m->hm.code[s] < 0) {
+                slots.push_back(s);
+                groups.push_back(-1 - m->hm.code[s]);
+            }
+    } catch (const std::bad_alloc&) {
+        set_error("swe_diagnostics: out of host memory");
+        return SWE_ENOMEM;
+    }
     const size_t nb = slots.size(), words = kDiagWords + kSmallWords + nb;
     cudaError_t e = cudaMalloc((void**)&m->diag_dev, words * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&m->diag_host, words * sizeof(double));
@@ -193,7 +199,7 @@ int diag_workspace(swe_mesh* m) {
         drop_diag_workspace(m);
         return dfail(e, "swe_diagnostics: workspace");
     }
-    m->diag_edge_group = groups;
+    m->diag_edge_group.swap(groups);
     m->diag_bytes = (int64_t)(words * sizeof(double) + kDiagMaxBlocks * kDiagWords * sizeof(double) +
                               std::max<size_t>(nb, 1) * (sizeof(long long) + sizeof(int)));
     m->device_bytes += m->diag_bytes;

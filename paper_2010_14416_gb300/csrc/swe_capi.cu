@@ -180,7 +180,7 @@ int flush_topo(swe_mesh* m) {
     }
     m->topo_dirty = false;
     m->act_valid = false;   // static activity may have changed
-    drop_diag_workspace(m);   // the boundary edges' groups
+    m->diag_groups_old = true;
     drop_graph(m);
     return SWE_OK;
 }

@@ -168,10 +168,21 @@ struct DiagDeviceGuard {
 
 // The mesh's diagnostics workspace: device words [results | status block | q of
 // the boundary edges], their pinned host copy, and the boundary edges (slot,
-// group) in a fixed order.  Laid out on the first call and after a change of
-// boundary groups.
+// group) in a fixed order.  Laid out on the first call; a change of boundary
+// groups renews the groups.
 int diag_workspace(swe_mesh* m) {
-    if (m->diag_dev) return SWE_OK;
+    if (m->diag_dev) {
+        if (!m->diag_groups_old) return SWE_OK;
+        const size_t nb = m->diag_edge_group.size();
+        for (size_t k = 0; k < nb; ++k) m->diag_edge_group[k] = -1 - m->hm.code[m->diag_edge[k]];
+        if (nb) {
+            const cudaError_t e = cudaMemcpyAsync(m->diag_groups, m->diag_edge_group.data(), nb * sizeof(int),
+                                                  cudaMemcpyHostToDevice, m->stream);
+            if (e != cudaSuccess) return dfail(e, "swe_diagnostics: boundary groups");
+        }
+        m->diag_groups_old = false;
+        return SWE_OK;
+    }
     std::vector<long long> slots;
     std::vector<int> groups;
     try {
@@ -200,6 +211,8 @@ int diag_workspace(swe_mesh* m) {
         return dfail(e, "swe_diagnostics: workspace");
     }
     m->diag_edge_group.swap(groups);
+    m->diag_edge.swap(slots);
+    m->diag_groups_old = false;
     m->diag_bytes = (int64_t)(words * sizeof(double) + kDiagMaxBlocks * kDiagWords * sizeof(double) +
                               std::max<size_t>(nb, 1) * (sizeof(long long) + sizeof(int)));
     m->device_bytes += m->diag_bytes;
@@ -292,6 +305,7 @@ void drop_diag_workspace(swe_mesh* m) {
     m->diag_slots = nullptr;
     m->diag_groups = nullptr;
     m->diag_edge_group.clear();
+    m->diag_edge.clear();
     m->device_bytes -= m->diag_bytes;
     m->diag_bytes = 0;
 }

@@ -201,7 +201,9 @@ struct swe_mesh {
     long long* diag_slots = nullptr;
     int* diag_groups = nullptr;
     int64_t diag_bytes = 0;
+    std::vector<long long> diag_edge;   // the boundary edges and their groups
     std::vector<int> diag_edge_group;
+    bool diag_groups_old = false;       // the groups have changed since
     // reverse step of swe_adjoint: SWE_ADJOINT_TRANSPOSE or SWE_ADJOINT_DUAL
     int adjoint_method = SWE_ADJOINT_TRANSPOSE;
 };

@@ -81,3 +81,25 @@ def test_run_to_steady_state_balances_inflow_and_outflow():
     assert q_in == pytest.approx(30.0, rel=1e-12)
     assert q_out == pytest.approx(q_in, rel=1e-3)
     m.close()
+
+
+@pytest.mark.parametrize("precision", [capi.SWE_FP64, capi.SWE_FP32])
+def test_boundary_changes_between_diagnostics(precision):
+    # each change of groups shows in the next diagnostics, as on a mesh that had
+    # them from the start
+    mi = mg.river(160, 32, seed=5)
+    m, _ = _pair(mi, precision)
+    m.diagnostics()
+    for q in (500.0, 900.0):
+        m.set_bc(mi.bcs[0][0], mg.BC_INFLOW, q)
+        d = m.diagnostics()
+        assert d["discharge"][-1] == pytest.approx(-q, rel=1e-6) and d["discharge"][1] == 0.0
+    m.set_bc(mi.bcs[1][0], mg.BC_WALL)
+    d = m.diagnostics()
+    fresh, _ = _pair(mi, precision)
+    for pairs, kind, value in ((mi.bcs[0][0], mg.BC_INFLOW, 500.0), (mi.bcs[0][0], mg.BC_INFLOW, 900.0),
+                               (mi.bcs[1][0], mg.BC_WALL, 0.0)):
+        fresh.set_bc(pairs, kind, value)
+    assert np.array_equal(d["discharge"], fresh.diagnostics()["discharge"]) and d["n_groups"] == 6
+    m.close()
+    fresh.close()

@@ -130,21 +130,22 @@ template <typename T>
 int upload_static(swe_mesh* m) {
     const HostMesh& H = m->hm;
     const int64_t n = H.n_cells;
-    std::vector<V4<T>> A(n), B(n), R(n);
+    std::vector<V4<T>> A(n), B(n), R(sizeof(T) == 8 ? n : 0);
     std::vector<T> gm2(n), zt(n);
     std::vector<unsigned> perm(n), inv(n);
     const std::vector<int4> topo = make_topo(m);
     for (int64_t c = 0; c < n; ++c) {
-        double ln[6], len[3] = {0.0, 0.0, 0.0};
-        for (int j = 0; j < 3; ++j) {
-            ln[2 * j] = H.ln[6 * c + 2 * j];
-            ln[2 * j + 1] = H.ln[6 * c + 2 * j + 1];
-            if (sizeof(T) == 8) len[j] = host_unit_normal(ln[2 * j], ln[2 * j + 1]);
+        double ln[6];
+        std::memcpy(ln, &H.ln[6 * c], sizeof ln);
+        if (sizeof(T) == 8) {
+            R[c].x = (T)host_unit_normal(ln[0], ln[1]);
+            R[c].y = (T)host_unit_normal(ln[2], ln[3]);
+            R[c].z = (T)host_unit_normal(ln[4], ln[5]);
+            R[c].w = (T)0;
         }
         A[c].x = (T)ln[0]; A[c].y = (T)ln[1];
         A[c].z = (T)ln[2]; A[c].w = (T)ln[3];
         B[c].x = (T)ln[4]; B[c].y = (T)ln[5];
-        R[c].x = (T)len[0]; R[c].y = (T)len[1]; R[c].z = (T)len[2]; R[c].w = (T)0;
         B[c].z = (T)H.inv_area[c]; B[c].w = (T)H.rin[c];
         gm2[c] = (T)(m->cfg.g * H.m[c] * H.m[c]);
         zt[c] = (T)H.z[c];

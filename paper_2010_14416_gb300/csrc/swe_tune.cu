@@ -169,7 +169,7 @@ cudaError_t tune_loop(swe_mesh* m, size_t state_bytes) {
     for (int kind = 0; kind < 2 && e == cudaSuccess; ++kind) {
         const int64_t steps = kind ? 2 * graph : std::min(16, graph - 1);
         double best[2] = {1e300, 1e300};
-        for (int r = 0; r < 6 && e == cudaSuccess; ++r)        // the first round warms up
+        for (int r = 0; r < 4 && e == cudaSuccess; ++r)        // the first round warms up
             for (int way = 0; way < 2 && e == cudaSuccess; ++way) {
                 put_back();
                 m->loop_short = m->loop_long = way;

@@ -7,16 +7,19 @@
 // lambda^N = dL/dU^N, accumulating dL/dz and dL/dm on the way.  Cell i's
 // update is U_i + Phi(U_i, m_i, R_i), R_i = (1/|Omega_i|) sum_e E_ie, where
 // E_ie is the edge's flux-and-bed-source contribution (Eq 13, 30, 37).  One
-// reverse step is two gathers, no atomics:
-//   phase 1 (cell i): recompute R_i; differentiate Phi on 7-component duals
-//     (h, hu, hv, g m^2, R) -> own term a_i, dL/dm_i, nu_i = (dPhi/dR)^T lambda / |Omega_i|
-//   phase 2 (cell j): differentiate each edge term E_je and the neighbour's
-//     E_ie on 4-component duals (h_j, hu_j, hv_j, z_j):
+// reverse step, without atomics:
+//   phase 1 (cell i): R_i again, from the edge terms that the forward kept or
+//     inline; the transpose of Phi -> own term a_i, dL/dm_i,
+//     nu_i = (dPhi/dR)^T lambda / |Omega_i|
+//   phase 2:
 //     lambda^n_j = a_j + sum_e (dE_je)^T nu_j + (dE_ie)^T nu_i,  dL/dz_j likewise.
-// Both phases run the forward's own templated edge and friction functions,
-// so the derivatives are those of the branches the forward takes.
-// States are recomputed segment by segment from checkpoints taken every k
-// steps of the forward run.
+// By default the transposes are written out by hand and phase 2 takes each
+// interior edge once for both of its cells, then sums a cell's edges in the
+// same kernel as the step before's phase 1.  SWE_ADJOINT_DUAL differentiates
+// the forward's formulas on dual numbers instead (seven components for Phi,
+// four for an edge, from both cells), as a check.  Either follows the branches
+// that the forward takes.  Where the states of all steps do not fit, they are
+// recomputed segment by segment from checkpoints.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -95,14 +95,6 @@ struct Ar<Dual<N>> {
         for (int j = 0; j < N; ++j) r.d[j] = k * x.d[j];
         return r;
     }
-    static __device__ __forceinline__ D rsqrt_(const D& x) {
-        D r;
-        r.v = 1.0 / sqrt(x.v);
-        const double k = -0.5 * r.v / x.v;
-#pragma unroll
-        for (int j = 0; j < N; ++j) r.d[j] = k * x.d[j];
-        return r;
-    }
     static __device__ __forceinline__ D div_(const D& a, const D& b) { return a / b; }
     static __device__ __forceinline__ D rcp_(const D& x) { return D(1.0) / x; }
     static __device__ __forceinline__ D pow_m73(const D& h) {

@@ -185,23 +185,19 @@ struct EnsArgs {
 // ---- precision-specific arithmetic ------------------------------------------------
 // The FP32 instantiation is compiled with fast-math: division, reciprocal and
 // square root map to the hardware approximations (a few ulp), which the
-// 1e-4 FP32 tolerance absorbs.  The FP64 instantiation keeps IEEE division
-// and square root.
+// 1e-4 FP32 tolerance absorbs.  The double one (IEEE division and square root)
+// serves the first CFL step of a state; the FP64 steps have their own
+// arithmetic (swe_f64.cuh).
 template <typename T> struct Ar;
 template <> struct Ar<float> {
     static __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
-    static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
     static __device__ __forceinline__ float div_(float a, float b) { return __fdividef(a, b); }
     static __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
-    // h^(-7/3) through the hardware base-2 exp/log pair
-    static __device__ __forceinline__ float pow_m73(float h) { return exp2f(-7.0f / 3.0f * __log2f(h)); }
 };
 template <> struct Ar<double> {
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-    static __device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
     static __device__ __forceinline__ double div_(double a, double b) { return a / b; }
     static __device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
-    static __device__ __forceinline__ double pow_m73(double h) { return 1.0 / (h * h * cbrt(h)); }
 };
 
 // h^(-1/3) in double, for the friction factor h^(-7/3) = r^7 and 1/h = r^3
@@ -2003,7 +1999,7 @@ __global__ void riemann_batch_kernel(long long n, const T* __restrict__ hL, cons
 // instruction holds its SM quarter for 64 clocks, four quarters together reach
 // one per 19, so warps should be spread evenly (4,000 cells: 9,663 -> 9,134 us
 // for 500 steps).  FP32 steps measured the same to 2 % slower with it.
-constexpr long long kSpreadCells = 152LL * 12 * 32;   // 12 one-warp blocks per SM
+constexpr long long kSpreadCells = 152LL * 12 * 32;   // 12 one-warp blocks on each of GB300's 152 SMs
 template <typename T>
 __host__ __device__ inline unsigned step_threads(long long n, unsigned grid, int block) {
     if (sizeof(T) == 4) return (unsigned)block;

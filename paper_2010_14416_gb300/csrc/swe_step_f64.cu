@@ -1,4 +1,4 @@
-// FP64 instantiation of the step kernels (IEEE division and square root).
+// FP64 instantiation of the step kernels (arithmetic: swe_f64.cuh).
 #include "swe_launch.cuh"
 
 namespace swe {

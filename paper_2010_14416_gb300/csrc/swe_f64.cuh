@@ -389,12 +389,13 @@ __device__ __forceinline__ void riemann_any(double hL, double unL, double utL, d
                                             double g2, double h_dry, double& G1, double& G2, double& G3, double* speeds,
                                             bool hll_only) {
     double PL, PR;
+    const bool g_ok = __double2hiint(g2) >= 0;   // (roots of negative numbers: NaN in Rare only)
     if (in_range<-64, 24>(hL) && in_range<-64, 24>(hR) && in_range<-100, 40>(unL) && in_range<-100, 40>(utL) &&
-        in_range<-100, 40>(unR) && in_range<-100, 40>(utR) && in_range<-64, 24>(g2)) {
+        in_range<-100, 40>(unR) && in_range<-100, 40>(utR) && in_range<-64, 24>(g2) && g_ok) {
         riemann<Soft>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
     } else if (in_range<-200, 100>(hL) && in_range<-200, 100>(hR) && in_range<-400, 100>(unL) &&
                in_range<-400, 100>(utL) && in_range<-400, 100>(unR) && in_range<-400, 100>(utR) &&
-               in_range<-64, 64>(g2)) {
+               in_range<-64, 64>(g2) && g_ok) {
         riemann<Hard>(hL, unL, utL, hR, unR, utR, g2, h_dry, G1, G2, G3, PL, PR, speeds, hll_only);
     } else {
         const FluxAndSpeeds r = riemann_rare(hL, unL, utL, hR, unR, utR, g2, h_dry, hll_only);

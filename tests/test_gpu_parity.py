@@ -802,3 +802,26 @@ def test_riemann_flux_far_from_any_flow_fp64():
         assert np.all(np.abs(gs - ref_s) <= (1e-13 + root) * 4 * c), (s, gs, ref_s)
         scale = np.array([h * c, h * c * c, h * c * c], np.longdouble)
         assert np.all(np.abs(gg - ref_g) <= 1e-13 * 4 * scale + 1e-320), (s, gg, ref_g)
+
+
+@pytest.mark.parametrize("flux", [capi.SWE_FLUX_HLLC, capi.SWE_FLUX_HLL])
+def test_riemann_flux_without_gravity_fp64(flux):
+    # the flux alone takes any g.  Without gravity the wave speeds are the
+    # velocities (no star depth exists where they converge, and none is needed);
+    # negative g has no wave speeds: NaN, not a number that looks like a flux
+    st = [(1.0, -1.0, 2.0, 3.0, 0.5, -1.0), (2.0, 1.0, 0.5, 1.0, 2.0, 0.25), (1.0, -3.0, 0.5, 2.0, -1.0, 4.0),
+          (1.0, 1.0, 0.0, 2.0, -1.0, 0.0), (4.0, -0.5, 1.0, 0.25, -2.0, 1.0)]
+    dev = [torch.tensor(c, dtype=torch.float64, device="cuda") for c in zip(*st)]
+    G = [torch.empty(len(st), dtype=torch.float64, device="cuda") for _ in range(3)]
+    for g in (0.0, -9.81):
+        capi.riemann_flux(capi.SWE_FP64, *dev, *G, g=g, flux=flux)
+        got = torch.stack(G, 1).cpu().numpy()
+        for k, (hL, uL, vL, hR, uR, vR) in enumerate(st):
+            if g < 0.0:
+                assert np.all(np.isnan(got[k])), (g, st[k], got[k])
+                continue
+            FL, FR = [np.array([h * u, h * u * u, h * u * v]) for h, u, v in ((hL, uL, vL), (hR, uR, vR))]
+            dU = np.array([hR - hL, hR * uR - hL * uL, hR * vR - hL * vL])
+            F = FL if uL >= 0.0 else (FR if uR <= 0.0 else (uR * FL - uL * FR + uL * uR * dU) / (uR - uL))
+            n = 3 if flux == capi.SWE_FLUX_HLL else 2   # (HLLC: S* is 0/0 here, either side's tangential velocity)
+            assert np.allclose(got[k][:n], F[:n], rtol=1e-14, atol=1e-14), (st[k], got[k], F)

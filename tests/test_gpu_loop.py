@@ -179,3 +179,19 @@ def test_the_autotuner_chooses_between_the_loop_and_its_shape(precision, nx, ny)
     # on the smallest meshes the loop is the faster by a third and more
     if nx == 60:
         assert m.debug_loop() == done + 20 + 101 + 48 + 5
+
+
+def test_no_loop_on_larger_meshes_nor_under_capture():
+    large = _mesh(mg.river(700, 110, seed=2, n_bumps=10), capi.SWE_FP32)   # 154,000 cells
+    large.step(20)
+    assert large.debug_loop() == 0
+    m = _mesh(mg.river(60, 12, seed=4, n_bumps=20), capi.SWE_FP64)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    m.set_stream(stream)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        m.step(6, sync=False)
+    assert m.debug_loop() == 0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert m.info()["status"] == 0
